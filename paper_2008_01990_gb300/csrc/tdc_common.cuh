@@ -496,6 +496,8 @@ cudaError_t launch_cauchy_like_prep(int64_t m, int64_t n, const double* A, int64
                                     const double* w, const double* u, const double* v, int32_t* org, double* tau,
                                     double* scol, int32_t* eb, int32_t* cexp, int32_t* eA,
                                     unsigned long long* maxsq, bool scale, cudaStream_t s);
+cudaError_t launch_row_max(int64_t m, int64_t n, const double* A, int64_t lda, unsigned long long* maxsq,
+                           cudaStream_t s);
 cudaError_t launch_cauchy_like_patch(GemmSeg* seg, const int32_t* eA, cudaStream_t s);
 cudaError_t launch_seg_dense(const GemmSeg& seg, cudaStream_t s);
 cudaError_t launch_struct(const GemmSeg* segs, int nseg, const StructArgs& A, cudaStream_t s);
