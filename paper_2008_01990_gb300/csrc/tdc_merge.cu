@@ -1,8 +1,9 @@
 // tdc_merge.cu -- the merge step of Cuppen's divide and conquer on the GPU,
 // level by level over every node of every problem in the plan:
 //   k_dmod      corner modification of the split points (Eq. (T2))
-//   k_leaf      leaf eigensolves (Algorithm 1, "QR"): two warps per leaf, or
-//   k_leaf_multi  a lane per leaf for leaves of at most 32 rows
+//   k_leaf      leaf eigensolves (Algorithm 1, "QR"): two warps per leaf;
+//   k_leaf_rows   rows in the registers of a few lanes, for leaves of at most 32 rows;
+//   k_leaf_multi  a lane per leaf for many leaves of 17 to 32 rows
 //   k_prepare   z (Eq. (T3)) from the children's boundary rows, merge of the
 //               two sorted spectra, deflation scan (Section 3.2, Eq. (T3-def)),
 //               compaction
@@ -20,6 +21,8 @@
 //   k_sign_out  sign convention and eigenvalue output
 #include <float.h>
 #include <math.h>
+
+#include <utility>
 
 #include "tdc_common.cuh"
 
@@ -278,13 +281,216 @@ __global__ void __launch_bounds__(64) k_leaf(Plan P, int64_t nleaves) {
   }
 }
 
+// Leaves of at most LM = 8, 16 or 32 rows: GL = LM / R lanes per leaf, each holding R rows
+// of the eigenvector block, and all of the leaf's d and e, in registers.  Every lane of a
+// leaf runs the same implicit QL/QR chase (the recurrence of EISPACK's imtql2, run from the
+// top) and applies each rotation to its own rows at once, so a leaf needs no shared memory,
+// no barrier and no hand-over of rotations.  Bound by FP64 issue: an FP64 warp instruction
+// holds its quarter of the SM for 64 clocks (measured, whatever the number of active lanes),
+// and a rotation takes 19 of them for the chase and 4 R for the rows.  With few leaves R = 1
+// is shortest (the leaves spread over the SMs), with many a larger R shares a chase among
+// more leaves of the warp.  64 leaves of 16 rows: 1393 -> 415 us.
+// f(0), ..., f(N-1) with the index a compile-time constant in each call, so that register
+// arrays indexed by it are scalars from the start (an unrolled loop with tests on a runtime
+// k was turned back into indexed accesses of local memory)
+template <class F, int... I>
+__device__ __forceinline__ void static_for_impl(F&& f, std::integer_sequence<int, I...>) {
+  (f(std::integral_constant<int, I>()), ...);
+}
+template <int N, class F>
+__device__ __forceinline__ void static_for(F&& f) {
+  static_for_impl(f, std::make_integer_sequence<int, N>());
+}
+
+// Helpers of the chase: a warp's FP64 instructions go through its quarter of the SM one per
+// 64 clocks (measured, dependent or not, and a comparison counts as one), so what integer
+// instructions can do they do.  in_range: 2^-960 <= x < 2^960 for x >= 0; twice(x) = 2 x
+// by the exponent field; rsqrt_cubic: the hardware estimate y (error e of
+// 1 - x y^2 near 2^-20) refined once to y (1 + e/2 + 3 e^2 / 8), which leaves 5 e^3 / 16.
+__device__ __forceinline__ bool in_range(double x) {
+  const unsigned ex = (unsigned)__double2hiint(x) >> 20;
+  return ex >= 63u && ex < 1983u;
+}
+__device__ __forceinline__ double twice(double x) {
+  const int h = __double2hiint(x);
+  if ((h & 0x7ff00000) == 0) return x + x;
+  return __hiloint2double(h + 0x100000, __double2loint(x));
+}
+__device__ __forceinline__ double rsqrt_cubic(double x) {
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  const double e = fma(-(x * y), y, 1.0);
+  return fma(y * e, fma(0.375, e, 0.5), y);
+}
+
+template <int LM, int R, int NL>
+__global__ void __launch_bounds__(32) k_leaf_rows(Plan P, int64_t nleaves) {
+  constexpr int GL = LM / R;  // lanes per leaf; NL leaves per warp
+  static_assert(NL * GL <= 32, "leaves of a warp");
+  __shared__ double s_d[NL][LM];
+  __shared__ int s_rank[NL][LM];
+  const int lane = threadIdx.x, slot = lane / GL, gl = lane % GL;
+  // spare lanes (NL GL < 32) follow a leaf of the warp, so that its branches stay uniform
+  const int64_t gid = (int64_t)blockIdx.x * NL + slot % NL;
+  const bool live = gid < nleaves, writes = live && slot < NL;
+  int pi = 0, L = 0;
+  int64_t lo = 0;
+  if (live) {
+    int x = 0, y = P.nprob - 1;
+    while (x < y) {
+      const int m = (x + y + 1) >> 1;
+      if (P.prob[m].leaf0 <= gid) x = m; else y = m - 1;
+    }
+    pi = x;
+    const Problem& pr = P.prob[pi];
+    lo = node_bound(gid - pr.leaf0, pr.n, pr.depth);
+    L = (int)(node_bound(gid - pr.leaf0 + 1, pr.n, pr.depth) - lo);
+  }
+  const Problem& pr = P.prob[pi];
+  double d[LM], e[LM], z[R][LM];
+#pragma unroll
+  for (int k = 0; k < LM; ++k) {
+    d[k] = k < L ? P.v.dmod[pr.voff + lo + k] : 0.0;
+    e[k] = k < L - 1 ? input_entry(P.e[pr.off_de + lo + k], pr.escale) : 0.0;
+#pragma unroll
+    for (int i = 0; i < R; ++i) z[i][k] = (gl + i * GL == k) ? 1.0 : 0.0;
+  }
+  const int max_sweeps = 40 * LM;
+  for (int sweep = 0;; ++sweep) {
+    // negligible off-diagonals, |e_k| <= eps (|d_k| + |d_k+1|): by the exponents first (e_k
+    // above 2^-50 of the larger of the two is not), in FP64 only where those leave it open
+    unsigned nz = 0;
+    static_for<LM - 1>([&](auto kc) {
+      constexpr int k = kc.value;
+      const int xe = (__double2hiint(e[k]) >> 20) & 0x7ff;
+      const int xd = max((__double2hiint(d[k]) >> 20) & 0x7ff, (__double2hiint(d[k + 1]) >> 20) & 0x7ff);
+      bool neg = false;
+      if (xe < xd - 50 || xe == 0) neg = fabs(e[k]) <= kEps * (fabs(d[k]) + fabs(d[k + 1]));
+      if (neg) e[k] = 0.0; else nz |= 1u << k;
+    });
+    if (sweep >= max_sweeps && nz) {
+      nz = 0;
+      set_status(P.status, TDC_ENOCONV);
+    }
+    if (!__any_sync(0xffffffffu, nz != 0)) break;
+    int pp = 0, q = 0;
+    double mu = 0.0;
+    if (nz) {  // trailing unreduced block [pp, q]: e[q-1] != 0, e[q..] == 0
+      q = 32 - __clz(nz);
+      const unsigned below = ~nz & ((1u << (q - 1)) - 1u);
+      pp = below ? 32 - __clz(below) : 0;
+      // Wilkinson shift: eigenvalue of the trailing 2 x 2 block nearer to d[q]
+      double dq = 0.0, dq1 = 0.0, bq = 0.0;
+      static_for<LM - 1>([&](auto kc) {
+        constexpr int k = kc.value;
+        if (k == q - 1) {
+          dq1 = d[k];
+          dq = d[k + 1];
+          bq = e[k];
+        }
+      });
+      const double hd = 0.5 * (dq1 - dq);
+      const double t2 = fma(hd, hd, bq * bq);
+      if (in_range(t2)) {
+        const double hh = t2 * rsqrt_cubic(t2);
+        mu = dq - bq * bq * rcp_nr(hd + copysign(hh, hd));
+      } else {
+        const double hh = hypot(hd, bq);
+        mu = dq - bq * (bq / (hd + copysign(hh, hd)));
+      }
+    }
+    double c = 1.0, sn = 1.0, g = 0.0, pv = 0.0;
+    static_for<LM - 1>([&](auto kc) {
+      constexpr int k = kc.value;
+      if (k >= pp && k < q) {
+        if (k == pp) g = d[k] - mu;
+        const double f = sn * e[k], b = c * e[k];
+        const double t2 = fma(g, g, f * f);
+        double r;
+        if (in_range(t2)) {
+          const double ri = rsqrt_cubic(t2);
+          r = t2 * ri;
+          sn = f * ri;
+          c = g * ri;
+        } else {
+          r = hypot(f, g);
+          sn = r != 0.0 ? f / r : 0.0;
+          c = r != 0.0 ? g / r : 1.0;
+        }
+        if constexpr (k > 0) {
+          if (k > pp) e[k - 1] = r;
+        }
+        g = d[k] - pv;
+        r = fma(d[k + 1] - g, sn, twice(b) * c);
+        pv = sn * r;
+        d[k] = g + pv;
+        g = fma(c, r, -b);
+#pragma unroll
+        for (int i = 0; i < R; ++i) {
+          const double v = z[i][k], w = z[i][k + 1];
+          z[i][k] = fma(sn, w, c * v);
+          z[i][k + 1] = fma(c, w, -(sn * v));
+        }
+        if (k == q - 1) {
+          d[k + 1] -= pv;
+          e[k] = g;
+        }
+      }
+    });
+  }
+  // ascending order (stable): the rank of each eigenvalue
+#pragma unroll
+  for (int k = 0; k < LM; ++k)
+    if (gl == 0 && writes) s_d[slot][k] = d[k];
+  __syncwarp();
+  for (int k = gl; k < (writes ? L : 0); k += GL) {
+    const double v = s_d[slot][k];
+    int rk = 0;
+    for (int m = 0; m < L; ++m) {
+      const double w = s_d[slot][m];
+      rk += (w < v || (w == v && m < k)) ? 1 : 0;
+    }
+    s_rank[slot][k] = rk;
+  }
+  __syncwarp();
+  if (!writes) return;
+  const int par = pr.depth & 1;
+  const int64_t ld = par ? pr.n : pr.ld0;
+  double* dst = (par ? P.Q1 + pr.qoff1 : P.Q0 + pr.off_q) + lo + lo * ld;
+  double* lam = P.lam2[par] + pr.voff + lo;
+  double* bf = P.bf2[par] + pr.voff + lo;
+  double* bl = P.bl2[par] + pr.voff + lo;
+#pragma unroll
+  for (int k = 0; k < LM; ++k) {
+    if (k < L) {
+      const int rk = s_rank[slot][k];
+#pragma unroll
+      for (int i = 0; i < R; ++i) {
+        const int r = gl + i * GL;
+        if (r < L) dst[r + rk * ld] = z[i][k];
+        if (r == 0) {
+          lam[rk] = d[k];
+          bf[rk] = z[i][k];
+        }
+        if (r == L - 1) bl[rk] = z[i][k];
+      }
+    }
+  }
+}
+
+template <int LM, int R, int NL = 32 * R / LM>
+static cudaError_t launch_leaf_rows(const Plan& P, int64_t nleaves, cudaStream_t s) {
+  k_leaf_rows<LM, R, NL><<<(unsigned)((nleaves + NL - 1) / NL), 32, 0, s>>>(P, nleaves);
+  return cudaGetLastError();
+}
+
 // Many small leaves per block.  The sequential bulge chase costs one warp
 // instruction per FP64 operation whether one lane or 32 are active, so here lane l
 // of warp 0 runs the whole QR iteration of leaf l (its own deflation scan, shift
 // and chase) and the G leaves of the block advance together; warps 1.. apply each
 // round's rotations to the leaves' eigenvector blocks (one row per lane, the
-// rotations of consecutive rounds double-buffered).  Used when leaves have at
-// most 32 rows; every leaf gets the same arithmetic as in k_leaf.
+// rotations of consecutive rounds double-buffered).  Used for many leaves of 17 to 32
+// rows, where k_leaf_rows has a whole warp for one leaf; same arithmetic as in k_leaf.
 __global__ void __launch_bounds__(1024) k_leaf_multi(Plan P, int64_t nleaves, int Lm, int G) {
   extern __shared__ double sm[];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -461,10 +667,30 @@ __global__ void __launch_bounds__(1024) k_leaf_multi(Plan P, int64_t nleaves, in
   }
 }
 
+// Leaves of at most 16 rows take k_leaf_rows with one row a lane while that is at most one
+// warp per quarter SM (608 quarters; 1024 leaves of 16 rows: 420 us
+// against 464 with R = 2), two rows to twice that, four beyond (12,000 leaves: 2.07 ms; the
+// lane-per-leaf kernel took 4.67 ms, and 1.39 ms for 64 leaves).  Leaves of 17 to 32 rows: under
+// 64 leaves k_leaf's two warps a leaf (10 leaves: 540 us, k_leaf_rows 681), to 4000
+// k_leaf_rows (1000 leaves: 2.4 ms, k_leaf_multi 5.3), beyond k_leaf_multi, whose time grows
+// by 1.06 us a leaf against 1.3.
 cudaError_t launch_leaves(const Plan& P, int64_t nleaves, int max_leaf, cudaStream_t s) {
   if (nleaves == 0) return cudaSuccess;
   if (max_leaf > kMaxLeaf) return cudaErrorInvalidValue;
+  constexpr int64_t kQuarters = 4 * 152;
+  if (max_leaf <= 8) {
+    if (nleaves <= kQuarters) return launch_leaf_rows<8, 1, 1>(P, nleaves, s);
+    if (nleaves <= 4 * kQuarters) return launch_leaf_rows<8, 1>(P, nleaves, s);
+    return launch_leaf_rows<8, 4>(P, nleaves, s);
+  }
+  if (max_leaf <= 16) {
+    if (nleaves <= kQuarters) return launch_leaf_rows<16, 1, 1>(P, nleaves, s);
+    if (nleaves <= 2 * kQuarters) return launch_leaf_rows<16, 1>(P, nleaves, s);
+    if (nleaves <= 4 * kQuarters) return launch_leaf_rows<16, 2>(P, nleaves, s);
+    return launch_leaf_rows<16, 4>(P, nleaves, s);
+  }
   if (max_leaf <= 32 && nleaves >= 64) {
+    if (nleaves <= 4000) return launch_leaf_rows<32, 1>(P, nleaves, s);
     // G leaves per block within a shared-memory budget, one apply warp per 32 rows
     const int Lm = max_leaf;
     // per leaf: Q block, d, e and two rotation buffers; pp/q of both buffers, the
