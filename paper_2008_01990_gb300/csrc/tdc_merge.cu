@@ -1364,96 +1364,180 @@ __device__ int secular_fp64(const double* D, const double* z, int K, int j, doub
   return passes;
 }
 
-// FP64 iteration for root j from a close starting point (the FP32 estimate)
-// with a single pass over all poles.  In that pass, at tau1, the term of each
-// lane's pole in the window [j-15, j+16] (the 32 poles nearest the root) is kept
-// apart from the far terms, whose sums of t, t r and t r^2 (r = 1/(delta_i - tau1))
-// are kept per side.  The following iterates tau = tau1 + e re-evaluate only the
-// window terms; the far sums follow from
+// Sums over the warp of two values (a in every lane, b in every lane), by a reduce-scatter:
+// the first step leaves the lower half-warp with a's partial sums and the upper one with
+// b's, so the five steps take 5 FP64 additions instead of 10 (one holds its quarter of the
+// SM for 64 clocks).
+__device__ __forceinline__ void warp_sum2(double& a, double& b) {
+  const bool up = threadIdx.x & 16;
+  double v = up ? b : a;
+  v += __shfl_xor_sync(0xffffffffu, up ? a : b, 16);
+#pragma unroll
+  for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  a = __shfl_sync(0xffffffffu, v, 0);
+  b = __shfl_sync(0xffffffffu, v, 16);
+}
+__device__ __forceinline__ float warp_sumf(float v) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+
+// FP64 Newton iteration for root j from a close starting point (the FP32 estimate), as a
+// rule with a single pass over all poles.  In that pass, at tau1, the far terms (outside the
+// window of the 32 poles nearest the root, one per lane) are summed: t, t r and t r^2 with
+// r = 1/(delta_i - tau1).  The iterates tau = tau1 + e re-evaluate only the window terms;
+// the far sums follow from
 //   t_i(tau1 + e) = t_i / (1 - e r_i) = t_i (1 + e r_i + (e r_i)^2) + rest_i,
 //   |sum of rest_i| <= (sum of far |t_i|) q^3 / (1 - q),  q = |e| / (distance from
-//   tau1 to the nearest far pole),
-// (their slopes likewise, to first order, for the model only).  A root is
-// accepted when |g| plus that bound passes the convergence test.  Returns true
-// when accepted (tau updated, conv set); otherwise tau is the last iterate,
-// lo / hi hold the bracket, and the caller continues with full passes.
-__device__ bool secular_certified(const double* D, const double* z, const double* zz, int K, int j, double irho,
-                                  int org, double& tau, double& lo, double& hi, bool& conv) {
+//   tau1 to the nearest far pole).
+// What decides the root's accuracy, the sums of t and of t r and the value g, is FP64; the
+// slope, the sums of magnitudes and the tests are FP32.  A root is accepted when |g| plus
+// the bound is at rounding level of 1/rho + sum |t|, or after a Newton step h below 2^-33 of
+// the distance to the nearest pole: the quadratic error (2^-66) and the FP32 slope's (2^-20
+// of h) are then below the rounding of tau.  A step that leaves the expansion's range
+// (q >= 4e-6) starts another pass there.  Returns true when accepted (tau updated); else tau
+// is the last iterate inside the bracket and the caller continues with the safeguarded
+// iteration.  Bound by FP64 issue: 16 FP64 instructions a root, 20 an iterate and 10 a pole
+// and pass of 32; the earlier form (four FP64 sums, divisions and a square root an iterate)
+// took 24,000 clocks a root of a small merge, this one 5,000.
+__device__ bool secular_certified(const double* D, const double* zz, int K, int j, double irho, int org, double width,
+                                  double& tau, int max_passes, int& passes) {
   const int lane = threadIdx.x & 31;
+  const float irf = (float)irho, wf = (float)width;
+  if (!(irf > 1e-18f && irf < 1e18f && wf > 1e-30f)) return false;  // FP32 tests out of range
+  const bool last = j == K - 1;
   const double dorg = D[org];
-  const double dl = D[j] - dorg, dr = (j < K - 1) ? D[j + 1] - dorg : 0.0;
-  const int wlo = j - 15, whi = j + 16;
-  const int iw = wlo + ((lane - wlo) & 31);  // this lane's window pole
-  const bool wv = iw >= 0 && iw < K, wleft = iw <= j;
+  const int w0 = max(0, min(j - 15, K - 32));
+  const int iw = w0 + ((lane - w0) & 31);  // this lane's window pole
+  const bool wv = iw < K;
   const double zw2 = wv ? zz[iw] : 0.0, dw = wv ? D[iw] - dorg : 0.0;
-  const double tau1 = tau;
-  double a0 = 0.0, a1 = 0.0, a2 = 0.0, b0 = 0.0, b1 = 0.0, b2 = 0.0, wt = 0.0, wd = 0.0;
-  // this lane's poles are i = lane (mod 32): those below the window lie left of the
-  // root, its one window pole iw is kept apart, those above the window lie right
-  // of it -- three branch-free ranges
-  for (int i = lane; i < wlo; i += 32) {
-    const double r = rcp_nr((D[i] - dorg) - tau1);
-    const double t = zz[i] * r, tr = t * r;
-    a0 += t; a1 += tr; a2 = fma(tr, r, a2);
-  }
-  if (wv) {
-    const double r = rcp_nr(dw - tau1);
-    wt = zw2 * r;
-    wd = wt * r;
-  }
-  for (int i = iw + 32; i < K; i += 32) {
-    const double r = rcp_nr((D[i] - dorg) - tau1);
-    const double t = zz[i] * r, tr = t * r;
-    b0 += t; b1 += tr; b2 = fma(tr, r, b2);
-  }
-  a0 = warp_sum(a0); a1 = warp_sum(a1); a2 = warp_sum(a2);
-  b0 = warp_sum(b0); b1 = warp_sum(b1); b2 = warp_sum(b2);
-  // distance from tau1 to the nearest far pole (poles are sorted)
-  double dmin = HUGE_VAL;
-  if (wlo - 1 >= 0) dmin = fmin(dmin, fabs((D[wlo - 1] - dorg) - tau1));
-  if (whi + 1 < K) dmin = fmin(dmin, fabs((D[whi + 1] - dorg) - tau1));
-  conv = false;
-  double tc = tau1;
-  for (int k = 0; k < 8; ++k) {
-    const double e = tc - tau1;
-    const double q = fabs(e) / dmin;
-    // beyond q ~ eps^(1/3) the expansion is no better than a full evaluation
-    if (!(q < 4e-6)) break;
-    if (k > 0) {  // window terms at tc
-      wt = 0.0;
-      wd = 0.0;
+  const float zwf = (float)zw2;
+  double tau1 = tau;
+  for (passes = 1; passes <= max_passes; ++passes) {
+    double F = 0.0, A1 = 0.0;
+    float S = 0.0f, A2 = 0.0f, A1f = 0.0f, rdmin = 0.0f;
+    if (K > 32) {
+      // this lane's far poles are i = lane (mod 32): those below the window lie left of the
+      // root, those above it right
+      double a0 = 0.0, b0 = 0.0, a2 = 0.0;
+      for (int i = lane; i < w0; i += 32) {
+        const double r = rcp_nr((D[i] - dorg) - tau1);
+        const double t = zz[i] * r, tr = t * r;
+        a0 += t; A1 += tr; a2 = fma(tr, r, a2);
+      }
+      for (int i = iw + 32; i < K; i += 32) {
+        const double r = rcp_nr((D[i] - dorg) - tau1);
+        const double t = zz[i] * r, tr = t * r;
+        b0 += t; A1 += tr; a2 = fma(tr, r, a2);
+      }
+      F = a0 + b0;
+      S = warp_sumf((float)(b0 - a0));
+      A2 = warp_sumf((float)a2);
+      warp_sum2(F, A1);
+      A1f = (float)A1;
+      // 1 / (distance from tau1 to the nearest far pole), below the window (lower half-warp)
+      // and above it (poles are sorted)
+      const int in = lane < 16 ? w0 - 1 : w0 + 32;
+      float rd = 0.0f;
+      if (in >= 0 && in < K) rd = __fdividef(1.0f, fabsf((float)((D[in] - dorg) - tau1)));
+      rdmin = fmaxf(rd, __shfl_xor_sync(0xffffffffu, rd, 16));
+    }
+    const double A2d = (double)A2;
+    double tc = tau1, e = 0.0;
+    float ef = 0.0f, q = 0.0f;
+    for (int it = 0; it < 8; ++it) {
+      float wsf = 0.0f, wdf = 0.0f;
+      double wt = 0.0;
       if (wv) {
-        const double r = rcp_nr(dw - tc);
-        wt = zw2 * r;
-        wd = wt * r;
+        const double dl = dw - tc;
+        wt = zw2 * rcp_nr(dl);
+        const float rf = __fdividef(1.0f, (float)dl), tf = zwf * rf;
+        wsf = fabsf(tf);
+        wdf = tf * rf;
+      }
+      wsf = warp_sumf(wsf);
+      wdf = warp_sumf(wdf);
+      const double gv = (irho + F + e * fma(e, A2d, A1)) + warp_sum(wt);
+      const float gf = (float)gv, sabs = irf + S + wsf;
+      const float rest = it > 0 ? S * q * q * q / (1.0f - q) : 0.0f;
+      tau = tc;
+      if (fabsf(gf) + rest <= 8.0f * (float)kEps * sabs) return true;
+      const float gp = A1f + 2.0f * ef * A2 + wdf;
+      const float tf = fabsf((float)tc), dist = last ? tf : fminf(tf, wf - tf);
+      if (!(gp > 0.0f && gp < 1e37f && dist > 1e-36f)) return false;
+      const float h = -gf / gp;
+      if (!(fabsf(h) <= 0.015625f * dist)) return false;
+      tc += (double)h;
+      if (fabsf(h) <= 0x1p-33f * dist && rest <= (float)kEps * sabs) {
+        tau = tc;
+        return true;
+      }
+      e = tc - tau1;
+      ef = (float)e;
+      q = fabsf(ef) * rdmin;
+      if (!(q < 4e-6f)) break;
+    }
+    tau = tc;
+    tau1 = tc;
+  }
+  passes = max_passes;
+  return false;
+}
+
+// One step of the FP32 pre-iterations.  R and Rp: value and slope at tau of 1/rho plus the
+// terms of every pole but the own one (the frame's origin, weight y), so that
+// g = R - y / tau.  a / b, da / db: the sums left and right of the root, the own term
+// included.  Close to the own pole (|tau| below an eighth of the interval) the step solves
+//   R + Rp (t - tau) = y / t,
+// the own pole exact: t comes out with full relative accuracy however small it is (as tau
+// plus a correction it keeps 1e-7 of the old tau, so a root 1e-20 of the interval from its
+// pole took the twelve steps allowed and arrived useless: 20 % of the roots of merges of
+// 100 poles of random matrices).  Else the two-pole model of g (interior roots) or the
+// one-pole one (the last root).  Falls back to the bracket's midpoint.
+__device__ __forceinline__ float fp32_step(bool last, bool left, float y, float R, float Rp, float irho, float a,
+                                           float da, float b, float db, float gv, float width, float tau, float lo,
+                                           float hi) {
+  float s;
+  const float c = R - Rp * tau;
+  asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(s) : "f"(fmaf(c, c, 4.0f * Rp * y)));
+  float tn;
+  if (left) tn = c > 0.0f ? __fdividef(2.0f * y, c + s) : __fdividef(s - c, 2.0f * Rp);
+  else tn = c < 0.0f ? __fdividef(2.0f * y, c - s) : -__fdividef(c + s, 2.0f * Rp);
+  if (tn > lo && tn < hi && fabsf(tn) <= 0.125f * width) return tn;
+  // p = d_j - lambda, q = d_j+1 - lambda in the current frame
+  const float p = left ? -tau : -(width + tau);
+  float h = 0.0f;
+  bool ok = true;
+  if (last) {
+    const float A = irho + (a - da * p) + b;
+    if (A != 0.0f) h = p + __fdividef(da * p * p, A); else ok = false;
+  } else {
+    const float q = left ? width - tau : -tau;
+    const float A = irho + (a - da * p) + (b - db * q);
+    const float B = A * (p + q) + da * p * p + db * q * q;
+    const float C = p * q * gv;
+    if (A == 0.0f) {
+      h = __fdividef(C, B);
+    } else {
+      const float disc = B * B - 4.0f * A * C;
+      if (disc < 0.0f) {
+        ok = false;
+      } else {
+        asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(s) : "f"(disc));
+        const float w = B + copysignf(s, B);
+        const float h1 = (w != 0.0f) ? __fdividef(2.0f * C, w) : 0.0f;
+        const float h2 = __fdividef(w, 2.0f * A);
+        const bool in1 = (h1 > p && h1 < q), in2 = (h2 > p && h2 < q);
+        if (in1 && (!in2 || fabsf(h1) <= fabsf(h2))) h = h1;
+        else if (in2) h = h2;
+        else ok = false;
       }
     }
-    const double wtl = warp_sum((wv && wleft) ? wt : 0.0), wtr = warp_sum((wv && !wleft) ? wt : 0.0);
-    const double wdl = warp_sum((wv && wleft) ? wd : 0.0), wdr = warp_sum((wv && !wleft) ? wd : 0.0);
-    const double rest = k > 0 ? (b0 - a0) * (q * q * q) / (1.0 - q) : 0.0;
-    const double psi = a0 + e * (a1 + e * a2) + wtl, dpsi = a1 + 2.0 * e * a2 + wdl;
-    const double phi = b0 + e * (b1 + e * b2) + wtr, dphi = b1 + 2.0 * e * b2 + wdr;
-    const double gv = irho + psi + phi;
-    if (gv == 0.0 || fabs(gv) + rest <= 8.0 * kEps * (irho + (phi - psi))) {
-      tau = tc;
-      conv = true;
-      return true;
-    }
-    if (fabs(gv) > rest) {
-      if (gv < 0.0) lo = tc; else hi = tc;
-    }
-    const double tn = model_step(j, K, irho, dl, dr, tc, gv, psi, dpsi, phi, dphi, lo, hi);
-    // a vanishing step counts only where g is known to rounding level
-    const bool exact_g = rest <= kEps * (irho + (phi - psi));
-    if (exact_g && (fabs(tn - tc) <= 2.0 * kEps * fabs(tc) || (hi - lo) <= 2.0 * kEps * fmax(fabs(lo), fabs(hi)))) {
-      tau = tn;
-      conv = true;
-      return true;
-    }
-    tc = tn;
   }
-  tau = tc;
-  return false;
+  tn = tau + h;
+  if (!ok || !(tn > lo && tn < hi) || !isfinite(tn)) tn = 0.5f * (lo + hi);
+  return tn;
 }
 
 // FP32 pre-iteration for root j: width = d_{j+1} - d_j, or for the last root
@@ -1475,7 +1559,7 @@ __device__ bool secular_fp32(const double* D, const float2* xz, const float* xlo
   const bool wv = iw >= 0 && iw < K;
   float dw = wv ? (float)(D[iw] - D[j]) : 0.0f;
   int o = j;
-  float xo = xz[j].x, xlo_o = xlo[j];
+  float xo = xz[j].x, xlo_o = xlo[j], yo = xz[j].y;
   float lo = 0.0f, hi = width, tau = 0.5f * width;
   for (int it = 0; it < 12; ++it) {
     // it == 0 for the last root: the sum of the other poles' terms at tau = 0
@@ -1484,7 +1568,7 @@ __device__ bool secular_fp32(const double* D, const float2* xz, const float* xlo
     for (int i = lane; i < K; i += 32) {
       const float2 v = xz[i];
       const float del = (i == iw) ? dw : (v.x - xo) + (xlo[i] - xlo_o);
-      if (last && it == 0 && i == j) continue;
+      if (i == o) continue;  // the own pole's term is added below
       float r;
       asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(del - tv));
       const float t = v.y * r;
@@ -1500,58 +1584,37 @@ __device__ bool secular_fp32(const double* D, const float2* xz, const float* xlo
     }
     if (last && it == 0) {
       const float den = irho + a;
-      const float t0 = den > 0.0f ? xz[j].y / den : -1.0f;
+      const float t0 = den > 0.0f ? __fdividef(yo, den) : -1.0f;
       if (t0 > 0.0f && t0 < width) tau = t0;
       continue;
     }
-    const float gv = irho + a + b;
+    float R = irho + a + b, Rp = da + db;
+    float ro;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(ro) : "f"(-tau));
+    const float to = yo * ro;
+    if (o == j) { a += to; da = fmaf(to, ro, da); }
+    else { b += to; db = fmaf(to, ro, db); }
+    const float gv = R + to;
     if (!isfinite(gv)) return false;
     if (gv == 0.0f) break;
     if (it == 0 && !last && gv < 0.0f) {
-      // root in the upper half: continue in the frame of pole j+1 (same point)
+      // root in the upper half: continue in the frame of pole j+1 (same point); the two
+      // poles change their parts in R and Rp
       o = j + 1;
       xo = xz[j + 1].x;
       xlo_o = xlo[j + 1];
+      yo = xz[j + 1].y;
       dw = wv ? (float)(D[iw] - D[j + 1]) : 0.0f;
+      const float tq = -yo * ro;  // the new own term: its distance is the old one's negative
+      R = gv - tq;
+      Rp = fmaf(to, ro, Rp) + tq * ro;
       tau = -0.5f * width;
       lo = -width;
       hi = 0.0f;
     }
     if (gv < 0.0f) lo = tau; else hi = tau;
-    // p = d_j - lambda, q = d_j+1 - lambda in the current frame
-    const float p = o == j ? -tau : -(width + tau);
-    float h = 0.0f;
-    bool ok = true;
-    if (last) {
-      const float b1 = da * p * p;
-      const float A = irho + (a - b1 / p) + b;
-      if (A != 0.0f) h = p + b1 / A; else ok = false;
-    } else {
-      const float q = o == j ? width - tau : -tau;
-      const float b1 = da * p * p, b2 = db * q * q;
-      const float A = irho + (a - b1 / p) + (b - b2 / q);
-      const float B = A * (p + q) + b1 + b2;
-      const float C = p * q * gv;
-      if (A == 0.0f) {
-        h = C / B;
-      } else {
-        const float disc = B * B - 4.0f * A * C;
-        if (disc < 0.0f) {
-          ok = false;
-        } else {
-          const float w = B + copysignf(sqrtf(disc), B);
-          const float h1 = (w != 0.0f) ? 2.0f * C / w : 0.0f;
-          const float h2 = w / (2.0f * A);
-          const bool in1 = (h1 > p && h1 < q), in2 = (h2 > p && h2 < q);
-          if (in1 && (!in2 || fabsf(h1) <= fabsf(h2))) h = h1;
-          else if (in2) h = h2;
-          else ok = false;
-        }
-      }
-    }
-    float tn = tau + h;
-    if (!ok || !(tn > lo && tn < hi) || !isfinite(tn)) tn = 0.5f * (lo + hi);
-    const bool small = fabsf(tn - tau) <= 2e-7f * fabsf(tau);
+    const float tn = fp32_step(last, o == j, yo, R, Rp, irho, a, da, b, db, gv, width, tau, lo, hi);
+    const bool small = fabsf(tn - tau) <= 1e-5f * fabsf(tau);
     tau = tn;
     if (small || (hi - lo) <= 4e-7f * fmaxf(fabsf(lo), fabsf(hi))) break;
   }
@@ -1570,7 +1633,7 @@ __device__ bool secular_fp32(const double* D, const float2* xz, const float* xlo
 __device__ void secular_root(const double* D, const double* z, const double* zz, const float2* xz, const float* xlo,
                              int K, int j,
                              double rho, int max_iter, int& org_out, double& tau_out, int& iters, bool& conv) {
-  const double irho = 1.0 / rho;
+  const double irho = in_range(rho) ? rcp_nr(rho) : 1.0 / rho;
   int org;
   double lo, hi, tau;
   double psi, dpsi, phi, dphi, sabs;
@@ -1591,10 +1654,14 @@ __device__ void secular_root(const double* D, const double* z, const double* zz,
     tau = (double)t32;
     if (org == j) { lo = 0.0; hi = width; } else { lo = -width; hi = 0.0; }
     if (!(tau > lo && tau < hi)) tau = 0.5 * (lo + hi);
-    const bool tried = max_iter >= 2;
-    if (!tried || !secular_certified(D, z, zz, K, j, irho, org, tau, lo, hi, conv)) {
+    int tried = 0;
+    conv = max_iter >= 2 && secular_certified(D, zz, K, j, irho, org, width, tau, min(max_iter - 1, 4), tried);
+    if (conv) {
+      passes = tried;
+    } else {
+      if (!(tau > lo && tau < hi)) tau = 0.5 * (lo + hi);
       secular_sums(D, z, K, j, D[org], tau, psi, dpsi, phi, dphi, sabs);
-      if (tried) ++passes;
+      passes += tried;
       passes += secular_fp64(D, z, K, j, irho, org, tau, lo, hi, psi, dpsi, phi, dphi, sabs, max_iter, conv);
     }
     // an interior root that converged nearer the other pole: continue from that pole
@@ -1638,7 +1705,7 @@ __device__ bool secular_fp32_thread(const float2* xz, const float* xlo, int K, i
                                     int& org_out, float& tau_out) {
   const bool last = j == K - 1;
   int o = j;
-  float xo = xz[j].x, xlo_o = xlo[j];
+  float xo = xz[j].x, xlo_o = xlo[j], yo = xz[j].y;
   float lo = 0.0f, hi = width, tau = 0.5f * width;
   for (int it = 0; it < 12; ++it) {
     const float tv = (last && it == 0) ? 0.0f : tau;
@@ -1654,62 +1721,43 @@ __device__ bool secular_fp32_thread(const float2* xz, const float* xlo, int K, i
       acc += t;
       dacc = fmaf(t, r, dacc);
     };
-    const int jl = (last && it == 0) ? j : j + 1;  // the last root's first pass leaves out pole j
-    for (int i = 0; i < jl; ++i) term(i, a, da);
-    for (int i = j + 1; i < K; ++i) term(i, b, db);
+    // the own pole's term is added below
+    for (int i = 0; i < j; ++i) term(i, a, da);
+    if (o != j) term(j, a, da);
+    if (o == j && j + 1 < K) term(j + 1, b, db);
+    for (int i = j + 2; i < K; ++i) term(i, b, db);
     if (last && it == 0) {
       const float den = irho + a;
-      const float t0 = den > 0.0f ? xz[j].y / den : -1.0f;
+      const float t0 = den > 0.0f ? __fdividef(yo, den) : -1.0f;
       if (t0 > 0.0f && t0 < width) tau = t0;
       continue;
     }
-    const float gv = irho + a + b;
+    float R = irho + a + b, Rp = da + db;
+    float ro;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(ro) : "f"(-tau));
+    const float to = yo * ro;
+    if (o == j) { a += to; da = fmaf(to, ro, da); }
+    else { b += to; db = fmaf(to, ro, db); }
+    const float gv = R + to;
     if (!isfinite(gv)) return false;
     if (gv == 0.0f) break;
     if (it == 0 && !last && gv < 0.0f) {
-      // root in the upper half: continue in the frame of pole j+1 (same point)
+      // root in the upper half: continue in the frame of pole j+1 (same point); the two
+      // poles change their parts in R and Rp
       o = j + 1;
       xo = xz[j + 1].x;
       xlo_o = xlo[j + 1];
+      yo = xz[j + 1].y;
+      const float tq = -yo * ro;
+      R = gv - tq;
+      Rp = fmaf(to, ro, Rp) + tq * ro;
       tau = -0.5f * width;
       lo = -width;
       hi = 0.0f;
     }
     if (gv < 0.0f) lo = tau; else hi = tau;
-    // p = d_j - lambda, q2 = d_j+1 - lambda in the current frame
-    const float p = o == j ? -tau : -(width + tau);
-    float h = 0.0f;
-    bool ok = true;
-    if (last) {
-      const float b1 = da * p * p;
-      const float A = irho + (a - b1 / p) + b;
-      if (A != 0.0f) h = p + b1 / A; else ok = false;
-    } else {
-      const float q2 = o == j ? width - tau : -tau;
-      const float b1 = da * p * p, b2 = db * q2 * q2;
-      const float A = irho + (a - b1 / p) + (b - b2 / q2);
-      const float B = A * (p + q2) + b1 + b2;
-      const float C = p * q2 * gv;
-      if (A == 0.0f) {
-        h = C / B;
-      } else {
-        const float disc = B * B - 4.0f * A * C;
-        if (disc < 0.0f) {
-          ok = false;
-        } else {
-          const float w = B + copysignf(sqrtf(disc), B);
-          const float h1 = (w != 0.0f) ? 2.0f * C / w : 0.0f;
-          const float h2 = w / (2.0f * A);
-          const bool in1 = (h1 > p && h1 < q2), in2 = (h2 > p && h2 < q2);
-          if (in1 && (!in2 || fabsf(h1) <= fabsf(h2))) h = h1;
-          else if (in2) h = h2;
-          else ok = false;
-        }
-      }
-    }
-    float tn = tau + h;
-    if (!ok || !(tn > lo && tn < hi) || !isfinite(tn)) tn = 0.5f * (lo + hi);
-    const bool small = fabsf(tn - tau) <= 2e-7f * fabsf(tau);
+    const float tn = fp32_step(last, o == j, yo, R, Rp, irho, a, da, b, db, gv, width, tau, lo, hi);
+    const bool small = fabsf(tn - tau) <= 1e-5f * fabsf(tau);
     tau = tn;
     if (small || (hi - lo) <= 4e-7f * fmaxf(fabsf(lo), fabsf(hi))) break;
   }
@@ -1719,69 +1767,80 @@ __device__ bool secular_fp32_thread(const float2* xz, const float* xlo, int K, i
   return true;
 }
 
-// The certified FP64 iteration of secular_certified for one thread: one full pass
-// at tau1 keeps the six poles j-2 .. j+3 apart from the far sums (t, t r, t r^2 per
-// side), the following iterates re-evaluate only those six; same remainder bound
-// and acceptance test.
+// The Newton iteration of secular_certified for one thread: one full pass at tau1 keeps the
+// six poles j-2 .. j+3 apart from the far sums, the following iterates re-evaluate only those
+// six; same remainder bound and acceptance, with the rounding bound of the two recursive far
+// sums (terms of one sign each: at most one unit roundoff of the sum per addition) added to
+// the threshold, so that a root whose |g| is below what this pass can resolve is not
+// rejected.  No second pass: what it does not accept goes to a warp.
 __device__ bool secular_certified_thread(const double* D, const double* zz, int K, int j, double irho, int org,
-                                         double& tau, double& lo, double& hi, bool& conv) {
+                                         double width, double& tau) {
+  constexpr int kWin = 6;
+  const float irf = (float)irho, wf = (float)width;
+  if (!(irf > 1e-18f && irf < 1e18f && wf > 1e-30f)) return false;  // FP32 tests out of range
+  const bool last = j == K - 1;
   const double dorg = D[org];
-  const double dl = D[j] - dorg, dr = (j < K - 1) ? D[j + 1] - dorg : 0.0;
-  const int wlo = max(0, j - 2), whi = min(K - 1, j + 3);
-  const double tau1 = tau;
-  double a0 = 0.0, a1 = 0.0, a2 = 0.0, b0 = 0.0, b1 = 0.0, b2 = 0.0;
-  for (int i = 0; i < wlo; ++i) {
-    const double r = rcp_nr((D[i] - dorg) - tau1);
+  const int w0 = max(0, j - 2), w1 = min(K, j + 4);
+  double tc = tau;
+  double a0 = 0.0, A1 = 0.0, a2 = 0.0, b0 = 0.0;
+  for (int i = 0; i < w0; ++i) {
+    const double r = rcp_nr((D[i] - dorg) - tc);
     const double t = zz[i] * r, tr = t * r;
-    a0 += t; a1 += tr; a2 = fma(tr, r, a2);
+    a0 += t; A1 += tr; a2 = fma(tr, r, a2);
   }
-  for (int i = whi + 1; i < K; ++i) {
-    const double r = rcp_nr((D[i] - dorg) - tau1);
+  for (int i = w1; i < K; ++i) {
+    const double r = rcp_nr((D[i] - dorg) - tc);
     const double t = zz[i] * r, tr = t * r;
-    b0 += t; b1 += tr; b2 = fma(tr, r, b2);
+    b0 += t; A1 += tr; a2 = fma(tr, r, a2);
   }
-  double dmin = HUGE_VAL;
-  if (wlo - 1 >= 0) dmin = fmin(dmin, fabs((D[wlo - 1] - dorg) - tau1));
-  if (whi + 1 < K) dmin = fmin(dmin, fabs((D[whi + 1] - dorg) - tau1));
-  // rounding bound of the two recursive far sums (terms of one sign each: at most
-  // one unit roundoff of the sum per addition), added to the acceptance threshold
-  // so that a root whose |g| is below what this pass can resolve is not rejected
-  const double sum_err = kEps * ((double)wlo * fabs(a0) + (double)(K - 1 - whi) * fabs(b0));
-  conv = false;
-  double tc = tau1;
-  for (int k = 0; k < 8; ++k) {
-    const double e = tc - tau1;
-    const double q = fabs(e) / dmin;
-    if (!(q < 4e-6)) break;
-    double wl = 0.0, wr = 0.0, wdl = 0.0, wdr = 0.0;
-    for (int i = wlo; i <= whi; ++i) {
-      const double r = rcp_nr((D[i] - dorg) - tc);
-      const double t = zz[i] * r;
-      if (i <= j) { wl += t; wdl = fma(t, r, wdl); }
-      else { wr += t; wdr = fma(t, r, wdr); }
+  float rdmin = 0.0f;
+  if (w0 > 0) rdmin = __fdividef(1.0f, fabsf((float)((D[w0 - 1] - dorg) - tc)));
+  if (w1 < K) rdmin = fmaxf(rdmin, __fdividef(1.0f, fabsf((float)((D[w1] - dorg) - tc))));
+  double dw[kWin], zw[kWin];
+#pragma unroll
+  for (int k = 0; k < kWin; ++k) {
+    const bool in = w0 + k < w1;
+    dw[k] = in ? D[w0 + k] - dorg : 0.0;
+    zw[k] = in ? zz[w0 + k] : 0.0;
+  }
+  const float fa = (float)fabs(a0), fb = (float)b0, S = fa + fb, A1f = (float)A1, A2f = (float)a2;
+  const float sum_err = (float)kEps * ((float)w0 * fa + (float)(K - w1) * fb);
+  const double F = a0 + b0, tau1 = tc;
+  double e = 0.0;
+  float ef = 0.0f, q = 0.0f;
+  for (int it = 0; it < 8; ++it) {
+    double W = 0.0;
+    float ws = 0.0f, wd = 0.0f;
+#pragma unroll
+    for (int k = 0; k < kWin; ++k) {
+      if (w0 + k < w1) {
+        const double dl = dw[k] - tc;
+        W = fma(zw[k], rcp_nr(dl), W);
+        const float rf = __fdividef(1.0f, (float)dl), tf = (float)zw[k] * rf;
+        ws += fabsf(tf);
+        wd = fmaf(tf, rf, wd);
+      }
     }
-    const double rest = k > 0 ? (b0 - a0) * (q * q * q) / (1.0 - q) : 0.0;
-    const double psi = a0 + e * (a1 + e * a2) + wl, dpsi = a1 + 2.0 * e * a2 + wdl;
-    const double phi = b0 + e * (b1 + e * b2) + wr, dphi = b1 + 2.0 * e * b2 + wdr;
-    const double gv = irho + psi + phi;
-    if (gv == 0.0 || fabs(gv) + rest <= 8.0 * kEps * (irho + (phi - psi)) + sum_err) {
+    const double gv = (irho + F + e * fma(e, a2, A1)) + W;
+    const float gf = (float)gv, sabs = irf + S + ws;
+    const float rest = it > 0 ? S * q * q * q / (1.0f - q) : 0.0f;
+    tau = tc;
+    if (fabsf(gf) + rest <= 8.0f * (float)kEps * sabs + sum_err) return true;
+    const float gp = A1f + 2.0f * ef * A2f + wd;
+    const float tf = fabsf((float)tc), dist = last ? tf : fminf(tf, wf - tf);
+    if (!(gp > 0.0f && gp < 1e37f && dist > 1e-36f)) return false;
+    const float h = -__fdividef(gf, gp);
+    if (!(fabsf(h) <= 0.015625f * dist)) return false;
+    tc += (double)h;
+    if (fabsf(h) <= 0x1p-33f * dist && rest <= (float)kEps * sabs) {
       tau = tc;
-      conv = true;
       return true;
     }
-    if (fabs(gv) > rest + sum_err) {
-      if (gv < 0.0) lo = tc; else hi = tc;
-    }
-    const double tn = model_step(j, K, irho, dl, dr, tc, gv, psi, dpsi, phi, dphi, lo, hi);
-    const bool exact_g = rest <= kEps * (irho + (phi - psi));
-    if (exact_g && (fabs(tn - tc) <= 2.0 * kEps * fabs(tc) || (hi - lo) <= 2.0 * kEps * fmax(fabs(lo), fabs(hi)))) {
-      tau = tn;
-      conv = true;
-      return true;
-    }
-    tc = tn;
+    e = tc - tau1;
+    ef = (float)e;
+    q = fabsf(ef) * rdmin;
+    if (!(q < 4e-6f)) return false;
   }
-  tau = tc;
   return false;
 }
 
@@ -1797,7 +1856,7 @@ __device__ void secular_root_thread(const double* D, const double* z, const doub
                                     const float* xlo, int K,
                                     int j, double rho, int max_iter, bool single, int& org_out, double& tau_out,
                                     int& iters, bool& conv) {
-  const double irho = 1.0 / rho;
+  const double irho = in_range(rho) ? rcp_nr(rho) : 1.0 / rho;
   const bool last = j == K - 1;
   int org;
   double lo, hi, tau, psi, dpsi, phi, dphi, sabs, width;
@@ -1823,7 +1882,8 @@ __device__ void secular_root_thread(const double* D, const double* z, const doub
     tau = (double)t32;
     if (org == j) { lo = 0.0; hi = width; } else { lo = -width; hi = 0.0; }
     if (!(tau > lo && tau < hi)) tau = 0.5 * (lo + hi);
-    if (!secular_certified_thread(D, zz, K, j, irho, org, tau, lo, hi, conv)) return;
+    conv = secular_certified_thread(D, zz, K, j, irho, org, width, tau);
+    if (!conv) return;
     if (!last && ((org == j) ? (tau > 0.5 * width) : (tau < -0.5 * width))) {
       conv = false;
       return;
@@ -1837,12 +1897,8 @@ __device__ void secular_root_thread(const double* D, const double* z, const doub
     tau = (double)t32;
     if (org == j) { lo = 0.0; hi = width; } else { lo = -width; hi = 0.0; }
     if (!(tau > lo && tau < hi)) tau = 0.5 * (lo + hi);
-    const bool tried = max_iter >= 2;
-    if (!tried || !secular_certified_thread(D, zz, K, j, irho, org, tau, lo, hi, conv)) {
-      secular_sums<1>(D, z, K, j, D[org], tau, psi, dpsi, phi, dphi, sabs);
-      if (tried) ++passes;
-      passes += secular_fp64<1>(D, z, K, j, irho, org, tau, lo, hi, psi, dpsi, phi, dphi, sabs, max_iter, conv);
-    }
+    secular_sums<1>(D, z, K, j, D[org], tau, psi, dpsi, phi, dphi, sabs);
+    passes += secular_fp64<1>(D, z, K, j, irho, org, tau, lo, hi, psi, dpsi, phi, dphi, sabs, max_iter, conv);
     const bool far = !last && conv && ((org == j) ? (tau > 0.5 * width) : (tau < -0.5 * width));
     if (far) {
       if (org == j) { org = j + 1; tau -= width; lo -= width; hi -= width; }
@@ -2042,8 +2098,10 @@ __global__ void __launch_bounds__(kSecThreads) k_secular_fixup(Plan P, int level
   }
 }
 
-// Warp per root over the merges with K > small_k (for_warp_roots).
-__global__ void __launch_bounds__(kSecThreads) k_secular(Plan P, int level, int64_t M, int small_k, bool listed) {
+// Warp per root over the merges with K > small_k (for_warp_roots).  At most 80 registers a
+// thread: four warps then fit on an SM beside a resident CTA of the split product (96 x 576
+// of the 65,536 registers), whose stream runs during the next level's roots.
+__global__ void __launch_bounds__(kSecThreads, 6) k_secular(Plan P, int level, int64_t M, int small_k, bool listed) {
   for_warp_roots(P, M, small_k, listed, [&](int64_t g, int K, int jw) {
     const Node nd = make_node(P, level, g);
     const int64_t v0 = nd.v0;
