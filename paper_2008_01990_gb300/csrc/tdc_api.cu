@@ -301,8 +301,8 @@ static void build_plan(HostPlan& H, int32_t batch, const int64_t* n_host, const 
       mx = std::max(mx, nm);
       mn = std::min(mn, p.n >> l);
       const int64_t n1 = (nm + 1) / 2;
-      int bm, bn;
-      dense_tile_dims(nm, bm, bn);
+      int bm, bn;  // a bound for either tile size: the grid walks the tiles counted on the device
+      dense_tile_dims(nm, true, bm, bn);
       const int64_t rt = 2 * ((n1 + bm - 1) / bm);
       tiles += (((int64_t)1) << l) * rt * ((nm + bn - 1) / bn);
     }
@@ -589,6 +589,10 @@ static int run_plan(HostPlan& H, const tdc_opts& o, const double* d, const doubl
     Plan P = PP[l & 1];
     const bool ss = H.ss && H.ss_level[l] && LL.max_n >= P.struct_min_K;
     P.struct_split = ss ? 1 : 0;
+    P.dense_small = (P.split_min_K > 0 && P.split_min_K <= kDenseSmallK) ||
+                            LL.nslots * LL.max_n < kDenseFewTiles * kDenseBM * kDenseBN
+                        ? 1
+                        : 0;
     if (l + 2 < H.T) err = cudaStreamWaitEvent(s, evG[l + 2], 0);
     const size_t a0 = mark();
     if (err == cudaSuccess) err = launch_prepare(P, LL, s);

@@ -207,7 +207,7 @@ struct Plan {
   int32_t struct_min_K; // merges with K >= this use the structured path (0: never)
   int32_t struct_m;     // tile size of the structured path
   int32_t struct_split; // 1: the structured path's products run on the split tensor-core GEMM
-  int32_t pad_;
+  int32_t dense_small;  // the level's FP64 merges all take the small tiles (dense_tile_dims)
   const int32_t* ss_accept;  // per merge part (2g + p): 1 if the structured split path took it
 };
 
@@ -672,12 +672,20 @@ cudaError_t launch_gk_build(int64_t n, const double* d, const double* e, double*
 cudaError_t launch_gk_extract(int64_t n, const double* lam, const double* Q, int64_t ldq, double* sigma, double* U,
                               int64_t ldu, double* VT, int64_t ldvt, cudaStream_t s);
 constexpr int kDenseBM = 128, kDenseBN = 64, kDenseBK = 16;
-// merges of order n <= kDenseSmallN take 32 x 32 tiles: their halves have at most 64
-// rows, so a 128-row tile would leave most of its FP64 multiply-adds on padding
+// FP64 tiles of 32 x 32 instead of 128 x 64: merges of order n <= kDenseSmallN (their halves
+// have at most 64 rows), and whole levels (Plan::dense_small) whose FP64 merges have few
+// poles or that hold few tiles.  A 32-row tile generates each Qhat entry for 32 rows instead of
+// 128 (6 operations: 19 % against 5 %), but pads less (K of about 100: 128 columns against
+// 64 + 64, halves of a few hundred rows) and spreads a lone merge over the SMs: the FP64
+// tiles of a batch of 512 problems 17.5 -> 15.2 ms, of one matrix of n = 1024 531 -> 142 us.
 constexpr int kDenseSmallN = 128, kDenseSmallBM = 32, kDenseSmallBN = 32;
-__host__ __device__ inline void dense_tile_dims(int64_t n, int& bm, int& bn) {
-  bm = n <= kDenseSmallN ? kDenseSmallBM : kDenseBM;
-  bn = n <= kDenseSmallN ? kDenseSmallBN : kDenseBN;
+// merges this wide or wider keep the large tiles where they fill the chip
+constexpr int kDenseSmallK = 256;
+constexpr int64_t kDenseFewTiles = 2 * 152;
+__host__ __device__ inline void dense_tile_dims(int64_t n, bool small, int& bm, int& bn) {
+  small = small || n <= kDenseSmallN;
+  bm = small ? kDenseSmallBM : kDenseBM;
+  bn = small ? kDenseSmallBN : kDenseBN;
 }
 // merges of order n <= kTinyN (halves of at most 16 rows and poles, K <= 32) off the
 // split and structured paths take a warp each (k_gemm_tiny) instead of tiles

@@ -8,11 +8,12 @@
 // column j goes to the node's eigenvector column posr[j].
 //
 // One CTA computes a 128 x 64 tile with 256 threads (8 x 4 outputs each) on
-// the FP64 pipe -- 32 x 32 (2 x 2 each) for merges of order <= 128, whose halves
-// have at most 64 rows; per 16-deep k-step it stages the Qtilde tile in shared
-// memory and generates the 16 x 64 (16 x 32) Qhat tile there (8 FP64 operations
-// per entry, amortised over the tile's rows).  Tiles of all merges of the level
-// form one work list (prefix in MergeInfo::tiles) that a fixed grid walks.
+// the FP64 pipe -- 32 x 32 (2 x 2 each) for small merges and levels of few tiles
+// (dense_tile_dims); per 16-deep k-step it stages the Qtilde tile in shared
+// memory and generates the 16 x 64 (16 x 32) Qhat tile there (6 FP64 operations
+// per entry, amortised over the tile's rows; the normaliser s_j scales the column
+// at the end).  Tiles of all merges of the level form one work list (prefix in
+// MergeInfo::tiles) that a fixed grid walks.  Bound by the FP64 pipe.
 // Merges of order <= 32 take a warp each instead (k_gemm_tiny).
 #include <float.h>
 
@@ -63,7 +64,7 @@ template <int TBM, int TBN, bool kRowFast>
 __device__ __forceinline__ void dense_tile(const Plan& P, const Node& nd, int64_t g, int64_t local, double* As,
                                            double* Us, DenseCols& sc) {
   constexpr int TM = TBM / 16, TN = TBN / 16;
-  static_assert(TBM % 16 == 0 && TBN % 16 == 0 && TBN <= BN && TBM * BK <= BM * BK, "tile shape");
+  static_assert(TBM % 16 == 0 && TBN % 16 == 0 && TBN <= BN && TBM <= BM, "tile shape");
   const int tid = threadIdx.x;
   const int ty = kRowFast ? (tid & 15) : (tid >> 4);  // row group: TM rows
   const int tx = kRowFast ? (tid >> 4) : (tid & 15);  // column group: TN columns
@@ -134,7 +135,7 @@ __device__ __forceinline__ void dense_tile(const Plan& P, const Node& nd, int64_
       const int idx = tid + e * kThreads;
       const int k = idx / TBN, c = idx % TBN;
       const double del = (sc.Dq[k] - sc.Do[c]) - sc.Tau[c];
-      Us[k * TBN + c] = (sc.Zq[k] * sc.S[c]) * rcp_nr(del);
+      Us[k * TBN + c] = sc.Zq[k] * rcp_nr(del);
     }
     __syncthreads();
 #pragma unroll
@@ -155,19 +156,23 @@ __device__ __forceinline__ void dense_tile(const Plan& P, const Node& nd, int64_
   for (int c = 0; c < TN; ++c) {
     const int pos = sc.Pos[tx * TN + c];
     if (pos < 0 || pos >= n) continue;
+    const double sj = sc.S[tx * TN + c];
     double* out = nd.dst + (int64_t)pos * nd.ldd;
 #pragma unroll
     for (int i = 0; i < TM; ++i) {
       const int row = r0 + ty * TM + i;
-      if (row < rend) out[row] = acc[i][c];
+      if (row < rend) out[row] = acc[i][c] * sj;
     }
   }
 }
 }  // namespace
 
-__global__ void __launch_bounds__(kThreads, 2) k_gemm_dense(Plan P, int level, int64_t M) {
-  __shared__ double As[BK * BM];
-  __shared__ double Us[BK * BN];
+// kSmall: every FP64 merge of the level takes 32 x 32 tiles (five blocks a SM hide each
+// other's loads and barriers).
+template <bool kSmall>
+__global__ void __launch_bounds__(kThreads, kSmall ? 5 : 2) k_gemm_dense(Plan P, int level, int64_t M) {
+  __shared__ double As[BK * (kSmall ? kDenseSmallBM : BM)];
+  __shared__ double Us[BK * (kSmall ? kDenseSmallBN : BN)];
   __shared__ DenseCols sc;
   const int64_t total = P.m.tiles[M];
   for (int64_t w = blockIdx.x; w < total; w += gridDim.x) {
@@ -180,10 +185,10 @@ __global__ void __launch_bounds__(kThreads, 2) k_gemm_dense(Plan P, int level, i
     const int64_t g = a;
     const Node nd = make_node(P, level, g);
     int bm, bn;
-    dense_tile_dims(nd.hi - nd.lo, bm, bn);
-    if (bm == kDenseSmallBM)
+    dense_tile_dims(nd.hi - nd.lo, kSmall, bm, bn);
+    if (kSmall || bm == kDenseSmallBM)
       dense_tile<kDenseSmallBM, kDenseSmallBN, true>(P, nd, g, w - P.m.tiles[g], As, Us, sc);
-    else
+    else if constexpr (!kSmall)
       dense_tile<BM, BN, false>(P, nd, g, w - P.m.tiles[g], As, Us, sc);
   }
 }
@@ -355,7 +360,8 @@ cudaError_t launch_gemm_dense(const Plan& P, const LevelLaunch& L, int64_t max_t
   int64_t grid = max_tiles;
   const int64_t cap = 152 * 8;
   if (grid > cap) grid = cap;
-  k_gemm_dense<<<(unsigned)grid, kThreads, 0, s>>>(P, L.level, L.merges);
+  if (P.dense_small) k_gemm_dense<true><<<(unsigned)grid, kThreads, 0, s>>>(P, L.level, L.merges);
+  else k_gemm_dense<false><<<(unsigned)grid, kThreads, 0, s>>>(P, L.level, L.merges);
   return cudaGetLastError();
 }
 

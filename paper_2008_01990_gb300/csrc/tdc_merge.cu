@@ -2596,7 +2596,7 @@ __global__ void __launch_bounds__(1024) k_finalize(Plan P, int level) {
   if (threadIdx.x == 0) {
     // GEMM tiles of this merge: (row tiles of top + bottom parts) x column tiles
     int bm, bn;
-    dense_tile_dims(n, bm, bn);
+    dense_tile_dims(n, P.dense_small != 0, bm, bn);
     const int64_t rt = (n1 + bm - 1) / bm + (n - n1 + bm - 1) / bm;
     const int64_t ct = (K + bn - 1) / bn;
     const bool split = P.split_min_K > 0 && K >= P.split_min_K;
