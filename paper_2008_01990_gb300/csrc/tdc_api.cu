@@ -1545,7 +1545,26 @@ int sytrd_run(int64_t n, double* A, int64_t lda, double* d, double* e, double* t
     U.status = st;
     U.budget = op.spin_budget;
     U.chunk_steps = op.split_chunk_k / 16;
+    const int64_t res = trd_resident_max();
     for (int64_t p = 0; p < n - 2; p += kTrdNb) {
+      if (n - p <= res) {  // the rest in one launch; the exchange uses V's space (128 n doubles)
+        TrdResident R;
+        memset(&R, 0, sizeof(R));
+        R.A = A;
+        R.lda = lda;
+        R.t0 = p;
+        R.m = (int32_t)(n - p);
+        R.d = d;
+        R.e = e;
+        R.tau = tau;
+        R.xy = P.V;
+        R.xc = R.xy + 2 * (n - p);
+        R.bar = P.bar;
+        R.status = st;
+        R.budget = op.spin_budget;
+        if (launch_trd_resident(R, grid, s) != cudaSuccess) return TDC_ECUDA;
+        break;
+      }
       P.p = p;
       P.nbp = (int32_t)std::min<int64_t>(kTrdNb, n - 2 - p);
       if (launch_trd_panel(P, grid, s) != cudaSuccess) return TDC_ECUDA;

@@ -417,6 +417,22 @@ __device__ __forceinline__ double rsqrt_nr(double x) {
   return y;
 }
 
+// The same with one third-order refinement: y (1 + e/2 + 3 e^2 / 8), e = 1 - x y^2 near 2^-20,
+// leaves 5 e^3 / 16; five FP64 operations instead of seven.
+__device__ __forceinline__ double rsqrt_cubic(double x) {
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  const double e = fma(-(x * y), y, 1.0);
+  return fma(y * e, fma(0.375, e, 0.5), y);
+}
+
+// 2^-960 <= x < 2^960 for x >= 0, by the exponent field (an FP64 comparison holds its
+// quarter of the SM for 64 clocks like any other FP64 instruction).
+__device__ __forceinline__ bool in_range(double x) {
+  const unsigned ex = (unsigned)__double2hiint(x) >> 20;
+  return ex >= 63u && ex < 1983u;
+}
+
 __device__ __forceinline__ double warp_sum(double v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
@@ -544,6 +560,22 @@ struct TrdPanel {
   int* status;
   long long budget;
 };
+// the resident end of the reduction (k_trd_resident): trailing matrix of order m <= kTrdResMax
+// at A(t0, t0)
+constexpr int kTrdResMax = 1824;
+struct TrdResident {
+  double* A;
+  int64_t lda, t0;
+  int32_t m;
+  double* d;
+  double* e;
+  double* tau;
+  double* xy;      // the exchanged vectors, 2 x m each: y and the next column
+  double* xc;
+  unsigned* bar;   // arrival counter
+  int* status;
+  long long budget;
+};
 struct TrdUpdate {
   double* A;
   int64_t lda, n, t0;  // trailing matrix A(t0:n, t0:n)
@@ -588,6 +620,8 @@ struct OrmStep {
 int trd_panel_grid();
 cudaError_t launch_sym_fill(int64_t n, double* A, int64_t lda, cudaStream_t s);
 cudaError_t launch_trd_panel(const TrdPanel& P, int grid, cudaStream_t s);
+int64_t trd_resident_max();
+cudaError_t launch_trd_resident(const TrdResident& P, int grid, cudaStream_t s);
 cudaError_t launch_trd_update(const TrdUpdate& U, cudaStream_t s);
 cudaError_t launch_trd_tail(int64_t n, const double* A, int64_t lda, double* d, double* e, double* tau,
                             cudaStream_t s);

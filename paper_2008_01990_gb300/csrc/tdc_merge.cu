@@ -304,23 +304,11 @@ __device__ __forceinline__ void static_for(F&& f) {
 
 // Helpers of the chase: a warp's FP64 instructions go through its quarter of the SM one per
 // 64 clocks (measured, dependent or not, and a comparison counts as one), so what integer
-// instructions can do they do.  in_range: 2^-960 <= x < 2^960 for x >= 0; twice(x) = 2 x
-// by the exponent field; rsqrt_cubic: the hardware estimate y (error e of
-// 1 - x y^2 near 2^-20) refined once to y (1 + e/2 + 3 e^2 / 8), which leaves 5 e^3 / 16.
-__device__ __forceinline__ bool in_range(double x) {
-  const unsigned ex = (unsigned)__double2hiint(x) >> 20;
-  return ex >= 63u && ex < 1983u;
-}
+// instructions can do they do (in_range; twice(x) = 2 x by the exponent field).
 __device__ __forceinline__ double twice(double x) {
   const int h = __double2hiint(x);
   if ((h & 0x7ff00000) == 0) return x + x;
   return __hiloint2double(h + 0x100000, __double2loint(x));
-}
-__device__ __forceinline__ double rsqrt_cubic(double x) {
-  double y;
-  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-  const double e = fma(-(x * y), y, 1.0);
-  return fma(y * e, fma(0.375, e, 0.5), y);
 }
 
 template <int LM, int R, int NL>

@@ -465,6 +465,238 @@ __global__ void __launch_bounds__(kTrdThreads, 1) k_trd_panel(TrdPanel P) {
   }
 }
 
+// ---------------------------------------------------------------------------
+// The end of the reduction, once the trailing matrix fits the SMs' shared memory: the
+// columns of the m x m trailing matrix lie spread over the blocks (column c in block
+// c mod G, whole columns of the symmetric matrix), each reflector's rank-2 update is applied
+// to them in FP64 as soon as it is known, and a column costs one exchange between the
+// blocks.  At step k every block holds x = column k below its diagonal.  (1) A warp per own
+// column c applies the previous reflector's update to it and takes its dot with x, while
+// four other warps form the reflector (beta, tau, 1 / (alpha - beta)) from ||x||.
+// (2) y_c = (A v)_c and the updated column k + 1 go to memory; the blocks meet at an arrival
+// counter (release reductions, one acquire-polling thread a block) and read both.  (3) Every
+// block forms w = tau y - (tau^2 / 2)(v^T y) v and the next column's
+// x = A(:, k+1) - v w_{k+1} - w for itself.
+// The counter is the cheapest meeting point measured (152 blocks, 600 entries, clocks a
+// round): counter 4200, entries tagged with the step that all readers poll for 7400, a flag a
+// block 7900 (stores to lines that other SMs poll are slow; reductions are not).
+// The vectors are double-buffered by the step's parity: a block writes step k + 2 only after
+// it has read all of step k + 1, whose writers had read all of step k.  A block leaves once
+// it owns no column past k + 1; the counter's next target leaves it out.
+// All blocks are resident (cooperative launch); polls are bounded and report TDC_ETIMEOUT.
+//
+// Bound by the FP64 pipe (3 multiply-adds an entry of the square a column, 7 an entry of the
+// vectors, at 2 a clock and SM) and by the exchange.  The blocked panel kernel needs one
+// multiply-add an entry but two grid barriers a column and the panel's products.  Order
+// 1000: 16.7 -> 6.8 ms for the whole reduction; orders 1792 and below at the end of n = 4096: 36.6 -> 20.3.
+constexpr int kResThreads = 512;
+constexpr int kResCols = 12;  // columns a block at most: warps 0-11 take one each, 12-15 the reflector
+constexpr int kResRows = (kTrdResMax + kResThreads - 1) / kResThreads;
+
+// Sum of 512 partials by the four warps wq = 0..3 (128 entries each; named barrier `bar`):
+// the total in every lane of warp wq = 0.
+__device__ __forceinline__ double sum512(const double* part, double* quad, int wq, int bar) {
+  const int lane = threadIdx.x & 31;
+  const double* p = part + wq * 128 + lane;
+  double t = (p[0] + p[32]) + (p[64] + p[96]);
+  t = warp_sum(t);
+  if (lane == 0) quad[wq] = t;
+  asm volatile("bar.sync %0, 128;" ::"r"(bar) : "memory");
+  return wq == 0 ? (quad[0] + quad[1]) + (quad[2] + quad[3]) : 0.0;
+}
+
+__global__ void __launch_bounds__(kResThreads, 1) k_trd_resident(TrdResident P) {
+  extern __shared__ double sm[];
+  __shared__ double s_ss[kResThreads], s_vy[kResThreads], s_quad[8], s_dot[kResCols];
+  __shared__ double s_alpha, s_tau, s_sc, s_beta, s_y1, s_g, s_w1;
+  __shared__ int s_fail;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int m = P.m, G = gridDim.x, b = blockIdx.x;
+  if (b >= m) return;
+  const int ncb = (m - b + G - 1) / G, clast = b + (ncb - 1) * G;
+  double* cols = sm;  // ncb columns of m
+  double* vp = cols + (int64_t)ncb * m;
+  double* wp = vp + m;
+  double* xs = wp + m;
+  double* __restrict__ A = P.A + P.t0 + P.t0 * P.lda;
+  for (int q = 0; q < ncb; ++q)
+    for (int r = tid; r < m; r += kResThreads) cols[q * m + r] = A[r + (int64_t)(b + q * G) * P.lda];
+  double a[kResRows], v[kResRows];
+#pragma unroll
+  for (int i = 0; i < kResRows; ++i) {
+    const int r = tid + i * kResThreads;
+    a[i] = r < m ? A[r] : 0.0;
+    v[i] = 0.0;
+    if (r < m) {
+      vp[r] = 0.0;
+      wp[r] = 0.0;
+    }
+  }
+  if (tid == 0) s_fail = 0;
+  volatile int* vfail = &s_fail;
+  unsigned target = 0;
+  for (int k = 0; k + 2 < m; ++k) {
+    target += (unsigned)min(G, m - 1 - k);  // the blocks owning a column past k
+    double* xy = P.xy + (int64_t)(k & 1) * m;
+    double* xc = P.xc + (int64_t)(k & 1) * m;
+    double ss = 0.0;
+#pragma unroll
+    for (int i = 0; i < kResRows; ++i) {
+      const int r = tid + i * kResThreads;
+      if (r > k && r < m) {
+        xs[r] = r > k + 1 ? a[i] : 0.0;
+        if (r > k + 1) ss = fma(a[i], a[i], ss);
+        else s_alpha = a[i];
+      }
+    }
+    s_ss[tid] = ss;
+    __syncthreads();
+    // (1) update and dots; the reflector
+    if (warp < ncb) {
+      const int c = b + warp * G;
+      if (c > k) {
+        double* __restrict__ col = cols + warp * m;
+        const double vc = -vp[c], wc = -wp[c];
+        double dot = 0.0;
+        // the next rows' loads go out before this row's multiply-adds
+        int r = k + 1 + lane;
+        double c0 = 0.0, v0 = 0.0, w0 = 0.0, x0 = 0.0;
+        if (r < m) {
+          c0 = col[r]; v0 = vp[r]; w0 = wp[r]; x0 = xs[r];
+        }
+        for (; r < m; r += 32) {
+          const int r2 = r + 32;
+          double c1 = 0.0, v1 = 0.0, w1 = 0.0, x1 = 0.0;
+          if (r2 < m) {
+            c1 = col[r2]; v1 = vp[r2]; w1 = wp[r2]; x1 = xs[r2];
+          }
+          const double x = fma(w0, vc, fma(v0, wc, c0));
+          col[r] = x;
+          if (c == k + 1) xc[r] = x;
+          dot = fma(x, x0, dot);
+          c0 = c1; v0 = v1; w0 = w1; x0 = x1;
+        }
+        dot = warp_sum(dot);
+        if (lane == 0) s_dot[warp] = dot;
+      }
+    } else if (warp >= kResCols) {
+      const double s = sum512(s_ss, s_quad, warp - kResCols, 1);
+      if (warp == kResCols && lane == 0) {
+        const double alpha = s_alpha;
+        double t = 0.0, beta = alpha, sc = 0.0;
+        if (s > 0.0) {
+          const double t2 = fma(alpha, alpha, s);
+          if (in_range(t2)) {
+            const double ri = -copysign(rsqrt_cubic(t2), alpha);  // 1 / beta
+            beta = t2 * ri;
+            sc = rcp_nr(alpha - beta);
+            t = (beta - alpha) * ri;
+          } else {
+            beta = -copysign(sqrt(t2), alpha);
+            t = (beta - alpha) / beta;
+            sc = 1.0 / (alpha - beta);
+          }
+        }
+        s_tau = t;
+        s_sc = sc;
+        s_beta = beta;
+      }
+    }
+    __syncthreads();
+    const double tau = s_tau, sc = s_sc;
+    const bool leave = clast < k + 2;
+    if (warp == 0) {
+      const int c = b + lane * G;
+      if (lane < ncb && c > k) xy[c] = fma(sc, s_dot[lane], cols[lane * m + k + 1]);
+      __syncwarp();
+      // (2) y and column k + 1 of every block
+      if (lane == 0) {
+        asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(P.bar) : "memory");
+        long long polls = 0;
+        while (!leave && ld_acquire_u32(P.bar) < target && polls <= P.budget) ++polls;
+        if (polls > P.budget) *vfail = 1;
+      }
+    }
+    if (leave) return;
+    __syncthreads();
+    if (*vfail) {
+      if (tid == 0) set_status(P.status, TDC_ETIMEOUT);
+      return;
+    }
+    double y[kResRows], cn[kResRows];
+#pragma unroll
+    for (int i = 0; i < kResRows; ++i) {
+      const int r = tid + i * kResThreads;
+      const bool in = r > k && r < m;
+      y[i] = in ? __ldcg(xy + r) : 0.0;
+      cn[i] = in ? __ldcg(xc + r) : 0.0;
+    }
+    double vy = 0.0;
+#pragma unroll
+    for (int i = 0; i < kResRows; ++i) {
+      const int r = tid + i * kResThreads;
+      if (r > k && r < m) {
+        v[i] = r == k + 1 ? 1.0 : a[i] * sc;
+        vy = fma(v[i], y[i], vy);
+        if (r == k + 1) s_y1 = y[i];
+      }
+    }
+    s_vy[tid] = vy;
+    __syncthreads();
+    // (3) w and the next column
+    if (warp < 4) {
+      const double t = sum512(s_vy, s_quad + 4, warp, 2);
+      if (tid == 0) {
+        const double g = 0.5 * tau * tau * t;
+        s_g = g;
+        s_w1 = fma(tau, s_y1, -g);
+      }
+    }
+    __syncthreads();
+    const double g = s_g, w1 = s_w1;
+    // the writer of column k's results: any block that is still here
+    const bool mine = (m - 1 - k % min(G, m - 2 - k)) % G == b;
+    double* __restrict__ Ak = A + (int64_t)k * P.lda;
+#pragma unroll
+    for (int i = 0; i < kResRows; ++i) {
+      const int r = tid + i * kResThreads;
+      if (r >= m || r < k) continue;
+      if (r == k) {
+        if (mine) {
+          P.d[P.t0 + k] = a[i];
+          Ak[k] = a[i];
+        }
+        continue;
+      }
+      const double w = fma(-g, v[i], tau * y[i]);
+      vp[r] = v[i];
+      wp[r] = w;
+      a[i] = fma(-v[i], w1, cn[i]) - w;
+      if (mine) {
+        if (r == k + 1) {
+          P.e[P.t0 + k] = s_beta;
+          P.tau[P.t0 + k] = tau;
+          Ak[r] = s_beta;
+        } else {
+          Ak[r] = v[i];
+        }
+      }
+    }
+  }
+  // the last 2 x 2 block (only the owner of column m - 1 is left)
+  __syncthreads();
+  const int q = ncb - 1;
+#pragma unroll
+  for (int i = 0; i < kResRows; ++i) {
+    const int r = tid + i * kResThreads;
+    if (r == m - 2) A[r + (int64_t)(m - 2) * P.lda] = a[i];
+    if (r == m - 1) {
+      A[r + (int64_t)(m - 2) * P.lda] = a[i];
+      A[r + (int64_t)r * P.lda] = fma(-2.0 * vp[r], wp[r], cols[q * m + r]);
+    }
+  }
+}
+
 // Largest |W(t0:n, 0:nb)| as the bits of a non-negative double (zero beforehand).
 __global__ void __launch_bounds__(256) k_trd_wmax(int64_t t0, int64_t n, int nb, const double* W, int64_t ld,
                                                  unsigned long long* wmax) {
@@ -673,6 +905,44 @@ cudaError_t launch_trd_panel(const TrdPanel& P, int grid, cudaStream_t s) {
   void* args[] = {&arg};
   return cudaLaunchCooperativeKernel((const void*)k_trd_panel, dim3(grid), dim3(kTrdThreads), args,
                                      trd_panel_smem(P.n), s);
+}
+
+static size_t trd_resident_smem(int64_t m, int grid) {
+  return sizeof(double) * (size_t)(((m + grid - 1) / grid + 3) * m);
+}
+
+// The largest trailing order k_trd_resident takes on this device (0: none).
+int64_t trd_resident_max() {
+  static int64_t best[64] = {0};
+  static bool known[64] = {false};
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
+  if (!known[dev]) {
+    const int grid = trd_panel_grid();
+    int optin = 0;
+    cudaFuncAttributes fa;
+    if (grid <= 0 || cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess ||
+        cudaFuncGetAttributes(&fa, k_trd_resident) != cudaSuccess)
+      return 0;
+    const int64_t room = (int64_t)optin - (int64_t)fa.sharedSizeBytes;
+    if (room <= 0 || cudaFuncSetAttribute(k_trd_resident, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)room) !=
+                         cudaSuccess)
+      return 0;
+    int64_t m = std::min<int64_t>(kTrdResMax, (int64_t)kResCols * grid);
+    while (m > 0 && (int64_t)trd_resident_smem(m, grid) > room) --m;
+    best[dev] = m;
+    known[dev] = true;
+  }
+  return best[dev];
+}
+
+cudaError_t launch_trd_resident(const TrdResident& P, int grid, cudaStream_t s) {
+  cudaError_t e = cudaMemsetAsync(P.bar, 0, sizeof(unsigned), s);
+  if (e != cudaSuccess) return e;
+  TrdResident arg = P;
+  void* args[] = {&arg};
+  return cudaLaunchCooperativeKernel((const void*)k_trd_resident, dim3((unsigned)grid), dim3(kResThreads), args,
+                                     trd_resident_smem(P.m, grid), s);
 }
 
 cudaError_t launch_trd_update(const TrdUpdate& U, cudaStream_t s) {
