@@ -69,16 +69,45 @@ __device__ bool grid_barrier(unsigned* ctr, unsigned& target, long long budget, 
   return *s_flag != 0;
 }
 
-// sum over a block's warps in warp order of values held by lane 0 of each warp (thread 0
-// gets the result)
+// sum over a block's warps of values held by lane 0 of each warp (thread 0 gets the result)
 __device__ __forceinline__ double block_sum_lane0(double v, double* s_red) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   if (lane == 0) s_red[warp] = v;
   __syncthreads();
+  return warp == 0 ? warp_sum(lane < (int)(blockDim.x >> 5) ? s_red[lane] : 0.0) : 0.0;
+}
+
+// Sum over the grid's blocks of their partials p[b], by a warp (every lane gets it): loads of
+// 8 x 32 blocks go out together.
+__device__ __forceinline__ double sum_blocks(const double* p) {
+  const int lane = threadIdx.x & 31, G = (int)gridDim.x;
   double t = 0.0;
-  if (threadIdx.x == 0)
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += s_red[w];
-  return t;
+  for (int b0 = lane; b0 < G; b0 += 256) {
+    double v[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) v[u] = b0 + 32 * u < G ? p[b0 + 32 * u] : 0.0;
+#pragma unroll
+    for (int u = 0; u < 8; ++u)
+      if (b0 - lane + 32 * u < G) t += v[u];
+  }
+  return warp_sum(t);
+}
+
+// The reflector of a column with first entry alpha and the others' squared norm s > 0: beta,
+// tau = (beta - alpha) / beta and 1 / (alpha - beta), from refined hardware reciprocals (an
+// FP64 square root and two divisions take 2,400 clocks of one thread, these 700).
+__device__ __forceinline__ void reflector(double alpha, double s, double& tau, double& beta, double& sc) {
+  const double t2 = fma(alpha, alpha, s);
+  if (in_range(t2)) {
+    const double ri = -copysign(rsqrt_cubic(t2), alpha);  // 1 / beta
+    beta = t2 * ri;
+    sc = rcp_nr(alpha - beta);
+    tau = (beta - alpha) * ri;
+  } else {
+    beta = -copysign(sqrt(t2), alpha);
+    tau = (beta - alpha) / beta;
+    sc = 1.0 / (alpha - beta);
+  }
 }
 
 }  // namespace
@@ -108,129 +137,89 @@ __global__ void __launch_bounds__(256) k_sym_fill(int64_t n, double* A, int64_t 
   }
 }
 
-constexpr int kProdChunk = 16;  // columns a block takes at once in the symv
-
-// Sums over the 32 lanes of each of C per-lane values (C a power of two <= 32): a
-// reduce-scatter (every step keeps half of the values and adds the partner's other
-// half), then butterflies; lanes l with l mod (32 / C) = 0 end with the sum of value
-// l / (32 / C).  C = 16 takes 16 FP64 adds instead of the 80 of a butterfly per value:
-// FP64 adds are scarce on this chip.
-template <int C>
-__device__ __forceinline__ double warp_reduce_cols(double (&v)[C]) {
+// Dots of one (p2 NULL) or two columns with x over m rows by a warp (x_0 counts as 0): the
+// next rows' entries are loaded before the current rows' multiply-adds, 2 U loads a lane and
+// column in flight.  Plain loads: V, W and x change between the columns of a panel.
+template <int U, bool kPair, bool kSmem>
+__device__ __forceinline__ void warp_dots(const double* p1, const double* p2, int64_t m, const double* s_x,
+                                          const double* xk, double& s1, double& s2) {
   const int lane = threadIdx.x & 31;
-  int o = 16;
+  double a1 = 0.0, a2 = 0.0, c1[U], c2[U];
 #pragma unroll
-  for (int cnt = C; cnt > 1; cnt >>= 1, o >>= 1) {
-    const int half = cnt >> 1;
-    const bool up = lane & o;
+  for (int u = 0; u < U; ++u) {
+    const int64_t i = lane + 32 * u;
+    c1[u] = i < m ? p1[i] : 0.0;
+    if (kPair) c2[u] = i < m ? p2[i] : 0.0;
+  }
+  for (int64_t i0 = lane; i0 < m; i0 += 32 * U) {
+    double n1[U], n2[U];
 #pragma unroll
-    for (int i = 0; i < half; ++i) {
-      const double send = up ? v[i] : v[i + half], keep = up ? v[i + half] : v[i];
-      v[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+    for (int u = 0; u < U; ++u) {
+      const int64_t i = i0 + 32 * (U + u);
+      n1[u] = i < m ? p1[i] : 0.0;
+      if (kPair) n2[u] = i < m ? p2[i] : 0.0;
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int64_t i = i0 + 32 * u;
+      if (i < m) {
+        const double x = kSmem ? s_x[i] : (i == 0 ? 0.0 : xk[i]);
+        a1 = fma(c1[u], x, a1);
+        if (kPair) a2 = fma(c2[u], x, a2);
+      }
+      c1[u] = n1[u];
+      if (kPair) c2[u] = n2[u];
     }
   }
-  double r = v[0];
-#pragma unroll
-  for (; o > 0; o >>= 1) r += __shfl_xor_sync(0xffffffffu, r, o);
-  return r;
-}
-
-// Dots of nc <= C columns (base + q * stride, q < nc) with v over m rows: the block's
-// threads stride over the rows, loading the next row's entries before the current row's
-// multiply-adds, then reduce per column; writes y / pw / pv on threads q < nc and returns
-// (thread 0) sum_q v_col(q) dot_q for the A columns.
-template <int C, bool kSmem>
-__device__ __forceinline__ double chunk_dots(const double* base, int64_t stride, int nc, int64_t m,
-                                             const double* s_x, const double* xk, double sc, double* s_part,
-                                             double* s_vy, const TrdPanel& P, int64_t k, int kind, int64_t c0) {
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int32_t st32 = (int32_t)stride;
-  const int64_t bd = blockDim.x;
-  double acc[C], cur[C];
-#pragma unroll
-  for (int q = 0; q < C; ++q) {
-    acc[q] = 0.0;
-    cur[q] = (tid < m && q < nc) ? base[tid + q * st32] : 0.0;
-  }
-  for (int64_t i = tid; i < m; i += bd) {
-    const int64_t i2 = i + bd;
-    double nxt[C];
-#pragma unroll
-    for (int q = 0; q < C; ++q) nxt[q] = (i2 < m && q < nc) ? base[i2 + q * st32] : 0.0;
-    const double v = i == 0 ? 1.0 : (kSmem ? s_x[i] : xk[i]) * sc;
-#pragma unroll
-    for (int q = 0; q < C; ++q) {
-      if (q < nc) acc[q] = fma(cur[q], v, acc[q]);
-      cur[q] = nxt[q];
-    }
-  }
-  constexpr int kSpan = 32 / C;
-  const double r = warp_reduce_cols<C>(acc);
-  if ((lane & (kSpan - 1)) == 0) s_part[warp * kProdChunk + lane / kSpan] = r;
-  __syncthreads();
-  if (tid < nc) {
-    double t = 0.0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += s_part[w * kProdChunk + tid];
-    const int64_t c = c0 + tid;  // index within its kind
-    if (kind == 0) {
-      P.y[k + 1 + c] = t;
-      s_vy[tid] = (c == 0 ? 1.0 : (kSmem ? s_x[c] : xk[c]) * sc) * t;
-    } else if (kind == 1) {
-      P.pw[c] = t;
-    } else {
-      P.pv[c] = t;
-    }
-  }
-  __syncthreads();
-  double vy = 0.0;
-  if (kind == 0 && tid == 0)
-    for (int q = 0; q < nc; ++q) vy += s_vy[q];
-  return vy;
-}
-
-template <bool kSmem>
-__device__ __forceinline__ double chunk_dots_n(const double* base, int64_t stride, int nc, int64_t m,
-                                               const double* s_x, const double* xk, double sc, double* s_part,
-                                               double* s_vy, const TrdPanel& P, int64_t k, int kind, int64_t c0) {
-  if (nc > 8) return chunk_dots<16, kSmem>(base, stride, nc, m, s_x, xk, sc, s_part, s_vy, P, k, kind, c0);
-  if (nc > 4) return chunk_dots<8, kSmem>(base, stride, nc, m, s_x, xk, sc, s_part, s_vy, P, k, kind, c0);
-  if (nc > 2) return chunk_dots<4, kSmem>(base, stride, nc, m, s_x, xk, sc, s_part, s_vy, P, k, kind, c0);
-  if (nc > 1) return chunk_dots<2, kSmem>(base, stride, nc, m, s_x, xk, sc, s_part, s_vy, P, k, kind, c0);
-  return chunk_dots<1, kSmem>(base, stride, nc, m, s_x, xk, sc, s_part, s_vy, P, k, kind, c0);
+  if (kPair) warp_sum2(a1, a2);
+  else a1 = warp_sum(a1);
+  s1 = a1;
+  s2 = a2;
 }
 
 // The symv A22 v and the panel dots W^T v, V^T v as column dots over rows k+1..n-1: the m
-// columns of A22 are cut into equal runs over the blocks, and so are the 2j panel
-// columns (j of W, then j of V); a block takes its runs kProdChunk columns at a time.
-// v_0 = 1 and v_i = x_i sc, x from the shared copy (kSmem) or from global memory.
-// Returns (thread 0) the block's part of v^T A22 v.
+// columns of A22 and the 2j panel columns (j of W, then j of V) form one list cut into equal
+// runs over the blocks; a warp takes whole columns of its block's run, two at a time, so that
+// a column costs five FP64 additions of reduction and no block barrier (rows over the block's
+// 512 threads, 16 columns at a time, took 4,100 clocks of additions and two barriers per
+// chunk: 72 -> 48 us a column at order 4096, 29 -> 19 at 2000).  v_0 = 1 and v_i = x_i sc: the sums run over
+// x_i, i >= 1, and are scaled once.  x from the shared copy (kSmem, its entry 0 zero) or from
+// global memory.  Returns (lane 0 of each warp) its part of v^T A22 v.
 template <bool kSmem>
-__device__ double panel_products(const TrdPanel& P, int64_t k, int j, double sc, const double* s_x,
-                                 double* s_part, double* s_vy) {
+__device__ double panel_products(const TrdPanel& P, int64_t k, int j, double sc, const double* s_x) {
   const int64_t n = P.n, m = n - k - 1;
-  const double* __restrict__ xk = P.x + k + 1;
+  const double* xk = P.x + k + 1;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  constexpr int kWarps = kTrdThreads / 32;
+  const int64_t items = m + 2 * (int64_t)j;
+  const int64_t per = (items + gridDim.x - 1) / gridDim.x;
+  const int64_t i0 = blockIdx.x * per, i1 = i0 + per < items ? i0 + per : items;
+  auto column = [&](int64_t t) -> const double* {
+    if (t < m) return P.A + (k + 1 + t) * P.lda + k + 1;
+    return (t < m + j ? P.W + (t - m) * n : P.V + (t - m - j) * n) + k + 1;
+  };
   double vy = 0.0;
-  {
-    const int64_t per = (m + gridDim.x - 1) / gridDim.x;
-    const int64_t c0 = blockIdx.x * per, c1 = c0 + per < m ? c0 + per : m;
-    for (int64_t cb = c0; cb < c1; cb += kProdChunk) {
-      const int nc = (int)(c1 - cb < kProdChunk ? c1 - cb : kProdChunk);
-      vy += chunk_dots_n<kSmem>(P.A + (k + 1 + cb) * P.lda + k + 1, P.lda, nc, m, s_x, xk, sc, s_part, s_vy, P,
-                                k, 0, cb);
-    }
-  }
-  const int64_t items = 2 * (int64_t)j;
-  if (items > 0) {
-    const int64_t per = (items + gridDim.x - 1) / gridDim.x;
-    const int64_t c0 = blockIdx.x * per, c1 = c0 + per < items ? c0 + per : items;
-    for (int64_t cb = c0; cb < c1;) {
-      const int kind = cb < j ? 1 : 2;
-      const int64_t seg_end = cb < j ? j : items, lim = c1 < seg_end ? c1 : seg_end;
-      const int nc = (int)(lim - cb < kProdChunk ? lim - cb : kProdChunk);
-      const int64_t col = kind == 1 ? cb : cb - j;
-      const double* base = (kind == 1 ? P.W : P.V) + col * n + k + 1;
-      chunk_dots_n<kSmem>(base, n, nc, m, s_x, xk, sc, s_part, s_vy, P, k, kind, col);
-      cb += nc;
+  for (int64_t t = i0 + warp; t < i1; t += 2 * kWarps) {
+    const int64_t t2 = t + kWarps;
+    const double* p1 = column(t);
+    const double* p2 = t2 < i1 ? column(t2) : nullptr;
+    double s1, s2 = 0.0;
+    if (p2) warp_dots<4, true, kSmem>(p1, p2, m, s_x, xk, s1, s2);
+    else warp_dots<8, false, kSmem>(p1, p1, m, s_x, xk, s1, s2);
+    if (lane == 0) {
+      for (int h = 0; h < 2; ++h) {
+        const int64_t c = h ? t2 : t;
+        if (h && !p2) break;
+        const double d = fma(sc, h ? s2 : s1, h ? p2[0] : p1[0]);
+        if (c < m) {
+          P.y[k + 1 + c] = d;
+          vy = fma(c == 0 ? 1.0 : (kSmem ? s_x[c] : xk[c]) * sc, d, vy);
+        } else if (c < m + j) {
+          P.pw[c - m] = d;
+        } else {
+          P.pv[c - m - j] = d;
+        }
+      }
     }
   }
   return vy;
@@ -245,14 +234,11 @@ __global__ void __launch_bounds__(kTrdThreads, 1) k_trd_panel(TrdPanel P) {
   extern __shared__ double s_x[];  // x(k+1 : n) when P.vsm
   __shared__ double s_vk[kTrdNb], s_wk[kTrdNb], s_pw[kTrdNb], s_pv[kTrdNb];
   __shared__ double s_red[kTrdThreads / 32];
-  __shared__ double s_part[(kTrdThreads / 32) * kProdChunk];
-  __shared__ double s_vy[kProdChunk];
   __shared__ double s_scal[8];
   __shared__ int s_flag;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   constexpr int kWarps = kTrdThreads / 32;
   const int64_t n = P.n, ld = P.n;
-  const int64_t G = (int64_t)gridDim.x * blockDim.x, g = (int64_t)blockIdx.x * blockDim.x + tid;
   const int64_t rstep = (int64_t)gridDim.x * kWarps;  // warp-per-row stride
   unsigned target = 0;
   double* __restrict__ A = P.A;
@@ -262,7 +248,7 @@ __global__ void __launch_bounds__(kTrdThreads, 1) k_trd_panel(TrdPanel P) {
   for (int j = 0; j < P.nbp; ++j) {
     const int64_t k = P.p + j;
     // ---- (1) finish w of column j-1, update column k with the panel so far
-    double tprev = 0.0, gam = 0.0;
+    double tprev = 0.0, hg = 0.0;  // tau of column j-1; tau^2 / 2 (v^T y - 2 pw^T pv)
     // the warp's first row: its loads go out with the prelude's
     const int64_t r0 = k + blockIdx.x + (int64_t)gridDim.x * warp;
     double vrc[4] = {0.0, 0.0, 0.0, 0.0}, wrc[4] = {0.0, 0.0, 0.0, 0.0};
@@ -285,19 +271,29 @@ __global__ void __launch_bounds__(kTrdThreads, 1) k_trd_panel(TrdPanel P) {
     }
     if (j > 0) {
       // one round trip: row k of the panel, the dots of column j-1, the partials of
-      // v^T A22 v, y_k and tau_{k-1}
-      for (int c = tid; c < j; c += blockDim.x) {
-        s_vk[c] = P.Vr[k * nb + c];
-        if (c < j - 1) {
-          s_pw[c] = P.pw[c];
-          s_pv[c] = P.pv[c];
-          s_wk[c] = P.Wr[k * nb + c];
+      // v^T A22 v, y_k and tau_{k-1}; warp 0 sums pw^T pv and row k's part as they arrive
+      if (warp == 0) {
+        double q = 0.0, f = 0.0;
+        for (int c = lane; c < j; c += 32) {
+          const double vk = P.Vr[k * nb + c];
+          s_vk[c] = vk;
+          if (c < j - 1) {
+            const double a = P.pw[c], b = P.pv[c], wk = P.Wr[k * nb + c];
+            s_pw[c] = a;
+            s_pv[c] = b;
+            s_wk[c] = wk;
+            q = fma(a, b, q);
+            f = fma(vk, a, fma(wk, b, f));
+          }
+        }
+        warp_sum2(q, f);
+        if (lane == 0) {
+          s_scal[7] = q;
+          s_scal[0] = f;
         }
       }
       if (warp == kWarps - 1) {
-        double t = 0.0;
-        for (int b = lane; b < (int)gridDim.x; b += 32) t += P.pvy[b];
-        t = warp_sum(t);
+        const double t = sum_blocks(P.pvy);
         if (lane == 0) {
           s_scal[4] = t;
           s_scal[5] = P.y[k];
@@ -306,22 +302,14 @@ __global__ void __launch_bounds__(kTrdThreads, 1) k_trd_panel(TrdPanel P) {
       }
       __syncthreads();
       tprev = s_scal[6];
-      if (warp == 0) {
-        double q = 0.0, f = 0.0;
-        for (int c = lane; c < j - 1; c += 32) {
-          q = fma(s_pw[c], s_pv[c], q);
-          f = fma(s_vk[c], s_pw[c], fma(s_wk[c], s_pv[c], f));
-        }
-        q = warp_sum(q);
-        f = warp_sum(f);
-        if (lane == 0) {
-          const double gm = tprev * (s_scal[4] - 2.0 * q);
-          s_scal[0] = gm;
-          s_wk[j - 1] = tprev * (s_scal[5] - f) - 0.5 * tprev * gm * s_vk[j - 1];
-        }
+      if (tid == 0) {
+        const double gm = tprev * fma(-2.0, s_scal[7], s_scal[4]);
+        const double h = 0.5 * tprev * gm;
+        s_wk[j - 1] = fma(-h, s_vk[j - 1], tprev * (s_scal[5] - s_scal[0]));
+        s_scal[1] = h;
       }
       __syncthreads();
-      gam = s_scal[0];
+      hg = s_scal[1];
     }
     double ss = 0.0;
     for (int64_t r = r0; r < n; r += rstep) {
@@ -352,12 +340,11 @@ __global__ void __launch_bounds__(kTrdThreads, 1) k_trd_panel(TrdPanel P) {
             u = fma(vrc[q], s_wk[c], fma(wrc[q], s_vk[c], u));
           }
         }
-        f = warp_sum(f);
-        u = warp_sum(u);
+        warp_sum2(f, u);
       }
       if (lane == 0) {
         if (j > 0) {
-          const double wr = (r == k) ? s_wk[j - 1] : tprev * (yv - f) - 0.5 * tprev * gam * vlast;
+          const double wr = (r == k) ? s_wk[j - 1] : fma(-hg, vlast, tprev * (yv - f));
           P.W[r + (j - 1) * ld] = wr;
           P.Wr[r * nb + j - 1] = wr;
           u = fma(vlast, s_wk[j - 1], fma(wr, s_vk[j - 1], u));
@@ -381,20 +368,16 @@ __global__ void __launch_bounds__(kTrdThreads, 1) k_trd_panel(TrdPanel P) {
     // ---- (2) the reflector of column k (one round trip: the partials and x), then A22 v
     // and the panel dots
     const int64_t m = n - k - 1;
-    if (P.vsm)
-      for (int64_t i = tid; i < m; i += blockDim.x) s_x[i] = P.x[k + 1 + i];
-    if (warp == 0) {
+    if (warp != 0) {  // warp 0 has the reflector
+      if (P.vsm)
+        for (int64_t i = tid - 32; i < m; i += kTrdThreads - 32) s_x[i] = i == 0 ? 0.0 : P.x[k + 1 + i];
+    } else {
       const double alpha = P.x[k + 1];
-      double s = 0.0;
-      for (int b = lane; b < (int)gridDim.x; b += 32) s += P.ps[b];
-      s = warp_sum(s);
+      const double s = sum_blocks(P.ps);
       if (lane == 0) {
         double t = 0.0, beta = alpha, sc = 0.0;
         if (s > 0.0) {
-          const double nrm = sqrt(fma(alpha, alpha, s));
-          beta = -copysign(nrm, alpha);
-          t = (beta - alpha) / beta;
-          sc = 1.0 / (alpha - beta);
+          reflector(alpha, s, t, beta, sc);
         }
         s_scal[1] = t;
         s_scal[2] = sc;
@@ -403,19 +386,24 @@ __global__ void __launch_bounds__(kTrdThreads, 1) k_trd_panel(TrdPanel P) {
     }
     __syncthreads();
     const double sc = s_scal[2];
-    if (g == 0) {
+    if (blockIdx.x == 0 && tid == 0) {
       P.tau[k] = s_scal[1];
       P.e[k] = s_scal[3];
       A[k + 1 + k * lda] = s_scal[3];
     }
-    for (int64_t r = P.p + 1 + g; r < n; r += G) {
-      const double v = r <= k ? 0.0 : (r == k + 1 ? 1.0 : (P.vsm ? s_x[r - k - 1] : P.x[r]) * sc);
-      P.V[r + j * ld] = v;
-      P.Vr[r * nb + j] = v;
-      if (r >= k + 2) A[r + k * lda] = v;
+    // v to the panel and the reduced matrix: the block's run of rows, by its last warp
+    if (warp == kWarps - 1) {
+      const int64_t rows = n - P.p - 1, per = (rows + gridDim.x - 1) / gridDim.x;
+      const int64_t ra = P.p + 1 + blockIdx.x * per, rb = ra + per < n ? ra + per : n;
+      for (int64_t r = ra + lane; r < rb; r += 32) {
+        const double v = r <= k ? 0.0 : (r == k + 1 ? 1.0 : (P.vsm ? s_x[r - k - 1] : P.x[r]) * sc);
+        P.V[r + j * ld] = v;
+        P.Vr[r * nb + j] = v;
+        if (r >= k + 2) A[r + k * lda] = v;
+      }
     }
-    const double vy = P.vsm ? panel_products<true>(P, k, j, sc, s_x, s_part, s_vy)
-                            : panel_products<false>(P, k, j, sc, s_x, s_part, s_vy);
+    const double vy = block_sum_lane0(P.vsm ? panel_products<true>(P, k, j, sc, s_x)
+                                            : panel_products<false>(P, k, j, sc, s_x), s_red);
     if (tid == 0) P.pvy[blockIdx.x] = vy;
     if (!grid_barrier(P.bar, target, P.budget, P.status, &s_flag)) return;
   }
@@ -585,17 +573,7 @@ __global__ void __launch_bounds__(kResThreads, 1) k_trd_resident(TrdResident P) 
         const double alpha = s_alpha;
         double t = 0.0, beta = alpha, sc = 0.0;
         if (s > 0.0) {
-          const double t2 = fma(alpha, alpha, s);
-          if (in_range(t2)) {
-            const double ri = -copysign(rsqrt_cubic(t2), alpha);  // 1 / beta
-            beta = t2 * ri;
-            sc = rcp_nr(alpha - beta);
-            t = (beta - alpha) * ri;
-          } else {
-            beta = -copysign(sqrt(t2), alpha);
-            t = (beta - alpha) / beta;
-            sc = 1.0 / (alpha - beta);
-          }
+          reflector(alpha, s, t, beta, sc);
         }
         s_tau = t;
         s_sc = sc;
