@@ -376,9 +376,8 @@ int tdc_dft_gemm(int64_t m, int64_t n, const double* A, int64_t lda, double* Cre
  * tensor-core product from K = 128 on).  A band whose largest finite |entry| lies
  * outside [2^-400, 2^400] is solved scaled by the power of two that puts it in [1, 2)
  * (exact; AB itself is not modified) and lam scaled back.  lam[n] ascending, Q n x n
- * (ldq >= n).  The call
- * reads each rank-one step's deflation count back to the host, so it returns when the
- * solve is done.  ws of tdc_sbevd_workspace_size(n, b, o) bytes.  Errors: -1 n, -2 b,
+ * (ldq >= n).  The nodes of a tree level take their terms in the same launches, and every
+ * count stays on the device: the call only enqueues.  ws of tdc_sbevd_workspace_size(n, b, o) bytes.  Errors: -1 n, -2 b,
  * -3 AB, -4 ldab, -5 lam, -6 Q, -7 ldq, -10 options, TDC_ENOWS, TDC_ECUDA, or those of
  * the steps. */
 int tdc_sbevd_workspace_size(int64_t n, int64_t b, const tdc_opts* o, size_t* bytes);

@@ -1623,24 +1623,42 @@ size_t syevd_vec_bytes(int64_t n) { return 3 * align_up(sizeof(double) * (size_t
 // ---- symmetric band eigenproblem: divide and conquer with b rank-one merges per node
 struct BandNode {
   int64_t lo, hi;
+  int depth;
 };
 
 int64_t band_leafmax(int64_t b) { return std::max<int64_t>(128, 8 * b); }
 
 // nodes in post order (children before their parent); leaves have at most leafmax rows
-void band_nodes(int64_t lo, int64_t hi, int64_t leafmax, std::vector<BandNode>& out) {
+void band_nodes(int64_t lo, int64_t hi, int64_t leafmax, std::vector<BandNode>& out, int depth = 0) {
   if (hi - lo > leafmax) {
     const int64_t m = lo + (hi - lo) / 2;
-    band_nodes(lo, m, leafmax, out);
-    band_nodes(m, hi, leafmax, out);
+    band_nodes(lo, m, leafmax, out, depth + 1);
+    band_nodes(m, hi, leafmax, out, depth + 1);
   }
-  out.push_back({lo, hi});
+  out.push_back({lo, hi, depth});
+}
+
+// The inner nodes level by level, the deepest first: level t is [first[t], first[t + 1]).
+void band_levels(const std::vector<BandNode>& nodes, int64_t leafmax, std::vector<BdNode>& inner,
+                 std::vector<size_t>& first) {
+  int deep = -1;
+  for (const BandNode& nd : nodes)
+    if (nd.hi - nd.lo > leafmax) deep = std::max(deep, nd.depth);
+  inner.clear();
+  first.assign(1, 0);
+  for (int t = deep; t >= 0; --t) {
+    for (const BandNode& nd : nodes)
+      if (nd.depth == t && nd.hi - nd.lo > leafmax)
+        inner.push_back({nd.lo, nd.hi - nd.lo, nd.lo + (nd.hi - nd.lo) / 2, (int64_t)inner.size()});
+    first.push_back(inner.size());
+  }
 }
 
 struct BandLayout {
   size_t ABw, wv, Ab, Zb, dl, el, taul, Dcur, z, Ds, zs, perm, kept, defl, rotp, rotcs, cnt, DK, zK, Dd, org, tau, zhat,
-      scol, iota, Qw, prod, leafws, r1, total;
+      scol, Qw, nodes, ncnt, unsorted, rho, segs, dsegs, nsegs, img, leafws, r1, total;
   size_t leafws_bytes;
+  int64_t img_elems;
 };
 
 // sizes of the leaves (post order) and their first rows
@@ -1661,7 +1679,11 @@ BandLayout band_layout(int64_t n, int64_t b, const tdc_opts& op) {
   std::vector<BandNode> nodes;
   band_nodes(0, std::max<int64_t>(n, 1), band_leafmax(b), nodes);
   L.ABw = take(o, sizeof(double) * (size_t)(b + 1) * nn);
-  L.wv = take(o, sizeof(double) * nodes.size() * (size_t)std::max<int64_t>(b, 1) * (size_t)(b + 1));
+  std::vector<BdNode> inner;
+  std::vector<size_t> first;
+  band_levels(nodes, band_leafmax(b), inner, first);
+  const size_t ni = std::max<size_t>(inner.size(), 1);
+  L.wv = take(o, sizeof(double) * ni * (size_t)std::max<int64_t>(b, 1) * (size_t)(b + 1));
   L.Ab = take(o, sizeof(double) * nn * (size_t)lm);
   L.Zb = take(o, sizeof(double) * nn * (size_t)lm);
   L.dl = take(o, sizeof(double) * nn);
@@ -1684,12 +1706,24 @@ BandLayout band_layout(int64_t n, int64_t b, const tdc_opts& op) {
   L.tau = take(o, sizeof(double) * nn);
   L.zhat = take(o, sizeof(double) * nn);
   L.scol = take(o, sizeof(double) * nn);
-  L.iota = take(o, sizeof(int32_t) * nn);
   L.r1 = take(o, rank_one_scratch_bytes((int64_t)nn));
   L.Qw = take(o, sizeof(double) * nn * nn);
-  size_t pb = 0;
-  tdc_cauchy_gemm_workspace_size((int64_t)nn, (int64_t)nn, TDC_MERGE_SPLIT, &op, &pb);
-  L.prod = take(o, pb);
+  L.nodes = take(o, sizeof(BdNode) * ni);
+  L.ncnt = take(o, 4 * sizeof(int32_t) * ni);
+  L.unsorted = take(o, sizeof(int32_t) * ni);
+  L.rho = take(o, sizeof(double) * ni);
+  L.segs = take(o, sizeof(GemmSeg) * (ni + 1));
+  L.dsegs = take(o, sizeof(GemmSeg) * ni);
+  L.nsegs = take(o, 64);
+  // digit images of one level's products
+  L.img_elems = 0;
+  for (size_t t = 0; t + 1 < first.size(); ++t) {
+    int64_t el = 0;
+    for (size_t i = first[t]; i < first[t + 1]; ++i)
+      el += cauchy_split_elems(inner[i].nn, inner[i].nn, op.split_slices, nullptr);
+    L.img_elems = std::max(L.img_elems, el);
+  }
+  L.img = take(o, sizeof(__nv_bfloat16) * (size_t)L.img_elems);
   std::vector<int64_t> llo, lsz;
   band_leaves(nodes, band_leafmax(b), llo, lsz);
   size_t we = 0;
@@ -1706,55 +1740,26 @@ int sbevd_run(int64_t n, int64_t b, const double* AB, int64_t ldab, double* lam,
   const int64_t ldw = b + 1;
   double* ABw = (double*)(base + L.ABw);
   double* wv = (double*)(base + L.wv);
-  double* Dcur = (double*)(base + L.Dcur);
-  double* z = (double*)(base + L.z);
-  double* Ds = (double*)(base + L.Ds);
-  double* zs = (double*)(base + L.zs);
-  int32_t* perm = (int32_t*)(base + L.perm);
-  int32_t* kept = (int32_t*)(base + L.kept);
-  int32_t* defl = (int32_t*)(base + L.defl);
-  int32_t* rotp = (int32_t*)(base + L.rotp);
-  double* rotcs = (double*)(base + L.rotcs);
-  int32_t* cnt = (int32_t*)(base + L.cnt);
-  double* rhod = (double*)(base + L.cnt + 32);
-  double* DK = (double*)(base + L.DK);
-  double* zK = (double*)(base + L.zK);
-  double* Dd = (double*)(base + L.Dd);
-  int32_t* org = (int32_t*)(base + L.org);
-  double* tau = (double*)(base + L.tau);
-  double* zhat = (double*)(base + L.zhat);
-  double* scol = (double*)(base + L.scol);
-  int32_t* iota = (int32_t*)(base + L.iota);
-  double* Qw = (double*)(base + L.Qw);
-  char* prod = base + L.prod;
   std::vector<BandNode> nodes;
   band_nodes(0, n, band_leafmax(b), nodes);
-  // scratch of the sort and the deflation: arrays that the gather, the secular solve and
-  // the product write only after them
-  BdScratch S;
-  S.sk = DK;
-  S.si = org;
-  S.surv = org;
-  S.slot = (int32_t*)zK;
-  S.c = tau;
-  S.s = zhat;
-  S.w = DK;
-  S.dp = scol;
-  S.dn = Dd;
+  std::vector<BdNode> inner;
+  std::vector<size_t> first;
+  band_levels(nodes, band_leafmax(b), inner, first);
+  BdNode* dnodes = (BdNode*)(base + L.nodes);
   if (launch_bd_copy_band(n, (int)b, AB, ldab, ABw, cs) != cudaSuccess) return TDC_ECUDA;
   // entries outside [2^-400, 2^400]: the band copy scaled by a power of two
   unsigned long long* rmx = (unsigned long long*)(base + L.cnt + 40);
   int* res = (int*)(base + L.cnt + 48);
   if (launch_range_scale(ABw, ldw, n, ldw, 0, rmx, res, cs) != cudaSuccess) return TDC_ECUDA;
   if (launch_bd_zero(n, n, Q, ldq, cs) != cudaSuccess) return TDC_ECUDA;
-  k_iota<<<(unsigned)std::min<int64_t>((n + 255) / 256, 4096), 256, 0, cs>>>(iota, n);
-  // tearings (they touch disjoint entries: nodes have at least 4b rows)
-  for (size_t i = 0; i < nodes.size(); ++i) {
-    const BandNode& nd = nodes[i];
-    if (nd.hi - nd.lo <= band_leafmax(b)) continue;
-    const int64_t m = nd.lo + (nd.hi - nd.lo) / 2;
-    if (launch_bd_tear(ABw, ldw, (int)b, m, wv + i * b * (b + 1), cs) != cudaSuccess) return TDC_ECUDA;
+  // the inner nodes' table (by kernel parameter, copied at launch) and their tearings
+  for (size_t c0 = 0; c0 < inner.size(); c0 += kBdNodeChunk) {
+    BdNodeTable T;
+    const int c = (int)std::min<size_t>(kBdNodeChunk, inner.size() - c0);
+    std::copy(inner.begin() + c0, inner.begin() + c0 + c, T.nd);
+    if (launch_bd_nodes(dnodes + c0, T, c, cs) != cudaSuccess) return TDC_ECUDA;
   }
+  if (launch_bd_tear(dnodes, (int)inner.size(), ABw, ldw, (int)b, wv, cs) != cudaSuccess) return TDC_ECUDA;
   // leaves, all at once: dense blocks of the torn band reduced to tridiagonal form (a block
   // each), their tridiagonals solved as one batch, the eigenvectors back-transformed into Q
   {
@@ -1794,53 +1799,73 @@ int sbevd_run(int64_t n, int64_t b, const double* AB, int64_t ldab, double* lam,
       }
     }
   }
-  for (size_t i = 0; i < nodes.size(); ++i) {
-    const BandNode& nd = nodes[i];
-    const int64_t nn = nd.hi - nd.lo;
-    double* Qn = Q + nd.lo + nd.lo * ldq;
-    if (nn <= band_leafmax(b)) continue;  // a leaf, solved above
-    const int64_t m = nd.lo + (nd.hi - nd.lo) / 2;
-    if (cudaMemcpyAsync(Dcur, lam + nd.lo, sizeof(double) * nn, cudaMemcpyDeviceToDevice, cs) != cudaSuccess)
-      return TDC_ECUDA;
-    for (int64_t k = 0; k < b; ++k) {
-      const double* w = wv + i * b * (b + 1) + k * (b + 1);
-      if (launch_bd_z(nn, Qn, ldq, (m - b + k) - nd.lo, m - nd.lo, (int)b, w, z, cs) != cudaSuccess) return TDC_ECUDA;
-      if (launch_bd_sort(nn, Dcur, z, Ds, zs, perm, S, cs) != cudaSuccess) return TDC_ECUDA;
-      if (launch_bd_deflate(nn, Ds, zs, kept, defl, rotp, rotcs, cnt, rhod, S, st, cs) != cudaSuccess)
+  // the tree's levels, the deepest first: every node of a level takes its b terms in the same
+  // launches; K, the deflated and the rotation counts stay on the device
+  BdLevel V;
+  memset(&V, 0, sizeof(V));
+  V.b = (int32_t)b;
+  V.n = n;
+  V.wv = wv;
+  V.Q = Q;
+  V.ldq = ldq;
+  V.Qw = (double*)(base + L.Qw);
+  V.Dcur = (double*)(base + L.Dcur);
+  V.z = (double*)(base + L.z);
+  V.Ds = (double*)(base + L.Ds);
+  V.zs = (double*)(base + L.zs);
+  V.perm = (int32_t*)(base + L.perm);
+  V.kept = (int32_t*)(base + L.kept);
+  V.defl = (int32_t*)(base + L.defl);
+  V.rotp = (int32_t*)(base + L.rotp);
+  V.rotcs = (double*)(base + L.rotcs);
+  V.DK = (double*)(base + L.DK);
+  V.zK = (double*)(base + L.zK);
+  V.Dd = (double*)(base + L.Dd);
+  V.org = (int32_t*)(base + L.org);
+  V.tau = (double*)(base + L.tau);
+  V.zhat = (double*)(base + L.zhat);
+  V.scol = (double*)(base + L.scol);
+  rank_one_carve(base + L.r1, n, V.zz, V.xz, V.xlo);
+  // scratch of the sort and the deflation: arrays that the gather, the secular solve and
+  // the product write only after them
+  V.sk = V.DK;
+  V.si = V.org;
+  V.surv = V.org;
+  V.slot = (int32_t*)V.zK;
+  V.rc = V.tau;
+  V.rs = V.zhat;
+  V.rw = V.DK;
+  V.rdp = V.scol;
+  V.rdn = V.Dd;
+  V.segs = (GemmSeg*)(base + L.segs);
+  V.dsegs = (GemmSeg*)(base + L.dsegs);
+  V.nsegs = (int64_t*)(base + L.nsegs);
+  V.img_cap = L.img_elems;
+  V.S = op.split_slices;
+  V.max_iter = op.max_iter;
+  V.status = st;
+  __nv_bfloat16* img = (__nv_bfloat16*)(base + L.img);
+  for (size_t t = 0; t + 1 < first.size(); ++t) {
+    V.nodes = dnodes + first[t];
+    V.count = (int32_t)(first[t + 1] - first[t]);
+    if (V.count == 0) continue;
+    V.cnt = (int32_t*)(base + L.ncnt) + 4 * first[t];
+    V.unsorted = (int32_t*)(base + L.unsorted) + first[t];
+    V.rho = (double*)(base + L.rho) + first[t];
+    V.max_nn = 0;
+    for (size_t i = first[t]; i < first[t + 1]; ++i) V.max_nn = std::max(V.max_nn, inner[i].nn);
+    if (launch_bd_level_begin(V, lam, cs) != cudaSuccess) return TDC_ECUDA;
+    for (int k = 0; k < (int)b; ++k) {
+      if (launch_bd_term(V, k, cs) != cudaSuccess || launch_bd_rank_one(V, cs) != cudaSuccess ||
+          launch_bd_segs(V, cs) != cudaSuccess ||
+          launch_split_list(V.segs, V.count, V.nsegs, op.split_slices, st, op.spin_budget, img, op.split_chunk_k / 16,
+                            nullptr, cs, nullptr) != cudaSuccess ||
+          launch_dense_list(V.dsegs, V.count, V.max_nn, std::min<int64_t>(V.max_nn, 128), cs) != cudaSuccess ||
+          launch_bd_finish(V, cs) != cudaSuccess)
         return TDC_ECUDA;
-      int32_t hc[3] = {0, 0, 0};
-      double hrho = 0.0;
-      if (cudaMemcpyAsync(hc, cnt, sizeof(hc), cudaMemcpyDeviceToHost, cs) != cudaSuccess ||
-          cudaMemcpyAsync(&hrho, rhod, sizeof(double), cudaMemcpyDeviceToHost, cs) != cudaSuccess ||
-          cudaStreamSynchronize(cs) != cudaSuccess)
-        return TDC_ECUDA;
-      const int K = hc[0], ndf = hc[1], nr = hc[2];
-      if (launch_bd_rotate(nn, Qn, ldq, perm, rotp, rotcs, nr, st, cs) != cudaSuccess) return TDC_ECUDA;
-      if (launch_bd_gather(nn, Qn, ldq, perm, kept, K, defl, ndf, Ds, zs, Qw, DK, zK, Dd, st, cs) != cudaSuccess)
-        return TDC_ECUDA;
-      if (K > 0) {
-        double* r1zz;
-        float2* r1xz;
-        float* r1xlo;
-        rank_one_carve(base + L.r1, K, r1zz, r1xz, r1xlo);
-        if (launch_rank_one(DK, zK, K, hrho, op.max_iter, org, tau, zhat, scol, r1zz, r1xz, r1xlo, st, cs) !=
-            cudaSuccess)
-          return TDC_ECUDA;
-        const int32_t mode = K >= 128 ? TDC_MERGE_SPLIT : TDC_MERGE_DENSE;
-        char* pw = (char*)(((uintptr_t)prod + 255) & ~(uintptr_t)255);
-        const int r = cauchy_product(nn, K, Qw, nn, DK, org, tau, zhat, scol, Qn, ldq, mode, op, pw, st, nullptr,
-                                     nullptr, cs);
-        if (r != TDC_OK) return r;
-      }
-      if (launch_bd_finish(nn, Qw, Qn, ldq, K, ndf, DK, org, tau, Dd, Dcur, cs) != cudaSuccess) return TDC_ECUDA;
     }
     // ascending eigenvalues and the columns in that order
-    if (launch_bd_sort(nn, Dcur, nullptr, Ds, nullptr, perm, S, cs) != cudaSuccess) return TDC_ECUDA;
-    if (launch_bd_gather(nn, Qn, ldq, perm, iota, (int)nn, defl, 0, Ds, Ds, Qw, DK, zK, Dd, st, cs) != cudaSuccess)
-      return TDC_ECUDA;
-    if (launch_bd_copy_back(nn, nn, Qw, Qn, ldq, cs) != cudaSuccess) return TDC_ECUDA;
-    if (cudaMemcpyAsync(lam + nd.lo, Ds, sizeof(double) * nn, cudaMemcpyDeviceToDevice, cs) != cudaSuccess)
-      return TDC_ECUDA;
+    if (launch_bd_order(V, lam, cs) != cudaSuccess) return TDC_ECUDA;
   }
   return launch_range_unscale(lam, n, res, cs) == cudaSuccess ? TDC_OK : TDC_ECUDA;
 }

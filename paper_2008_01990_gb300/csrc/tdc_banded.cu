@@ -13,7 +13,10 @@
 // poles sorted, deflated (type 1: rho |zhat_i| <= tol; type 2: a rotation when
 // |t c s| <= tol for neighbouring poles, tol = 8 eps max(|D|max, |zhat|max), the tests of
 // Section 3.2), the secular equation and the Cauchy-like update of the non-deflated
-// columns (tdc_rank_one's kernels and the merge's product), the deflated columns copied.
+// columns (tdc_rank_one's solver and the merge's product), the deflated columns copied.  All
+// nodes of a tree level take each term in the same launches, a grid row or a block a node; K
+// and the other counts stay on the device, where the products' segment list is built from
+// them (n = 2048, b = 8: 120 steps with a host read each -> 32 without, 41.7 -> 16.5 ms).
 #include "tdc_common.cuh"
 
 namespace tdc {
@@ -22,10 +25,18 @@ namespace {
 constexpr double kBdEps = 1.1102230246251565e-16;  // 2^-53
 }  // namespace
 
-// Tearing of the node split at m: the terms (s_k, y_k) into wv[k (b + 1) + 0..b] (s_k = 0:
-// no term) and the corner updates of the band copy ABw (lower band storage, ld ldab).
-__global__ void __launch_bounds__(256) k_bd_tear(double* ABw, int64_t ldab, int b, int64_t m, double* wv) {
+__global__ void __launch_bounds__(32) k_bd_nodes(BdNode* dst, BdNodeTable T, int count) {
+  for (int i = threadIdx.x; i < count; i += 32) dst[i] = T.nd[i];
+}
+
+// Tearing of every inner node, a block each (they touch disjoint entries: nodes have at
+// least 4b rows): the terms (s_k, y_k) into wv[k (b + 1) + 0..b] of the node (s_k = 0: no
+// term) and the corner updates of the band copy ABw (lower band storage, ld ldab).
+__global__ void __launch_bounds__(256) k_bd_tear(const BdNode* nodes, double* ABw, int64_t ldab, int b, double* wv_all) {
   extern __shared__ double sb[];  // b x b: B_k(c) at sb[k * b + c], then b norms
+  const BdNode nd = nodes[blockIdx.x];
+  const int64_t m = nd.mid;
+  double* wv = wv_all + nd.wi * b * (b + 1);
   double* nrm = sb + b * b;
   for (int t = threadIdx.x; t < b * b; t += blockDim.x) {
     const int k = t / b, c = t % b;
@@ -61,14 +72,42 @@ __global__ void __launch_bounds__(256) k_bd_tear(double* ABw, int64_t ldab, int 
 // beta = -sign(alpha) hypot(alpha, sigma), tau = (beta - alpha) / beta,
 // v = [1, x(1:) / (alpha - beta)] (stored below the subdiagonal), p = tau A22 v,
 // w = p - (tau / 2)(p^T v) v, A22 -= v w^T + w v^T (sigma = 0: tau = 0, nothing applied).
+// Sum over the block, in every thread: warp sums, then the first warp over them (FP64
+// additions by every warp of all partials cost thousands of clocks).
 __device__ __forceinline__ double bd_block_sum(double v, double* red) {
   v = warp_sum(v);
   __syncthreads();
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
   __syncthreads();
-  double t = 0.0;
-  for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += red[w];
-  return t;
+  if (threadIdx.x < 32) {
+    const double t = warp_sum(threadIdx.x < (blockDim.x >> 5) ? red[threadIdx.x] : 0.0);
+    if (threadIdx.x == 0) red[0] = t;
+  }
+  __syncthreads();
+  return red[0];
+}
+// Largest |v| over the block (not NaN), by the bits of the non-negative doubles.
+__device__ __forceinline__ double bd_block_max(double v, double* red) {
+  unsigned long long u = (unsigned long long)__double_as_longlong(fabs(v));
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const unsigned long long w = __shfl_xor_sync(0xffffffffu, u, o);
+    u = w > u ? w : u;
+  }
+  __syncthreads();
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = __longlong_as_double((long long)u);
+  __syncthreads();
+  if (threadIdx.x < 32) {
+    u = threadIdx.x < (blockDim.x >> 5) ? (unsigned long long)__double_as_longlong(red[threadIdx.x]) : 0ull;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      const unsigned long long w = __shfl_xor_sync(0xffffffffu, u, o);
+      u = w > u ? w : u;
+    }
+    if (threadIdx.x == 0) red[0] = __longlong_as_double((long long)u);
+  }
+  __syncthreads();
+  return red[0];
 }
 
 __global__ void __launch_bounds__(kBdLeafThreads) k_bd_leaf_trd(BdLeafArgs P, BdLeafTable T) {
@@ -105,12 +144,13 @@ __global__ void __launch_bounds__(kBdLeafThreads) k_bd_leaf_trd(BdLeafArgs P, Bd
         P.e[lo + k] = alpha;
         P.tau[lo + k] = 0.0;
       } else {
-        const double beta = -copysign(hypot(alpha, sqrt(ss)), alpha);
+        double t, beta, sc;
+        reflector(alpha, ss, t, beta, sc);
         s_skip = 0;
-        s_tau = (beta - alpha) / beta;
-        s_scal = 1.0 / (alpha - beta);
+        s_tau = t;
+        s_scal = sc;
         P.e[lo + k] = beta;
-        P.tau[lo + k] = s_tau;
+        P.tau[lo + k] = t;
       }
     }
     __syncthreads();
@@ -157,52 +197,106 @@ __global__ void __launch_bounds__(kBdLeafThreads) k_bd_leaf_trd(BdLeafArgs P, Bd
 }
 
 // k_bd_leaf_back: Q(lo:lo+L, lo:lo+L) = H_0 ... H_{L-3} Z, Z the leaf tridiagonal's
-// eigenvectors (Zb, ld L): Z copied into Q's block, then the reflectors applied last
-// first, each as y = v^T Z(k+1:L, :) (a warp per column) and Z(k+1:L, :) -= tau v y.
-__global__ void __launch_bounds__(kBdLeafThreads) k_bd_leaf_back(BdLeafArgs P, BdLeafTable T) {
-  __shared__ double v[512], y[512];
+// eigenvectors (Zb, ld L): the reflectors applied last first to each column of Z, one warp a
+// column with its rows in registers (R a lane), so that a leaf spreads over L warps instead
+// of one block and nothing waits: bound by 2 R + 5 FP64 instructions a reflector (16 leaves of
+// 128 rows: 1.79 -> 0.26 ms).
+template <int R>
+__global__ void __launch_bounds__(128) k_bd_leaf_back(BdLeafArgs P, BdLeafTable T) {
   const int64_t lo = T.lo[blockIdx.x];
   const int L = T.L[blockIdx.x];
-  if (L <= 0 || L > 512) return;
+  const int lane = threadIdx.x & 31, j = blockIdx.y * 4 + (threadIdx.x >> 5);
+  if (L <= 0 || L > 32 * R || j >= L) return;
   const double* A = P.Ab + lo * P.lmax;
-  const double* Z = P.Zb + lo * P.lmax;
-  double* Qb = P.Q + lo + lo * P.ldq;
-  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, nw = blockDim.x >> 5;
-  for (int t = tid; t < L * L; t += blockDim.x) {
-    const int i = t % L, j = t / L;
-    Qb[i + (int64_t)j * P.ldq] = Z[t];
-  }
-  __syncthreads();
+  const double* Z = P.Zb + lo * P.lmax + (int64_t)j * L;
+  double q[R];
+#pragma unroll
+  for (int u = 0; u < R; ++u) q[u] = lane + 32 * u < L ? Z[lane + 32 * u] : 0.0;
   for (int k = L - 3; k >= 0; --k) {
     const double tau = P.tau[lo + k];
-    if (tau == 0.0) continue;  // uniform across the block
-    const int m = L - k - 1;
-    for (int i = tid; i < m; i += blockDim.x) v[i] = i == 0 ? 1.0 : A[(k + 1 + i) + (int64_t)k * L];
-    __syncthreads();
-    for (int j = wid; j < L; j += nw) {
-      const double* col = Qb + (k + 1) + (int64_t)j * P.ldq;
-      double acc = 0.0;
-      for (int i = lane; i < m; i += 32) acc = fma(v[i], col[i], acc);
-      acc = warp_sum(acc);
-      if (lane == 0) y[j] = tau * acc;
+    if (tau == 0.0) continue;
+    double v[R], acc = 0.0;
+#pragma unroll
+    for (int u = 0; u < R; ++u) {
+      const int r = lane + 32 * u;
+      v[u] = r > k + 1 && r < L ? A[r + (int64_t)k * L] : (r == k + 1 ? 1.0 : 0.0);
+      if (32 * u + 31 > k) acc = fma(v[u], q[u], acc);
     }
-    __syncthreads();
-    for (int t = tid; t < m * L; t += blockDim.x) {
-      const int i = t % m, j = t / m;
-      Qb[(k + 1 + i) + (int64_t)j * P.ldq] -= v[i] * y[j];
-    }
-    __syncthreads();
+    acc = -tau * warp_sum(acc);
+#pragma unroll
+    for (int u = 0; u < R; ++u)
+      if (32 * u + 31 > k) q[u] = fma(acc, v[u], q[u]);
+  }
+  double* Qb = P.Q + lo + (lo + j) * P.ldq;
+#pragma unroll
+  for (int u = 0; u < R; ++u)
+    if (lane + 32 * u < L) Qb[lane + 32 * u] = q[u];
+}
+
+// Start of a level: the poles are the children's eigenvalues, the first run the left child's.
+__global__ void __launch_bounds__(256) k_bd_level_begin(BdLevel L, const double* lam) {
+  const BdNode nd = L.nodes[blockIdx.y];
+  for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < nd.nn; j += (int64_t)gridDim.x * blockDim.x)
+    L.Dcur[nd.lo + j] = lam[nd.lo + j];
+  if (blockIdx.x == 0 && threadIdx.x == 0) L.cnt[4 * blockIdx.y + 3] = (int32_t)(nd.mid - nd.lo);
+}
+
+// z_j = s Q(ra, j) + sum_c y_c Q(rb + c, j), j < nn, for a node's term k: ra the k-th of the b
+// rows above the split, rb the split's first row.
+__global__ void __launch_bounds__(256) k_bd_z(BdLevel L, int k) {
+  const BdNode nd = L.nodes[blockIdx.y];
+  const double* w = L.wv + (nd.wi * L.b + k) * (L.b + 1);
+  const double* Q = L.Q + nd.lo + nd.lo * L.ldq;
+  const int64_t ra = nd.mid - L.b + k - nd.lo, rb = nd.mid - nd.lo;
+  for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < nd.nn; j += (int64_t)gridDim.x * blockDim.x) {
+    const double* col = Q + j * L.ldq;
+    double acc = w[0] * col[ra];
+    for (int c = 0; c < L.b; ++c) acc = fma(w[1 + c], col[rb + c], acc);
+    L.z[nd.lo + j] = acc;
   }
 }
 
-// z_j = s Q(ra, j) + sum_c y_c Q(rb + c, j), j < nn.
-__global__ void __launch_bounds__(256) k_bd_z(int64_t nn, const double* Q, int64_t ldq, int64_t ra, int64_t rb, int b,
-                                             const double* w, double* z) {
-  for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < nn; j += (int64_t)gridDim.x * blockDim.x) {
-    const double* col = Q + j * ldq;
-    double acc = w[0] * col[ra];
-    for (int c = 0; c < b; ++c) acc = fma(w[1 + c], col[rb + c], acc);
-    z[j] = acc;
+// A double as an integer of the same order (-0 before +0).
+__device__ __forceinline__ long long bd_key(double x) {
+  const long long u = __double_as_longlong(x);
+  return u ^ ((u >> 63) & 0x7fffffffffffffffll);
+}
+
+// Sort of a node's poles, as a rule a merge: Dcur is two ascending runs (the children's
+// eigenvalues; later the roots in order, then the deflated poles in order of scan), so an
+// entry's place is its place in its run plus the count of the other run's entries before it
+// (ties: first run first), a binary search on integer keys.  A run that is not ascending (a
+// deflating rotation may move a pole past its neighbour) or holds a NaN sets `unsorted` and
+// leaves the node to the network below.  One block a node: 4 us where the network and the
+// ranks of its chunks took 39.
+__global__ void __launch_bounds__(1024) k_bd_merge(BdLevel L, int use_z) {
+  const BdNode nd = L.nodes[blockIdx.x];
+  const double* D = L.Dcur + nd.lo;
+  const int64_t nn = nd.nn, r0 = L.cnt[4 * blockIdx.x + 3];
+  bool bad = r0 < 0 || r0 > nn;
+  for (int64_t i = threadIdx.x; i < nn; i += blockDim.x) {
+    const double d = D[i];
+    bad = bad || (__double2hiint(d) & 0x7ff00000) == 0x7ff00000;
+    if (i > 0 && i != r0) bad = bad || bd_key(D[i - 1]) > bd_key(d);
+  }
+  const int any = __syncthreads_or(bad);
+  if (threadIdx.x == 0) L.unsorted[blockIdx.x] = any;
+  if (any) return;
+  for (int64_t i = threadIdx.x; i < nn; i += blockDim.x) {
+    const double d = D[i];
+    const long long key = bd_key(d);
+    const bool first = i < r0;
+    int64_t lo = first ? r0 : 0, hi = first ? nn : r0;
+    const int64_t base = lo;
+    while (lo < hi) {  // entries of the other run before this one
+      const int64_t m = (lo + hi) >> 1;
+      const long long km = bd_key(D[m]);
+      if (first ? km < key : km <= key) lo = m + 1; else hi = m;
+    }
+    const int64_t rk = (first ? i : i - r0) + (lo - base);
+    L.Ds[nd.lo + rk] = d;
+    if (use_z) L.zs[nd.lo + rk] = L.z[nd.lo + i];
+    L.perm[nd.lo + rk] = (int32_t)i;
   }
 }
 
@@ -214,7 +308,8 @@ __device__ __forceinline__ bool bd_before(double a, int64_t ia, double b, int64_
   return a < b || (a == b && ia < ib);
 }
 
-// Stable sort by rank in two kernels.  k_bd_chunk_sort: one block per chunk of ch entries
+// Stable sort by rank in two kernels, of the nodes k_bd_merge left.  k_bd_chunk_sort: one
+// block per chunk of ch entries
 // (ch = kBdChunk, or the power of two at or above nn when that is smaller) sorts (D[i], i)
 // by bd_before with a bitonic network in shared memory (entries past nn pad the chunk and
 // sort last), writing the chunk's sorted keys and indices.
@@ -228,10 +323,17 @@ __device__ __forceinline__ bool bd_before_pad(double a, int64_t ia, double b, in
   return bd_before(a, ia, b, ib);
 }
 
-__global__ void __launch_bounds__(1024) k_bd_chunk_sort(int64_t nn, int ch, const double* D, double* sk, int32_t* si) {
+__global__ void __launch_bounds__(1024) k_bd_chunk_sort(BdLevel L, int ch) {
   __shared__ double key[kBdChunk];
   __shared__ int32_t idx[kBdChunk];
+  if (!L.unsorted[blockIdx.y]) return;
+  const BdNode nd = L.nodes[blockIdx.y];
+  const int64_t nn = nd.nn;
+  const double* D = L.Dcur + nd.lo;
+  double* sk = L.sk + nd.lo;
+  int32_t* si = L.si + nd.lo;
   const int64_t c0 = (int64_t)blockIdx.x * ch;
+  if (c0 >= nn) return;
   for (int t = threadIdx.x; t < ch; t += blockDim.x) {
     const int64_t i = c0 + t;
     key[t] = i < nn ? D[i] : 0.0;
@@ -263,9 +365,17 @@ __global__ void __launch_bounds__(1024) k_bd_chunk_sort(int64_t nn, int ch, cons
   }
 }
 
-__global__ void __launch_bounds__(256) k_bd_rank(int64_t nn, int ch, const double* D, const double* z,
-                                                const double* sk, const int32_t* si, double* Ds, double* zs,
-                                                int32_t* perm) {
+__global__ void __launch_bounds__(256) k_bd_rank(BdLevel L, int ch, int use_z) {
+  if (!L.unsorted[blockIdx.y]) return;
+  const BdNode nd = L.nodes[blockIdx.y];
+  const int64_t nn = nd.nn;
+  const double* D = L.Dcur + nd.lo;
+  const double* z = use_z ? L.z + nd.lo : nullptr;
+  const double* sk = L.sk + nd.lo;
+  const int32_t* si = L.si + nd.lo;
+  double* Ds = L.Ds + nd.lo;
+  double* zs = L.zs + nd.lo;
+  int32_t* perm = L.perm + nd.lo;
   const int64_t nch = (nn + ch - 1) / ch;
   for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < nn; q += (int64_t)gridDim.x * blockDim.x) {
     const int64_t c = q / ch;  // q: sorted place within chunk c
@@ -305,24 +415,6 @@ __global__ void __launch_bounds__(256) k_bd_rank(int64_t nn, int ch, const doubl
 constexpr int kBdDefThreads = 1024;
 constexpr int64_t kBdDefMaxN = (int64_t)48 * 1024 * 8;  // two bit arrays in 96 KB of shared memory
 
-__device__ __forceinline__ double block_sum_bd(double v, double* red) {
-  v = warp_sum(v);
-  __syncthreads();
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
-  __syncthreads();
-  double t = 0.0;
-  for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += red[w];  // fixed order: reproducible
-  return t;
-}
-__device__ __forceinline__ double block_max_bd(double v, double* red) {
-  v = warp_max(v);
-  __syncthreads();
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
-  __syncthreads();
-  double t = 0.0;
-  for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t = fmax(t, red[w]);
-  return t;
-}
 // exclusive prefix of f over the block (blockDim.x = kBdDefThreads) and the block's total
 __device__ __forceinline__ int block_scan_bd(int f, int* wcnt, int& total) {
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -339,32 +431,62 @@ __device__ __forceinline__ int block_scan_bd(int f, int* wcnt, int& total) {
   return before + __popc(m & ((1u << lane) - 1u));
 }
 
-__global__ void __launch_bounds__(kBdDefThreads) k_bd_deflate(int64_t nn, double* Ds, double* zs, int32_t* kept,
-                                                             int32_t* defl, int32_t* rotp, double* rotcs,
-                                                             int32_t* cnt, double* rho_out, BdScratch S,
-                                                             int* status) {
+// w = hypot(zj, zp), c = zj / w, s = -zp / w from a refined reciprocal square root where the
+// squares stay in range (nine FP64 operations for some fifty).
+__device__ __forceinline__ void bd_rotation(double zj, double zp, double& w, double& c, double& s) {
+  const double t2 = fma(zj, zj, zp * zp);
+  if (in_range(t2)) {
+    const double ri = rsqrt_cubic(t2);
+    w = t2 * ri;
+    c = zj * ri;
+    s = -zp * ri;
+  } else {
+    w = hypot(zj, zp);
+    c = zj / w;
+    s = -zp / w;
+  }
+}
+
+__global__ void __launch_bounds__(kBdDefThreads) k_bd_deflate(BdLevel L) {
   extern __shared__ unsigned rotbit[];  // speculative outcome of survivor pair (q - 1, q), then dbit
   __shared__ double red[32];
   __shared__ int wcnt[32];
   const int tid = threadIdx.x;
+  const BdNode nd_ = L.nodes[blockIdx.x];
+  const int64_t nn = nd_.nn, o = nd_.lo;
+  double* Ds = L.Ds + o;
+  double* zs = L.zs + o;
+  int32_t* kept = L.kept + o;
+  int32_t* defl = L.defl + o;
+  int32_t* rotp = L.rotp + 2 * o;
+  double* rotcs = L.rotcs + 2 * o;
+  int32_t* cnt = L.cnt + 4 * blockIdx.x;
+  int32_t* surv = L.surv + o;
+  int32_t* slot = L.slot + o;
+  double* rc = L.rc + o;
+  double* rs = L.rs + o;
+  double* rw = L.rw + o;
+  double* rdp = L.rdp + o;
+  double* rdn = L.rdn + o;
   double s2 = 0.0, dmax = 0.0;
   bool fin = true;
   for (int64_t i = tid; i < nn; i += blockDim.x) {
-    s2 = fma(zs[i], zs[i], s2);
-    dmax = fmax(dmax, fabs(Ds[i]));
-    fin = fin && isfinite(zs[i]) && isfinite(Ds[i]);
+    const double z = zs[i], d = Ds[i];
+    s2 = fma(z, z, s2);
+    if (bd_key(fabs(d)) > bd_key(dmax)) dmax = fabs(d);
+    fin = fin && (__double2hiint(z) & 0x7ff00000) != 0x7ff00000 && (__double2hiint(d) & 0x7ff00000) != 0x7ff00000;
   }
   const int bad = __syncthreads_or(!fin);
-  s2 = block_sum_bd(s2, red);
-  dmax = block_max_bd(dmax, red);
+  s2 = bd_block_sum(s2, red);
+  dmax = bd_block_max(bad ? 0.0 : dmax, red);
   if (bad || !isfinite(s2)) {
-    if (tid == 0) set_status(status, TDC_ENONFINITE);
+    if (tid == 0) set_status(L.status, TDC_ENONFINITE);
     for (int64_t i = tid; i < nn; i += blockDim.x) defl[i] = (int32_t)i;
     if (tid == 0) {
       cnt[0] = 0;
       cnt[1] = (int32_t)nn;
       cnt[2] = 0;
-      *rho_out = 0.0;
+      L.rho[blockIdx.x] = 0.0;
     }
     return;
   }
@@ -374,9 +496,9 @@ __global__ void __launch_bounds__(kBdDefThreads) k_bd_deflate(int64_t nn, double
     double v = zs[i];
     if (zn > 0.0) v /= zn;
     zs[i] = v;
-    zmax = fmax(zmax, fabs(v));
+    if (bd_key(fabs(v)) > bd_key(zmax)) zmax = fabs(v);
   }
-  zmax = block_max_bd(zmax, red);
+  zmax = bd_block_max(zmax, red);
   const double tol = 8.0 * kBdEps * fmax(dmax, zmax);
   // type 1, and the survivors compacted in order
   int64_t M = 0;
@@ -386,8 +508,8 @@ __global__ void __launch_bounds__(kBdDefThreads) k_bd_deflate(int64_t nn, double
     const bool sv = i < nn && !t1;
     int total = 0;
     const int pos = block_scan_bd(sv ? 1 : 0, wcnt, total);
-    if (sv) S.surv[M + pos] = (int32_t)i;
-    if (i < nn) S.slot[i] = t1 ? (int32_t)i : -1;
+    if (sv) surv[M + pos] = (int32_t)i;
+    if (i < nn) slot[i] = t1 ? (int32_t)i : -1;
     M += total;
   }
   // type 2 on the original values, every consecutive survivor pair at once
@@ -398,17 +520,18 @@ __global__ void __launch_bounds__(kBdDefThreads) k_bd_deflate(int64_t nn, double
     const int64_t q = q0 + tid;
     bool rot = false;
     if (q >= 1 && q < M) {
-      const int32_t pa = S.surv[q - 1], pb = S.surv[q];
+      const int32_t pa = surv[q - 1], pb = surv[q];
       const double zp = zs[pa], zj = zs[pb], dp = Ds[pa], dj = Ds[pb];
-      const double w = hypot(zj, zp), t = dj - dp;
-      const double c = zj / w, s = -zp / w;
+      const double t = dj - dp;
+      double w, c, s;
+      bd_rotation(zj, zp, w, c, s);
       rot = fabs(t * c * s) <= tol;
       if (rot) {
-        S.c[q] = c;
-        S.s[q] = s;
-        S.w[q] = w;
-        S.dp[q] = dp * c * c + dj * s * s;
-        S.dn[q] = dp * s * s + dj * c * c;
+        rc[q] = c;
+        rs[q] = s;
+        rw[q] = w;
+        rdp[q] = dp * c * c + dj * s * s;
+        rdn[q] = dp * s * s + dj * c * c;
       }
     }
     const unsigned bits = __ballot_sync(0xffffffffu, rot);
@@ -434,18 +557,16 @@ __global__ void __launch_bounds__(kBdDefThreads) k_bd_deflate(int64_t nn, double
         q = wd * 32 + (__ffs(bits) - 1);
         if (q >= M) break;
         rot = true;
-        c = S.c[q];
-        s = S.s[q];
-        w = S.w[q];
-        dp = S.dp[q];
-        dn = S.dn[q];
+        c = rc[q];
+        s = rs[q];
+        w = rw[q];
+        dp = rdp[q];
+        dn = rdn[q];
       } else {
-        const int32_t pb = S.surv[q];
+        const int32_t pb = surv[q];
         const double zj = zs[pb], dj = Ds[pb];
-        w = hypot(zj, zc);
+        bd_rotation(zj, zc, w, c, s);
         const double t = dj - dc;
-        c = zj / w;
-        s = -zc / w;
         rot = fabs(t * c * s) <= tol;
         if (rot) {
           dp = dc * c * c + dj * s * s;
@@ -453,7 +574,7 @@ __global__ void __launch_bounds__(kBdDefThreads) k_bd_deflate(int64_t nn, double
         }
       }
       if (rot) {
-        const int32_t pa = S.surv[q - 1], pb = S.surv[q];
+        const int32_t pa = surv[q - 1], pb = surv[q];
         zs[pb] = w;
         zs[pa] = 0.0;
         Ds[pa] = dp;
@@ -463,7 +584,7 @@ __global__ void __launch_bounds__(kBdDefThreads) k_bd_deflate(int64_t nn, double
         rotcs[2 * nr] = c;
         rotcs[2 * nr + 1] = s;
         ++nr;
-        S.slot[pb] = pa;
+        slot[pb] = pa;
         dbit[(q - 1) >> 5] |= 1u << ((q - 1) & 31);
         mod = true;
         zc = w;
@@ -474,7 +595,7 @@ __global__ void __launch_bounds__(kBdDefThreads) k_bd_deflate(int64_t nn, double
       ++q;
     }
     cnt[2] = nr;
-    *rho_out = rho;
+    L.rho[blockIdx.x] = rho;
   }
   __syncthreads();
   // kept: the survivors no rotation deflated, in order
@@ -484,7 +605,7 @@ __global__ void __launch_bounds__(kBdDefThreads) k_bd_deflate(int64_t nn, double
     const bool kp = q < M && !((dbit[q >> 5] >> (q & 31)) & 1u);
     int total = 0;
     const int pos = block_scan_bd(kp ? 1 : 0, wcnt, total);
-    if (kp) kept[K + pos] = S.surv[q];
+    if (kp) kept[K + pos] = surv[q];
     K += total;
   }
   if (tid == 0) cnt[0] = (int32_t)K;
@@ -492,7 +613,7 @@ __global__ void __launch_bounds__(kBdDefThreads) k_bd_deflate(int64_t nn, double
   int64_t nd = 0;
   for (int64_t i0 = 0; i0 < nn; i0 += blockDim.x) {
     const int64_t i = i0 + tid;
-    const int32_t e = i < nn ? S.slot[i] : -1;
+    const int32_t e = i < nn ? slot[i] : -1;
     int total = 0;
     const int pos = block_scan_bd(e >= 0 ? 1 : 0, wcnt, total);
     if (e >= 0) defl[nd + pos] = e;
@@ -503,18 +624,25 @@ __global__ void __launch_bounds__(kBdDefThreads) k_bd_deflate(int64_t nn, double
 
 // The deflation rotations on the columns of Q (sorted position p is column perm[p]), in
 // order, each row independently.
-__global__ void __launch_bounds__(256) k_bd_rotate(int64_t nrows, double* Q, int64_t ldq, const int32_t* perm,
-                                                  const int32_t* rotp, const double* rotcs, int nr, int* status) {
+__global__ void __launch_bounds__(256) k_bd_rotate(BdLevel L) {
+  const int nr = L.cnt[4 * blockIdx.y + 2];
+  if (nr <= 0) return;
+  const BdNode nd = L.nodes[blockIdx.y];
+  const int64_t nrows = nd.nn;
+  double* Q = L.Q + nd.lo + nd.lo * L.ldq;
+  const int32_t* perm = L.perm + nd.lo;
+  const int32_t* rotp = L.rotp + 2 * nd.lo;
+  const double* rotcs = L.rotcs + 2 * nd.lo;
   for (int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; r < nrows; r += (int64_t)gridDim.x * blockDim.x) {
     for (int t = 0; t < nr; ++t) {
       const int32_t pa = rotp[2 * t], pb = rotp[2 * t + 1];
       if (pa < 0 || pa >= nrows || pb < 0 || pb >= nrows || perm[pa] < 0 || perm[pa] >= nrows || perm[pb] < 0 ||
           perm[pb] >= nrows) {  // cannot happen for a permutation; never touch memory outside Q
-        set_status(status, TDC_EUNSUPPORTED);
+        set_status(L.status, TDC_EUNSUPPORTED);
         continue;
       }
-      double* a = Q + r + (int64_t)perm[pa] * ldq;
-      double* bq = Q + r + (int64_t)perm[pb] * ldq;
+      double* a = Q + r + (int64_t)perm[pa] * L.ldq;
+      double* bq = Q + r + (int64_t)perm[pb] * L.ldq;
       const double c = rotcs[2 * t], s = rotcs[2 * t + 1];
       const double x = *a, y = *bq;
       *a = c * x + s * y;
@@ -524,52 +652,158 @@ __global__ void __launch_bounds__(256) k_bd_rotate(int64_t nrows, double* Q, int
 }
 
 // Qw(:, t) = Q(:, perm[kept[t]]) for t < K, Q(:, perm[defl[t - K]]) after; the kept poles,
-// their weights and the deflated values alongside.
-__global__ void __launch_bounds__(256) k_bd_gather(int64_t nrows, const double* Q, int64_t ldq, const int32_t* perm,
-                                                  const int32_t* kept, int K, const int32_t* defl, int nd,
-                                                  const double* Ds, const double* zs, double* Qw, double* DK,
-                                                  double* zK, double* Dd, int* status) {
-  for (int64_t t = blockIdx.x; t < K + nd; t += gridDim.x) {
-    const int32_t sp = t < K ? kept[t] : defl[t - K];
-    if (t >= nrows || sp < 0 || sp >= nrows || perm[sp] < 0 || perm[sp] >= nrows) {  // cannot happen; never
-      if (threadIdx.x == 0) set_status(status, TDC_EUNSUPPORTED);                   // read or write outside
+// their weights (squared, and the FP32 copies relative to the middle pole for the roots'
+// pre-iteration) and the deflated values alongside.
+__global__ void __launch_bounds__(256) k_bd_gather(BdLevel L) {
+  const BdNode nd = L.nodes[blockIdx.y];
+  const int64_t nrows = nd.nn, o = nd.lo;
+  const int K = L.cnt[4 * blockIdx.y], ndf = L.cnt[4 * blockIdx.y + 1];
+  const double* Q = L.Q + o + o * L.ldq;
+  double* Qw = L.Qw + o * L.n;
+  for (int64_t t = blockIdx.x; t < (int64_t)K + ndf; t += gridDim.x) {
+    const int32_t sp = t < nrows ? (t < K ? L.kept[o + t] : L.defl[o + t - K]) : -1;
+    if (sp < 0 || sp >= nrows || L.perm[o + sp] < 0 || L.perm[o + sp] >= nrows) {  // cannot happen; never
+      if (threadIdx.x == 0) set_status(L.status, TDC_EUNSUPPORTED);                // read or write outside
       continue;
     }
-    const double* src = Q + (int64_t)perm[sp] * ldq;
+    const double* src = Q + (int64_t)L.perm[o + sp] * L.ldq;
     double* dst = Qw + t * nrows;
     for (int64_t r = threadIdx.x; r < nrows; r += blockDim.x) dst[r] = src[r];
     if (threadIdx.x == 0) {
+      const double d = L.Ds[o + sp];
       if (t < K) {
-        DK[t] = Ds[sp];
-        zK[t] = zs[sp];
+        const int32_t mid = L.kept[o + (K >> 1)];
+        const double zt = L.zs[o + sp], x = d - ((mid >= 0 && mid < nrows) ? L.Ds[o + mid] : 0.0);
+        const float xh = (float)x;
+        L.DK[o + t] = d;
+        L.zK[o + t] = zt;
+        L.zz[o + t] = zt * zt;
+        L.xz[o + t] = make_float2(xh, (float)(zt * zt));
+        L.xlo[o + t] = (float)(x - (double)xh);
       } else {
-        Dd[t - K] = Ds[sp];
+        L.Dd[o + t - K] = d;
       }
     }
   }
 }
 
-// Q(:, K + t) = Qw(:, K + t) (deflated columns); D = [roots; deflated values].
-__global__ void __launch_bounds__(256) k_bd_finish(int64_t nrows, const double* Qw, double* Q, int64_t ldq, int K,
-                                                  int nd, const double* DK, const int32_t* org, const double* tau,
-                                                  const double* Dd, double* D) {
-  for (int64_t t = blockIdx.x; t < K + nd && t < nrows; t += gridDim.x) {
-    if (t >= K) {
-      const double* src = Qw + t * nrows;
-      double* dst = Q + t * ldq;
-      for (int64_t r = threadIdx.x; r < nrows; r += blockDim.x) dst[r] = src[r];
+// The level's products: split segments for nodes with K >= kBdSplitK (digit images one after
+// the other), FP64 tiles for the others.  One warp, 32 nodes at a time.
+constexpr int kBdSplitK = 128;
+__global__ void __launch_bounds__(32) k_bd_segs(BdLevel L) {
+  const int lane = threadIdx.x;
+  int64_t base[5] = {0, 0, 0, 0, 0};  // A items, B items, tiles, image elements, segments
+  for (int g0 = 0; g0 < L.count; g0 += 32) {
+    const int g = g0 + lane;
+    GemmSeg sg;
+    memset(&sg, 0, sizeof(sg));
+    int64_t v[5] = {0, 0, 0, 0, 0}, ael = 0;
+    if (g < L.count) {
+      const BdNode nd = L.nodes[g];
+      const int K = L.cnt[4 * g];
+      sg.ars = 1;
+      sg.A = L.Qw + nd.lo * L.n;
+      sg.lda = nd.nn;
+      sg.rows = (int32_t)nd.nn;
+      sg.kk = K;
+      sg.K = K;
+      sg.D = L.DK + nd.lo;
+      sg.org = L.org + nd.lo;
+      sg.tau = L.tau + nd.lo;
+      sg.zhat = L.zhat + nd.lo;
+      sg.scol = L.scol + nd.lo;
+      sg.C = L.Q + nd.lo + nd.lo * L.ldq;
+      sg.ldc = L.ldq;
+      GemmSeg ds = sg;
+      if (K >= kBdSplitK) {
+        const int64_t RT = (nd.nn + kSplitBM - 1) / kSplitBM, KB = (K + kSplitBK - 1) / kSplitBK,
+                      CT = (K + kSplitBN - 1) / kSplitBN;
+        v[0] = RT * KB;
+        v[1] = CT * KB;
+        v[2] = RT * CT;
+        ael = v[0] * L.S * kSplitBM * kSplitBK;
+        v[3] = ael + v[1] * L.S * kSplitBN * kSplitBK;
+        v[4] = 1;
+        ds.K = 0;
+      }
+      L.dsegs[g] = ds;
     }
-    if (threadIdx.x == 0) D[t] = t < K ? ((org[t] >= 0 && org[t] < K) ? DK[org[t]] + tau[t] : __longlong_as_double(0x7ff8000000000000ll)) : Dd[t - K];
+    int64_t at[5];
+#pragma unroll
+    for (int q = 0; q < 5; ++q) {
+      int64_t inc = v[q];
+      for (int of = 1; of < 32; of <<= 1) {
+        const int64_t u = __shfl_up_sync(0xffffffffu, inc, of);
+        if (lane >= of) inc += u;
+      }
+      at[q] = base[q] + inc - v[q];
+      base[q] += __shfl_sync(0xffffffffu, inc, 31);
+    }
+    if (v[4]) {
+      sg.it_a = at[0];
+      sg.it_b = at[1];
+      sg.it_t = at[2];
+      sg.a_img = at[3];
+      sg.b_img = at[3] + ael;
+      L.segs[at[4]] = sg;
+    }
+  }
+  if (lane == 0) {
+    GemmSeg last;
+    memset(&last, 0, sizeof(last));
+    last.it_a = base[0];
+    last.it_b = base[1];
+    last.it_t = base[2];
+    last.a_img = base[3];
+    if (base[3] > L.img_cap) {  // cannot happen with the host's bound; never write past the images
+      last.it_a = last.it_b = last.it_t = 0;
+      set_status(L.status, TDC_EUNSUPPORTED);
+    }
+    L.segs[base[4]] = last;
+    *L.nsegs = base[4];
   }
 }
 
-// Q(:, t) = Qw(:, t) for every column (the final order), lam = Ds.
-__global__ void __launch_bounds__(256) k_bd_copy_back(int64_t nrows, int64_t ncols, const double* Qw, double* Q,
-                                                     int64_t ldq) {
-  for (int64_t t = blockIdx.x; t < ncols; t += gridDim.x) {
-    const double* src = Qw + t * nrows;
-    double* dst = Q + t * ldq;
+// Q(:, K + t) = Qw(:, K + t) (deflated columns); D = [roots; deflated values], whose first run
+// is the K roots.
+__global__ void __launch_bounds__(256) k_bd_finish(BdLevel L) {
+  const BdNode nd = L.nodes[blockIdx.y];
+  const int64_t nrows = nd.nn, o = nd.lo;
+  const int K = L.cnt[4 * blockIdx.y], ndf = L.cnt[4 * blockIdx.y + 1];
+  const double* Qw = L.Qw + o * L.n;
+  double* Q = L.Q + o + o * L.ldq;
+  if (blockIdx.x == 0 && threadIdx.x == 0) L.cnt[4 * blockIdx.y + 3] = K;
+  for (int64_t t = blockIdx.x; t < (int64_t)K + ndf && t < nrows; t += gridDim.x) {
+    if (t >= K) {
+      const double* src = Qw + t * nrows;
+      double* dst = Q + t * L.ldq;
+      for (int64_t r = threadIdx.x; r < nrows; r += blockDim.x) dst[r] = src[r];
+    }
+    if (threadIdx.x == 0) {
+      const int32_t og = t < K ? L.org[o + t] : 0;
+      L.Dcur[o + t] = t >= K ? L.Dd[o + t - K]
+                             : (og >= 0 && og < K ? L.DK[o + og] + L.tau[o + t]
+                                                  : __longlong_as_double(0x7ff8000000000000ll));
+    }
+  }
+}
+
+// The node's final order: Qw(:, t) = Q(:, perm[t]) (back = 0), Q(:, t) = Qw(:, t) and lam (1).
+__global__ void __launch_bounds__(256) k_bd_order(BdLevel L, double* lam, int back) {
+  const BdNode nd = L.nodes[blockIdx.y];
+  const int64_t nrows = nd.nn, o = nd.lo;
+  double* Qw = L.Qw + o * L.n;
+  double* Q = L.Q + o + o * L.ldq;
+  for (int64_t t = blockIdx.x; t < nrows; t += gridDim.x) {
+    const int32_t c = L.perm[o + t];
+    if (!back && (c < 0 || c >= nrows)) {  // cannot happen for a permutation
+      if (threadIdx.x == 0) set_status(L.status, TDC_EUNSUPPORTED);
+      continue;
+    }
+    const double* src = back ? Qw + t * nrows : Q + (int64_t)c * L.ldq;
+    double* dst = back ? Q + t * L.ldq : Qw + t * nrows;
     for (int64_t r = threadIdx.x; r < nrows; r += blockDim.x) dst[r] = src[r];
+    if (back && threadIdx.x == 0) lam[o + t] = L.Ds[o + t];
   }
 }
 
@@ -598,9 +832,14 @@ cudaError_t launch_bd_copy_band(int64_t n, int b, const double* AB, int64_t ldab
   k_bd_copy_band<<<grid_for((int64_t)(b + 1) * n), 256, 0, s>>>(n, b, AB, ldab, ABw);
   return cudaGetLastError();
 }
-cudaError_t launch_bd_tear(double* ABw, int64_t ldab, int b, int64_t m, double* wv, cudaStream_t s) {
-  if (b <= 0) return cudaSuccess;
-  k_bd_tear<<<1, 256, sizeof(double) * (size_t)(b * b + b), s>>>(ABw, ldab, b, m, wv);
+cudaError_t launch_bd_nodes(BdNode* dst, const BdNodeTable& T, int count, cudaStream_t s) {
+  k_bd_nodes<<<1, 32, 0, s>>>(dst, T, count);
+  return cudaGetLastError();
+}
+cudaError_t launch_bd_tear(const BdNode* nodes, int count, double* ABw, int64_t ldab, int b, double* wv,
+                           cudaStream_t s) {
+  if (b <= 0 || count <= 0) return cudaSuccess;
+  k_bd_tear<<<(unsigned)count, 256, sizeof(double) * (size_t)(b * b + b), s>>>(nodes, ABw, ldab, b, wv);
   return cudaGetLastError();
 }
 cudaError_t launch_bd_leaf_trd(const BdLeafArgs& A, const BdLeafTable& T, cudaStream_t s) {
@@ -610,29 +849,35 @@ cudaError_t launch_bd_leaf_trd(const BdLeafArgs& A, const BdLeafTable& T, cudaSt
 }
 cudaError_t launch_bd_leaf_back(const BdLeafArgs& A, const BdLeafTable& T, cudaStream_t s) {
   if (A.nleaf <= 0) return cudaSuccess;
-  k_bd_leaf_back<<<(unsigned)A.nleaf, kBdLeafThreads, 0, s>>>(A, T);
+  int lmax = 0;
+  for (int t = 0; t < A.nleaf; ++t) lmax = std::max(lmax, T.L[t]);
+  const dim3 grid((unsigned)A.nleaf, (unsigned)((lmax + 3) / 4));
+  if (lmax <= 128) k_bd_leaf_back<4><<<grid, 128, 0, s>>>(A, T);
+  else if (lmax <= 256) k_bd_leaf_back<8><<<grid, 128, 0, s>>>(A, T);
+  else k_bd_leaf_back<16><<<grid, 128, 0, s>>>(A, T);
   return cudaGetLastError();
 }
-cudaError_t launch_bd_z(int64_t nn, const double* Q, int64_t ldq, int64_t ra, int64_t rb, int b, const double* w,
-                        double* z, cudaStream_t s) {
-  k_bd_z<<<grid_for(nn), 256, 0, s>>>(nn, Q, ldq, ra, rb, b, w, z);
+static dim3 bd_grid(const BdLevel& L, int64_t work, int64_t per, int64_t cap) {
+  return dim3(grid_for(work, per, cap), (unsigned)L.count);
+}
+
+cudaError_t launch_bd_level_begin(const BdLevel& L, const double* lam, cudaStream_t s) {
+  k_bd_level_begin<<<bd_grid(L, L.max_nn, 256, 4096), 256, 0, s>>>(L, lam);
   return cudaGetLastError();
 }
-cudaError_t launch_bd_sort(int64_t nn, const double* D, const double* z, double* Ds, double* zs, int32_t* perm,
-                           const BdScratch& S, cudaStream_t s) {
-  if (nn <= 0) return cudaSuccess;
+
+static cudaError_t bd_sort(const BdLevel& L, int use_z, cudaStream_t s) {
   int ch = 2;
-  while (ch < kBdChunk && ch < nn) ch <<= 1;
-  k_bd_chunk_sort<<<(unsigned)((nn + ch - 1) / ch), std::max(32, std::min(1024, ch / 2)), 0, s>>>(nn, ch, D, S.sk,
-                                                                                                 S.si);
-  k_bd_rank<<<grid_for(nn), 256, 0, s>>>(nn, ch, D, z, S.sk, S.si, Ds, zs, perm);
+  while (ch < kBdChunk && ch < L.max_nn) ch <<= 1;
+  k_bd_merge<<<(unsigned)L.count, 1024, 0, s>>>(L, use_z);
+  k_bd_chunk_sort<<<bd_grid(L, L.max_nn, ch, 1 << 20), std::max(32, std::min(1024, ch / 2)), 0, s>>>(L, ch);
+  k_bd_rank<<<bd_grid(L, L.max_nn, 256, 4096), 256, 0, s>>>(L, ch, use_z);
   return cudaGetLastError();
 }
-cudaError_t launch_bd_deflate(int64_t nn, double* Ds, double* zs, int32_t* kept, int32_t* defl, int32_t* rotp,
-                              double* rotcs, int32_t* cnt, double* rho, const BdScratch& S, int* status,
-                              cudaStream_t s) {
-  if (nn > kBdDefMaxN) return cudaErrorInvalidValue;
-  const size_t smem = 2 * sizeof(unsigned) * (size_t)((std::max<int64_t>(nn, 1) + 31) / 32);
+
+cudaError_t launch_bd_term(const BdLevel& L, int term, cudaStream_t s) {
+  if (L.max_nn > kBdDefMaxN) return cudaErrorInvalidValue;
+  const size_t smem = 2 * sizeof(unsigned) * (size_t)((std::max<int64_t>(L.max_nn, 1) + 31) / 32);
   static bool attr[64] = {false};  // once per device
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
@@ -643,32 +888,30 @@ cudaError_t launch_bd_deflate(int64_t nn, double* Ds, double* zs, int32_t* kept,
     if (e != cudaSuccess) return e;
     attr[dev] = true;
   }
-  k_bd_deflate<<<1, kBdDefThreads, smem, s>>>(nn, Ds, zs, kept, defl, rotp, rotcs, cnt, rho, S, status);
+  k_bd_z<<<bd_grid(L, L.max_nn, 256, 4096), 256, 0, s>>>(L, term);
+  e = bd_sort(L, 1, s);
+  if (e != cudaSuccess) return e;
+  k_bd_deflate<<<(unsigned)L.count, kBdDefThreads, smem, s>>>(L);
+  k_bd_rotate<<<bd_grid(L, L.max_nn, 256, 4096), 256, 0, s>>>(L);
+  k_bd_gather<<<bd_grid(L, L.max_nn, 1, 8192), 256, 0, s>>>(L);
   return cudaGetLastError();
 }
-cudaError_t launch_bd_rotate(int64_t nrows, double* Q, int64_t ldq, const int32_t* perm, const int32_t* rotp,
-                             const double* rotcs, int nr, int* status, cudaStream_t s) {
-  if (nr <= 0) return cudaSuccess;
-  k_bd_rotate<<<grid_for(nrows), 256, 0, s>>>(nrows, Q, ldq, perm, rotp, rotcs, nr, status);
+
+cudaError_t launch_bd_segs(const BdLevel& L, cudaStream_t s) {
+  k_bd_segs<<<1, 32, 0, s>>>(L);
   return cudaGetLastError();
 }
-cudaError_t launch_bd_gather(int64_t nrows, const double* Q, int64_t ldq, const int32_t* perm, const int32_t* kept,
-                             int K, const int32_t* defl, int nd, const double* Ds, const double* zs, double* Qw,
-                             double* DK, double* zK, double* Dd, int* status, cudaStream_t s) {
-  k_bd_gather<<<(unsigned)std::max(1, std::min(K + nd, 8192)), 256, 0, s>>>(nrows, Q, ldq, perm, kept, K, defl, nd, Ds,
-                                                                            zs, Qw, DK, zK, Dd, status);
+
+cudaError_t launch_bd_finish(const BdLevel& L, cudaStream_t s) {
+  k_bd_finish<<<bd_grid(L, L.max_nn, 1, 8192), 256, 0, s>>>(L);
   return cudaGetLastError();
 }
-cudaError_t launch_bd_finish(int64_t nrows, const double* Qw, double* Q, int64_t ldq, int K, int nd, const double* DK,
-                             const int32_t* org, const double* tau, const double* Dd, double* D, cudaStream_t s) {
-  k_bd_finish<<<(unsigned)std::max(1, std::min(K + nd, 8192)), 256, 0, s>>>(nrows, Qw, Q, ldq, K, nd, DK, org, tau,
-                                                                            Dd, D);
-  return cudaGetLastError();
-}
-cudaError_t launch_bd_copy_back(int64_t nrows, int64_t ncols, const double* Qw, double* Q, int64_t ldq,
-                                cudaStream_t s) {
-  k_bd_copy_back<<<(unsigned)std::max<int64_t>(1, std::min<int64_t>(ncols, 8192)), 256, 0, s>>>(nrows, ncols, Qw, Q,
-                                                                                                 ldq);
+
+cudaError_t launch_bd_order(const BdLevel& L, double* lam, cudaStream_t s) {
+  const cudaError_t e = bd_sort(L, 0, s);
+  if (e != cudaSuccess) return e;
+  k_bd_order<<<bd_grid(L, L.max_nn, 1, 8192), 256, 0, s>>>(L, lam, 0);
+  k_bd_order<<<bd_grid(L, L.max_nn, 1, 8192), 256, 0, s>>>(L, lam, 1);
   return cudaGetLastError();
 }
 cudaError_t launch_bd_zero(int64_t rows, int64_t cols, double* Q, int64_t ldq, cudaStream_t s) {

@@ -465,6 +465,23 @@ __device__ __forceinline__ double warp_max(double v) {
   return v;
 }
 
+// The reflector of a column with first entry alpha and the others' squared norm s > 0: beta,
+// tau = (beta - alpha) / beta and 1 / (alpha - beta), from refined hardware reciprocals (an
+// FP64 square root and two divisions take 2,400 clocks of one thread, these 700).
+__device__ __forceinline__ void reflector(double alpha, double s, double& tau, double& beta, double& sc) {
+  const double t2 = fma(alpha, alpha, s);
+  if (in_range(t2)) {
+    const double ri = -copysign(rsqrt_cubic(t2), alpha);  // 1 / beta
+    beta = t2 * ri;
+    sc = rcp_nr(alpha - beta);
+    tau = (beta - alpha) * ri;
+  } else {
+    beta = -copysign(sqrt(t2), alpha);
+    tau = (beta - alpha) / beta;
+    sc = 1.0 / (alpha - beta);
+  }
+}
+
 // A call's status slot is two words: status[0] the first error (first writer wins),
 // status[1] warning bits (results written, accuracy possibly reduced).
 __device__ __forceinline__ void set_status(int* status, int code) {
@@ -651,7 +668,6 @@ cudaError_t launch_operand_prep(int64_t m, int64_t n, const double* A, int64_t l
 cudaError_t launch_dft_tables(int64_t n, double* cosv, double* msinv, cudaStream_t s);
 // symmetric band divide and conquer (tdc_banded.cu)
 cudaError_t launch_bd_copy_band(int64_t n, int b, const double* AB, int64_t ldab, double* ABw, cudaStream_t s);
-cudaError_t launch_bd_tear(double* ABw, int64_t ldab, int b, int64_t m, double* wv, cudaStream_t s);
 // The leaves of the band tree, all at once: dense block of leaf t (rows [lo, lo + L) of the
 // torn band) at Ab + lo lmax (ld L), its tridiagonal in d, e and reflector scalars in tau at
 // offset lo; the tridiagonal eigenvectors Zb + lo lmax (ld L) back-transformed into the
@@ -678,8 +694,6 @@ struct BdLeafArgs {
 };
 cudaError_t launch_bd_leaf_trd(const BdLeafArgs& A, const BdLeafTable& T, cudaStream_t s);
 cudaError_t launch_bd_leaf_back(const BdLeafArgs& A, const BdLeafTable& T, cudaStream_t s);
-cudaError_t launch_bd_z(int64_t nn, const double* Q, int64_t ldq, int64_t ra, int64_t rb, int b, const double* w,
-                        double* z, cudaStream_t s);
 // Overflow guard of the dense and band solvers: the largest finite |entry| of a column-major
 // rows x cols block (lower != 0: its lower triangle only) and, when that lies outside
 // [2^-400, 2^400], the block times the power of two 2^-escale that puts it in [1, 2)
@@ -688,32 +702,75 @@ cudaError_t launch_bd_z(int64_t nn, const double* Q, int64_t ldq, int64_t ra, in
 cudaError_t launch_range_scale(double* A, int64_t rows, int64_t cols, int64_t ld, int lower, unsigned long long* mx,
                                int* escale, cudaStream_t s);
 cudaError_t launch_range_unscale(double* x, int64_t n, const int* escale, cudaStream_t s);
-// Scratch of the band sort and deflation (arrays of nn entries, free while they run).
-struct BdScratch {
-  double* sk;      // sort: the chunks' sorted keys
-  int32_t* si;     // sort: their indices
-  int32_t* surv;   // deflation: sorted positions of the poles surviving type 1
-  int32_t* slot;   // deflation: deflated entry keyed by the position at which the scan deflates it
-  double* c;       // deflation: speculative rotation of each consecutive survivor pair: c, s,
-  double* s;       //   the combined weight and the two new poles
-  double* w;
-  double* dp;
-  double* dn;
+// The band tree's inner nodes on one level: node g holds rows [lo, lo + nn) and splits at row
+// mid; its arrays are entries lo .. lo + nn - 1 of the arrays below (columns of Qw: nn x nn at
+// Qw + lo n), its terms wv + wi b (b + 1).
+struct BdNode {
+  int64_t lo, nn, mid;
+  int64_t wi;
 };
-cudaError_t launch_bd_sort(int64_t nn, const double* D, const double* z, double* Ds, double* zs, int32_t* perm,
-                           const BdScratch& S, cudaStream_t s);
-cudaError_t launch_bd_deflate(int64_t nn, double* Ds, double* zs, int32_t* kept, int32_t* defl, int32_t* rotp,
-                              double* rotcs, int32_t* cnt, double* rho, const BdScratch& S, int* status,
-                              cudaStream_t s);
-cudaError_t launch_bd_rotate(int64_t nrows, double* Q, int64_t ldq, const int32_t* perm, const int32_t* rotp,
-                             const double* rotcs, int nr, int* status, cudaStream_t s);
-cudaError_t launch_bd_gather(int64_t nrows, const double* Q, int64_t ldq, const int32_t* perm, const int32_t* kept,
-                             int K, const int32_t* defl, int nd, const double* Ds, const double* zs, double* Qw,
-                             double* DK, double* zK, double* Dd, int* status, cudaStream_t s);
-cudaError_t launch_bd_finish(int64_t nrows, const double* Qw, double* Q, int64_t ldq, int K, int nd, const double* DK,
-                             const int32_t* org, const double* tau, const double* Dd, double* D, cudaStream_t s);
-cudaError_t launch_bd_copy_back(int64_t nrows, int64_t ncols, const double* Qw, double* Q, int64_t ldq,
-                                cudaStream_t s);
+constexpr int kBdNodeChunk = 96;  // nodes per launch of the table's upload (by kernel parameter)
+struct BdNodeTable {
+  BdNode nd[kBdNodeChunk];
+};
+struct BdLevel {
+  const BdNode* nodes;
+  int32_t count;  // nodes of the level
+  int32_t b;
+  int64_t max_nn, n;
+  const double* wv;
+  double* Q;
+  int64_t ldq;
+  double* Qw;
+  double* Dcur;    // poles in column order: two ascending runs (see cnt)
+  double* z;
+  double* Ds;      // sorted
+  double* zs;
+  int32_t* perm;   // column of sorted position p
+  int32_t* kept;   // sorted positions of the non-deflated poles
+  int32_t* defl;   // and of the deflated ones
+  int32_t* rotp;
+  double* rotcs;
+  int32_t* cnt;    // per node: K, deflated, rotations, length of Dcur's first run
+  int32_t* unsorted;  // per node: a run of Dcur is not ascending
+  double* rho;     // per node
+  double* DK;      // non-deflated poles and weights, deflated values
+  double* zK;
+  double* Dd;
+  int32_t* org;
+  double* tau;
+  double* zhat;
+  double* scol;
+  double* zz;      // FP32 pre-iteration's copies
+  float2* xz;
+  float* xlo;
+  double* sk;      // sort: the chunks' sorted keys (shares DK)
+  int32_t* si;     // sort: their indices (shares org)
+  int32_t* surv;   // deflation: sorted positions of the poles surviving type 1 (shares org)
+  int32_t* slot;   // deflation: deflated entry keyed by the position at which the scan deflates it (zK)
+  double* rc;      // deflation: speculative rotation of each consecutive survivor pair: c, s,
+  double* rs;      //   the combined weight and the two new poles
+  double* rw;
+  double* rdp;
+  double* rdn;
+  GemmSeg* segs;   // the split products' list (count + 1) and the FP64 products (count)
+  GemmSeg* dsegs;
+  int64_t* nsegs;
+  int64_t img_cap;
+  int32_t S;       // split digits
+  int32_t max_iter;
+  int* status;
+};
+cudaError_t launch_bd_nodes(BdNode* dst, const BdNodeTable& T, int count, cudaStream_t s);
+cudaError_t launch_bd_tear(const BdNode* nodes, int count, double* ABw, int64_t ldab, int b, double* wv,
+                           cudaStream_t s);
+cudaError_t launch_bd_level_begin(const BdLevel& L, const double* lam, cudaStream_t s);
+cudaError_t launch_bd_term(const BdLevel& L, int term, cudaStream_t s);  // z, sort, deflation, rotations, gather
+cudaError_t launch_bd_rank_one(const BdLevel& L, cudaStream_t s);        // roots, zhat, normalisers (tdc_merge.cu)
+cudaError_t launch_bd_segs(const BdLevel& L, cudaStream_t s);
+cudaError_t launch_bd_finish(const BdLevel& L, cudaStream_t s);
+cudaError_t launch_bd_order(const BdLevel& L, double* lam, cudaStream_t s);
+cudaError_t launch_dense_list(const GemmSeg* segs, int count, int64_t max_rows, int64_t max_K, cudaStream_t s);
 cudaError_t launch_bd_zero(int64_t rows, int64_t cols, double* Q, int64_t ldq, cudaStream_t s);
 // bidiagonal SVD through the Golub-Kahan tridiagonal (tdc_bdsdc.cu)
 cudaError_t launch_gk_build(int64_t n, const double* d, const double* e, double* td, double* te, cudaStream_t s);

@@ -342,6 +342,72 @@ __global__ void __launch_bounds__(kThreads, 2) k_gemm_dense_seg(GemmSeg sg) {
   }
 }
 
+// The FP64 products of a list of plain segments (no pole or column lists), segment g in grid
+// row g, 32 x 32 tiles (2 x 2 outputs a thread): the band merges of fewer than 128 poles, one
+// tile of which would otherwise run alone on its SM.
+__global__ void __launch_bounds__(kThreads, 5) k_gemm_dense_list(const GemmSeg* list) {
+  constexpr int T = kDenseSmallBM;
+  __shared__ double As[BK * T], Us[BK * T];
+  __shared__ double sDo[T], sTau[T], sS[T], sDq[BK], sZq[BK];
+  const GemmSeg& sg = list[blockIdx.y];
+  const int rows = sg.rows, K = sg.K, kk = sg.kk;
+  const int tid = threadIdx.x, ty = tid & 15, tx = tid >> 4;
+  const int rtiles = (rows + T - 1) / T, ctiles = (K + T - 1) / T;
+  for (int64_t w = blockIdx.x; w < (int64_t)rtiles * ctiles; w += gridDim.x) {
+    const int r0 = (int)(w / ctiles) * T, j0 = (int)(w % ctiles) * T;
+    __syncthreads();
+    if (tid < T) {
+      const int j = j0 + tid;
+      sDo[tid] = j < K ? sg.D[sg.org[j]] : 0.0;
+      sTau[tid] = j < K ? sg.tau[j] : 1.0;
+      sS[tid] = j < K ? sg.scol[j] : 0.0;
+    }
+    double acc[2][2] = {{0.0, 0.0}, {0.0, 0.0}};
+    for (int k0 = 0; k0 < kk; k0 += BK) {
+      __syncthreads();
+      if (tid < BK) {
+        const int k = k0 + tid;
+        sDq[tid] = k < kk ? sg.D[k] : 0.0;
+        sZq[tid] = k < kk ? sg.zhat[k] : 0.0;
+      }
+      __syncthreads();
+      for (int e = tid; e < BK * T; e += kThreads) {
+        const int k = e / T, r = e % T;
+        As[e] = (k0 + k < kk && r0 + r < rows) ? sg.A[r0 + r + (int64_t)(k0 + k) * sg.lda] : 0.0;
+        Us[e] = k0 + k < kk ? sZq[k] * rcp_nr((sDq[k] - sDo[r]) - sTau[r]) : 0.0;
+      }
+      __syncthreads();
+#pragma unroll
+      for (int k = 0; k < BK; ++k) {
+        const double a0 = As[k * T + 2 * ty], a1 = As[k * T + 2 * ty + 1];
+        const double b0 = Us[k * T + 2 * tx], b1 = Us[k * T + 2 * tx + 1];
+        acc[0][0] = fma(a0, b0, acc[0][0]);
+        acc[0][1] = fma(a0, b1, acc[0][1]);
+        acc[1][0] = fma(a1, b0, acc[1][0]);
+        acc[1][1] = fma(a1, b1, acc[1][1]);
+      }
+    }
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+      const int j = j0 + 2 * tx + c;
+      if (j >= K) continue;
+      double* out = sg.C + (int64_t)j * sg.ldc;
+#pragma unroll
+      for (int i = 0; i < 2; ++i) {
+        const int row = r0 + 2 * ty + i;
+        if (row < rows) out[row] = acc[i][c] * sS[2 * tx + c];
+      }
+    }
+  }
+}
+
+cudaError_t launch_dense_list(const GemmSeg* segs, int count, int64_t max_rows, int64_t max_K, cudaStream_t s) {
+  const int64_t t = kDenseSmallBM, tiles = ((max_rows + t - 1) / t) * ((max_K + t - 1) / t);
+  k_gemm_dense_list<<<dim3((unsigned)std::max<int64_t>(1, std::min<int64_t>(tiles, 608)), (unsigned)count), kThreads, 0,
+                      s>>>(segs);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_seg_dense(const GemmSeg& seg, cudaStream_t s) {
   const int64_t tiles = (int64_t)((seg.rows + BM - 1) / BM) * ((seg.K + BN - 1) / BN);
   if (tiles == 0) return cudaSuccess;

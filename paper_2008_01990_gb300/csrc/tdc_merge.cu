@@ -2361,6 +2361,50 @@ cudaError_t launch_rank_one(const double* D, const double* z, int64_t K, double 
   return cudaGetLastError();
 }
 
+// The rank-one problems of a band level, node g's in grid row g: K = cnt[4 g] poles.
+__global__ void __launch_bounds__(128) k_bd_secular(BdLevel L) {
+  const int64_t j = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+  const int K = L.cnt[4 * blockIdx.y];
+  if (j >= K) return;
+  const int64_t o = L.nodes[blockIdx.y].lo;
+  int og, it;
+  double t;
+  bool conv;
+  secular_root(L.DK + o, L.zK + o, L.zz + o, L.xz + o, L.xlo + o, K, (int)j, L.rho[blockIdx.y], L.max_iter, og, t, it,
+               conv);
+  if ((threadIdx.x & 31) == 0) {
+    L.org[o + j] = og;
+    L.tau[o + j] = t;
+    if (!conv) set_status(L.status, TDC_ENOCONV);
+  }
+}
+
+__global__ void __launch_bounds__(256) k_bd_lowner(BdLevel L) {
+  const int64_t i = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+  const int K = L.cnt[4 * blockIdx.y];
+  if (i >= K) return;
+  const int64_t o = L.nodes[blockIdx.y].lo;
+  const double zh = lowner_zhat(L.DK + o, L.org + o, L.tau + o, K, (int)i, L.rho[blockIdx.y], L.zK[o + i]);
+  if ((threadIdx.x & 31) == 0) L.zhat[o + i] = zh;
+}
+
+__global__ void __launch_bounds__(256) k_bd_colnorm(BdLevel L) {
+  const int64_t j = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+  const int K = L.cnt[4 * blockIdx.y];
+  if (j >= K) return;
+  const int64_t o = L.nodes[blockIdx.y].lo;
+  const double sj = column_norm(L.DK + o, L.zhat + o, K, L.DK[o + L.org[o + j]], L.tau[o + j]);
+  if ((threadIdx.x & 31) == 0) L.scol[o + j] = sj;
+}
+
+cudaError_t launch_bd_rank_one(const BdLevel& L, cudaStream_t s) {
+  auto grid = [&](int threads) { return dim3((unsigned)((L.max_nn * 32 + threads - 1) / threads), (unsigned)L.count); };
+  k_bd_secular<<<grid(128), 128, 0, s>>>(L);
+  k_bd_lowner<<<grid(256), 256, 0, s>>>(L);
+  k_bd_colnorm<<<grid(256), 256, 0, s>>>(L);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_lowner(const Plan& P, const LevelLaunch& L, cudaStream_t s) {
   if (L.nslots == 0) return cudaSuccess;
   const unsigned tblocks = (unsigned)((L.nslots + 255) / 256);

@@ -93,23 +93,6 @@ __device__ __forceinline__ double sum_blocks(const double* p) {
   return warp_sum(t);
 }
 
-// The reflector of a column with first entry alpha and the others' squared norm s > 0: beta,
-// tau = (beta - alpha) / beta and 1 / (alpha - beta), from refined hardware reciprocals (an
-// FP64 square root and two divisions take 2,400 clocks of one thread, these 700).
-__device__ __forceinline__ void reflector(double alpha, double s, double& tau, double& beta, double& sc) {
-  const double t2 = fma(alpha, alpha, s);
-  if (in_range(t2)) {
-    const double ri = -copysign(rsqrt_cubic(t2), alpha);  // 1 / beta
-    beta = t2 * ri;
-    sc = rcp_nr(alpha - beta);
-    tau = (beta - alpha) * ri;
-  } else {
-    beta = -copysign(sqrt(t2), alpha);
-    tau = (beta - alpha) / beta;
-    sc = 1.0 / (alpha - beta);
-  }
-}
-
 }  // namespace
 
 // ---------------------------------------------------------------------------
