@@ -480,6 +480,9 @@ def sbevd(AB: torch.Tensor, opts: Opts | None = None, stream=None, check: bool =
     ws = workspace(nb.value, AB.device)
     _check("tdc_sbevd", lib().tdc_sbevd(n, b, _ptr(ABc), max(b1, 1), _ptr(lam), _ptr(Q), max(n, 1), _ptr(ws),
                                         ws.numel(), ctypes.byref(opts) if opts else None, _stream(stream)))
+    if stream is not None:  # the call only enqueues: its buffers live until that stream is done with them
+        for t in (ABc, lam, Q, ws):
+            t.record_stream(stream)
     if check:
         _check("tdc_sbevd (device status)", sync_status(stream))
     return lam[:n], Q
