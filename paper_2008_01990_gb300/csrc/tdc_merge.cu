@@ -2160,25 +2160,33 @@ __device__ double lowner_zhat(const double* D, const int* org, const double* tau
   }
   dnorm(pn, en);
   dnorm(pd, ed);
+  if (W == 32) {
+    // reduce-scatter: the lower half-warp multiplies the numerators, the upper one the
+    // denominators (5 FP64 multiplications instead of 10)
+    const bool up = threadIdx.x & 16;
+    double v = (up ? pd : pn) * __shfl_xor_sync(0xffffffffu, up ? pn : pd, 16);
+    int e = (up ? ed : en) + __shfl_xor_sync(0xffffffffu, up ? en : ed, 16);
+    dnorm(v, e);
 #pragma unroll
-  for (int o = 16; o > 0 && W == 32; o >>= 1) {
-    const double qn = __shfl_xor_sync(0xffffffffu, pn, o), qd = __shfl_xor_sync(0xffffffffu, pd, o);
-    const int gn = __shfl_xor_sync(0xffffffffu, en, o), gd = __shfl_xor_sync(0xffffffffu, ed, o);
-    pn *= qn;
-    pd *= qd;
-    en += gn;
-    ed += gd;
-    dnorm(pn, en);
-    dnorm(pd, ed);
+    for (int o = 8; o > 0; o >>= 1) {
+      v *= __shfl_xor_sync(0xffffffffu, v, o);
+      e += __shfl_xor_sync(0xffffffffu, e, o);
+      dnorm(v, e);
+    }
+    pn = __shfl_sync(0xffffffffu, v, 0);
+    en = __shfl_sync(0xffffffffu, e, 0);
+    pd = __shfl_sync(0xffffffffu, v, 16);
+    ed = __shfl_sync(0xffffffffu, e, 16);
   }
   // zhat_i^2 = (pn / pd) 2^(en - ed), with an even exponent for the root
-  double r = pn / pd;
+  double r = in_range(fabs(pd)) ? pn * rcp_nr(pd) : pn / pd;
   int E = en - ed;
   if (E & 1) {
     r *= 2.0;
     E -= 1;
   }
-  return copysign(ldexp(sqrt(r), E / 2), zsign);
+  const double q = in_range(r) ? r * rsqrt_cubic(r) : sqrt(r);
+  return copysign(ldexp(q, E / 2), zsign);
 }
 
 __global__ void __launch_bounds__(256) k_lowner(Plan P, int level, int64_t M, int small_k, bool listed) {
@@ -2213,7 +2221,7 @@ __device__ double column_norm(const double* D, const double* zh, int K, double d
     acc = fma(u, u, acc);
   }
   if (W == 32) acc = warp_sum(acc);
-  return 1.0 / sqrt(acc);
+  return in_range(acc) ? rsqrt_nr(acc) : 1.0 / sqrt(acc);
 }
 
 // The same pass for a merge below the top level, which also forms its boundary
@@ -2249,11 +2257,15 @@ __device__ double column_norm_rows(const Plan& P, int64_t v0, int K, int j, bool
     if (need_f) f = x; else l = x;
   }
   if (W == 32) {
-    acc = warp_sum(acc);
-    f = warp_sum(f);
-    l = warp_sum(l);
+    if (need_f && need_l) {
+      warp_sum3(acc, f, l);
+    } else if (need_f) {
+      warp_sum2(acc, f);
+    } else {
+      warp_sum2(acc, l);
+    }
   }
-  const double sj = 1.0 / sqrt(acc);
+  const double sj = in_range(acc) ? rsqrt_nr(acc) : 1.0 / sqrt(acc);
   if (W == 1 || (threadIdx.x & 31) == 0) {
     P.v.rf[v0 + j] = sj * f;
     P.v.rl[v0 + j] = sj * l;
