@@ -97,6 +97,7 @@ struct HostPlan {
   std::vector<LevelLaunch> levels;  // index l
   int64_t Mmax = 1;
   std::vector<int64_t> max_tiles;   // GEMM tile upper bound per level
+  int64_t far = 0;                  // doubles of the largest level's far-field tables
   int64_t img_elems = 0;            // digit images of the split path (bf16 elements)
   int64_t max_passes = 0;           // most split passes of a level
   int split_S = 0;                  // 0: split path off
@@ -312,6 +313,7 @@ static void build_plan(HostPlan& H, int32_t batch, const int64_t* n_host, const 
     L.max_n = mx;
     L.min_n = c > 0 ? mn : 0;
     H.max_tiles[l] = tiles;
+    if (far_level(L)) H.far = std::max(H.far, L.merges * far_doubles(L.max_n));
     H.Mmax = std::max(H.Mmax, L.merges);
   }
 }
@@ -319,7 +321,7 @@ static void build_plan(HostPlan& H, int32_t batch, const int64_t* n_host, const 
 // workspace carving
 struct Layout {
   size_t prob, vec_d, vec_i, vec_b, minfo, tiles, stats, segs, img, srank, spiv, sy, svr, scolpiv, sw;
-  size_t ss_segs, ss_counts, ss_wcol0, ss_bcol, ss_wpos, ss_w, ss_r, ss_cexp, ss_item, ss_accept, q1, total;
+  size_t ss_segs, ss_counts, ss_wcol0, ss_bcol, ss_wpos, ss_w, ss_r, ss_cexp, ss_item, ss_accept, far, q1, total;
 };
 
 static constexpr int kVecD = 27;  // doubles per slot (13 vectors, 2 for rcs, 2 for skey, xlo, zz, 8 boundary rows)
@@ -361,6 +363,7 @@ static Layout layout_of(const HostPlan& H) {
   L.ss_cexp = o; o = align_up(o + sizeof(int32_t) * it * mm);
   L.ss_item = o; o = align_up(o + sizeof(int64_t) * 6 * it);
   L.ss_accept = o; o = align_up(o + (H.ss ? sizeof(int32_t) * 2 * (size_t)H.Mmax : 0));
+  L.far = o; o = align_up(o + sizeof(double) * (size_t)H.far);
   L.q1 = o; o = align_up(o + sizeof(double) * (size_t)H.Q1);
   L.total = o + 256;  // slack for aligning an unaligned base
   return L;
@@ -553,11 +556,12 @@ static int run_plan(HostPlan& H, const tdc_opts& o, const double* d, const doubl
     if (timing) spans.push_back({phase, {a0, a1}});
   };
   // kernel launches: problem upload, input scale, corner modification, leaves, 9 per level (14
-  // on levels that also run the thread-per-root variants), output
+  // on levels that also run the thread-per-root variants, 7 more with far-field tables), output
   int64_t launches = (int64_t)((H.prob.size() + kProbChunk - 1) / kProbChunk) + 4 + 9 * (int64_t)H.T;
   for (int l = 0; l < H.T; ++l) {
     if (l > 0) launches += 2;  // boundary rows: rotation and gather, output order
     if (H.levels[l].nslots >= kSmallMinSlots) launches += 5;
+    if (far_level(H.levels[l])) launches += 7;
     if (H.levels[l].merges > 0 && H.levels[l].min_n <= kTinyN) launches += 1;
     if (H.split_S && H.levels[l].max_n >= o.split_min_K)
       launches += 4 * (int64_t)H.split_chunks[l].size() + (H.split_chunks[l].size() > 1 ? 1 : 0);
@@ -589,6 +593,8 @@ static int run_plan(HostPlan& H, const tdc_opts& o, const double* d, const doubl
     Plan P = PP[l & 1];
     const bool ss = H.ss && H.ss_level[l] && LL.max_n >= P.struct_min_K;
     P.struct_split = ss ? 1 : 0;
+    P.far = far_level(LL) ? (double*)(base + L.far) : nullptr;
+    P.far_stride = far_doubles(LL.max_n);
     P.dense_small = (P.split_min_K > 0 && P.split_min_K <= kDenseSmallK) ||
                             LL.nslots * LL.max_n < kDenseFewTiles * kDenseBM * kDenseBN
                         ? 1
@@ -1656,7 +1662,7 @@ void band_levels(const std::vector<BandNode>& nodes, int64_t leafmax, std::vecto
 
 struct BandLayout {
   size_t ABw, wv, Ab, Zb, dl, el, taul, Dcur, z, Ds, zs, perm, kept, defl, rotp, rotcs, cnt, DK, zK, Dd, org, tau, zhat,
-      scol, Qw, nodes, ncnt, unsorted, rho, segs, dsegs, nsegs, img, leafws, r1, total;
+      scol, Qw, nodes, ncnt, unsorted, rho, segs, dsegs, nsegs, img, far, leafws, r1, total;
   size_t leafws_bytes;
   int64_t img_elems;
 };
@@ -1717,12 +1723,18 @@ BandLayout band_layout(int64_t n, int64_t b, const tdc_opts& op) {
   L.nsegs = take(o, 64);
   // digit images of one level's products
   L.img_elems = 0;
+  int64_t far = 0;
   for (size_t t = 0; t + 1 < first.size(); ++t) {
-    int64_t el = 0;
-    for (size_t i = first[t]; i < first[t + 1]; ++i)
+    int64_t el = 0, mx = 0;
+    for (size_t i = first[t]; i < first[t + 1]; ++i) {
       el += cauchy_split_elems(inner[i].nn, inner[i].nn, op.split_slices, nullptr);
+      mx = std::max(mx, inner[i].nn);
+    }
     L.img_elems = std::max(L.img_elems, el);
+    if (mx >= kFarMinN && (int64_t)(first[t + 1] - first[t]) <= kFarMaxMerges)
+      far = std::max(far, (int64_t)(first[t + 1] - first[t]) * far_doubles(mx));
   }
+  L.far = take(o, sizeof(double) * (size_t)far);
   L.img = take(o, sizeof(__nv_bfloat16) * (size_t)L.img_elems);
   std::vector<int64_t> llo, lsz;
   band_leaves(nodes, band_leafmax(b), llo, lsz);
@@ -1854,6 +1866,8 @@ int sbevd_run(int64_t n, int64_t b, const double* AB, int64_t ldab, double* lam,
     V.rho = (double*)(base + L.rho) + first[t];
     V.max_nn = 0;
     for (size_t i = first[t]; i < first[t + 1]; ++i) V.max_nn = std::max(V.max_nn, inner[i].nn);
+    V.far = V.max_nn >= kFarMinN && V.count <= kFarMaxMerges ? (double*)(base + L.far) : nullptr;
+    V.far_stride = far_doubles(V.max_nn);
     if (launch_bd_level_begin(V, lam, cs) != cudaSuccess) return TDC_ECUDA;
     for (int k = 0; k < (int)b; ++k) {
       if (launch_bd_term(V, k, cs) != cudaSuccess || launch_bd_rank_one(V, cs) != cudaSuccess ||

@@ -176,6 +176,31 @@ __device__ __forceinline__ double struct_entry(const GemmSeg& sg, int64_t k, int
   return sg.tgen[(k * j) % sg.toff];
 }
 
+// Far-field tables of the roots' sums (k_far_*): merges of K >= kFarMinK poles, blocks of
+// far_block(K) consecutive poles and roots, one record of kFarRec doubles a block, then
+// kFarM x 3 partial sums a block and split of its far poles.  A larger block makes the table
+// cheaper and the near sums of its roots longer (4 blocks): the two cost the same near
+// B = 2 sqrt(K), hence far_block.
+constexpr int kFarM = 20;        // Chebyshev nodes of a block
+constexpr int kFarRec = 5 * kFarM + 4;
+constexpr int kFarMinK = 1024;
+constexpr int kFarMinN = 2048;   // host: levels whose largest merge has at least this order
+constexpr int64_t kFarMaxMerges = 64;  // and at most so many merges
+constexpr int kFarSplit = 512;   // far poles a block of threads takes
+__host__ __device__ inline int far_block(int64_t K) { return K < 4096 ? 64 : (K < 12288 ? 128 : 256); }
+__host__ __device__ inline int64_t far_blocks_bound(int64_t K) { return (K + 63) / 64; }
+__host__ __device__ inline int64_t far_splits_bound(int64_t K) { return (K + kFarSplit - 1) / kFarSplit; }
+// doubles of one merge's table, for any K <= n
+__host__ inline int64_t far_doubles(int64_t n) {
+  if (n < kFarMinN) return 0;
+  int64_t best = 0;
+  for (int64_t K : {std::min<int64_t>(n, 4095), std::min<int64_t>(n, 12287), n}) {
+    const int64_t nb = (K + far_block(K) - 1) / far_block(K);
+    best = std::max(best, nb * (kFarRec + far_splits_bound(K) * 3 * kFarM));
+  }
+  return best;
+}
+
 struct Plan {
   const Problem* prob;  // sorted problems (device)
   int32_t nprob;        // problems in the plan
@@ -209,6 +234,8 @@ struct Plan {
   int32_t struct_split; // 1: the structured path's products run on the split tensor-core GEMM
   int32_t dense_small;  // the level's FP64 merges all take the small tiles (dense_tile_dims)
   const int32_t* ss_accept;  // per merge part (2g + p): 1 if the structured split path took it
+  double* far;          // far-field tables, one per merge of the level (NULL: none)
+  int64_t far_stride;   // doubles per table
 };
 
 // Scratch of the structured path: one slot per (segment, row tile I, column tile J).
@@ -520,6 +547,8 @@ struct LevelLaunch {
   int64_t max_n;      // largest merge order on the level
   int64_t min_n;      // smallest merge order on the level
 };
+// levels whose roots' sums use far-field tables
+inline bool far_level(const LevelLaunch& L) { return L.max_n >= kFarMinN && L.merges <= kFarMaxMerges; }
 cudaError_t launch_dmod(const Plan& P, cudaStream_t s);
 cudaError_t launch_leaves(const Plan& P, int64_t nleaves, int max_leaf, cudaStream_t s);
 // levels with at least this many slots also run the thread-per-root kernels
@@ -528,7 +557,7 @@ cudaError_t launch_prepare(const Plan& P, const LevelLaunch& L, cudaStream_t s);
 cudaError_t launch_rotate(const Plan& P, const LevelLaunch& L, cudaStream_t s);
 cudaError_t launch_boundary_rot(const Plan& P, const LevelLaunch& L, cudaStream_t s);
 cudaError_t launch_boundary_out(const Plan& P, const LevelLaunch& L, cudaStream_t s);
-cudaError_t launch_secular(const Plan& P, const LevelLaunch& L, cudaStream_t s);
+cudaError_t launch_secular(const Plan& P, const LevelLaunch& L, cudaStream_t s);  // with the far tables
 cudaError_t launch_lowner(const Plan& P, const LevelLaunch& L, cudaStream_t s);
 cudaError_t launch_finalize(const Plan& P, const LevelLaunch& L, cudaStream_t s);
 cudaError_t launch_copy_deflated(const Plan& P, const LevelLaunch& L, int sign_normalise, cudaStream_t s);
@@ -776,6 +805,8 @@ struct BdLevel {
   int32_t S;       // split digits
   int32_t max_iter;
   int* status;
+  double* far;     // far-field tables, one per node (NULL: none)
+  int64_t far_stride;
 };
 cudaError_t launch_bd_nodes(BdNode* dst, const BdNodeTable& T, int count, cudaStream_t s);
 cudaError_t launch_bd_tear(const BdNode* nodes, int count, double* ABw, int64_t ldab, int b, double* wv,

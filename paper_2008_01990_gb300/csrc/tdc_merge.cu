@@ -1358,6 +1358,368 @@ __device__ __forceinline__ float warp_sumf(float v) {
   return v;
 }
 
+__device__ __forceinline__ int dexp_field(double x) { return (__double2hiint(x) >> 20) & 0x7ff; }
+__device__ __forceinline__ double dscale(double x, int e) { return x * __hiloint2double((2046 - e) << 20, 0); }
+
+// (x, ex) -> mantissa in [1, 2) and exponent, for normal x (zero, subnormal and
+// non-finite values are left as they are)
+__device__ __forceinline__ void dnorm(double& x, int& ex) {
+  const int f = dexp_field(x);
+  if (f > 0 && f < 2047) {
+    x = dscale(x, f);
+    ex += f - 1023;
+  }
+}
+
+// The numerator prod_j (lambda_j - d_i) and the denominator prod of the paired
+// pole differences are accumulated as two separate products with their exponents
+// kept apart (one division per pole instead of one per term): both stay within
+// [2^-600, 2^600] and are renormalised when they leave it.
+// ---------------------------------------------------------------------------
+// Far-field tables.  The sums that every root (or pole) of a merge takes over all K poles --
+// the secular function, Loewner's product, the column norm and the boundary rows -- are, but
+// for the poles near it, smooth functions of its position: for a block of consecutive roots
+// whose interval has half-width h, the poles more than 4 h from its centre contribute a
+// function that the polynomial through kFarM Chebyshev points reproduces to
+//   |T_M(x) / T_M(t)| <= 2 / (4 + sqrt 15)^M = 2.4e-18  (M = 20, |t| >= 4)
+// of each term 1 / (t - x) (7e-17 for its square).  So a block's far sums are taken at its 20
+// points (k_far_nodes) instead of at its 64 to 256 roots, and a root adds their barycentric
+// interpolant to the direct sum over the near poles (about four blocks, FP64 as before).
+// Loewner's product enters by its logarithm; its far factors 1 + x, x the root's shift from
+// its pole over the pole's distance, are multiplied as 1 + E, E <- E + x + E x, so that a
+// point's product rounds by the size of E and not of 1 (a model of it in FP64 against 80-bit
+// sums: secular sums within 0.4 eps of sum |t| on average, norms 0.01 eps).
+// Where a block's interval is wide against its surroundings (graded or clustered spectra) the
+// near range grows to what the 4 h ask for; past 3/4 of the poles the block stays direct.
+// FP64 instructions a root at K = 16384 (direct sums in brackets): secular 580 (5180),
+// Loewner 480 (2560), norms with rows 620 (4600).  tridiag(1,2,1): n = 16384 57.3 -> 42.3 ms
+// (the sums over K >= 4096 had been 18 ms of it), harmonic chain n = 4999 6.74 -> 6.29 ms;
+// band n = 2048 (one such level) 16.2 -> 16.4 ms: there the tables cost what they save, hence
+// kFarMinN.
+// ---------------------------------------------------------------------------
+// record: points y[M] (relative to pole ref), barycentric weights w[M], f0, f1, f2[M]; then
+// {n0, n1} (the near poles), 1 / (3 h), {ref, -}, -.
+struct FarIn {
+  const double* D;
+  const double* zz;
+  const double* zh;
+  const double* pf;
+  const double* pl;
+  const double* tau;
+  const int* org;
+  int K;
+  double* tab;
+};
+
+__device__ __forceinline__ FarIn far_in(const Plan& P, int level, int64_t g) {
+  FarIn f;
+  f.K = P.m.K[g];
+  const int64_t v0 = f.K >= kFarMinK ? make_node(P, level, g).v0 : 0;
+  f.D = P.v.Dk + v0;
+  f.zz = P.v.zz + v0;
+  f.zh = P.v.zhat + v0;
+  f.pf = P.v.pf + v0;
+  f.pl = P.v.pl + v0;
+  f.tau = P.v.tau + v0;
+  f.org = P.v.org + v0;
+  f.tab = P.far + g * P.far_stride;
+  return f;
+}
+__device__ __forceinline__ FarIn far_in(const BdLevel& L, int, int64_t g) {
+  FarIn f;
+  const int64_t o = L.nodes[g].lo;
+  f.K = L.cnt[4 * g];
+  f.D = L.DK + o;
+  f.zz = L.zz + o;
+  f.zh = L.zhat + o;
+  f.pf = f.pl = nullptr;
+  f.tau = L.tau + o;
+  f.org = L.org + o;
+  f.tab = L.far + g * L.far_stride;
+  return f;
+}
+
+__device__ __forceinline__ int* far_range(double* rec) { return reinterpret_cast<int*>(rec + 5 * kFarM); }
+__device__ __forceinline__ const int* far_range(const double* rec) {
+  return reinterpret_cast<const int*>(rec + 5 * kFarM);
+}
+
+// The block's interval, its near poles, points and weights.
+template <typename C>
+__global__ void __launch_bounds__(32) k_far_setup(C ctx, int level) {
+  const FarIn f = far_in(ctx, level, blockIdx.y);
+  const int K = f.K, B = far_block(K), J = blockIdx.x, lane = threadIdx.x;
+  if (K < kFarMinK || (int64_t)J * B >= K) return;
+  double* rec = f.tab + (int64_t)J * kFarRec;
+  const int j0 = J * B, j1 = min(K - 1, j0 + B), ref = (j0 + j1) >> 1;
+  const double dref = f.D[ref], ya = f.D[j0] - dref, yb = f.D[j1] - dref;
+  const double yc = 0.5 * (ya + yb), h = 0.5 * (yb - ya);
+  int lo = 0, hi = K;  // first pole at or above yc - 4 h
+  while (lo < hi) {
+    const int m = (lo + hi) >> 1;
+    if (f.D[m] - dref < yc - 4.0 * h) lo = m + 1; else hi = m;
+  }
+  int n0 = lo;
+  hi = K;  // first pole above yc + 4 h
+  while (lo < hi) {
+    const int m = (lo + hi) >> 1;
+    if (f.D[m] - dref <= yc + 4.0 * h) lo = m + 1; else hi = m;
+  }
+  int n1 = lo;
+  // the window of 32 poles around every root of the block is near
+  n0 = min(n0, max(0, min(j0 - 16, K - 32)));
+  n1 = max(n1, min(K, max(j0 + B + 17, 32)));
+  if (n1 - n0 > K - K / 4 || !in_range(h)) {
+    n0 = 0;
+    n1 = K;
+  }
+  if (lane < kFarM) {
+    double sv, cv;
+    sincospi((2 * lane + 1) / (2.0 * kFarM), &sv, &cv);
+    rec[lane] = fma(h, cv, yc);
+    rec[kFarM + lane] = lane & 1 ? -sv : sv;
+    rec[2 * kFarM + lane] = 0.0;
+    rec[3 * kFarM + lane] = 0.0;
+    rec[4 * kFarM + lane] = 0.0;
+  }
+  if (lane == 0) {
+    int* r = far_range(rec);
+    r[0] = n0;
+    r[1] = n1;
+    rec[5 * kFarM + 1] = in_range(h) ? rcp_nr(3.0 * h) : 0.0;
+    r[4] = ref;
+    r[5] = 0;
+  }
+}
+
+// Reduce-scatter of C per-lane values (C a power of two): lane q 32 / C ends with value q's sum.
+template <int C>
+__device__ __forceinline__ double lane_scatter_sum(double (&v)[C]) {
+  int o = 16;
+#pragma unroll
+  for (int cnt = C; cnt > 1; cnt >>= 1, o >>= 1) {
+    const int half = cnt >> 1;
+    const bool up = threadIdx.x & o;
+#pragma unroll
+    for (int i = 0; i < half; ++i) {
+      const double send = up ? v[i] : v[i + half], keep = up ? v[i + half] : v[i];
+      v[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+    }
+  }
+  double r = v[0];
+#pragma unroll
+  for (; o > 0; o >>= 1) r += __shfl_xor_sync(0xffffffffu, r, o);
+  return r;
+}
+// The same for products kept as mantissa and exponent (dnorm).
+template <int C>
+__device__ __forceinline__ void lane_scatter_prod(double (&v)[C], int (&e)[C]) {
+  int o = 16;
+#pragma unroll
+  for (int cnt = C; cnt > 1; cnt >>= 1, o >>= 1) {
+    const int half = cnt >> 1;
+    const bool up = threadIdx.x & o;
+#pragma unroll
+    for (int i = 0; i < half; ++i) {
+      const double send = up ? v[i] : v[i + half], keep = up ? v[i + half] : v[i];
+      const int es = up ? e[i] : e[i + half], ek = up ? e[i + half] : e[i];
+      v[i] = keep * __shfl_xor_sync(0xffffffffu, send, o);
+      e[i] = ek + __shfl_xor_sync(0xffffffffu, es, o);
+      dnorm(v[i], e[i]);
+    }
+  }
+#pragma unroll
+  for (; o > 0; o >>= 1) {
+    v[0] *= __shfl_xor_sync(0xffffffffu, v[0], o);
+    e[0] += __shfl_xor_sync(0xffffffffu, e[0], o);
+    dnorm(v[0], e[0]);
+  }
+}
+
+// far poles of the block: left ones 0 .. nl - 1, right ones from n1 on (nr of them); Loewner's
+// factors stop one short of the near range on the left (root j lies below pole j + 1) and
+// leave the last root to the direct product
+__device__ __forceinline__ void far_counts(const int* range, int K, int mode, int& nl, int& nr) {
+  nl = range[0];
+  nr = K - range[1];
+  if (mode == 1) {
+    nl = max(nl - 1, 0);
+    nr = max(nr - 1, 0);
+  }
+}
+
+constexpr int kFarThreads = 128, kFarPer = kFarM / 4;  // a warp takes 5 of the points
+// mode 0: f0 = sum zz / (d - y), f1 = sum |.|; mode 1: f0 = log of Loewner's far product;
+// mode 2: f0 = sum (zh / (d - y))^2, with rows f1 = sum pf zh / (d - y), f2 likewise pl.
+// At most 80 registers: a block fits beside a CTA of the split product, whose stream runs at
+// the same time.
+template <int kMode, bool kRows, typename C>
+__global__ void __launch_bounds__(kFarThreads, 6) k_far_nodes(C ctx, int level) {
+  const FarIn f = far_in(ctx, level, blockIdx.z);
+  const int K = f.K, B = far_block(K), J = blockIdx.y;
+  if (K < kFarMinK || (int64_t)J * B >= K) return;
+  const double* rec = f.tab + (int64_t)J * kFarRec;
+  int nl, nr;
+  far_counts(far_range(rec), K, kMode, nl, nr);
+  const int n1 = far_range(rec)[1], nf = nl + nr;
+  const int a = blockIdx.x * kFarSplit, b = min(nf, a + kFarSplit);
+  if (a >= b) return;
+  const int lane = threadIdx.x & 31, m0 = (threadIdx.x >> 5) * kFarPer;
+  double y[kFarPer];
+#pragma unroll
+  for (int m = 0; m < kFarPer; ++m) y[m] = rec[m0 + m];
+  const double dref = f.D[far_range(rec)[4]];
+  constexpr int kSums = kMode == 0 ? 2 : (kMode == 1 ? 2 : (kRows ? 3 : 1));
+  double p[kSums][kFarPer];
+#pragma unroll
+  for (int c = 0; c < kSums; ++c)
+#pragma unroll
+    for (int m = 0; m < kFarPer; ++m) p[c][m] = kMode == 1 && c == 1 ? 1.0 : 0.0;
+  for (int q = a + lane; q < b; q += 32) {
+    const bool left = q < nl;
+    const int i = left ? q : q - nl + n1;
+    if constexpr (kMode == 0) {
+      const double d = f.D[i] - dref, z = f.zz[i];
+#pragma unroll
+      for (int m = 0; m < kFarPer; ++m) {
+        const double t = z * rcp_nr(d - y[m]);
+        if (left) p[1][m] += t; else p[0][m] += t;
+      }
+    } else if constexpr (kMode == 1) {
+      // factor 1 + x: on the left the root against its pole i, on the right against pole i + 1
+      const double di = f.D[i], dn = f.D[i + 1], tau = f.tau[i];
+      const bool at = f.org[i] == i;
+      const double d = (left ? di : dn) - dref;
+      const double g = left ? (at ? tau : tau + (dn - di)) : (at ? tau - (dn - di) : tau);
+#pragma unroll
+      for (int m = 0; m < kFarPer; ++m) {
+        const double dl = d - y[m], r = rcp_nr(dl), x = g * r;
+        const int ex = (__double2hiint(x) >> 20) & 0x7ff;
+        if (ex < 1021) p[0][m] = fma(p[0][m], x, p[0][m] + x);  // |x| < 1/4
+        else p[1][m] *= (dl + g) * r;
+      }
+    } else {
+      const double d = f.D[i] - dref, z = f.zh[i];
+      const double wf = kRows ? f.pf[i] : 0.0, wl = kRows ? f.pl[i] : 0.0;
+#pragma unroll
+      for (int m = 0; m < kFarPer; ++m) {
+        const double u = z * rcp_nr(d - y[m]);
+        p[0][m] = fma(u, u, p[0][m]);
+        if constexpr (kRows) {
+          p[1][m] = fma(wf, u, p[1][m]);
+          p[2][m] = fma(wl, u, p[2][m]);
+        }
+      }
+    }
+  }
+  const int64_t nb = (K + B - 1) / B;
+  double* part = f.tab + nb * kFarRec + ((int64_t)J * far_splits_bound(K) + blockIdx.x) * 3 * kFarM;
+  if constexpr (kMode == 1) {
+    double v4[4], v1[1];
+    int e4[4], e1[1];
+#pragma unroll
+    for (int m = 0; m < 4; ++m) {
+      v4[m] = p[1][m] * (1.0 + p[0][m]);
+      e4[m] = 0;
+      dnorm(v4[m], e4[m]);
+    }
+    v1[0] = p[1][4] * (1.0 + p[0][4]);
+    e1[0] = 0;
+    dnorm(v1[0], e1[0]);
+    lane_scatter_prod<4>(v4, e4);
+    lane_scatter_prod<1>(v1, e1);
+    if ((lane & 7) == 0) {
+      part[m0 + (lane >> 3)] = v4[0];
+      part[kFarM + m0 + (lane >> 3)] = (double)e4[0];
+    }
+    if (lane == 0) {
+      part[m0 + 4] = v1[0];
+      part[kFarM + m0 + 4] = (double)e1[0];
+    }
+  } else {
+#pragma unroll
+    for (int c = 0; c < kSums; ++c) {
+      double v4[4] = {p[c][0], p[c][1], p[c][2], p[c][3]};
+      const double x = lane_scatter_sum<4>(v4), z = warp_sum(p[c][4]);
+      if ((lane & 7) == 0) part[c * kFarM + m0 + (lane >> 3)] = x;
+      if (lane == 0) part[c * kFarM + m0 + 4] = z;
+    }
+  }
+}
+
+// The splits' partial sums (in order) into the record.
+template <int kMode, bool kRows, typename C>
+__global__ void __launch_bounds__(64) k_far_combine(C ctx, int level) {
+  const FarIn f = far_in(ctx, level, blockIdx.y);
+  const int K = f.K, B = far_block(K), J = blockIdx.x, tid = threadIdx.x;
+  if (K < kFarMinK || (int64_t)J * B >= K) return;
+  double* rec = f.tab + (int64_t)J * kFarRec;
+  int nl, nr;
+  far_counts(far_range(rec), K, kMode, nl, nr);
+  const int ns = (nl + nr + kFarSplit - 1) / kFarSplit;
+  const int64_t nb = (K + B - 1) / B;
+  const double* part = f.tab + nb * kFarRec + (int64_t)J * far_splits_bound(K) * 3 * kFarM;
+  if (kMode == 1) {
+    if (tid >= kFarM) return;
+    double v = 1.0;
+    int e = 0;
+    for (int q = 0; q < ns; ++q) {
+      v *= part[q * 3 * kFarM + tid];
+      e += (int)part[q * 3 * kFarM + kFarM + tid];
+      dnorm(v, e);
+    }
+    rec[2 * kFarM + tid] = log(v) + (double)e * 0.69314718055994530942;
+    return;
+  }
+  if (tid >= (kMode == 0 ? 2 : (kRows ? 3 : 1)) * kFarM) return;
+  double v = 0.0;
+  for (int q = 0; q < ns; ++q) v += part[q * 3 * kFarM + tid];
+  if (kMode == 0) {  // f0 = right + left, f1 = right - left
+    const int m = tid % kFarM;
+    double o = 0.0;
+    for (int q = 0; q < ns; ++q) o += part[q * 3 * kFarM + (tid < kFarM ? kFarM : 0) + m];
+    rec[2 * kFarM + tid] = tid < kFarM ? v + o : o - v;
+  } else {
+    rec[2 * kFarM + tid] = v;
+  }
+}
+
+template <int kMode, bool kRows, typename C>
+static cudaError_t launch_far(const C& ctx, int level, int64_t merges, int64_t max_n, cudaStream_t s) {
+  const unsigned nb = (unsigned)far_blocks_bound(max_n), ns = (unsigned)far_splits_bound(max_n);
+  if (kMode == 0) k_far_setup<C><<<dim3(nb, (unsigned)merges), 32, 0, s>>>(ctx, level);
+  k_far_nodes<kMode, kRows, C><<<dim3(ns, nb, (unsigned)merges), kFarThreads, 0, s>>>(ctx, level);
+  k_far_combine<kMode, kRows, C><<<dim3(nb, (unsigned)merges), 64, 0, s>>>(ctx, level);
+  return cudaGetLastError();
+}
+
+// The record of root (or pole) j's block; NULL: no table.
+__device__ __forceinline__ const double* far_record(const double* tab, int K, int j) {
+  return tab && K >= kFarMinK ? tab + (int64_t)(j / far_block(K)) * kFarRec : nullptr;
+}
+
+// Barycentric weights of the block's points for position x (relative to the block's pole
+// ref): bw in lanes below kFarM, and 1 / (x - y); a point that x falls on takes all of it.
+__device__ __forceinline__ void far_weights(const double* rec, double x, double& bw, double& rd) {
+  const int lane = threadIdx.x & 31;
+  bw = 0.0;
+  rd = 0.0;
+  bool hit = false;
+  if (lane < kFarM) {
+    const double d = x - rec[lane];
+    hit = !in_range(fabs(d));
+    if (!hit) {
+      rd = rcp_nr(d);
+      bw = rec[kFarM + lane] * rd;
+    }
+  }
+  const unsigned h = __ballot_sync(0xffffffffu, hit);
+  if (h) {
+    bw = lane == __ffs(h) - 1 ? 1.0 : 0.0;
+    rd = 0.0;
+  }
+}
+
 // FP64 Newton iteration for root j from a close starting point (the FP32 estimate), as a
 // rule with a single pass over all poles.  In that pass, at tau1, the far terms (outside the
 // window of the 32 poles nearest the root, one per lane) are summed: t, t r and t r^2 with
@@ -1377,7 +1739,7 @@ __device__ __forceinline__ float warp_sumf(float v) {
 // and pass of 32; the earlier form (four FP64 sums, divisions and a square root an iterate)
 // took 24,000 clocks a root of a small merge, this one 5,000.
 __device__ bool secular_certified(const double* D, const double* zz, int K, int j, double irho, int org, double width,
-                                  double& tau, int max_passes, int& passes) {
+                                  double& tau, int max_passes, int& passes, const double* far) {
   const int lane = threadIdx.x & 31;
   const float irf = (float)irho, wf = (float)width;
   if (!(irf > 1e-18f && irf < 1e18f && wf > 1e-30f)) return false;  // FP32 tests out of range
@@ -1388,6 +1750,8 @@ __device__ bool secular_certified(const double* D, const double* zz, int K, int 
   const bool wv = iw < K;
   const double zw2 = wv ? zz[iw] : 0.0, dw = wv ? D[iw] - dorg : 0.0;
   const float zwf = (float)zw2;
+  const int n0 = far ? far_range(far)[0] : 0, n1 = far ? far_range(far)[1] : K;
+  const bool use_far = n0 > 0 || n1 < K;
   double tau1 = tau;
   for (passes = 1; passes <= max_passes; ++passes) {
     double F = 0.0, A1 = 0.0;
@@ -1396,12 +1760,12 @@ __device__ bool secular_certified(const double* D, const double* zz, int K, int 
       // this lane's far poles are i = lane (mod 32): those below the window lie left of the
       // root, those above it right
       double a0 = 0.0, b0 = 0.0, a2 = 0.0;
-      for (int i = lane; i < w0; i += 32) {
+      for (int i = n0 + ((lane - n0) & 31); i < w0; i += 32) {
         const double r = rcp_nr((D[i] - dorg) - tau1);
         const double t = zz[i] * r, tr = t * r;
         a0 += t; A1 += tr; a2 = fma(tr, r, a2);
       }
-      for (int i = iw + 32; i < K; i += 32) {
+      for (int i = iw + 32; i < n1; i += 32) {
         const double r = rcp_nr((D[i] - dorg) - tau1);
         const double t = zz[i] * r, tr = t * r;
         b0 += t; A1 += tr; a2 = fma(tr, r, a2);
@@ -1415,8 +1779,29 @@ __device__ bool secular_certified(const double* D, const double* zz, int K, int 
       // and above it (poles are sorted)
       const int in = lane < 16 ? w0 - 1 : w0 + 32;
       float rd = 0.0f;
-      if (in >= 0 && in < K) rd = __fdividef(1.0f, fabsf((float)((D[in] - dorg) - tau1)));
+      if (in >= n0 && in < n1) rd = __fdividef(1.0f, fabsf((float)((D[in] - dorg) - tau1)));
       rdmin = fmaxf(rd, __shfl_xor_sync(0xffffffffu, rd, 16));
+    }
+    // the far poles' sum and slope by interpolation; Sf bounds their sum |t|, rd3 1 / distance
+    float Sf = 0.0f, rd3 = 0.0f;
+    if (use_far) {
+      double bw, rd, ff = 0.0;
+      far_weights(far, (dorg - D[far_range(far)[4]]) + tau1, bw, rd);
+      if (lane < kFarM) {
+        ff = far[2 * kFarM + lane];
+        Sf = (float)far[3 * kFarM + lane];
+      }
+      double num = bw * ff, den = bw;
+      warp_sum2(num, den);
+      const double rden = rcp_nr(den), p = num * rden;
+      const float slope = warp_sumf((float)(bw * (p - ff)) * (float)rd) * (float)rden;
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) Sf = fmaxf(Sf, __shfl_xor_sync(0xffffffffu, Sf, o));
+      rd3 = (float)far[5 * kFarM + 1];
+      rdmin = fmaxf(rdmin, rd3);
+      F += p;
+      A1 += (double)slope;
+      A1f += slope;
     }
     const double A2d = (double)A2;
     double tc = tau1, e = 0.0;
@@ -1434,8 +1819,11 @@ __device__ bool secular_certified(const double* D, const double* zz, int K, int 
       wsf = warp_sumf(wsf);
       wdf = warp_sumf(wdf);
       const double gv = (irho + F + e * fma(e, A2d, A1)) + warp_sum(wt);
-      const float gf = (float)gv, sabs = irf + S + wsf;
-      const float rest = it > 0 ? S * q * q * q / (1.0f - q) : 0.0f;
+      const float gf = (float)gv, sabs = irf + S + Sf + wsf;
+      // remainders: third order of the poles summed here, second of the far ones (whose FP32
+      // slope is good to 2^-20)
+      const float qf = fabsf(ef) * rd3;
+      const float rest = it > 0 ? S * q * q * q / (1.0f - q) + Sf * qf * (2.0f * qf + 0x1p-20f) : 0.0f;
       tau = tc;
       if (fabsf(gf) + rest <= 8.0f * (float)kEps * sabs) return true;
       const float gp = A1f + 2.0f * ef * A2 + wdf;
@@ -1607,7 +1995,8 @@ __device__ bool secular_fp32(const double* D, const float2* xz, const float* xlo
 // FP32 estimate is unusable, the origin comes from the sign of g at the midpoint.
 __device__ void secular_root(const double* D, const double* z, const double* zz, const float2* xz, const float* xlo,
                              int K, int j,
-                             double rho, int max_iter, int& org_out, double& tau_out, int& iters, bool& conv) {
+                             double rho, int max_iter, int& org_out, double& tau_out, int& iters, bool& conv,
+                             const double* far_tab = nullptr) {
   const double irho = in_range(rho) ? rcp_nr(rho) : 1.0 / rho;
   int org;
   double lo, hi, tau;
@@ -1630,7 +2019,8 @@ __device__ void secular_root(const double* D, const double* z, const double* zz,
     if (org == j) { lo = 0.0; hi = width; } else { lo = -width; hi = 0.0; }
     if (!(tau > lo && tau < hi)) tau = 0.5 * (lo + hi);
     int tried = 0;
-    conv = max_iter >= 2 && secular_certified(D, zz, K, j, irho, org, width, tau, min(max_iter - 1, 4), tried);
+    conv = max_iter >= 2 && secular_certified(D, zz, K, j, irho, org, width, tau, min(max_iter - 1, 4), tried,
+                                               last ? nullptr : far_record(far_tab, K, j));
     if (conv) {
       passes = tried;
     } else {
@@ -2088,7 +2478,7 @@ __global__ void __launch_bounds__(kSecThreads, 6) k_secular(Plan P, int level, i
     // so that it starts with the first wave of warps instead of ending the kernel
     const int j = jw == 0 ? K - 1 : jw - 1;
     secular_root(P.v.Dk + v0, P.v.zk + v0, P.v.zz + v0, P.v.xz + v0, P.v.xlo + v0, K, j, rho, P.max_iter, org, tau,
-                 it, conv);
+                 it, conv, P.far ? P.far + g * P.far_stride : nullptr);
     if ((threadIdx.x & 31) == 0) {
       P.v.org[v0 + j] = org;
       P.v.tau[v0 + j] = tau;
@@ -2107,6 +2497,10 @@ cudaError_t launch_secular(const Plan& P, const LevelLaunch& L, cudaStream_t s) 
   const int small_k = L.nslots >= kSmallMinSlots ? kSmallK : 0;
   const bool listed = small_k > 0;
   if (listed) k_root_scan<<<1, 512, 0, s>>>(P, L.merges, small_k);
+  if (P.far) {
+    const cudaError_t e = launch_far<0, false>(P, L.level, L.merges, L.max_n, s);
+    if (e != cudaSuccess) return e;
+  }
   k_secular<<<warp_root_grid(L, listed), kSecThreads, 0, s>>>(P, L.level, L.merges, small_k, listed);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess || small_k == 0) return e;
@@ -2124,30 +2518,15 @@ cudaError_t launch_secular(const Plan& P, const LevelLaunch& L, cudaStream_t s) 
 // ---------------------------------------------------------------------------
 // Exponent field of x, and x scaled by 2^(1023 - e) (into [1, 2) when e is the
 // exponent field of a normal x): integer work plus one multiplication.
-__device__ __forceinline__ int dexp_field(double x) { return (__double2hiint(x) >> 20) & 0x7ff; }
-__device__ __forceinline__ double dscale(double x, int e) { return x * __hiloint2double((2046 - e) << 20, 0); }
-
-// (x, ex) -> mantissa in [1, 2) and exponent, for normal x (zero, subnormal and
-// non-finite values are left as they are)
-__device__ __forceinline__ void dnorm(double& x, int& ex) {
-  const int f = dexp_field(x);
-  if (f > 0 && f < 2047) {
-    x = dscale(x, f);
-    ex += f - 1023;
-  }
-}
-
-// The numerator prod_j (lambda_j - d_i) and the denominator prod of the paired
-// pole differences are accumulated as two separate products with their exponents
-// kept apart (one division per pole instead of one per term): both stay within
-// [2^-600, 2^600] and are renormalised when they leave it.
 template <int W = 32>
 __device__ double lowner_zhat(const double* D, const int* org, const double* tau, int K, int i, double rho,
-                              double zsign) {
+                              double zsign, const double* far = nullptr) {
   const double di = D[i];
   double pn = 1.0, pd = 1.0;
   int en = 0, ed = 0;  // pn 2^en, pd 2^ed
-  for (int j = W == 32 ? (threadIdx.x & 31) : 0; j < K; j += W) {
+  // the near factors (all without a table): the far ones are left of jb and from je to K - 2
+  const int jb = far ? max(far_range(far)[0] - 1, 0) : 0, je = far ? far_range(far)[1] : K;
+  auto factor = [&](int j) {
     const double num = (D[org[j]] - di) + tau[j];
     const double den = (j == K - 1) ? rho : ((j < i) ? D[j] - di : D[j + 1] - di);
     pn *= num;
@@ -2157,7 +2536,10 @@ __device__ double lowner_zhat(const double* D, const int* org, const double* tau
       dnorm(pn, en);
       dnorm(pd, ed);
     }
-  }
+  };
+  const int lane = W == 32 ? (threadIdx.x & 31) : 0;
+  for (int j = jb + lane; j < je; j += W) factor(j);
+  if (je < K && lane == 0) factor(K - 1);
   dnorm(pn, en);
   dnorm(pd, ed);
   if (W == 32) {
@@ -2185,16 +2567,28 @@ __device__ double lowner_zhat(const double* D, const int* org, const double* tau
     r *= 2.0;
     E -= 1;
   }
-  const double q = in_range(r) ? r * rsqrt_cubic(r) : sqrt(r);
+  double q = in_range(r) ? r * rsqrt_cubic(r) : sqrt(r);
+  if (W == 32 && far && (jb > 0 || je < K)) {  // times the square root of the far product
+    double bw, rd;
+    far_weights(far, di - D[far_range(far)[4]], bw, rd);
+    double num = lane < kFarM ? bw * far[2 * kFarM + lane] : 0.0, den = bw;
+    warp_sum2(num, den);
+    const double lg = 0.5 * num * rcp_nr(den);
+    // exp(lg) as 2^k exp(rest), k even or odd alike: folded into the exponent
+    q *= exp(fmax(lg, -600.0));
+    if (lg < -600.0) q *= exp(lg + 600.0);
+  }
   return copysign(ldexp(q, E / 2), zsign);
 }
 
-__global__ void __launch_bounds__(256) k_lowner(Plan P, int level, int64_t M, int small_k, bool listed) {
+// 128 threads: a block fits on an SM beside a CTA of the split product.
+__global__ void __launch_bounds__(128) k_lowner(Plan P, int level, int64_t M, int small_k, bool listed) {
   for_warp_roots(P, M, small_k, listed, [&](int64_t g, int K, int j) {
     const Node nd = make_node(P, level, g);
     const int64_t v0 = nd.v0;
     const double zh =
-        lowner_zhat(P.v.Dk + v0, P.v.org + v0, P.v.tau + v0, K, j, 2.0 * fabs(nd.b), P.v.zk[v0 + j]);
+        lowner_zhat(P.v.Dk + v0, P.v.org + v0, P.v.tau + v0, K, j, 2.0 * fabs(nd.b), P.v.zk[v0 + j],
+                    P.far ? far_record(P.far + g * P.far_stride, K, j) : nullptr);
     if ((threadIdx.x & 31) == 0) P.v.zhat[v0 + j] = zh;
   });
 }
@@ -2214,13 +2608,26 @@ __global__ void __launch_bounds__(256) k_lowner_small(Plan P, int level, int64_t
 
 // s_j = 1 / sqrt(sum_i (zhat_i / delta_ij)^2), delta_ij = (d_i - d_org(j)) - tau_j.
 template <int W = 32>
-__device__ double column_norm(const double* D, const double* zh, int K, double dorg, double tj) {
+__device__ double column_norm(const double* D, const double* zh, int K, double dorg, double tj,
+                              const double* far = nullptr) {
   double acc = 0.0;
-  for (int i = W == 32 ? (threadIdx.x & 31) : 0; i < K; i += W) {
+  const int lane = W == 32 ? (threadIdx.x & 31) : 0;
+  const int n0 = far ? far_range(far)[0] : 0, n1 = far ? far_range(far)[1] : K;
+  for (int i = n0 + lane; i < n1; i += W) {
     const double u = zh[i] * rcp_nr((D[i] - dorg) - tj);
     acc = fma(u, u, acc);
   }
-  if (W == 32) acc = warp_sum(acc);
+  if (W == 32) {
+    if (n0 > 0 || n1 < K) {
+      double bw, rd;
+      far_weights(far, (dorg - D[far_range(far)[4]]) + tj, bw, rd);
+      double num = lane < kFarM ? bw * far[2 * kFarM + lane] : 0.0;
+      warp_sum3(acc, num, bw);
+      acc = fma(num, rcp_nr(bw), acc);
+    } else {
+      acc = warp_sum(acc);
+    }
+  }
   return in_range(acc) ? rsqrt_nr(acc) : 1.0 / sqrt(acc);
 }
 
@@ -2231,16 +2638,18 @@ __device__ double column_norm(const double* D, const double* zh, int K, double d
 // two more multiply-adds per term.  The leftmost node of a level skips the first
 // row and the rightmost the last (no merge reads them).
 template <int W = 32>
-__device__ double column_norm_rows(const Plan& P, int64_t v0, int K, int j, bool need_f, bool need_l) {
+__device__ double column_norm_rows(const Plan& P, int64_t v0, int K, int j, bool need_f, bool need_l,
+                                   const double* far = nullptr) {
   const double* D = P.v.Dk + v0;
   const double* zh = P.v.zhat + v0;
   const double* pf = P.v.pf + v0;
   const double* pl = P.v.pl + v0;
   const double dorg = D[P.v.org[v0 + j]], tj = P.v.tau[v0 + j];
   double acc = 0.0, f = 0.0, l = 0.0;
-  const int i0 = W == 32 ? (threadIdx.x & 31) : 0;
+  const int n0 = far ? far_range(far)[0] : 0, n1 = far ? far_range(far)[1] : K;
+  const int i0 = n0 + (W == 32 ? (threadIdx.x & 31) : 0);
   if (need_f && need_l) {
-    for (int i = i0; i < K; i += W) {
+    for (int i = i0; i < n1; i += W) {
       const double u = zh[i] * rcp_nr((D[i] - dorg) - tj);
       acc = fma(u, u, acc);
       f = fma(pf[i], u, f);
@@ -2249,7 +2658,7 @@ __device__ double column_norm_rows(const Plan& P, int64_t v0, int K, int j, bool
   } else {
     const double* pq = need_f ? pf : pl;
     double x = 0.0;
-    for (int i = i0; i < K; i += W) {
+    for (int i = i0; i < n1; i += W) {
       const double u = zh[i] * rcp_nr((D[i] - dorg) - tj);
       acc = fma(u, u, acc);
       x = fma(pq[i], u, x);
@@ -2263,6 +2672,18 @@ __device__ double column_norm_rows(const Plan& P, int64_t v0, int K, int j, bool
       warp_sum2(acc, f);
     } else {
       warp_sum2(acc, l);
+    }
+    if (n0 > 0 || n1 < K) {
+      double bw, rd;
+      far_weights(far, (dorg - D[far_range(far)[4]]) + tj, bw, rd);
+      const int lane = threadIdx.x & 31, at = lane < kFarM ? lane : 0;
+      double fa = bw * far[2 * kFarM + at], ff = bw * far[3 * kFarM + at], fl = bw * far[4 * kFarM + at];
+      bw = warp_sum(bw);
+      warp_sum3(fa, ff, fl);
+      const double r = rcp_nr(bw);
+      acc = fma(fa, r, acc);
+      if (need_f) f = fma(ff, r, f);
+      if (need_l) l = fma(fl, r, l);
     }
   }
   const double sj = in_range(acc) ? rsqrt_nr(acc) : 1.0 / sqrt(acc);
@@ -2289,16 +2710,18 @@ __global__ void __launch_bounds__(256) k_colnorm_small(Plan P, int level, int64_
   P.v.scol[v0 + j] = column_norm<1>(D, P.v.zhat + v0, K, D[P.v.org[v0 + j]], P.v.tau[v0 + j]);
 }
 
-__global__ void __launch_bounds__(256) k_colnorm(Plan P, int level, int64_t M, int small_k, bool listed) {
+__global__ void __launch_bounds__(128, 6) k_colnorm(Plan P, int level, int64_t M, int small_k, bool listed) {
   for_warp_roots(P, M, small_k, listed, [&](int64_t g, int K, int j) {
     const int64_t v0 = make_node(P, level, g).v0;
+    // the last root lies past the last block's interval: direct
+    const double* far = P.far && j < K - 1 ? far_record(P.far + g * P.far_stride, K, j) : nullptr;
     double sj;
     if (level > 0) {
       const int64_t idx = g & ((((int64_t)1) << level) - 1);
-      sj = column_norm_rows(P, v0, K, j, idx != 0, idx != (((int64_t)1) << level) - 1);
+      sj = column_norm_rows(P, v0, K, j, idx != 0, idx != (((int64_t)1) << level) - 1, far);
     } else {
       const double* D = P.v.Dk + v0;
-      sj = column_norm(D, P.v.zhat + v0, K, D[P.v.org[v0 + j]], P.v.tau[v0 + j]);
+      sj = column_norm(D, P.v.zhat + v0, K, D[P.v.org[v0 + j]], P.v.tau[v0 + j], far);
     }
     if ((threadIdx.x & 31) == 0) P.v.scol[v0 + j] = sj;
   });
@@ -2383,7 +2806,7 @@ __global__ void __launch_bounds__(128) k_bd_secular(BdLevel L) {
   double t;
   bool conv;
   secular_root(L.DK + o, L.zK + o, L.zz + o, L.xz + o, L.xlo + o, K, (int)j, L.rho[blockIdx.y], L.max_iter, og, t, it,
-               conv);
+               conv, L.far ? L.far + blockIdx.y * L.far_stride : nullptr);
   if ((threadIdx.x & 31) == 0) {
     L.org[o + j] = og;
     L.tau[o + j] = t;
@@ -2396,7 +2819,8 @@ __global__ void __launch_bounds__(256) k_bd_lowner(BdLevel L) {
   const int K = L.cnt[4 * blockIdx.y];
   if (i >= K) return;
   const int64_t o = L.nodes[blockIdx.y].lo;
-  const double zh = lowner_zhat(L.DK + o, L.org + o, L.tau + o, K, (int)i, L.rho[blockIdx.y], L.zK[o + i]);
+  const double zh = lowner_zhat(L.DK + o, L.org + o, L.tau + o, K, (int)i, L.rho[blockIdx.y], L.zK[o + i],
+                                L.far ? far_record(L.far + blockIdx.y * L.far_stride, K, (int)i) : nullptr);
   if ((threadIdx.x & 31) == 0) L.zhat[o + i] = zh;
 }
 
@@ -2405,16 +2829,21 @@ __global__ void __launch_bounds__(256) k_bd_colnorm(BdLevel L) {
   const int K = L.cnt[4 * blockIdx.y];
   if (j >= K) return;
   const int64_t o = L.nodes[blockIdx.y].lo;
-  const double sj = column_norm(L.DK + o, L.zhat + o, K, L.DK[o + L.org[o + j]], L.tau[o + j]);
+  const double sj = column_norm(L.DK + o, L.zhat + o, K, L.DK[o + L.org[o + j]], L.tau[o + j],
+                                L.far && j < K - 1 ? far_record(L.far + blockIdx.y * L.far_stride, K, (int)j) : nullptr);
   if ((threadIdx.x & 31) == 0) L.scol[o + j] = sj;
 }
 
 cudaError_t launch_bd_rank_one(const BdLevel& L, cudaStream_t s) {
   auto grid = [&](int threads) { return dim3((unsigned)((L.max_nn * 32 + threads - 1) / threads), (unsigned)L.count); };
+  cudaError_t e = cudaSuccess;
+  if (L.far) e = launch_far<0, false>(L, 0, L.count, L.max_nn, s);
   k_bd_secular<<<grid(128), 128, 0, s>>>(L);
+  if (e == cudaSuccess && L.far) e = launch_far<1, false>(L, 0, L.count, L.max_nn, s);
   k_bd_lowner<<<grid(256), 256, 0, s>>>(L);
+  if (e == cudaSuccess && L.far) e = launch_far<2, false>(L, 0, L.count, L.max_nn, s);
   k_bd_colnorm<<<grid(256), 256, 0, s>>>(L);
-  return cudaGetLastError();
+  return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 cudaError_t launch_lowner(const Plan& P, const LevelLaunch& L, cudaStream_t s) {
@@ -2423,11 +2852,17 @@ cudaError_t launch_lowner(const Plan& P, const LevelLaunch& L, cudaStream_t s) {
   const int small_k = L.nslots >= kSmallMinSlots ? kSmallK : 0;
   const bool listed = small_k > 0;  // block list left by launch_secular's k_root_scan
   const dim3 wgrid = warp_root_grid(L, listed);
-  k_lowner<<<wgrid, 256, 0, s>>>(P, L.level, L.merges, small_k, listed);
-  if (small_k) k_lowner_small<<<tblocks, 256, 0, s>>>(P, L.level, L.merges);
-  cudaError_t e = cudaGetLastError();
+  cudaError_t e = cudaSuccess;
+  if (P.far) e = launch_far<1, false>(P, L.level, L.merges, L.max_n, s);
   if (e != cudaSuccess) return e;
-  k_colnorm<<<wgrid, 256, 0, s>>>(P, L.level, L.merges, small_k, listed);
+  k_lowner<<<wgrid, 128, 0, s>>>(P, L.level, L.merges, small_k, listed);
+  if (small_k) k_lowner_small<<<tblocks, 256, 0, s>>>(P, L.level, L.merges);
+  e = cudaGetLastError();
+  if (e == cudaSuccess && P.far)
+    e = L.level > 0 ? launch_far<2, true>(P, L.level, L.merges, L.max_n, s)
+                    : launch_far<2, false>(P, L.level, L.merges, L.max_n, s);
+  if (e != cudaSuccess) return e;
+  k_colnorm<<<wgrid, 128, 0, s>>>(P, L.level, L.merges, small_k, listed);
   if (small_k) k_colnorm_small<<<tblocks, 256, 0, s>>>(P, L.level, L.merges);
   return cudaGetLastError();
 }
