@@ -681,7 +681,8 @@ static int run_plan(HostPlan& H, const tdc_opts& o, const double* d, const doubl
         }
         const size_t b5 = timing ? evs.size() - 1 : 0;
         err = launch_split_list(lists[k], (int)items, cnts[k], P.split_slices, P.status, P.spin_budget, P.img,
-                                P.split_chunk_steps, P.stats ? &P.stats->split_level_max : nullptr, sg, mid);
+                                P.split_chunk_steps, P.stats ? &P.stats->split_level_max : nullptr,
+                                LL.level > 0 ? kSpareSms : 0, sg, mid);
         const size_t b6 = mark_on(sg);
         span(5, b4, b5);
         span(6, b5, b6);
@@ -1098,7 +1099,7 @@ static int cauchy_product(int64_t m, int64_t K, const double* A, int64_t lda, co
     const int64_t* cnts[4] = {A.counts + 3, A.counts + 0, A.counts + 1, A.counts + 2};
     for (int k = 0; k < 4 && err == cudaSuccess; ++k)
       err = launch_split_list(lists[k], (int)L.T, cnts[k], op.split_slices, st, op.spin_budget, img,
-                              op.split_chunk_k / 16, nullptr, cs, nullptr);
+                              op.split_chunk_k / 16, nullptr, 0, cs, nullptr);
     // the plain split product, emptied by the gate when the structured path took the part
     if (err == cudaSuccess) {
       GemmSeg* plain = (GemmSeg*)(p + L.plain);
@@ -1873,7 +1874,7 @@ int sbevd_run(int64_t n, int64_t b, const double* AB, int64_t ldab, double* lam,
       if (launch_bd_term(V, k, cs) != cudaSuccess || launch_bd_rank_one(V, cs) != cudaSuccess ||
           launch_bd_segs(V, cs) != cudaSuccess ||
           launch_split_list(V.segs, V.count, V.nsegs, op.split_slices, st, op.spin_budget, img, op.split_chunk_k / 16,
-                            nullptr, cs, nullptr) != cudaSuccess ||
+                            nullptr, 0, cs, nullptr) != cudaSuccess ||
           launch_dense_list(V.dsegs, V.count, V.max_nn, std::min<int64_t>(V.max_nn, 128), cs) != cudaSuccess ||
           launch_bd_finish(V, cs) != cudaSuccess)
         return TDC_ECUDA;

@@ -579,7 +579,11 @@ cudaError_t launch_seg_split(const GemmSeg* segs_dev, int nseg, int S, int* stat
                              __nv_bfloat16* img, int chunk_steps, cudaStream_t s);
 cudaError_t launch_split_list(const GemmSeg* segs, int nseg_bound, const int64_t* dcount, int S, int* status,
                               long long spin_budget, __nv_bfloat16* img, int chunk_steps, unsigned int* lvl_max,
-                              cudaStream_t s, cudaEvent_t mid);
+                              int spare, cudaStream_t s, cudaEvent_t mid);
+// SMs that the products of a tree level leave to the next level's roots on the other stream
+// (the blocks of k_prepare and k_finalize fit beside no product block): at 16384 of
+// tridiag(1,2,1) 0 / 2 / 4 of them took 41.6 / 40.8 / 40.8 ms.  The last level needs none.
+constexpr int kSpareSms = 2;
 cudaError_t launch_srrsc(const GemmSeg* segs, int nseg, const StructArgs& A, cudaStream_t s);
 cudaError_t launch_struct_fallback(const GemmSeg* segs, int nseg, const StructArgs& A, cudaStream_t s);
 cudaError_t launch_ss_build(const SSArgs& A, cudaStream_t s);

@@ -451,58 +451,71 @@ constexpr int kEpiWarps = 16, kMmaWarp = 16, kLoadWarp = 17, kSplitThreads = 576
 constexpr int kEpiCols = BN / (kEpiWarps / 4);  // columns per epilogue warp
 static_assert(kEpiCols == 16, "epilogue column split: one 16-column TMEM load per level");
 
-// Level m < 5 of one hand-off (16 columns, exact integers held in FP32) into the
+// Level m < 5 of one hand-off (W columns from column W H, exact integers held in FP32) into the
 // 64-bit running sums: hi += P_m 2^sh with sh = 8 (4 - m).  An FP32 integer v with
 // |v| < 2^22 becomes an integer without the conversion unit (16 per clock per SM):
 // v + 1.5 2^23 lies in [2^23, 2^24), where the float's ulp is 1, so its bit pattern
-// is 0x4B400000 + v exactly; bias collects the 0x4B400000 2^sh this adds, removed
+// is 0x4B400000 + v exactly; the 0x4B400000 2^sh this adds (drain_bias) is removed
 // once per tile.  A thread holding a larger value (a level sum near the 2^24 limit)
 // forms the same 0x4B400000 + v with cvt instead.  The sums are kept modulo 2^64
 // (unsigned) and are exact once the bias is removed.
-__device__ __forceinline__ void add_level_int(const uint32_t (&r)[16], int sh, unsigned long long (&hi)[16],
-                                              unsigned long long& bias, float& gmax) {
+template <int W, int H>
+__device__ __forceinline__ void add_level_int(const uint32_t (&r)[W], int sh, unsigned long long (&hi)[16],
+                                              float& gmax) {
   float mx = 0.0f;
 #pragma unroll
-  for (int i = 0; i < 16; ++i) mx = fmaxf(mx, fabsf(__uint_as_float(r[i])));
+  for (int i = 0; i < W; ++i) mx = fmaxf(mx, fabsf(__uint_as_float(r[i])));
   gmax = fmaxf(gmax, mx);
   if (mx < 4194304.0f) {
 #pragma unroll
-    for (int i = 0; i < 16; ++i)
-      hi[i] += (unsigned long long)__float_as_uint(__uint_as_float(r[i]) + 12582912.0f) << sh;
+    for (int i = 0; i < W; ++i)
+      hi[W * H + i] += (unsigned long long)__float_as_uint(__uint_as_float(r[i]) + 12582912.0f) << sh;
   } else {
 #pragma unroll
-    for (int i = 0; i < 16; ++i)
-      hi[i] += (unsigned long long)((long long)__float2int_rn(__uint_as_float(r[i])) + 0x4B400000ll) << sh;
+    for (int i = 0; i < W; ++i)
+      hi[W * H + i] += (unsigned long long)((long long)__float2int_rn(__uint_as_float(r[i])) + 0x4B400000ll) << sh;
   }
-  bias += 0x4B400000ull << sh;
 }
 
 // One hand-off of the S level accumulators (this warp's 32 TMEM lanes, 16 columns at
-// ta): hi += sum_{m<5} P_m 2^(8(4-m)), lo += P_6 2^-8 then += P_5.  One level at a
-// time (16 registers; sixteen epilogue warps hide the load latency).  Summing these
+// ta): hi += sum_{m<5} P_m 2^(8(4-m)), lo += P_6 2^-8 then += P_5.  W columns of one
+// level at a time (W registers; sixteen epilogue warps hide the load latency).  Summing these
 // per hand-off gives the same integers as the per-tile Horner combination, and lo
 // the same FP32 roundings.
-template <int S>
-__device__ __forceinline__ void drain_levels(uint32_t ta, unsigned long long (&hi)[16], float (&lo)[16],
-                                             unsigned long long& bias, float& gmax) {
-  uint32_t a[16];
+template <int S, int W, int H>
+__device__ __forceinline__ void drain_part(uint32_t ta, unsigned long long (&hi)[16], float (&lo)[16], float& gmax) {
+  uint32_t a[W];
 #pragma unroll
   for (int m = 0; m < 5; ++m) {
     if (m < S) {
-      umma::tmem_ld16_nowait(ta + (uint32_t)(m * BN), a);
+      umma::tmem_ld_nowait(ta + (uint32_t)(m * BN + W * H), a);
       umma::tmem_wait_ld(a);
-      add_level_int(a, 8 * (4 - m), hi, bias, gmax);
+      add_level_int<W, H>(a, 8 * (4 - m), hi, gmax);
     }
   }
 #pragma unroll
   for (int m = 6; m >= 5; --m) {
     if (m < S) {
-      umma::tmem_ld16_nowait(ta + (uint32_t)(m * BN), a);
+      umma::tmem_ld_nowait(ta + (uint32_t)(m * BN + W * H), a);
       umma::tmem_wait_ld(a);
 #pragma unroll
-      for (int i = 0; i < 16; ++i) lo[i] += m == 6 ? __uint_as_float(a[i]) * 0.00390625f : __uint_as_float(a[i]);
+      for (int i = 0; i < W; ++i)
+        lo[W * H + i] += m == 6 ? __uint_as_float(a[i]) * 0.00390625f : __uint_as_float(a[i]);
     }
   }
+}
+template <int S, int W>
+__device__ __forceinline__ void drain_levels(uint32_t ta, unsigned long long (&hi)[16], float (&lo)[16],
+                                             float& gmax) {
+  drain_part<S, W, 0>(ta, hi, lo, gmax);
+  if constexpr (W == 8) drain_part<S, W, 1>(ta, hi, lo, gmax);
+}
+// what a hand-off's biased integers add to hi beyond the sums
+template <int S>
+__device__ __forceinline__ constexpr unsigned long long drain_bias() {
+  unsigned long long b = 0;
+  for (int m = 0; m < 5 && m < S; ++m) b += 0x4B400000ull << (8 * (4 - m));
+  return b;
 }
 
 // Bound of the waits on the give-up path (copies and MMAs already issued, which
@@ -551,10 +564,11 @@ __device__ __forceinline__ TileRef tile_ref(const GemmSeg* segs, int nseg, int64
 // kChunk: the accumulators are drained into the epilogue's running sums every ck
 // k-steps of a tile (the MMA warp waits for each drain), so that every level sum
 // covers at most 16 ck terms; without it they cover the tile's whole reduction.
-template <int S, bool kChunk>
-__global__ void __launch_bounds__(kSplitThreads, 1) k_gemm_split(const GemmSeg* segs, int nseg, const int64_t* dnseg,
-                                                                 const __nv_bfloat16* img, int* status,
-                                                                 long long budget, int ck, unsigned int* lvl_max) {
+// kShare: levels 8 columns at a time (see k_gemm_split_shared).
+template <int S, bool kChunk, bool kShare>
+__device__ __forceinline__ void gemm_split(const GemmSeg* segs, int nseg, const int64_t* dnseg,
+                                           const __nv_bfloat16* img, int* status, long long budget, int ck,
+                                           unsigned int* lvl_max) {
   if (dnseg) nseg = (int)*dnseg;
   extern __shared__ __align__(1024) uint8_t smem[];
   constexpr uint32_t a_bytes = S * kATileElems * 2, b_bytes = S * kBTileElems * 2;
@@ -710,7 +724,7 @@ __global__ void __launch_bounds__(kSplitThreads, 1) k_gemm_split(const GemmSeg* 
         // the same combination, accumulated over the tile's chunks: level m of a
         // chunk adds P_m 2^(8(4-m)) to hi (m < 5, exact) or its share to lo
         const int nch = t.KB > 0 ? (t.KB + ck - 1) / ck : 1;
-        unsigned long long hu[kEpiCols], bias = 0;
+        unsigned long long hu[kEpiCols];
         float lo[kEpiCols];
 #pragma unroll
         for (int i = 0; i < kEpiCols; ++i) {
@@ -723,7 +737,7 @@ __global__ void __launch_bounds__(kSplitThreads, 1) k_gemm_split(const GemmSeg* 
           okc = __all_sync(0xffffffffu, wait_or_fail(tfull, (uint32_t)(it & 1), budget, vfail));
           if (!okc) break;
           umma::tc_fence_after();
-          if (t.KB > 0) drain_levels<S>(tl + (uint32_t)c0, hu, lo, bias, gmax);
+          if (t.KB > 0) drain_levels<S, kShare ? 8 : 16>(tl + (uint32_t)c0, hu, lo, gmax);
           umma::tc_fence_before();
           __syncwarp();
           if (lane == 0) mbar_arrive(tempty);
@@ -732,6 +746,7 @@ __global__ void __launch_bounds__(kSplitThreads, 1) k_gemm_split(const GemmSeg* 
           if (lane == 0) *vfail = 1;
           break;
         }
+        const unsigned long long bias = t.KB > 0 ? (unsigned long long)nch * drain_bias<S>() : 0ull;
         long long hi[kEpiCols];
 #pragma unroll
         for (int i = 0; i < kEpiCols; ++i) hi[i] = (long long)(hu[i] - bias);
@@ -772,14 +787,15 @@ __global__ void __launch_bounds__(kSplitThreads, 1) k_gemm_split(const GemmSeg* 
       umma::tc_fence_after();
       double val[kEpiCols];
       {
-        unsigned long long hu[kEpiCols], bias = 0;
+        unsigned long long hu[kEpiCols];
+        const unsigned long long bias = t.KB > 0 ? drain_bias<S>() : 0ull;
         float lo[kEpiCols];
 #pragma unroll
         for (int i = 0; i < kEpiCols; ++i) {
           hu[i] = 0;
           lo[i] = 0.0f;
         }
-        if (t.KB > 0) drain_levels<S>(tl + (uint32_t)c0, hu, lo, bias, gmax);
+        if (t.KB > 0) drain_levels<S, kShare ? 8 : 16>(tl + (uint32_t)c0, hu, lo, gmax);
         long long hi[kEpiCols];
 #pragma unroll
         for (int i = 0; i < kEpiCols; ++i) hi[i] = (long long)(hu[i] - bias);
@@ -827,6 +843,26 @@ __global__ void __launch_bounds__(kSplitThreads, 1) k_gemm_split(const GemmSeg* 
   if (warp == 0) umma::tmem_dealloc(tmem, 512);
 }
 
+template <int S, bool kChunk>
+__global__ void __launch_bounds__(kSplitThreads, 1) k_gemm_split(const GemmSeg* segs, int nseg, const int64_t* dnseg,
+                                                                 const __nv_bfloat16* img, int* status,
+                                                                 long long budget, int ck, unsigned int* lvl_max) {
+  gemm_split<S, kChunk, false>(segs, nseg, dnseg, img, status, budget, ck, lvl_max);
+}
+// The form of a tree's products, beside which the next level's root kernels run on another
+// stream.  With 96 registers two of the SM's quarters have no registers left for a fifth warp
+// of more than 32, so that every root kernel waited for the end of the product (4 ms at
+// n = 16384); with 80 a block of 128 threads of up to 112 registers fits beside it.  The
+// price is 8-column drains (1.2 % at 4096 x 4096 x 4096), so products that run alone keep the
+// other form.  With kSpareSms SMs left free for the larger blocks: tridiag(1,2,1) n = 16384
+// 42.3 -> 40.1 ms, harmonic chain n = 4999 6.29 -> 6.23 ms.
+template <int S, bool kChunk>
+__global__ void __maxnreg__(80) k_gemm_split_shared(const GemmSeg* segs, int nseg, const int64_t* dnseg,
+                                                    const __nv_bfloat16* img, int* status, long long budget, int ck,
+                                                    unsigned int* lvl_max) {
+  gemm_split<S, kChunk, true>(segs, nseg, dnseg, img, status, budget, ck, lvl_max);
+}
+
 static cudaError_t launch_split_digits(const GemmSeg* segs, int nseg, const int64_t* dnseg, int S, int* status,
                                        __nv_bfloat16* img, cudaStream_t s) {
   k_split_a<<<152 * 8, 256, 0, s>>>(segs, nseg, dnseg, S, img, status);
@@ -839,37 +875,39 @@ static cudaError_t launch_split_digits(const GemmSeg* segs, int nseg, const int6
 template <int S, bool kChunk>
 static cudaError_t launch_split_mma_s(const GemmSeg* segs, int nseg, const int64_t* dnseg, int* status,
                                       long long budget, const __nv_bfloat16* img, int sms, int ck,
-                                      unsigned int* lvl_max, cudaStream_t s) {
+                                      unsigned int* lvl_max, bool share, cudaStream_t s) {
   const int smem = kStages * S * (kATileElems + kBTileElems) * 2 + 128;
-  cudaError_t e = cudaFuncSetAttribute(k_gemm_split<S, kChunk>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  const auto kernel = share ? k_gemm_split_shared<S, kChunk> : k_gemm_split<S, kChunk>;
+  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
-  k_gemm_split<S, kChunk><<<sms, kSplitThreads, smem, s>>>(segs, nseg, dnseg, img, status, budget, ck, lvl_max);
+  kernel<<<sms, kSplitThreads, smem, s>>>(segs, nseg, dnseg, img, status, budget, ck, lvl_max);
   return cudaGetLastError();
 }
 
-// ck > 0: drain the accumulators every ck k-steps
+// ck > 0: drain the accumulators every ck k-steps; spare: SMs left to kernels of another stream
 static cudaError_t launch_split_mma(const GemmSeg* segs, int nseg, const int64_t* dnseg, int S, int* status,
                                     long long budget, const __nv_bfloat16* img, int ck, unsigned int* lvl_max,
-                                    cudaStream_t s) {
+                                    int spare, cudaStream_t s) {
   int dev = 0, sms = 152;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  sms = sms > 4 * spare ? sms - spare : sms;
   if (ck > 0) {
     switch (S) {
-      case 3: return launch_split_mma_s<3, true>(segs, nseg, dnseg, status, budget, img, sms, ck, lvl_max, s);
-      case 4: return launch_split_mma_s<4, true>(segs, nseg, dnseg, status, budget, img, sms, ck, lvl_max, s);
-      case 5: return launch_split_mma_s<5, true>(segs, nseg, dnseg, status, budget, img, sms, ck, lvl_max, s);
-      case 6: return launch_split_mma_s<6, true>(segs, nseg, dnseg, status, budget, img, sms, ck, lvl_max, s);
-      case 7: return launch_split_mma_s<7, true>(segs, nseg, dnseg, status, budget, img, sms, ck, lvl_max, s);
+      case 3: return launch_split_mma_s<3, true>(segs, nseg, dnseg, status, budget, img, sms, ck, lvl_max, spare > 0, s);
+      case 4: return launch_split_mma_s<4, true>(segs, nseg, dnseg, status, budget, img, sms, ck, lvl_max, spare > 0, s);
+      case 5: return launch_split_mma_s<5, true>(segs, nseg, dnseg, status, budget, img, sms, ck, lvl_max, spare > 0, s);
+      case 6: return launch_split_mma_s<6, true>(segs, nseg, dnseg, status, budget, img, sms, ck, lvl_max, spare > 0, s);
+      case 7: return launch_split_mma_s<7, true>(segs, nseg, dnseg, status, budget, img, sms, ck, lvl_max, spare > 0, s);
       default: return cudaErrorInvalidValue;
     }
   }
   switch (S) {
-    case 3: return launch_split_mma_s<3, false>(segs, nseg, dnseg, status, budget, img, sms, 0, lvl_max, s);
-    case 4: return launch_split_mma_s<4, false>(segs, nseg, dnseg, status, budget, img, sms, 0, lvl_max, s);
-    case 5: return launch_split_mma_s<5, false>(segs, nseg, dnseg, status, budget, img, sms, 0, lvl_max, s);
-    case 6: return launch_split_mma_s<6, false>(segs, nseg, dnseg, status, budget, img, sms, 0, lvl_max, s);
-    case 7: return launch_split_mma_s<7, false>(segs, nseg, dnseg, status, budget, img, sms, 0, lvl_max, s);
+    case 3: return launch_split_mma_s<3, false>(segs, nseg, dnseg, status, budget, img, sms, 0, lvl_max, spare > 0, s);
+    case 4: return launch_split_mma_s<4, false>(segs, nseg, dnseg, status, budget, img, sms, 0, lvl_max, spare > 0, s);
+    case 5: return launch_split_mma_s<5, false>(segs, nseg, dnseg, status, budget, img, sms, 0, lvl_max, spare > 0, s);
+    case 6: return launch_split_mma_s<6, false>(segs, nseg, dnseg, status, budget, img, sms, 0, lvl_max, spare > 0, s);
+    case 7: return launch_split_mma_s<7, false>(segs, nseg, dnseg, status, budget, img, sms, 0, lvl_max, spare > 0, s);
     default: return cudaErrorInvalidValue;
   }
 }
@@ -893,26 +931,26 @@ cudaError_t launch_gemm_split(const Plan& P, const LevelLaunch& L, int64_t g0, i
   if (e != cudaSuccess) return e;
   if (mid) cudaEventRecord(mid, s);
   return launch_split_mma(P.segs, nseg, dn, P.split_slices, P.status, P.spin_budget, P.img, P.split_chunk_steps,
-                          P.stats ? &P.stats->split_level_max : nullptr, s);
+                          P.stats ? &P.stats->split_level_max : nullptr, L.level > 0 ? kSpareSms : 0, s);
 }
 
 // A segment list whose count lives on the device (*dcount; nseg_bound bounds it):
 // digit images, then the products; `mid` (optional) is recorded between the two.
 cudaError_t launch_split_list(const GemmSeg* segs, int nseg_bound, const int64_t* dcount, int S, int* status,
                               long long spin_budget, __nv_bfloat16* img, int chunk_steps, unsigned int* lvl_max,
-                              cudaStream_t s, cudaEvent_t mid) {
+                              int spare, cudaStream_t s, cudaEvent_t mid) {
   if (nseg_bound <= 0) return cudaSuccess;
   cudaError_t e = launch_split_digits(segs, nseg_bound, dcount, S, status, img, s);
   if (e != cudaSuccess) return e;
   if (mid) cudaEventRecord(mid, s);
-  return launch_split_mma(segs, nseg_bound, dcount, S, status, spin_budget, img, chunk_steps, lvl_max, s);
+  return launch_split_mma(segs, nseg_bound, dcount, S, status, spin_budget, img, chunk_steps, lvl_max, spare, s);
 }
 
 cudaError_t launch_seg_split(const GemmSeg* segs_dev, int nseg, int S, int* status, long long spin_budget,
                              __nv_bfloat16* img, int chunk_steps, cudaStream_t s) {
   cudaError_t e = launch_split_digits(segs_dev, nseg, nullptr, S, status, img, s);
   if (e != cudaSuccess) return e;
-  return launch_split_mma(segs_dev, nseg, nullptr, S, status, spin_budget, img, chunk_steps, nullptr, s);
+  return launch_split_mma(segs_dev, nseg, nullptr, S, status, spin_budget, img, chunk_steps, nullptr, 0, s);
 }
 
 }  // namespace tdc
