@@ -50,7 +50,6 @@ namespace {
 constexpr int BM = kSplitBM, BN = kSplitBN, BK = kSplitBK;
 constexpr int kATileElems = BM * BK;  // 2048 per slice (4 KB)
 constexpr int kBTileElems = BN * BK;  // 1024 per slice (2 KB)
-constexpr int kMaxS = 7;
 constexpr int kStages = 4;
 constexpr int kGroupRows = 8;
 
@@ -61,53 +60,64 @@ __host__ __device__ inline int64_t cdiv(int64_t a, int64_t b) { return (a + b - 
 __device__ __forceinline__ int core_off(int r, int k) { return (r >> 3) * (BK * 8) + (k >> 3) * 64 + (r & 7) * 8 + (k & 7); }
 
 
-// The S leading balanced base-256 digits of x (|x| <= 1 + O(eps)), as BF16 bit
-// patterns: F = round(x 2^56) as a two's-complement integer, written as
-// F = sum_s d_s 256^(6-s) with d_s in [-128, 127] for s >= 1 (the top digit carries
-// the rest, |d_0| <= 256).  Below the top digit the digits are zero-mean whatever
-// the sign of x, so sums of their products behave like random walks.  With
-// G = F + 128 (1 + 256 + ... + 256^5) the bytes of G below bit 48 are d_s + 128 and
-// G >> 48 is d_0, so the digits come out of 32-bit field extractions; a small
-// integer d becomes a float as (2^23 + 2^22 + d) - (2^23 + 2^22) on the FP32 pipe,
-// and its BF16 pattern is the float's upper half (exact: |d| <= 256).
-__device__ __forceinline__ void digits_bf16(double x, int S, uint32_t (&dg)[kMaxS]) {
-  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
-  const bool neg = (b >> 63) != 0;
-  int e = (int)((b >> 52) & 0x7FF);
-  unsigned long long m = b & 0xFFFFFFFFFFFFFull;
-  if (e) m |= 1ull << 52; else e = 1;
-  const int sh = e - 1019;  // |x| 2^56 = m * 2^(e - 1075 + 56)
-  unsigned long long mag;
-  if (sh >= 0) mag = (sh < 8) ? (m << sh) : 0ull;
-  else if (sh > -63) mag = ((m >> (-sh - 1)) + 1ull) >> 1;  // round half up
-  else mag = 0ull;
-  const long long F = neg ? -(long long)mag : (long long)mag;
-  const long long G = F + 0x808080808080ll;
-  const uint32_t lo = (uint32_t)G;
-  const int hi = (int)(G >> 32);
-  int d[kMaxS];
-  d[0] = hi >> 16;
-  d[1] = ((hi >> 8) & 255) - 128;
-  d[2] = (hi & 255) - 128;
-  d[3] = (int)(lo >> 24) - 128;
-  d[4] = (int)((lo >> 16) & 255) - 128;
-  d[5] = (int)((lo >> 8) & 255) - 128;
-  d[6] = (int)(lo & 255) - 128;
-#pragma unroll
-  for (int s = 0; s < kMaxS; ++s) {
-    const float f = __int_as_float(0x4B400000 + d[s]) - 12582912.0f;
-    dg[s] = (s < S) ? (__float_as_uint(f) >> 16) : 0u;
+// The balanced base-256 digits of x 2^-ae (magnitude <= 1 + O(eps)): F = round(x 2^(56-ae)) as
+// a two's-complement integer, written as F = sum_s d_s 256^(6-s) with d_s in [-128, 127] for
+// s >= 1 (the top digit carries the rest, |d_0| <= 256).  Below the top digit the digits are
+// zero-mean whatever the sign of x, so sums of their products behave like random walks.
+// Returned is G = F + 128 (1 + 256 + ... + 256^5): its bytes below bit 48 are d_s + 128 and
+// G >> 48 is d_0.  The scale enters by the exponent field (a subnormal x is multiplied first);
+// beyond the contract (16 and above, infinities, NaN) F is 0.
+__device__ __forceinline__ long long digit_word(double x, int ae) {
+  uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
+  uint32_t e = (hi >> 20) & 0x7FFu;
+  if (e - 1u >= 0x7FEu) {  // zero or subnormal (or not finite)
+    if (ae == 0 || e != 0) return 0x808080808080ll;
+    x *= pow2c(-ae);
+    ae = 0;
+    hi = (uint32_t)__double2hiint(x);
+    lo = (uint32_t)__double2loint(x);
+    e = (hi >> 20) & 0x7FFu;
+    if (e == 0) return 0x808080808080ll;
   }
+  const unsigned long long m = ((unsigned long long)((hi & 0xFFFFFu) | 0x100000u) << 32) | lo;
+  // |x| 2^(56-ae) = m 2^(e - ae - 1019); one bit more for the rounding (half up)
+  const uint32_t r = min((uint32_t)(1026 + ae) - e, 63u);  // above 63: below the last digit, or too large
+  const long long mag = (long long)((((m << 8) >> r) + 1) >> 1), sg = (long long)((int)hi >> 31);
+  return ((mag ^ sg) - sg) + 0x808080808080ll;
 }
 
-// Eight BF16 patterns (low halves of v[0..7]) into one 16-byte store.
-__device__ __forceinline__ uint4 pack8(const uint32_t* v) {
-  uint4 o;
-  o.x = v[0] | (v[1] << 16);
-  o.y = v[2] | (v[3] << 16);
-  o.z = v[4] | (v[5] << 16);
-  o.w = v[6] | (v[7] << 16);
-  return o;
+// Digit s of eight consecutive k as BF16 patterns (one 16-byte store).  A byte v = d + 128
+// becomes the BF16 number d without the FP32 pipe, two at a time: 0x4300 | (v & 127) is
+// 128 + (v & 127), to which -128 (v >= 128) or -256 is added, all exact in 8 bits.
+template <int s>
+__device__ __forceinline__ uint4 digit_pack(const long long (&g)[8]) {
+  uint32_t o[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const long long ga = g[2 * i], gb = g[2 * i + 1];
+    if constexpr (s == 0) {  // integers up to 256, through FP32: 1.5 2^23 + d
+      const float fa = __int_as_float(0x4B400000 + ((int)(ga >> 32) >> 16)) - 12582912.0f;
+      const float fb = __int_as_float(0x4B400000 + ((int)(gb >> 32) >> 16)) - 12582912.0f;
+      o[i] = __byte_perm(__float_as_uint(fa), __float_as_uint(fb), 0x7632);
+    } else {
+      constexpr int byte = (6 - s) & 3;
+      const uint32_t wa = s < 3 ? (uint32_t)(ga >> 32) : (uint32_t)ga, wb = s < 3 ? (uint32_t)(gb >> 32) : (uint32_t)gb;
+      const uint32_t v = __byte_perm(wa, wb, byte * 0x11 + (4 + byte) * 0x1100);  // bytes 0 and 2
+      const uint32_t a = (v & 0x007F007Fu) | 0x43004300u, b = (~v & 0x00800080u) | 0xC300C300u;
+      asm("add.rn.bf16x2 %0, %1, %2;" : "=r"(o[i]) : "r"(a), "r"(b));
+    }
+  }
+  return make_uint4(o[0], o[1], o[2], o[3]);
+}
+// the S slices of eight consecutive k of one row or column, `slice` elements apart
+__device__ __forceinline__ void store_digits(__nv_bfloat16* dst, int slice, int S, const long long (&g)[8]) {
+  *reinterpret_cast<uint4*>(dst) = digit_pack<0>(g);
+  *reinterpret_cast<uint4*>(dst + slice) = digit_pack<1>(g);
+  *reinterpret_cast<uint4*>(dst + 2 * slice) = digit_pack<2>(g);
+  if (S > 3) *reinterpret_cast<uint4*>(dst + 3 * slice) = digit_pack<3>(g);
+  if (S > 4) *reinterpret_cast<uint4*>(dst + 4 * slice) = digit_pack<4>(g);
+  if (S > 5) *reinterpret_cast<uint4*>(dst + 5 * slice) = digit_pack<5>(g);
+  if (S > 6) *reinterpret_cast<uint4*>(dst + 6 * slice) = digit_pack<6>(g);
 }
 
 __device__ __forceinline__ int find_seg(const GemmSeg* segs, int nseg, int64_t w, int which) {
@@ -319,106 +329,137 @@ __device__ __forceinline__ double level_value(long long I, int adj) {
   return scale2(__longlong_as_double(b - (58ll << 52)), adj);
 }
 
+// Digit tiles are taken in runs of neighbours along k: the segment search and the division that
+// place a tile cost as much as the digits of a thread's 8 elements.  A run is as long as the
+// grid's share of the tiles, at most kRun.
+//
+// Bound by latency and instructions rather than by the 22 bytes an element moves: taking every
+// tile by itself and every digit through FP32 cost 135 instructions an element.  The digits of
+// an 8192 x 8192 operand pair (top merge of tridiag(1,2,1) n = 16384) 1024 -> 603 us, all of
+// that solve 40.1 -> 37.9 ms, the 8192 x 8192 Cauchy-like product 5.66 -> 5.29 ms.
+constexpr int kRun = 8;
+struct DigitRun {
+  int64_t w, end;  // tiles [w, end)
+  int si, t, kb, KB;  // segment, row or column tile, k-tile, k-tiles of the segment
+};
+template <int kB>
+__device__ __forceinline__ void run_place(const GemmSeg* segs, DigitRun& r) {
+  const GemmSeg& sg = segs[r.si];
+  const int64_t local = r.w - (kB ? sg.it_b : sg.it_a);
+  r.KB = (int)cdiv(sg.kk, BK);
+  r.t = (int)(local / r.KB);
+  r.kb = (int)(local - (int64_t)r.t * r.KB);
+}
+template <int kB>
+__device__ __forceinline__ void run_next(const GemmSeg* segs, DigitRun& r) {
+  if (++r.w >= r.end || ++r.kb < r.KB) return;
+  r.kb = 0;
+  ++r.t;
+  if (r.w < (kB ? segs[r.si + 1].it_b : segs[r.si + 1].it_a)) return;
+  while (r.w >= (kB ? segs[r.si + 1].it_b : segs[r.si + 1].it_a)) ++r.si;  // ends: w < the terminator's
+  run_place<kB>(segs, r);
+}
+
 __global__ void __launch_bounds__(256) k_split_a(const GemmSeg* segs, int nseg, const int64_t* dnseg, int S,
                                                  __nv_bfloat16* img, int* status) {
   if (dnseg) nseg = (int)*dnseg;
-  const int64_t total = segs[nseg].it_a;
-  const int tid = threadIdx.x;
-  for (int64_t w = blockIdx.x; w < total; w += gridDim.x) {
-    const int si = find_seg(segs, nseg, w, 0);
-    const GemmSeg& sg = segs[si];
-    const int64_t local = w - sg.it_a;
-    const int KB = (int)cdiv(sg.kk, BK);
-    const int rt = (int)(local / KB), kb = (int)(local % KB);
-    const int64_t toff = sg.a_img + ((int64_t)rt * KB + kb) * S * kATileElems;
-    if (toff < 0 || toff + (int64_t)S * kATileElems > segs[nseg].a_img) {  // never write outside the images
-      if (threadIdx.x == 0) set_status(status, TDC_EUNSUPPORTED);
-      continue;
-    }
-    __nv_bfloat16* tile = img + toff;
-    for (int u = tid; u < BM * (BK / 8); u += blockDim.x) {
-      const int r = u % BM, kg = u / BM;  // BK/8 groups of 8 consecutive k
-      const int row = rt * BM + r;
-      uint32_t dig[8][kMaxS];
+  const int64_t total = segs[nseg].it_a, cap = segs[nseg].a_img;
+  const int64_t run = max((int64_t)1, min((int64_t)kRun, total / gridDim.x));
+  static_assert(BM * (BK / 8) == 256, "a thread takes 8 consecutive k of one row of a tile");
+  const int r = threadIdx.x % BM, k0 = (threadIdx.x / BM) * 8, off = core_off(r, k0);
+  for (int64_t c = blockIdx.x; c * run < total; c += gridDim.x) {
+    DigitRun R;
+    R.w = c * run;
+    R.end = min(total, R.w + run);
+    R.si = find_seg(segs, nseg, R.w, 0);
+    run_place<0>(segs, R);
+    for (; R.w < R.end; run_next<0>(segs, R)) {
+      const GemmSeg& sg = segs[R.si];
+      const int64_t toff = sg.a_img + ((int64_t)R.t * R.KB + R.kb) * S * kATileElems;
+      if (toff < 0 || toff + (int64_t)S * kATileElems > cap) {  // never write outside the images
+        if (threadIdx.x == 0) set_status(status, TDC_EUNSUPPORTED);
+        continue;
+      }
+      const int row = R.t * BM + r, q0 = R.kb * BK + k0;
+      const bool live = row < sg.rows;
+      const double* A = sg.A + (int64_t)row * sg.ars;
+      const int64_t kk = sg.kk, lda = sg.lda;
+      const int32_t *plist = sg.plist, *acol = sg.acol;
+      const int ae = min(max(sg.aexp, -1023), 1022);
+      double x[8];
 #pragma unroll
       for (int i = 0; i < 8; ++i) {
-        const int q = kb * BK + kg * 8 + i;
-        double x = 0.0;
-        if (q < sg.kk && row < sg.rows) {
-          const int p = sg.plist ? sg.plist[q] : q;
-          const int col = sg.acol ? sg.acol[p] : p;
-          x = sg.A[(int64_t)row * sg.ars + (int64_t)col * sg.lda];
-          if (sg.aexp) x *= pow2c(-sg.aexp);
+        const int q = q0 + i;
+        x[i] = 0.0;
+        if (live && q < kk) {
+          const int p = plist ? plist[q] : q;
+          x[i] = A[(int64_t)(acol ? acol[p] : p) * lda];
         }
-        digits_bf16(x, S, dig[i]);
       }
-      const int off = core_off(r, kg * 8);
+      long long g[8];
 #pragma unroll
-      for (int s = 0; s < kMaxS; ++s) {
-        if (s >= S) break;
-        uint32_t v[8];
-#pragma unroll
-        for (int i = 0; i < 8; ++i) v[i] = dig[i][s];
-        *reinterpret_cast<uint4*>(tile + (int64_t)s * kATileElems + off) = pack8(v);
-      }
+      for (int i = 0; i < 8; ++i) g[i] = digit_word(x[i], ae);
+      store_digits(img + toff + off, kATileElems, S, g);
     }
   }
 }
 
-// Two B tiles per block iteration: threads 0-127 and 128-255 each take one
-// (64 columns x BK/8 groups of 8 poles).
+// Threads 0-127 and 128-255 of a block each take their own run of B tiles (64 columns x BK/8
+// groups of 8 poles).
 static_assert(BN * (BK / 8) == 128, "k_split_b maps 128 threads onto one B tile");
 __global__ void __launch_bounds__(256) k_split_b(const GemmSeg* segs, int nseg, const int64_t* dnseg, int S,
                                                  __nv_bfloat16* img, int* status) {
   if (dnseg) nseg = (int)*dnseg;
-  const int64_t total = segs[nseg].it_b;
+  const int64_t total = segs[nseg].it_b, cap = segs[nseg].a_img;
+  const int64_t run = max((int64_t)1, min((int64_t)kRun, total / (2 * gridDim.x)));
   const int tid = threadIdx.x & 127;
-  for (int64_t w = 2 * (int64_t)blockIdx.x + (threadIdx.x >> 7); w < total; w += 2 * (int64_t)gridDim.x) {
-    const int si = find_seg(segs, nseg, w, 1);
-    const GemmSeg& sg = segs[si];
-    const int64_t local = w - sg.it_b;
-    const int KB = (int)cdiv(sg.kk, BK);
-    const int ct = (int)(local / KB), kb = (int)(local % KB);
-    const int64_t toff = sg.b_img + ((int64_t)ct * KB + kb) * S * kBTileElems;
-    if (toff < 0 || toff + (int64_t)S * kBTileElems > segs[nseg].a_img) {  // never write outside the images
-      if ((threadIdx.x & 127) == 0) set_status(status, TDC_EUNSUPPORTED);
-      continue;
-    }
-    __nv_bfloat16* tile = img + toff;
-    const int j = tid % BN, kg = tid / BN;  // 64 columns x BK/8 groups of 8 poles
-    const int jj = ct * BN + j;
+  const int j = tid % BN, k0 = (tid / BN) * 8, off = core_off(j, k0);
+  for (int64_t c = 2 * (int64_t)blockIdx.x + (threadIdx.x >> 7); c * run < total; c += 2 * (int64_t)gridDim.x) {
+    DigitRun R;
+    R.w = c * run;
+    R.end = min(total, R.w + run);
+    R.si = find_seg(segs, nseg, R.w, 1);
+    run_place<1>(segs, R);
     double dorg = 0.0, tj = 1.0, sj = 0.0;
-    if (jj < sg.K) {
-      if (sg.Bd || sg.tgen) {
-        sj = sg.cexp ? pow2c(-sg.cexp[jj]) : 1.0;
-      } else {
-        const int jr = sg.bcol ? sg.bcol[jj] : jj;
-        dorg = sg.D[sg.org[jr]];
-        tj = sg.tau[jr];
-        sj = sg.scol[jr];
+    int ae = 0, si0 = -1, t0 = -1;
+    for (; R.w < R.end; run_next<1>(segs, R)) {
+      const GemmSeg& sg = segs[R.si];
+      const int64_t toff = sg.b_img + ((int64_t)R.t * R.KB + R.kb) * S * kBTileElems;
+      if (toff < 0 || toff + (int64_t)S * kBTileElems > cap) {  // never write outside the images
+        if (tid == 0) set_status(status, TDC_EUNSUPPORTED);
+        continue;
       }
-    }
-    uint32_t dig[8][kMaxS];
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const int q = kb * BK + kg * 8 + i;
-      double u = 0.0;
-      if (q < sg.kk && q >= sg.bq0 && jj < sg.K) {
-        const int p = sg.plist ? sg.plist[q] : q;
-        if (sg.Bd) u = sg.Bd[p + (int64_t)jj * sg.ldb] * sj;
-        else if (sg.tgen) u = struct_entry(sg, p, jj) * sj;
-        else u = (sg.zhat[p] * sj) * rcp_nr((sg.D[p] - dorg) - tj);
+      const int jj = R.t * BN + j;
+      const bool live = jj < sg.K;
+      const bool given = sg.Bd || sg.tgen;
+      if (R.si != si0 || R.t != t0) {  // the column's data
+        si0 = R.si;
+        t0 = R.t;
+        ae = 0;
+        if (live && given) {
+          if (sg.cexp) ae = min(max(sg.cexp[jj], -1023), 1022);
+        } else if (live) {
+          const int jr = sg.bcol ? sg.bcol[jj] : jj;
+          dorg = sg.D[sg.org[jr]];
+          tj = sg.tau[jr];
+          sj = sg.scol[jr];
+        }
       }
-      digits_bf16(u, S, dig[i]);
-    }
-    const int off = core_off(j, kg * 8);
+      const int32_t* plist = sg.plist;
+      long long g[8];
 #pragma unroll
-    for (int s = 0; s < kMaxS; ++s) {
-      if (s >= S) break;
-      uint32_t v[8];
-#pragma unroll
-      for (int i = 0; i < 8; ++i) v[i] = dig[i][s];
-      *reinterpret_cast<uint4*>(tile + (int64_t)s * kBTileElems + off) = pack8(v);
+      for (int i = 0; i < 8; ++i) {
+        const int q = R.kb * BK + k0 + i;
+        double u = 0.0;
+        if (q < sg.kk && q >= sg.bq0 && live) {
+          const int p = plist ? plist[q] : q;
+          if (sg.Bd) u = sg.Bd[p + (int64_t)jj * sg.ldb];
+          else if (sg.tgen) u = struct_entry(sg, p, jj);
+          else u = (sg.zhat[p] * sj) * rcp_nr((sg.D[p] - dorg) - tj);
+        }
+        g[i] = digit_word(u, ae);
+      }
+      store_digits(img + toff + off, kBTileElems, S, g);
     }
   }
 }
@@ -865,10 +906,10 @@ __global__ void __maxnreg__(80) k_gemm_split_shared(const GemmSeg* segs, int nse
 
 static cudaError_t launch_split_digits(const GemmSeg* segs, int nseg, const int64_t* dnseg, int S, int* status,
                                        __nv_bfloat16* img, cudaStream_t s) {
-  k_split_a<<<152 * 8, 256, 0, s>>>(segs, nseg, dnseg, S, img, status);
+  k_split_a<<<152 * 5, 256, 0, s>>>(segs, nseg, dnseg, S, img, status);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  k_split_b<<<152 * 8, 256, 0, s>>>(segs, nseg, dnseg, S, img, status);
+  k_split_b<<<152 * 3, 256, 0, s>>>(segs, nseg, dnseg, S, img, status);
   return cudaGetLastError();
 }
 
