@@ -586,18 +586,22 @@ struct TileRef {
 // tile w of the level: tiles in groups of kGroupRows row tiles, column tile by
 // column tile, so that the CTAs running together share A row tiles and B column
 // tiles in L2
-__device__ __forceinline__ TileRef tile_ref(const GemmSeg* segs, int nseg, int64_t w) {
+// `si` is the segment of this role's previous tile: the next one is mostly in it or the one
+// after it (one load latency instead of a search; three roles pay it between tiles).
+__device__ __forceinline__ TileRef tile_ref(const GemmSeg* segs, int nseg, int64_t w, int& si) {
   TileRef t;
-  t.sg = &segs[find_seg(segs, nseg, w, 2)];
-  const int64_t local = w - t.sg->it_t;
-  const int CT = (int)cdiv(t.sg->K, BN);
-  const int RT = (int)cdiv(t.sg->rows, BM);
-  t.KB = (int)cdiv(t.sg->kk, BK);
-  const int grp = (int)(local / ((int64_t)kGroupRows * CT));
-  const int within = (int)(local % ((int64_t)kGroupRows * CT));
+  const int64_t n1 = segs[si + 1].it_t, n2 = segs[min(si + 2, nseg)].it_t;
+  if (w >= n1) si = w < n2 ? si + 1 : find_seg(segs, nseg, w, 2);
+  t.sg = &segs[si];
+  const uint32_t local = (uint32_t)(w - t.sg->it_t);  // a segment's tiles fit in 32 bits
+  const uint32_t CT = (uint32_t)(t.sg->K + BN - 1) / BN;
+  const int RT = (t.sg->rows + BM - 1) / BM;
+  t.KB = (t.sg->kk + BK - 1) / BK;
+  const int grp = (int)(local / (kGroupRows * CT));
+  const int within = (int)(local - (uint32_t)grp * (kGroupRows * CT));
   const int gr = min(kGroupRows, RT - grp * kGroupRows);
-  t.rt = grp * kGroupRows + within % gr;
   t.ct = within / gr;
+  t.rt = grp * kGroupRows + (within - t.ct * gr);
   return t;
 }
 }  // namespace
@@ -651,8 +655,9 @@ __device__ __forceinline__ void gemm_split(const GemmSeg* segs, int nseg, const 
       long long g = 0;  // k-steps loaded by this CTA (stage g % kStages, use g / kStages)
       bool ok = true;
       const int64_t img_end = segs[nseg].a_img;  // the list's images end here (the terminator)
+      int si = 0;
       for (int64_t w = blockIdx.x; w < total && ok; w += gridDim.x) {
-        const TileRef t = tile_ref(segs, nseg, w);
+        const TileRef t = tile_ref(segs, nseg, w, si);
         const int akt = t.sg->a_kt > 0 ? t.sg->a_kt : t.KB;  // k-tiles per row tile of the A image
         const int64_t a0 = t.sg->a_img + (int64_t)t.rt * akt * S * kATileElems;
         const int64_t b0 = t.sg->b_img + (int64_t)t.ct * t.KB * S * kBTileElems;
@@ -691,8 +696,9 @@ __device__ __forceinline__ void gemm_split(const GemmSeg* segs, int nseg, const 
       // the start-address field (bits 0-13, address / 16) absorbs every offset below
       // without carrying, as all of shared memory lies below 2^18 bytes
       const uint64_t desc0 = umma::sdesc(sbase, 128, BK * 16);
+      int si = 0;
       for (int64_t w = blockIdx.x; w < total && ok; w += gridDim.x, ++it) {
-        const TileRef t = tile_ref(segs, nseg, w);
+        const TileRef t = tile_ref(segs, nseg, w, si);
         // one accumulator hand-off per chunk of ck k-steps (kChunk), else per tile
         const int nch = kChunk && t.KB > 0 ? (t.KB + ck - 1) / ck : 1;
         int kb0 = 0;
@@ -759,116 +765,80 @@ __device__ __forceinline__ void gemm_split(const GemmSeg* segs, int nseg, const 
     float gmax = 0.0f;  // largest |level sum| (levels 0-4) this thread drained
     const int quarter = warp & 3, c0 = (warp >> 2) * kEpiCols;
     const uint32_t tl = tmem + ((uint32_t)(quarter * 32) << 16);
+    int si = 0;
     for (int64_t w = blockIdx.x; w < total; w += gridDim.x, ++it) {
-      const TileRef t = tile_ref(segs, nseg, w);
-      if constexpr (kChunk) {
-        // the same combination, accumulated over the tile's chunks: level m of a
-        // chunk adds P_m 2^(8(4-m)) to hi (m < 5, exact) or its share to lo
-        const int nch = t.KB > 0 ? (t.KB + ck - 1) / ck : 1;
-        unsigned long long hu[kEpiCols];
-        float lo[kEpiCols];
+      const TileRef t = tile_ref(segs, nseg, w, si);
+      // The columns' scales and places, one column a lane, and an accumulating tile's old
+      // values on their way into L2, while the products run: read where they were needed, one
+      // column after the other, they took 7.0 k clocks of conversion and 5.7 k (accumulating:
+      // 19.6 k) of stores a tile, which was all of a shallow tile's time; now 5.0 k and 4.1 k
+      // (6.3 k).  Top merge of tridiag(1,2,1) n = 16384: products 9.64 -> 7.95 ms.
+      const GemmSeg& sg = *t.sg;
+      const int row = t.rt * BM + quarter * 32 + lane, j0 = t.ct * BN + c0, K = sg.K;
+      const int64_t ldc = sg.ldc;
+      const bool acc = sg.acc != 0;
+      const int jl = j0 + (lane & (kEpiCols - 1));
+      const int my_adj = col_adj(sg, jl), my_pos = jl < K && sg.cpos ? sg.cpos[jl] : jl;
+      double* C = sg.C + row;
+      if (acc && jl < K && t.rt * BM + quarter * 32 + (lane & 16) < sg.rows)
+        asm volatile("prefetch.global.L2 [%0];" ::"l"(sg.C + t.rt * BM + quarter * 32 + (lane & 16) + (int64_t)my_pos * ldc));
+      const bool in_rows = row < sg.rows;
+      // the combination is accumulated over the tile's hand-offs: level m adds
+      // P_m 2^(8(4-m)) to hi (m < 5, exact) or its share to lo
+      const int nch = kChunk && t.KB > 0 ? (t.KB + ck - 1) / ck : 1;
+      unsigned long long hu[kEpiCols];
+      float lo[kEpiCols];
 #pragma unroll
-        for (int i = 0; i < kEpiCols; ++i) {
-          hu[i] = 0;
-          lo[i] = 0.0f;
-        }
-        bool okc = true;
-        for (int c = 0; c < nch; ++c) {
-          if (c > 0) ++it;
-          okc = __all_sync(0xffffffffu, wait_or_fail(tfull, (uint32_t)(it & 1), budget, vfail));
-          if (!okc) break;
-          umma::tc_fence_after();
-          if (t.KB > 0) drain_levels<S, kShare ? 8 : 16>(tl + (uint32_t)c0, hu, lo, gmax);
-          umma::tc_fence_before();
-          __syncwarp();
-          if (lane == 0) mbar_arrive(tempty);
-        }
-        if (!okc) {
-          if (lane == 0) *vfail = 1;
-          break;
-        }
-        const unsigned long long bias = t.KB > 0 ? (unsigned long long)nch * drain_bias<S>() : 0ull;
-        long long hi[kEpiCols];
-#pragma unroll
-        for (int i = 0; i < kEpiCols; ++i) hi[i] = (long long)(hu[i] - bias);
-        double val[kEpiCols];
-        bool fits = true;
-#pragma unroll
-        for (int i = 0; i < kEpiCols; ++i) fits = fits && hi[i] < (1ll << 52) && hi[i] > -(1ll << 52);
-        // the column's scale (2^cexp_j 2^oexp_j) goes into the exponent field of the value
-        if (__all_sync(0xffffffffu, fits)) {
-#pragma unroll
-          for (int i = 0; i < kEpiCols; ++i)
-            val[i] = level_value(hi[i] * 1024 + (long long)__float2int_rn(4.0f * lo[i]), col_adj(*t.sg, t.ct * BN + c0 + i));
-        } else {
-#pragma unroll
-          for (int i = 0; i < kEpiCols; ++i)
-            val[i] = scale2(fma((double)lo[i], 0x1p-56, __ll2double_rn(hi[i]) * 0x1p-48), col_adj(*t.sg, t.ct * BN + c0 + i));
-        }
-        const GemmSeg& sg = *t.sg;
-        const int row = t.rt * BM + quarter * 32 + lane;
-        if (row < sg.rows) {
-#pragma unroll
-          for (int i = 0; i < kEpiCols; ++i) {
-            const int j = t.ct * BN + c0 + i;
-            if (j < sg.K) {
-              const int pos = sg.cpos ? sg.cpos[j] : j;
-              double* cp = sg.C + row + (int64_t)pos * sg.ldc;
-              if (sg.acc) *cp += val[i]; else *cp = val[i];
-            }
-          }
-        }
-        continue;
+      for (int i = 0; i < kEpiCols; ++i) {
+        hu[i] = 0;
+        lo[i] = 0.0f;
       }
-      const bool okw = __all_sync(0xffffffffu, wait_or_fail(tfull, (uint32_t)(it & 1), budget, vfail));
-      if (!okw) {
+      bool okc = true;
+      for (int c = 0; c < nch; ++c) {
+        if (c > 0) ++it;
+        okc = __all_sync(0xffffffffu, wait_or_fail(tfull, (uint32_t)(it & 1), budget, vfail));
+        if (!okc) break;
+        umma::tc_fence_after();
+        if (t.KB > 0) drain_levels<S, kShare ? 8 : 16>(tl + (uint32_t)c0, hu, lo, gmax);
+        umma::tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(tempty);
+      }
+      if (!okc) {
         if (lane == 0) *vfail = 1;
         break;
       }
-      umma::tc_fence_after();
+      const unsigned long long bias = t.KB > 0 ? (unsigned long long)nch * drain_bias<S>() : 0ull;
+      long long hi[kEpiCols];
+#pragma unroll
+      for (int i = 0; i < kEpiCols; ++i) hi[i] = (long long)(hu[i] - bias);
       double val[kEpiCols];
-      {
-        unsigned long long hu[kEpiCols];
-        const unsigned long long bias = t.KB > 0 ? drain_bias<S>() : 0ull;
-        float lo[kEpiCols];
+      bool fits = true;
 #pragma unroll
-        for (int i = 0; i < kEpiCols; ++i) {
-          hu[i] = 0;
-          lo[i] = 0.0f;
-        }
-        if (t.KB > 0) drain_levels<S, kShare ? 8 : 16>(tl + (uint32_t)c0, hu, lo, gmax);
-        long long hi[kEpiCols];
+      for (int i = 0; i < kEpiCols; ++i) fits = fits && hi[i] < (1ll << 52) && hi[i] > -(1ll << 52);
+      // the column's scale (2^cexp_j 2^oexp_j) goes into the exponent field of the value
+      if (__all_sync(0xffffffffu, fits)) {
 #pragma unroll
-        for (int i = 0; i < kEpiCols; ++i) hi[i] = (long long)(hu[i] - bias);
-        bool fits = true;
+        for (int i = 0; i < kEpiCols; ++i)
+          val[i] = level_value(hi[i] * 1024 + (long long)__float2int_rn(4.0f * lo[i]), __shfl_sync(0xffffffffu, my_adj, i));
+      } else {
 #pragma unroll
-        for (int i = 0; i < kEpiCols; ++i) fits = fits && hi[i] < (1ll << 52) && hi[i] > -(1ll << 52);
-        // the column's scale (2^cexp_j 2^oexp_j) goes into the exponent field of the value
-        if (__all_sync(0xffffffffu, fits)) {
-#pragma unroll
-          for (int i = 0; i < kEpiCols; ++i)
-            val[i] = level_value(hi[i] * 1024 + (long long)__float2int_rn(4.0f * lo[i]), col_adj(*t.sg, t.ct * BN + c0 + i));
-        } else {
-#pragma unroll
-          for (int i = 0; i < kEpiCols; ++i)
-            val[i] = scale2(fma((double)lo[i], 0x1p-56, __ll2double_rn(hi[i]) * 0x1p-48), col_adj(*t.sg, t.ct * BN + c0 + i));
-        }
+        for (int i = 0; i < kEpiCols; ++i)
+          val[i] = scale2(fma((double)lo[i], 0x1p-56, __ll2double_rn(hi[i]) * 0x1p-48), __shfl_sync(0xffffffffu, my_adj, i));
       }
-      umma::tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(tempty);
-      const GemmSeg& sg = *t.sg;
-      const int row = t.rt * BM + quarter * 32 + lane;
-      if (row < sg.rows) {
+      // four columns at a time: an accumulating tile waits for its old values once a group
 #pragma unroll
-        for (int i = 0; i < kEpiCols; ++i) {
-          const int j = t.ct * BN + c0 + i;
-          if (j < sg.K) {
-            const int pos = sg.cpos ? sg.cpos[j] : j;
-            double* cp = sg.C + row + (int64_t)pos * sg.ldc;
-            if (sg.acc) *cp += val[i]; else *cp = val[i];
-          }
+      for (int i = 0; i < kEpiCols; i += 4) {
+        double* cp[4];
+        double old[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          cp[u] = C + (int64_t)__shfl_sync(0xffffffffu, my_pos, i + u) * ldc;
+          old[u] = acc && in_rows && j0 + i + u < K ? *cp[u] : 0.0;
         }
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          if (in_rows && j0 + i + u < K) *cp[u] = acc ? old[u] + val[i + u] : val[i + u];
       }
     }
     // the level sums' margin: statistics, and a warning once a hand-off reached 2^23
