@@ -312,7 +312,7 @@ __device__ __forceinline__ double twice(double x) {
 }
 
 template <int LM, int R, int NL>
-__global__ void __launch_bounds__(32) k_leaf_rows(Plan P, int64_t nleaves) {
+__global__ void __launch_bounds__(32) k_leaf_rows(Plan P, int64_t nleaves, const int* only) {
   constexpr int GL = LM / R;  // lanes per leaf; NL leaves per warp
   static_assert(NL * GL <= 32, "leaves of a warp");
   __shared__ double s_d[NL][LM];
@@ -320,7 +320,8 @@ __global__ void __launch_bounds__(32) k_leaf_rows(Plan P, int64_t nleaves) {
   const int lane = threadIdx.x, slot = lane / GL, gl = lane % GL;
   // spare lanes (NL GL < 32) follow a leaf of the warp, so that its branches stay uniform
   const int64_t gid = (int64_t)blockIdx.x * NL + slot % NL;
-  const bool live = gid < nleaves, writes = live && slot < NL;
+  const bool live = gid < nleaves && (!only || only[gid]), writes = live && slot < NL;
+  if (!__any_sync(0xffffffffu, live)) return;
   int pi = 0, L = 0;
   int64_t lo = 0;
   if (live) {
@@ -467,8 +468,8 @@ __global__ void __launch_bounds__(32) k_leaf_rows(Plan P, int64_t nleaves) {
 }
 
 template <int LM, int R, int NL = 32 * R / LM>
-static cudaError_t launch_leaf_rows(const Plan& P, int64_t nleaves, cudaStream_t s) {
-  k_leaf_rows<LM, R, NL><<<(unsigned)((nleaves + NL - 1) / NL), 32, 0, s>>>(P, nleaves);
+static cudaError_t launch_leaf_rows(const Plan& P, int64_t nleaves, cudaStream_t s, const int* only = nullptr) {
+  k_leaf_rows<LM, R, NL><<<(unsigned)((nleaves + NL - 1) / NL), 32, 0, s>>>(P, nleaves, only);
   return cudaGetLastError();
 }
 
@@ -655,6 +656,233 @@ __global__ void __launch_bounds__(1024) k_leaf_multi(Plan P, int64_t nleaves, in
   }
 }
 
+// Leaves of 9 to 16 rows: an FP32 solve, then FP64 refinement of all eigenpairs at once.
+// Warp 0 runs the QR iteration in FP32 (the chase above at 4 clocks an operation instead of
+// 64), which leaves X orthonormal and diagonalising T to about 1e-6.  Then, with
+//   G = X^T X, S = X^T T X, lam_j = S_jj / G_jj, s_ij = S_ij - (lam_i + lam_j) G_ij / 2,
+// the columns take X <- X + X E,
+//   E_ij = K_ij - G_ij / 2 (i != j), E_jj = (1 - G_jj) / 2, K_ij = s_ij / (lam_j - lam_i)
+// (the symmetric part restores orthonormality to second order, the antisymmetric K turns the
+// columns onto the eigenvectors; Ogita and Aishima, "Iterative refinement for symmetric
+// eigenvalue decomposition", 2018).  Where s_ij is not small against the gap, K_ij is the
+// tangent of the 2 x 2 problem's rotation, for which I + E is that rotation up to a scale.
+// The error is squared each time: two iterations as a rule.  s_ij at rounding level of
+// |lam_i| + |lam_j| counts as zero (the QR iteration's own criterion).  A leaf whose E does
+// not fall below 2^-30 in six iterations (clusters closer than FP32 resolves in groups of
+// three or more, entries below its range) is flagged and left to k_leaf_rows.
+// Per leaf of 16 rows 0.8 M FP64 clocks of one quarter SM become 35 k clocks of FP32 chase
+// and 10 k FP64 clocks an iteration over four quarters: 64 leaves 417 -> 54 us, 8192 leaves
+// 2.11 -> 1.38 ms.  Residual and orthogonality of 16-row leaves (eps): 5.3 and 10 -> 0.8 and
+// 0.95 for uniform entries, 6.0 and 5.5 -> 2.1 and 3.5 in one cluster, eigenvalues graded over
+// 2^-600 to 4.7e-16 of themselves (1.4e-15).
+constexpr int kRefLM = 16;
+__global__ void __launch_bounds__(128) k_leaf_refine(Plan P, int64_t nleaves, int* flag) {
+  constexpr int LM = kRefLM;
+  __shared__ double X[LM][LM + 1], Y[LM][LM + 1], E[LM][LM + 1];
+  __shared__ double s_d[LM], s_e[LM], s_lam[LM];
+  __shared__ int s_rank[LM], s_bad;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int64_t gid = blockIdx.x;
+  int x0 = 0, y0 = P.nprob - 1;
+  while (x0 < y0) {
+    const int m = (x0 + y0 + 1) >> 1;
+    if (P.prob[m].leaf0 <= gid) x0 = m; else y0 = m - 1;
+  }
+  const Problem& pr = P.prob[x0];
+  const int64_t lo = node_bound(gid - pr.leaf0, pr.n, pr.depth);
+  const int L = (int)(node_bound(gid - pr.leaf0 + 1, pr.n, pr.depth) - lo);
+  if (tid < LM) {
+    s_d[tid] = tid < L ? P.v.dmod[pr.voff + lo + tid] : 0.0;
+    s_e[tid] = tid < L - 1 ? input_entry(P.e[pr.off_de + lo + tid], pr.escale) : 0.0;
+  }
+  if (tid == 0) s_bad = 0;
+  __syncthreads();
+  if (warp == 0) {
+    // exponent of the largest entry, then the FP32 problem of scale one
+    int ex = lane < LM ? max((__double2hiint(s_d[lane]) >> 20) & 0x7ff, (__double2hiint(s_e[lane]) >> 20) & 0x7ff) : 0;
+    ex = __reduce_max_sync(0xffffffffu, ex);
+    const double sc = pow2c(1023 - max(ex, 1));
+    float d[LM], e[LM], z[LM];
+#pragma unroll
+    for (int k = 0; k < LM; ++k) {
+      d[k] = (float)(s_d[k] * sc);
+      e[k] = (float)(s_e[k] * sc);
+      z[k] = (lane & (LM - 1)) == k ? 1.0f : 0.0f;
+    }
+    int sweep = 0;
+    for (;; ++sweep) {
+      unsigned nz = 0;
+      static_for<LM - 1>([&](auto kc) {
+        constexpr int k = kc.value;
+        if (fabsf(e[k]) <= 6e-8f * (fabsf(d[k]) + fabsf(d[k + 1]))) e[k] = 0.0f; else nz |= 1u << k;
+      });
+      if (nz == 0 || sweep >= 6 * LM) {
+        if (nz && lane == 0) s_bad = 1;
+        break;
+      }
+      const int q = 32 - __clz(nz);
+      const unsigned below = ~nz & ((1u << (q - 1)) - 1u);
+      const int pp = below ? 32 - __clz(below) : 0;
+      float dq = 0.0f, dq1 = 0.0f, bq = 0.0f;
+      static_for<LM - 1>([&](auto kc) {
+        constexpr int k = kc.value;
+        if (k == q - 1) {
+          dq1 = d[k];
+          dq = d[k + 1];
+          bq = e[k];
+        }
+      });
+      const float hd = 0.5f * (dq1 - dq), hh = sqrtf(fmaf(hd, hd, bq * bq));
+      const float mu = dq - __fdividef(bq * bq, hd + copysignf(hh, hd));
+      float c = 1.0f, sn = 1.0f, g = 0.0f, pv = 0.0f;
+      static_for<LM - 1>([&](auto kc) {
+        constexpr int k = kc.value;
+        if (k >= pp && k < q) {
+          if (k == pp) g = d[k] - mu;
+          const float f = sn * e[k], b = c * e[k], t2 = fmaf(g, g, f * f);
+          float r = 0.0f;
+          if (t2 > 0.0f) {
+            const float ri = rsqrtf(t2);
+            r = t2 * ri;
+            sn = f * ri;
+            c = g * ri;
+          } else {
+            sn = 0.0f;
+            c = 1.0f;
+          }
+          if constexpr (k > 0) {
+            if (k > pp) e[k - 1] = r;
+          }
+          g = d[k] - pv;
+          r = fmaf(d[k + 1] - g, sn, 2.0f * b * c);
+          pv = sn * r;
+          d[k] = g + pv;
+          g = fmaf(c, r, -b);
+          const float v = z[k], w = z[k + 1];
+          z[k] = fmaf(sn, w, c * v);
+          z[k + 1] = fmaf(c, w, -(sn * v));
+          if (k == q - 1) {
+            d[k + 1] -= pv;
+            e[k] = g;
+          }
+        }
+      });
+    }
+    if (lane < LM) {
+#pragma unroll
+      for (int k = 0; k < LM; ++k) X[lane][k] = (double)z[k];
+    }
+  }
+  __syncthreads();
+  // refinement: thread (j, rows 2 g and 2 g + 1 of every 16 x 16 product)
+  const int j = tid & (LM - 1), i0 = 2 * (tid >> 4);
+  const bool live = j < L && i0 < L;
+  bool more = !s_bad;
+  for (int it = 0; more && it < 6; ++it) {
+    if (live) {
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        const int r = i0 + u;
+        double y = 0.0;
+        if (r < L) {
+          y = s_d[r] * X[r][j];
+          if (r > 0) y = fma(s_e[r - 1], X[r - 1][j], y);
+          if (r < L - 1) y = fma(s_e[r], X[r + 1][j], y);
+        }
+        Y[r][j] = y;
+      }
+    }
+    __syncthreads();
+    double S[2] = {0.0, 0.0}, G[2] = {0.0, 0.0};
+    if (live) {
+      for (int r = 0; r < L; ++r) {
+        const double a = X[r][i0], b = X[r][i0 + 1], yj = Y[r][j], xj = X[r][j];
+        S[0] = fma(a, yj, S[0]);
+        S[1] = fma(b, yj, S[1]);
+        G[0] = fma(a, xj, G[0]);
+        G[1] = fma(b, xj, G[1]);
+      }
+      if (j == i0) s_lam[j] = S[0] * rcp_nr(G[0]);
+      if (j == i0 + 1) s_lam[j] = S[1] * rcp_nr(G[1]);
+    }
+    __syncthreads();
+    bool big = false;
+    if (live) {
+      const double lj = s_lam[j];
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        const int i = i0 + u;
+        // one thread makes both entries of a pair, so that K is antisymmetric to the last bit
+        if (i == j) {
+          E[i][i] = fma(-0.5, G[u], 0.5);
+          big = big || !(fabs(E[i][i]) <= 0x1p-30);
+        } else if (i < j) {
+          const double li = s_lam[i], gap = lj - li, sm = fabs(li) + fabs(lj);
+          const double s = fma(-0.5 * (li + lj), G[u], S[u]);
+          double k = 0.0;
+          if (fabs(s) > kEps * sm) {
+            if (fabs(s) <= 0.015625 * fabs(gap)) {
+              k = s / gap;
+            } else {
+              const double t = gap / (2.0 * s);
+              k = copysign(1.0 / (fabs(t) + sqrt(fma(t, t, 1.0))), t);
+            }
+          }
+          E[i][j] = fma(-0.5, G[u], k);
+          E[j][i] = fma(-0.5, G[u], -k);
+          big = big || !(fabs(k) + fabs(G[u]) <= 0x1p-30);
+        }
+      }
+    }
+    more = __syncthreads_or(big);
+    double nx[2] = {0.0, 0.0};
+    if (live) {
+      for (int r = 0; r < L; ++r) {
+        const double er = E[r][j];
+        nx[0] = fma(X[i0][r], er, nx[0]);
+        nx[1] = fma(X[i0 + 1][r], er, nx[1]);
+      }
+      nx[0] += X[i0][j];
+      nx[1] += X[i0 + 1][j];
+    }
+    __syncthreads();
+    if (live) {
+      X[i0][j] = nx[0];
+      X[i0 + 1][j] = nx[1];
+    }
+    __syncthreads();
+  }
+  const bool bad = s_bad || more;
+  if (tid == 0) flag[gid] = bad ? 1 : 0;
+  if (bad) return;
+  if (tid < L) {
+    const double v = s_lam[tid];
+    int rk = 0;
+    for (int m = 0; m < L; ++m) {
+      const double w = s_lam[m];
+      rk += (w < v || (w == v && m < tid)) ? 1 : 0;
+    }
+    s_rank[tid] = rk;
+  }
+  __syncthreads();
+  const int par = pr.depth & 1;
+  const int64_t ld = par ? pr.n : pr.ld0;
+  double* dst = (par ? P.Q1 + pr.qoff1 : P.Q0 + pr.off_q) + lo + lo * ld;
+  const int64_t o = pr.voff + lo;
+  for (int t = tid; t < LM * LM; t += 128) {
+    const int r = t & (LM - 1), k = t >> 4;
+    if (r >= L || k >= L) continue;
+    const int rk = s_rank[k];
+    const double x = X[r][k];
+    dst[r + rk * ld] = x;
+    if (r == 0) {
+      P.lam2[par][o + rk] = s_lam[k];
+      P.bf2[par][o + rk] = x;
+    }
+    if (r == L - 1) P.bl2[par][o + rk] = x;
+  }
+}
+
 // Leaves of at most 16 rows take k_leaf_rows with one row a lane while that is at most one
 // warp per quarter SM (608 quarters; 1024 leaves of 16 rows: 420 us
 // against 464 with R = 2), two rows to twice that, four beyond (12,000 leaves: 2.07 ms; the
@@ -671,11 +899,15 @@ cudaError_t launch_leaves(const Plan& P, int64_t nleaves, int max_leaf, cudaStre
     if (nleaves <= 4 * kQuarters) return launch_leaf_rows<8, 1>(P, nleaves, s);
     return launch_leaf_rows<8, 4>(P, nleaves, s);
   }
-  if (max_leaf <= 16) {
-    if (nleaves <= kQuarters) return launch_leaf_rows<16, 1, 1>(P, nleaves, s);
-    if (nleaves <= 2 * kQuarters) return launch_leaf_rows<16, 1>(P, nleaves, s);
-    if (nleaves <= 4 * kQuarters) return launch_leaf_rows<16, 2>(P, nleaves, s);
-    return launch_leaf_rows<16, 4>(P, nleaves, s);
+  if (max_leaf <= kRefLM) {
+    int* flag = P.v.stag;  // the sort's scratch, unused here
+    k_leaf_refine<<<(unsigned)nleaves, 128, 0, s>>>(P, nleaves, flag);
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    if (nleaves <= kQuarters) return launch_leaf_rows<16, 1, 1>(P, nleaves, s, flag);
+    if (nleaves <= 2 * kQuarters) return launch_leaf_rows<16, 1>(P, nleaves, s, flag);
+    if (nleaves <= 4 * kQuarters) return launch_leaf_rows<16, 2>(P, nleaves, s, flag);
+    return launch_leaf_rows<16, 4>(P, nleaves, s, flag);
   }
   if (max_leaf <= 32 && nleaves >= 64) {
     if (nleaves <= 4000) return launch_leaf_rows<32, 1>(P, nleaves, s);
