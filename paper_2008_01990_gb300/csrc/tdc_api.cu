@@ -559,7 +559,7 @@ static int run_plan(HostPlan& H, const tdc_opts& o, const double* d, const doubl
   // on levels that also run the thread-per-root variants, 7 more with far-field tables), output
   int64_t launches = (int64_t)((H.prob.size() + kProbChunk - 1) / kProbChunk) + 4 + 9 * (int64_t)H.T;
   for (int l = 0; l < H.T; ++l) {
-    if (l > 0) launches += 2;  // boundary rows: rotation and gather, output order
+    if (l > 0 && H.levels[l].max_n > kBoundaryInFinalize) launches += 1;  // boundary rows
     if (H.levels[l].nslots >= kSmallMinSlots) launches += 5;
     if (far_level(H.levels[l])) launches += 7;
     if (H.levels[l].merges > 0 && H.levels[l].min_n <= kTinyN) launches += 1;
@@ -602,7 +602,6 @@ static int run_plan(HostPlan& H, const tdc_opts& o, const double* d, const doubl
     if (l + 2 < H.T) err = cudaStreamWaitEvent(s, evG[l + 2], 0);
     const size_t a0 = mark();
     if (err == cudaSuccess) err = launch_prepare(P, LL, s);
-    if (err == cudaSuccess) err = launch_boundary_rot(P, LL, s);
     if (err == cudaSuccess) err = cudaEventRecord(evR[l], s);
     const size_t a1 = mark();
     if (err == cudaSuccess) err = launch_secular(P, LL, s);
@@ -618,9 +617,23 @@ static int run_plan(HostPlan& H, const tdc_opts& o, const double* d, const doubl
     if (err == cudaSuccess) err = cudaStreamWaitEvent(sg, evR[l], 0);
     const size_t g0 = mark_on(sg);
     if (err == cudaSuccess) err = launch_rotate(P, LL, sg);
+    if (err == cudaSuccess) err = launch_tile_scan(P, LL, sg);
     size_t g1 = mark_on(sg);
     span(1, g0, g1);
+    // The plain split products' left digits too, where one pass takes the whole level and the
+    // structured path does not use the segment list first.  Not on levels whose roots fill the
+    // chip by themselves: there the digits only slow the roots down (adjoint of 256 problems of
+    // order 512: 21.4 ms with them early, 20.3 without).
+    const bool split = P.split_min_K > 0 && LL.max_n >= P.split_min_K;
+    const bool early = split && LL.nslots < kSmallMinSlots && H.split_chunks[l].size() == 1 && !ss &&
+                       (H.ss || P.struct_min_K <= 0 || LL.max_n < P.struct_min_K);
+    if (early && err == cudaSuccess) {
+      err = launch_gemm_split_left(P, LL, H.split_chunks[l][0].first, H.split_chunks[l][0].second, -1, sg);
+      const size_t g2 = mark_on(sg);
+      span(5, g1, g2);
+    }
     if (err == cudaSuccess) err = cudaStreamWaitEvent(sg, evE[l], 0);
+    g1 = mark_on(sg);
     if (err == cudaSuccess) err = launch_gemm_dense(P, LL, H.max_tiles[l], sg);
     if (err == cudaSuccess) err = launch_gemm_tiny(P, LL, sg);
     if (err == cudaSuccess && ss) {
@@ -703,7 +716,7 @@ static int run_plan(HostPlan& H, const tdc_opts& o, const double* d, const doubl
     const size_t a4 = mark_on(sg);
     span(4, g1, a4);
     size_t a6 = a4;
-    if (err == cudaSuccess && P.split_min_K > 0 && LL.max_n >= P.split_min_K) {
+    if (err == cudaSuccess && split) {
       // several passes on the host's bound: packed again on the device from the actual sizes
       const int npass = (int)H.split_chunks[l].size();
       if (npass > 1) err = launch_split_pack(P, LL, npass, sg);
@@ -716,7 +729,9 @@ static int run_plan(HostPlan& H, const tdc_opts& o, const double* d, const doubl
         }
         const size_t b5 = timing ? evs.size() - 1 : 0;
         const size_t b4 = a6;
-        if (err == cudaSuccess) err = launch_gemm_split(P, LL, ch.first, ch.second, npass > 1 ? pass : -1, sg, mid);
+        if (!early && err == cudaSuccess)
+          err = launch_gemm_split_left(P, LL, ch.first, ch.second, npass > 1 ? pass : -1, sg);
+        if (err == cudaSuccess) err = launch_gemm_split(P, LL, ch.first, ch.second, sg, mid);
         ++pass;
         a6 = mark_on(sg);
         span(5, b4, b5);

@@ -555,11 +555,14 @@ cudaError_t launch_leaves(const Plan& P, int64_t nleaves, int max_leaf, cudaStre
 constexpr int64_t kSmallMinSlots = 32768;
 cudaError_t launch_prepare(const Plan& P, const LevelLaunch& L, cudaStream_t s);
 cudaError_t launch_rotate(const Plan& P, const LevelLaunch& L, cudaStream_t s);
-cudaError_t launch_boundary_rot(const Plan& P, const LevelLaunch& L, cudaStream_t s);
+// levels of merges up to this order write their boundary rows at the end of k_finalize, the
+// longer ones from a grid of their own (one block a merge would be longer than the launch)
+constexpr int64_t kBoundaryInFinalize = 2048;
 cudaError_t launch_boundary_out(const Plan& P, const LevelLaunch& L, cudaStream_t s);
 cudaError_t launch_secular(const Plan& P, const LevelLaunch& L, cudaStream_t s);  // with the far tables
 cudaError_t launch_lowner(const Plan& P, const LevelLaunch& L, cudaStream_t s);
 cudaError_t launch_finalize(const Plan& P, const LevelLaunch& L, cudaStream_t s);
+cudaError_t launch_tile_scan(const Plan& P, const LevelLaunch& L, cudaStream_t s);
 cudaError_t launch_copy_deflated(const Plan& P, const LevelLaunch& L, int sign_normalise, cudaStream_t s);
 cudaError_t launch_sign_and_output(const Plan& P, int sign_normalise, cudaStream_t s);
 // Rank-one eigenproblem: secular roots, Loewner zhat, column normalisers.  zz (K doubles),
@@ -573,7 +576,9 @@ size_t rank_one_scratch_bytes(int64_t K);
 cudaError_t launch_gemm_dense(const Plan& P, const LevelLaunch& L, int64_t max_tiles, cudaStream_t s);
 cudaError_t launch_gemm_tiny(const Plan& P, const LevelLaunch& L, cudaStream_t s);
 cudaError_t launch_split_pack(const Plan& P, const LevelLaunch& L, int max_pass, cudaStream_t s);
-cudaError_t launch_gemm_split(const Plan& P, const LevelLaunch& L, int64_t g0, int64_t g1, int pass, cudaStream_t s,
+cudaError_t launch_gemm_split_left(const Plan& P, const LevelLaunch& L, int64_t g0, int64_t g1, int pass,
+                                   cudaStream_t s);
+cudaError_t launch_gemm_split(const Plan& P, const LevelLaunch& L, int64_t g0, int64_t g1, cudaStream_t s,
                               cudaEvent_t mid);
 cudaError_t launch_seg_split(const GemmSeg* segs_dev, int nseg, int S, int* status, long long spin_budget,
                              __nv_bfloat16* img, int chunk_steps, cudaStream_t s);

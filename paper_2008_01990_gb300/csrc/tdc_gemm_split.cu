@@ -874,13 +874,20 @@ __global__ void __maxnreg__(80) k_gemm_split_shared(const GemmSeg* segs, int nse
   gemm_split<S, kChunk, true>(segs, nseg, dnseg, img, status, budget, ck, lvl_max);
 }
 
-static cudaError_t launch_split_digits(const GemmSeg* segs, int nseg, const int64_t* dnseg, int S, int* status,
-                                       __nv_bfloat16* img, cudaStream_t s) {
+static cudaError_t launch_split_a(const GemmSeg* segs, int nseg, const int64_t* dnseg, int S, int* status,
+                                  __nv_bfloat16* img, cudaStream_t s) {
   k_split_a<<<152 * 5, 256, 0, s>>>(segs, nseg, dnseg, S, img, status);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
+  return cudaGetLastError();
+}
+static cudaError_t launch_split_b(const GemmSeg* segs, int nseg, const int64_t* dnseg, int S, int* status,
+                                  __nv_bfloat16* img, cudaStream_t s) {
   k_split_b<<<152 * 3, 256, 0, s>>>(segs, nseg, dnseg, S, img, status);
   return cudaGetLastError();
+}
+static cudaError_t launch_split_digits(const GemmSeg* segs, int nseg, const int64_t* dnseg, int S, int* status,
+                                       __nv_bfloat16* img, cudaStream_t s) {
+  const cudaError_t e = launch_split_a(segs, nseg, dnseg, S, status, img, s);
+  return e != cudaSuccess ? e : launch_split_b(segs, nseg, dnseg, S, status, img, s);
 }
 
 template <int S, bool kChunk>
@@ -929,16 +936,24 @@ cudaError_t launch_split_pack(const Plan& P, const LevelLaunch& L, int max_pass,
   return cudaGetLastError();
 }
 
-// Merges [g0, g1) of the level, or (pass >= 0) the device-packed pass of that number.
-cudaError_t launch_gemm_split(const Plan& P, const LevelLaunch& L, int64_t g0, int64_t g1, int pass, cudaStream_t s,
-                              cudaEvent_t mid) {
+// Merges [g0, g1) of the level, or (pass >= 0) the device-packed pass of that number: the
+// segments and the left operands' digits, which need the deflation's lists and the rotated
+// columns, then (launch_gemm_split) the right operands' digits and the products.
+cudaError_t launch_gemm_split_left(const Plan& P, const LevelLaunch& L, int64_t g0, int64_t g1, int pass,
+                                   cudaStream_t s) {
   if (P.split_min_K <= 0 || P.segs == nullptr || g1 <= g0) return cudaSuccess;
   k_split_segs<<<1, 1024, 0, s>>>(P, L.level, g0, g1, pass);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
+  return launch_split_a(P.segs, (int)(2 * (g1 - g0)), P.m.sseg, P.split_slices, P.status, P.img, s);
+}
+
+cudaError_t launch_gemm_split(const Plan& P, const LevelLaunch& L, int64_t g0, int64_t g1, cudaStream_t s,
+                              cudaEvent_t mid) {
+  if (P.split_min_K <= 0 || P.segs == nullptr || g1 <= g0) return cudaSuccess;
   const int nseg = (int)(2 * (g1 - g0));  // bound; the kernels read the compacted count
   const int64_t* dn = P.m.sseg;
-  e = launch_split_digits(P.segs, nseg, dn, P.split_slices, P.status, P.img, s);
+  const cudaError_t e = launch_split_b(P.segs, nseg, dn, P.split_slices, P.status, P.img, s);
   if (e != cudaSuccess) return e;
   if (mid) cudaEventRecord(mid, s);
   return launch_split_mma(P.segs, nseg, dn, P.split_slices, P.status, P.spin_budget, P.img, P.split_chunk_steps,

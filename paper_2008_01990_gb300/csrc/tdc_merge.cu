@@ -7,7 +7,7 @@
 //   k_prepare   z (Eq. (T3)) from the children's boundary rows, merge of the
 //               two sorted spectra, deflation scan (Section 3.2, Eq. (T3-def)),
 //               compaction
-//   k_boundary_rot  the children's boundary rows through the deflating rotations
+//               and the children's boundary rows through the deflating rotations
 //   k_rotate    plane rotations of deflation applied to Q's columns
 //   k_secular   secular equation (Eq. (secular)), one warp per root (a thread
 //               per root for small merges on many-merge levels), FP64, roots
@@ -1004,6 +1004,61 @@ __device__ __forceinline__ void type2_rot(double D, double z, double pD, double 
   di = __fma_rn(pD, s2, __dmul_rn(D, c2));
 }
 
+// ---------------------------------------------------------------------------
+// Boundary rows.  Each node's first and last eigenvector rows are kept apart
+// (P.v.bf, P.v.bl, by output column): the parent's z is made of them, so the
+// parent's roots do not need this node's full product.  At a merge, rbf = (first
+// row of Q1, 0) and rbl = (0, last row of Q2) take the deflating rotations as
+// k_rotate applies them to the columns of diag(Q1, Q2) (row 0 lies in the top
+// half, row n-1 in the bottom one); once the roots, zhat, the normalisers and the
+// output order are known, the node's rows are these vectors times Qhat for the
+// non-deflated columns (the same pole lists and entries as the products) and
+// copies for the deflated ones.  The top level has no parent and skips all this.
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ void boundary_rot(const Plan& P, const Node& nd, int64_t g) {
+  const int n = (int)(nd.hi - nd.lo), n1 = (int)(nd.mid - nd.lo);
+  const int64_t v0 = nd.v0;
+  double* rf = P.v.rbf + v0;
+  double* rl = P.v.rbl + v0;
+  for (int c = threadIdx.x; c < n; c += blockDim.x) {
+    rf[c] = c < n1 ? P.cbf[v0 + c] : 0.0;
+    rl[c] = c < n1 ? 0.0 : P.cbl[v0 + c];
+  }
+  const int nr = P.m.nrot[g];
+  __syncthreads();
+  const int nch = nr > 0 ? P.m.nchain[g] : 0;
+  for (int h = threadIdx.x; h < nch; h += blockDim.x) {
+    const int k0 = P.v.rch[v0 + h];
+    const int k1 = (h + 1 < nch) ? P.v.rch[v0 + h + 1] : nr;
+    for (int k = k0; k < k1; ++k) {
+      const int pj = P.v.rij[4 * (v0 + k) + 0];
+      const int ci = P.v.rij[4 * (v0 + k) + 1];
+      const int sup = P.v.rij[4 * (v0 + k) + 2];
+      const int sp = sup & 0xff, si = sup >> 8;
+      const double c = P.v.rcs[2 * (v0 + k)], s = P.v.rcs[2 * (v0 + k) + 1];
+      if ((sp | si) & 1) {
+        const double x = (sp & 1) ? rf[pj] : 0.0, y = (si & 1) ? rf[ci] : 0.0;
+        rf[pj] = c * x + s * y;
+        rf[ci] = c * y - s * x;
+      }
+      if ((sp | si) & 2) {
+        const double x = (sp & 2) ? rl[pj] : 0.0, y = (si & 2) ? rl[ci] : 0.0;
+        rl[pj] = c * x + s * y;
+        rl[ci] = c * y - s * x;
+      }
+    }
+  }
+  __syncthreads();
+  // by pole: the rotated rows at the pole's column, where the pole has support
+  const int K = P.m.K[g];
+  for (int i = threadIdx.x; i < K; i += blockDim.x) {
+    const int col = P.v.kept[v0 + i];
+    const int sup = P.v.kseg[v0 + i];
+    P.v.pf[v0 + i] = (sup & 1) ? rf[col] : 0.0;
+    P.v.pl[v0 + i] = (sup & 2) ? rl[col] : 0.0;
+  }
+}
+
 __global__ void __launch_bounds__(1024) k_prepare(Plan P, int level) {
   __shared__ double redd[64];
   __shared__ int redi[64];
@@ -1373,6 +1428,10 @@ __global__ void __launch_bounds__(1024) k_prepare(Plan P, int level) {
     if (P.stats && level < TDC_MAX_LEVELS)
       atomicAdd(&P.stats->gemm_flops[level],
                 2ull * ((unsigned long long)n1 * ot + (unsigned long long)(n - n1) * ob) * (unsigned long long)Kf);
+  }
+  if (level > 0) {
+    __syncthreads();
+    boundary_rot(P, nd, g);
   }
 }
 
@@ -3099,71 +3158,10 @@ cudaError_t launch_lowner(const Plan& P, const LevelLaunch& L, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-// ---------------------------------------------------------------------------
-// Boundary rows.  Each node's first and last eigenvector rows are kept apart
-// (P.v.bf, P.v.bl, by output column): the parent's z is made of them, so the
-// parent's roots do not need this node's full product.  At a merge, rbf = (first
-// row of Q1, 0) and rbl = (0, last row of Q2) take the deflating rotations as
-// k_rotate applies them to the columns of diag(Q1, Q2) (row 0 lies in the top
-// half, row n-1 in the bottom one); once the roots, zhat, the normalisers and the
-// output order are known, the node's rows are these vectors times Qhat for the
-// non-deflated columns (the same pole lists and entries as the products) and
-// copies for the deflated ones.  The top level has no parent and skips all this.
-// ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(1024) k_boundary_rot(Plan P, int level) {
-  const int64_t g = blockIdx.x;
-  const Node nd = make_node(P, level, g);
-  const int n = (int)(nd.hi - nd.lo), n1 = (int)(nd.mid - nd.lo);
-  const int64_t v0 = nd.v0;
-  double* rf = P.v.rbf + v0;
-  double* rl = P.v.rbl + v0;
-  for (int c = threadIdx.x; c < n; c += blockDim.x) {
-    rf[c] = c < n1 ? P.cbf[v0 + c] : 0.0;
-    rl[c] = c < n1 ? 0.0 : P.cbl[v0 + c];
-  }
-  const int nr = P.m.nrot[g];
-  __syncthreads();
-  const int nch = nr > 0 ? P.m.nchain[g] : 0;
-  for (int h = threadIdx.x; h < nch; h += blockDim.x) {
-    const int k0 = P.v.rch[v0 + h];
-    const int k1 = (h + 1 < nch) ? P.v.rch[v0 + h + 1] : nr;
-    for (int k = k0; k < k1; ++k) {
-      const int pj = P.v.rij[4 * (v0 + k) + 0];
-      const int ci = P.v.rij[4 * (v0 + k) + 1];
-      const int sup = P.v.rij[4 * (v0 + k) + 2];
-      const int sp = sup & 0xff, si = sup >> 8;
-      const double c = P.v.rcs[2 * (v0 + k)], s = P.v.rcs[2 * (v0 + k) + 1];
-      if ((sp | si) & 1) {
-        const double x = (sp & 1) ? rf[pj] : 0.0, y = (si & 1) ? rf[ci] : 0.0;
-        rf[pj] = c * x + s * y;
-        rf[ci] = c * y - s * x;
-      }
-      if ((sp | si) & 2) {
-        const double x = (sp & 2) ? rl[pj] : 0.0, y = (si & 2) ? rl[ci] : 0.0;
-        rl[pj] = c * x + s * y;
-        rl[ci] = c * y - s * x;
-      }
-    }
-  }
-  __syncthreads();
-  // by pole: the rotated rows at the pole's column, where the pole has support
-  const int K = P.m.K[g];
-  for (int i = threadIdx.x; i < K; i += blockDim.x) {
-    const int col = P.v.kept[v0 + i];
-    const int sup = P.v.kseg[v0 + i];
-    P.v.pf[v0 + i] = (sup & 1) ? rf[col] : 0.0;
-    P.v.pl[v0 + i] = (sup & 2) ? rl[col] : 0.0;
-  }
-}
-
 // The node's boundary rows in output order: root j's entries (formed with the
 // column norms) go to column posr[j]; deflated entry q copies its (rotated)
-// column's entries to column posd[q].
-__global__ void __launch_bounds__(256) k_boundary_out(Plan P, int level) {
-  const int64_t g = blockIdx.x;
-  const int t = blockIdx.y * blockDim.x + threadIdx.x;
-  const int K = P.m.K[g];
-  const int64_t v0 = make_node(P, level, g).v0;
+// column's entries to column posd[q].  Slot t of the merge: root t or entry t - K.
+__device__ __forceinline__ void boundary_out(const Plan& P, int64_t v0, int K, int defl, int t) {
   if (t < K) {
     const int o = P.v.posr[v0 + t];
     P.v.bf[v0 + o] = P.v.rf[v0 + t];
@@ -3171,22 +3169,19 @@ __global__ void __launch_bounds__(256) k_boundary_out(Plan P, int level) {
     return;
   }
   const int q = t - K;
-  if (q >= P.m.nd[g]) return;
+  if (q >= defl) return;
   const int c = P.v.dcol[v0 + q], sp = P.v.dseg[v0 + q], o = P.v.posd[v0 + q];
   P.v.bf[v0 + o] = (sp & 1) ? P.v.rbf[v0 + c] : 0.0;
   P.v.bl[v0 + o] = (sp & 2) ? P.v.rbl[v0 + c] : 0.0;
 }
 
-cudaError_t launch_boundary_rot(const Plan& P, const LevelLaunch& L, cudaStream_t s) {
-  if (L.level == 0 || L.merges == 0) return cudaSuccess;
-  int threads = 256;
-  while (threads > 32 && threads / 2 >= L.max_n) threads /= 2;
-  k_boundary_rot<<<(unsigned)L.merges, threads, 0, s>>>(P, L.level);
-  return cudaGetLastError();
+__global__ void __launch_bounds__(256) k_boundary_out(Plan P, int level) {
+  const int64_t g = blockIdx.x;
+  boundary_out(P, make_node(P, level, g).v0, P.m.K[g], P.m.nd[g], blockIdx.y * blockDim.x + threadIdx.x);
 }
 
 cudaError_t launch_boundary_out(const Plan& P, const LevelLaunch& L, cudaStream_t s) {
-  if (L.level == 0 || L.nslots == 0) return cudaSuccess;
+  if (L.level == 0 || L.nslots == 0 || L.max_n <= kBoundaryInFinalize) return cudaSuccess;
   k_boundary_out<<<dim3((unsigned)L.merges, (unsigned)((L.max_n + 255) / 256)), 256, 0, s>>>(P, L.level);
   return cudaGetLastError();
 }
@@ -3217,12 +3212,12 @@ __device__ __forceinline__ bool key_less(unsigned long long ka, int ta, unsigned
 // of kSortChunk entries run in shared memory, the wider ones in global memory.
 static constexpr int kSortChunk = 2048;
 
-__global__ void __launch_bounds__(1024) k_finalize(Plan P, int level) {
+__global__ void __launch_bounds__(1024) k_finalize(Plan P, int level, bool rows_out) {
   __shared__ unsigned long long sk[kSortChunk];
   __shared__ int stg[kSortChunk];
   const int64_t g = blockIdx.x;
   const Node nd = make_node(P, level, g);
-  const int n = (int)(nd.hi - nd.lo), n1 = (int)(nd.mid - nd.lo);
+  const int n = (int)(nd.hi - nd.lo);
   const int64_t v0 = nd.v0;
   const int K = P.m.K[g];
   int P2 = 1;
@@ -3291,44 +3286,54 @@ __global__ void __launch_bounds__(1024) k_finalize(Plan P, int level) {
     if (t < K) P.v.posr[v0 + t] = p;
     else if (t < n) P.v.posd[v0 + t - K] = p;
   }
-  if (threadIdx.x == 0) {
-    // GEMM tiles of this merge: (row tiles of top + bottom parts) x column tiles
-    int bm, bn;
-    dense_tile_dims(n, P.dense_small != 0, bm, bn);
-    const int64_t rt = (n1 + bm - 1) / bm + (n - n1 + bm - 1) / bm;
-    const int64_t ct = (K + bn - 1) / bn;
-    const bool split = P.split_min_K > 0 && K >= P.split_min_K;
-    const bool tiny = tiny_merge(n, K, P.m.ntop[g], P.m.nbot[g], P.split_min_K, P.struct_min_K);
-    P.m.tiles[g + 1] = (K > 0 && !split && !tiny) ? rt * ct : 0;
+  if (rows_out) {
+    __syncthreads();
+    const int defl = P.m.nd[g];
+    for (int t = threadIdx.x; t < n; t += blockDim.x) boundary_out(P, v0, K, defl, t);
   }
 }
 
-__global__ void k_tile_scan(Plan P, int64_t M) {
-  // single block exclusive scan of P.m.tiles[1..M] into a prefix with tiles[0] = 0
-  __shared__ int64_t part[1024];
+// The level's tiles of the FP64 products, (row tiles of top + bottom parts) x column tiles of
+// each merge, as a prefix with tiles[0] = 0: one block, from the deflation's counts alone, so
+// that it runs on the products' stream while the roots are being found.
+__global__ void __launch_bounds__(1024) k_tile_scan(Plan P, int level, int64_t M) {
+  __shared__ int64_t sc[4][32];
+  auto count = [&](int64_t g) -> int64_t {
+    const Node nd = make_node(P, level, g);
+    const int n = (int)(nd.hi - nd.lo), n1 = (int)(nd.mid - nd.lo), K = P.m.K[g];
+    int bm, bn;
+    dense_tile_dims(n, P.dense_small != 0, bm, bn);
+    const bool split = P.split_min_K > 0 && K >= P.split_min_K;
+    if (K <= 0 || split || tiny_merge(n, K, P.m.ntop[g], P.m.nbot[g], P.split_min_K, P.struct_min_K)) return 0;
+    return (int64_t)((n1 + bm - 1) / bm + (n - n1 + bm - 1) / bm) * ((K + bn - 1) / bn);
+  };
   const int64_t per = (M + blockDim.x - 1) / blockDim.x;
   const int64_t a = min(M, (int64_t)threadIdx.x * per), b = min(M, a + per);
-  int64_t s = 0;
-  for (int64_t i = a; i < b; ++i) s += P.m.tiles[i + 1];
-  part[threadIdx.x] = s;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    int64_t run = 0;
-    for (int i = 0; i < (int)blockDim.x; ++i) { int64_t t = part[i]; part[i] = run; run += t; }
+  int64_t v[4] = {0, 0, 0, 0};
+  for (int64_t i = a; i < b; ++i) {
+    const int64_t c = count(i);
+    P.m.tiles[i + 1] = c;
+    v[0] += c;
   }
-  __syncthreads();
-  int64_t run = part[threadIdx.x];
-  for (int64_t i = a; i < b; ++i) { run += P.m.tiles[i + 1]; P.m.tiles[i + 1] = run; }
+  block_excl_scan4(v, sc);
+  int64_t run = v[0];
+  for (int64_t i = a; i < b; ++i) {
+    run += P.m.tiles[i + 1];
+    P.m.tiles[i + 1] = run;
+  }
   if (threadIdx.x == 0) P.m.tiles[0] = 0;
+}
+
+cudaError_t launch_tile_scan(const Plan& P, const LevelLaunch& L, cudaStream_t s) {
+  if (L.merges == 0) return cudaSuccess;
+  k_tile_scan<<<1, L.merges > 512 ? 1024 : 128, 0, s>>>(P, L.level, L.merges);
+  return cudaGetLastError();
 }
 
 cudaError_t launch_finalize(const Plan& P, const LevelLaunch& L, cudaStream_t s) {
   int threads = 512;
   while (threads > 64 && threads / 2 >= L.max_n) threads /= 2;
-  k_finalize<<<(unsigned)L.merges, threads, 0, s>>>(P, L.level);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  k_tile_scan<<<1, 512, 0, s>>>(P, L.merges);
+  k_finalize<<<(unsigned)L.merges, threads, 0, s>>>(P, L.level, L.level > 0 && L.max_n <= kBoundaryInFinalize);
   return cudaGetLastError();
 }
 
