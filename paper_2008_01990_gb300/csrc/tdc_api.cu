@@ -303,7 +303,7 @@ static void build_plan(HostPlan& H, int32_t batch, const int64_t* n_host, const 
       mn = std::min(mn, p.n >> l);
       const int64_t n1 = (nm + 1) / 2;
       int bm, bn;  // a bound for either tile size: the grid walks the tiles counted on the device
-      dense_tile_dims(nm, true, bm, bn);
+      dense_tile_dims(nm, kDenseSmall, bm, bn);
       const int64_t rt = 2 * ((n1 + bm - 1) / bm);
       tiles += (((int64_t)1) << l) * rt * ((nm + bn - 1) / bn);
     }
@@ -558,6 +558,7 @@ static int run_plan(HostPlan& H, const tdc_opts& o, const double* d, const doubl
   // kernel launches: problem upload, input scale, corner modification, leaves, 9 per level (14
   // on levels that also run the thread-per-root variants, 7 more with far-field tables), output
   int64_t launches = (int64_t)((H.prob.size() + kProbChunk - 1) / kProbChunk) + 4 + 9 * (int64_t)H.T;
+  if (H.max_leaf > 8 && H.max_leaf <= 16) launches += 1;  // refined leaves and those left over
   for (int l = 0; l < H.T; ++l) {
     if (l > 0 && H.levels[l].max_n > kBoundaryInFinalize) launches += 1;  // boundary rows
     if (H.levels[l].nslots >= kSmallMinSlots) launches += 5;
@@ -597,8 +598,8 @@ static int run_plan(HostPlan& H, const tdc_opts& o, const double* d, const doubl
     P.far_stride = far_doubles(LL.max_n);
     P.dense_small = (P.split_min_K > 0 && P.split_min_K <= kDenseSmallK) ||
                             LL.nslots * LL.max_n < kDenseFewTiles * kDenseBM * kDenseBN
-                        ? 1
-                        : 0;
+                        ? (LL.nslots >= kSmallMinSlots ? kDenseTall : kDenseSmall)
+                        : kDenseLarge;
     if (l + 2 < H.T) err = cudaStreamWaitEvent(s, evG[l + 2], 0);
     const size_t a0 = mark();
     if (err == cudaSuccess) err = launch_prepare(P, LL, s);

@@ -232,7 +232,7 @@ struct Plan {
   int32_t struct_min_K; // merges with K >= this use the structured path (0: never)
   int32_t struct_m;     // tile size of the structured path
   int32_t struct_split; // 1: the structured path's products run on the split tensor-core GEMM
-  int32_t dense_small;  // the level's FP64 merges all take the small tiles (dense_tile_dims)
+  int32_t dense_small;  // DenseTiles: whether the level's FP64 merges all take small tiles, and which
   const int32_t* ss_accept;  // per merge part (2g + p): 1 if the structured split path took it
   double* far;          // far-field tables, one per merge of the level (NULL: none)
   int64_t far_stride;   // doubles per table
@@ -843,10 +843,18 @@ constexpr int kDenseSmallN = 128, kDenseSmallBM = 32, kDenseSmallBN = 32;
 // merges this wide or wider keep the large tiles where they fill the chip
 constexpr int kDenseSmallK = 256;
 constexpr int64_t kDenseFewTiles = 2 * 152;
-__host__ __device__ inline void dense_tile_dims(int64_t n, bool small, int& bm, int& bn) {
-  small = small || n <= kDenseSmallN;
+// Levels of many merges (kSmallMinSlots) take 64 rows to a small tile, which halves the
+// generation's share, where the halves fill them (an even number of 32-row tiles, or 12 and
+// more): the FP64 tiles of a batch of 256 x 512 12.6 -> 12.0 ms.  One problem keeps 32, for the
+// number of blocks.
+enum DenseTiles { kDenseLarge = 0, kDenseSmall = 1, kDenseTall = 2 };  // Plan::dense_small
+constexpr int kDenseTallBM = 64;
+__host__ __device__ inline void dense_tile_dims(int64_t n, int mode, int& bm, int& bn) {
+  const bool small = mode != kDenseLarge || n <= kDenseSmallN;
   bm = small ? kDenseSmallBM : kDenseBM;
   bn = small ? kDenseSmallBN : kDenseBN;
+  const int64_t t = ((n + 1) / 2 + kDenseSmallBM - 1) / kDenseSmallBM;
+  if (mode == kDenseTall && (t % 2 == 0 || t >= 12)) bm = kDenseTallBM;
 }
 // merges of order n <= kTinyN (halves of at most 16 rows and poles, K <= 32) off the
 // split and structured paths take a warp each (k_gemm_tiny) instead of tiles

@@ -8,8 +8,8 @@
 // column j goes to the node's eigenvector column posr[j].
 //
 // One CTA computes a 128 x 64 tile with 256 threads (8 x 4 outputs each) on
-// the FP64 pipe -- 32 x 32 (2 x 2 each) for small merges and levels of few tiles
-// (dense_tile_dims); per 16-deep k-step it stages the Qtilde tile in shared
+// the FP64 pipe -- 32 x 32 (2 x 2 each) or 64 x 32 for small merges and levels of few
+// tiles (dense_tile_dims); per 16-deep k-step it stages the Qtilde tile in shared
 // memory and generates the 16 x 64 (16 x 32) Qhat tile there (6 FP64 operations
 // per entry, amortised over the tile's rows; the normaliser s_j scales the column
 // at the end).  Tiles of all merges of the level form one work list (prefix in
@@ -179,12 +179,13 @@ __device__ __forceinline__ void dense_tile(const Plan& P, const Node& nd, int64_
 }
 }  // namespace
 
-// kSmall: every FP64 merge of the level takes 32 x 32 tiles (five blocks a SM hide each
-// other's loads and barriers).
-template <bool kSmall>
-__global__ void __launch_bounds__(kThreads, kSmall ? 5 : 2) k_gemm_dense(Plan P, int level, int64_t M) {
-  __shared__ double As[BK * (kSmall ? kDenseSmallBM : BM)];
-  __shared__ double Us[BK * (kSmall ? kDenseSmallBN : BN)];
+// kMode small: every FP64 merge of the level takes 32 x 32 tiles (five blocks a SM hide each
+// other's loads and barriers); tall: those or 64 x 32.
+template <int kMode>
+__global__ void __launch_bounds__(kThreads, kMode == kDenseSmall ? 5 : (kMode == kDenseTall ? 3 : 2))
+    k_gemm_dense(Plan P, int level, int64_t M) {
+  __shared__ double As[BK * (kMode == kDenseSmall ? kDenseSmallBM : (kMode == kDenseTall ? kDenseTallBM : BM))];
+  __shared__ double Us[BK * (kMode == kDenseLarge ? BN : kDenseSmallBN)];
   __shared__ DenseCols sc;
   const int64_t total = P.m.tiles[M];
   for (int64_t w = blockIdx.x; w < total; w += gridDim.x) {
@@ -197,10 +198,12 @@ __global__ void __launch_bounds__(kThreads, kSmall ? 5 : 2) k_gemm_dense(Plan P,
     const int64_t g = a;
     const Node nd = make_node(P, level, g);
     int bm, bn;
-    dense_tile_dims(nd.hi - nd.lo, kSmall, bm, bn);
-    if (kSmall || bm == kDenseSmallBM)
+    dense_tile_dims(nd.hi - nd.lo, kMode, bm, bn);
+    if (kMode == kDenseSmall || bm == kDenseSmallBM)
       dense_tile<kDenseSmallBM, kDenseSmallBN, true>(P, nd, g, w - P.m.tiles[g], As, Us, sc);
-    else if constexpr (!kSmall)
+    else if constexpr (kMode == kDenseTall)
+      dense_tile<kDenseTallBM, kDenseSmallBN, true>(P, nd, g, w - P.m.tiles[g], As, Us, sc);
+    else if constexpr (kMode == kDenseLarge)
       dense_tile<BM, BN, false>(P, nd, g, w - P.m.tiles[g], As, Us, sc);
   }
 }
@@ -438,8 +441,10 @@ cudaError_t launch_gemm_dense(const Plan& P, const LevelLaunch& L, int64_t max_t
   int64_t grid = max_tiles;
   const int64_t cap = 152 * 8;
   if (grid > cap) grid = cap;
-  if (P.dense_small) k_gemm_dense<true><<<(unsigned)grid, kThreads, 0, s>>>(P, L.level, L.merges);
-  else k_gemm_dense<false><<<(unsigned)grid, kThreads, 0, s>>>(P, L.level, L.merges);
+  const auto kernel = P.dense_small == kDenseTall    ? k_gemm_dense<kDenseTall>
+                      : P.dense_small == kDenseSmall ? k_gemm_dense<kDenseSmall>
+                                                     : k_gemm_dense<kDenseLarge>;
+  kernel<<<(unsigned)grid, kThreads, 0, s>>>(P, L.level, L.merges);
   return cudaGetLastError();
 }
 

@@ -3302,7 +3302,7 @@ __global__ void __launch_bounds__(1024) k_tile_scan(Plan P, int level, int64_t M
     const Node nd = make_node(P, level, g);
     const int n = (int)(nd.hi - nd.lo), n1 = (int)(nd.mid - nd.lo), K = P.m.K[g];
     int bm, bn;
-    dense_tile_dims(n, P.dense_small != 0, bm, bn);
+    dense_tile_dims(n, P.dense_small, bm, bn);
     const bool split = P.split_min_K > 0 && K >= P.split_min_K;
     if (K <= 0 || split || tiny_merge(n, K, P.m.ntop[g], P.m.nbot[g], P.split_min_K, P.struct_min_K)) return 0;
     return (int64_t)((n1 + bm - 1) / bm + (n - n1 + bm - 1) / bm) * ((K + bn - 1) / bn);
