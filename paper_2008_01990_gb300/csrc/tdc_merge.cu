@@ -2,13 +2,15 @@
 // level by level over every node of every problem in the plan:
 //   k_dmod      corner modification of the split points (Eq. (T2))
 //   k_leaf      leaf eigensolves (Algorithm 1, "QR"): two warps per leaf;
+//   k_leaf_refine FP32 iteration refined in FP64, for leaves of 9 to 16 rows;
 //   k_leaf_rows   rows in the registers of a few lanes, for leaves of at most 32 rows;
 //   k_leaf_multi  a lane per leaf for many leaves of 17 to 32 rows
 //   k_prepare   z (Eq. (T3)) from the children's boundary rows, merge of the
 //               two sorted spectra, deflation scan (Section 3.2, Eq. (T3-def)),
-//               compaction
-//               and the children's boundary rows through the deflating rotations
+//               compaction;
+//               the children's boundary rows through the deflating rotations
 //   k_rotate    plane rotations of deflation applied to Q's columns
+//   k_far_*     far poles' sums of large merges at Chebyshev points
 //   k_secular   secular equation (Eq. (secular)), one warp per root (a thread
 //               per root for small merges on many-merge levels), FP64, roots
 //               stored as (origin pole, offset) (Eq. (d-lambda))
@@ -883,13 +885,13 @@ __global__ void __launch_bounds__(128) k_leaf_refine(Plan P, int64_t nleaves, in
   }
 }
 
-// Leaves of at most 16 rows take k_leaf_rows with one row a lane while that is at most one
-// warp per quarter SM (608 quarters; 1024 leaves of 16 rows: 420 us
-// against 464 with R = 2), two rows to twice that, four beyond (12,000 leaves: 2.07 ms; the
-// lane-per-leaf kernel took 4.67 ms, and 1.39 ms for 64 leaves).  Leaves of 17 to 32 rows: under
-// 64 leaves k_leaf's two warps a leaf (10 leaves: 540 us, k_leaf_rows 681), to 4000
-// k_leaf_rows (1000 leaves: 2.4 ms, k_leaf_multi 5.3), beyond k_leaf_multi, whose time grows
-// by 1.06 us a leaf against 1.3.
+// Leaves of 9 to 16 rows take k_leaf_refine; those it leaves, and leaves of at most 8 rows, take
+// k_leaf_rows with one row a lane while that is at most one warp per quarter SM (608
+// quarters; 1024 leaves of 16 rows: 420 us against 464 with R = 2), two rows to twice that,
+// four beyond (12,000 leaves: 2.07 ms; the lane-per-leaf kernel took 4.67 ms, and 1.39 ms
+// for 64 leaves).  Leaves of 17 to 32 rows: under 64 leaves k_leaf's two warps a leaf (10
+// leaves: 540 us, k_leaf_rows 681), to 4000 k_leaf_rows (1000 leaves: 2.4 ms, k_leaf_multi
+// 5.3), beyond k_leaf_multi, whose time grows by 1.06 us a leaf against 1.3.
 cudaError_t launch_leaves(const Plan& P, int64_t nleaves, int max_leaf, cudaStream_t s) {
   if (nleaves == 0) return cudaSuccess;
   if (max_leaf > kMaxLeaf) return cudaErrorInvalidValue;
