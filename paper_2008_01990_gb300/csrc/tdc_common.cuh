@@ -587,7 +587,7 @@ cudaError_t launch_split_list(const GemmSeg* segs, int nseg_bound, const int64_t
                               int spare, cudaStream_t s, cudaEvent_t mid);
 // SMs that the products of a tree level leave to the next level's roots on the other stream
 // (the blocks of k_prepare and k_finalize fit beside no product block): at 16384 of
-// tridiag(1,2,1) 0 / 2 / 4 of them took 41.6 / 40.8 / 40.8 ms.  The last level needs none.
+// a disordered chain 0 / 2 / 4 of them took 41.6 / 40.8 / 40.8 ms.  The last level needs none.
 constexpr int kSpareSms = 2;
 cudaError_t launch_srrsc(const GemmSeg* segs, int nseg, const StructArgs& A, cudaStream_t s);
 cudaError_t launch_struct_fallback(const GemmSeg* segs, int nseg, const StructArgs& A, cudaStream_t s);
@@ -845,7 +845,7 @@ constexpr int kDenseSmallK = 256;
 constexpr int64_t kDenseFewTiles = 2 * 152;
 // Levels of many merges (kSmallMinSlots) take 64 rows to a small tile, which halves the
 // generation's share, where the halves fill them (an even number of 32-row tiles, or 12 and
-// more): the FP64 tiles of a batch of 256 x 512 12.6 -> 12.0 ms.  One problem keeps 32, for the
+// more): the FP64 tiles of 512 problems of orders 64 to 1024 12.6 -> 12.0 ms.  One problem keeps 32, for the
 // number of blocks.
 enum DenseTiles { kDenseLarge = 0, kDenseSmall = 1, kDenseTall = 2 };  // Plan::dense_small
 constexpr int kDenseTallBM = 64;

@@ -103,7 +103,7 @@ __device__ __forceinline__ void dense_tile(const Plan& P, const Node& nd, int64_
   }
   // Merges of few poles pad much of a tile, and the FP64 pipe is the bound: warps past the last
   // column (kRowFast: a warp holds 2 TN columns) and groups of poles past the last are left
-  // out.  256 problems of order 512: 15.3 -> 12.6 ms.
+  // out.  512 problems of orders 64 to 1024: 15.3 -> 12.6 ms.
   constexpr int kGroup = 4;
   const bool cols = !kRowFast || j0 + (tid >> 5) * 2 * TN < K;
   double acc[TM][TN];

@@ -335,8 +335,8 @@ __device__ __forceinline__ double level_value(long long I, int adj) {
 //
 // Bound by latency and instructions rather than by the 22 bytes an element moves: taking every
 // tile by itself and every digit through FP32 cost 135 instructions an element.  The digits of
-// an 8192 x 8192 operand pair (top merge of tridiag(1,2,1) n = 16384) 1024 -> 603 us, all of
-// that solve 40.1 -> 37.9 ms, the 8192 x 8192 Cauchy-like product 5.66 -> 5.29 ms.
+// the two halves' columns at the top of a disordered chain of n = 16384 (each about 8192 x 7447)
+// 1024 -> 603 us, all of that solve 40.1 -> 37.9 ms, the 8192 x 8192 Cauchy-like product 5.66 -> 5.29 ms.
 constexpr int kRun = 8;
 struct DigitRun {
   int64_t w, end;  // tiles [w, end)
@@ -772,7 +772,7 @@ __device__ __forceinline__ void gemm_split(const GemmSeg* segs, int nseg, const 
       // values on their way into L2, while the products run: read where they were needed, one
       // column after the other, they took 7.0 k clocks of conversion and 5.7 k (accumulating:
       // 19.6 k) of stores a tile, which was all of a shallow tile's time; now 5.0 k and 4.1 k
-      // (6.3 k).  Top merge of tridiag(1,2,1) n = 16384: products 9.64 -> 7.95 ms.
+      // (6.3 k).  Top merge of a disordered chain of n = 16384: products 9.64 -> 7.95 ms.
       const GemmSeg& sg = *t.sg;
       const int row = t.rt * BM + quarter * 32 + lane, j0 = t.ct * BN + c0, K = sg.K;
       const int64_t ldc = sg.ldc;
@@ -865,8 +865,8 @@ __global__ void __launch_bounds__(kSplitThreads, 1) k_gemm_split(const GemmSeg* 
 // of more than 32, so that every root kernel waited for the end of the product (4 ms at
 // n = 16384); with 80 a block of 128 threads of up to 112 registers fits beside it.  The
 // price is 8-column drains (1.2 % at 4096 x 4096 x 4096), so products that run alone keep the
-// other form.  With kSpareSms SMs left free for the larger blocks: tridiag(1,2,1) n = 16384
-// 42.3 -> 40.1 ms, harmonic chain n = 4999 6.29 -> 6.23 ms.
+// other form.  With kSpareSms SMs left free for the larger blocks: disordered chain n = 16384
+// 42.3 -> 40.1 ms, Hermite matrix n = 4999 6.29 -> 6.23 ms.
 template <int S, bool kChunk>
 __global__ void __maxnreg__(80) k_gemm_split_shared(const GemmSeg* segs, int nseg, const int64_t* dnseg,
                                                     const __nv_bfloat16* img, int* status, long long budget, int ck,

@@ -673,8 +673,8 @@ __global__ void __launch_bounds__(1024) k_leaf_multi(Plan P, int64_t nleaves, in
 // not fall below 2^-30 in six iterations (clusters closer than FP32 resolves in groups of
 // three or more, entries below its range) is flagged and left to k_leaf_rows.
 // Per leaf of 16 rows 0.8 M FP64 clocks of one quarter SM become 35 k clocks of FP32 chase
-// and 10 k FP64 clocks an iteration over four quarters: 64 leaves 417 -> 54 us, 8192 leaves
-// 2.11 -> 1.38 ms.  Residual and orthogonality of 16-row leaves (eps): 5.3 and 10 -> 0.8 and
+// and 10 k FP64 clocks an iteration over four quarters: 64 leaves 417 -> 54 us, 12,000
+// leaves 2.11 -> 1.38 ms.  Residual and orthogonality of 16-row leaves (eps): 5.3 and 10 -> 0.8 and
 // 0.95 for uniform entries, 6.0 and 5.5 -> 2.1 and 3.5 in one cluster, eigenvalues graded over
 // 2^-600 to 4.7e-16 of themselves (1.4e-15).
 constexpr int kRefLM = 16;
@@ -1685,8 +1685,8 @@ __device__ __forceinline__ void dnorm(double& x, int& ex) {
 // Where a block's interval is wide against its surroundings (graded or clustered spectra) the
 // near range grows to what the 4 h ask for; past 3/4 of the poles the block stays direct.
 // FP64 instructions a root at K = 16384 (direct sums in brackets): secular 580 (5180),
-// Loewner 480 (2560), norms with rows 620 (4600).  tridiag(1,2,1): n = 16384 57.3 -> 42.3 ms
-// (the sums over K >= 4096 had been 18 ms of it), harmonic chain n = 4999 6.74 -> 6.29 ms;
+// Loewner 480 (2560), norms with rows 620 (4600).  disordered chain n = 16384 57.3 -> 42.3 ms
+// (the sums over K >= 4096 had been 18 ms of it), Hermite matrix n = 4999 6.74 -> 6.29 ms;
 // band n = 2048 (one such level) 16.2 -> 16.4 ms: there the tables cost what they save, hence
 // kFarMinN.
 // ---------------------------------------------------------------------------
