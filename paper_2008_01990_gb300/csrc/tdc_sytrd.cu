@@ -32,6 +32,7 @@
 // split products cut along k into segments (partial sums added in a fixed order), then
 // X += V Z with Z = -T Y is one more split product.
 #include "tdc_common.cuh"
+#include "tdc_trd_rule.cuh"
 
 namespace tdc {
 
@@ -452,8 +453,9 @@ __global__ void __launch_bounds__(kTrdThreads, 1) k_trd_panel(TrdPanel P) {
 // round): counter 4200, entries tagged with the step that all readers poll for 7400, a flag a
 // block 7900 (stores to lines that other SMs poll are slow; reductions are not).
 // The vectors are double-buffered by the step's parity: a block writes step k + 2 only after
-// it has read all of step k + 1, whose writers had read all of step k.  A block leaves once
-// it owns no column past k + 1; the counter's next target leaves it out.
+// it has read all of step k + 1, whose writers had read all of step k.  That holds because the
+// blocks arriving at a step are exactly those its target counts (tdc_trd_rule.cuh): a block
+// leaves once it owns no column past k + 1, and one that owns none past column 0 never arrives.
 // All blocks are resident (cooperative launch); polls are bounded and report TDC_ETIMEOUT.
 //
 // Bound by the FP64 pipe (3 multiply-adds an entry of the square a column, 7 an entry of the
@@ -484,7 +486,8 @@ __global__ void __launch_bounds__(kResThreads, 1) k_trd_resident(TrdResident P) 
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int m = P.m, G = gridDim.x, b = blockIdx.x;
   if (b >= m) return;
-  const int ncb = (m - b + G - 1) / G, clast = b + (ncb - 1) * G;
+  const int ncb = (m - b + G - 1) / G, clast = trd_res_last(b, m, G);
+  if (!trd_res_takes_part(clast, 0)) return;  // owns column 0 alone (m <= G), which every block reads for itself
   double* cols = sm;  // ncb columns of m
   double* vp = cols + (int64_t)ncb * m;
   double* wp = vp + m;
@@ -507,7 +510,7 @@ __global__ void __launch_bounds__(kResThreads, 1) k_trd_resident(TrdResident P) 
   volatile int* vfail = &s_fail;
   unsigned target = 0;
   for (int k = 0; k + 2 < m; ++k) {
-    target += (unsigned)min(G, m - 1 - k);  // the blocks owning a column past k
+    target += (unsigned)trd_res_arrivals(k, m, G);
     double* xy = P.xy + (int64_t)(k & 1) * m;
     double* xc = P.xc + (int64_t)(k & 1) * m;
     double ss = 0.0;
@@ -565,7 +568,7 @@ __global__ void __launch_bounds__(kResThreads, 1) k_trd_resident(TrdResident P) 
     }
     __syncthreads();
     const double tau = s_tau, sc = s_sc;
-    const bool leave = clast < k + 2;
+    const bool leave = !trd_res_takes_part(clast, k + 1);
     if (warp == 0) {
       const int c = b + lane * G;
       if (lane < ncb && c > k) xy[c] = fma(sc, s_dot[lane], cols[lane * m + k + 1]);
@@ -616,7 +619,7 @@ __global__ void __launch_bounds__(kResThreads, 1) k_trd_resident(TrdResident P) 
     __syncthreads();
     const double g = s_g, w1 = s_w1;
     // the writer of column k's results: any block that is still here
-    const bool mine = (m - 1 - k % min(G, m - 2 - k)) % G == b;
+    const bool mine = trd_res_writer(k, m, G) == b;
     double* __restrict__ Ak = A + (int64_t)k * P.lda;
 #pragma unroll
     for (int i = 0; i < kResRows; ++i) {
