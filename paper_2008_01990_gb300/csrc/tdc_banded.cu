@@ -516,6 +516,7 @@ __global__ void __launch_bounds__(kBdDefThreads) k_bd_deflate(BdLevel L) {
   const int64_t nwords = (M + 31) / 32;
   unsigned* dbit = rotbit + (nn + 31) / 32;  // survivor q deflated by a rotation
   for (int64_t w = tid; w < nwords; w += blockDim.x) dbit[w] = 0u;
+  __syncthreads();  // the survivors' list is complete: each pair below reads entries of other threads
   for (int64_t q0 = 0; q0 < M; q0 += blockDim.x) {
     const int64_t q = q0 + tid;
     bool rot = false;
