@@ -17,6 +17,8 @@
 // nodes of a tree level take each term in the same launches, a grid row or a block a node; K
 // and the other counts stay on the device, where the products' segment list is built from
 // them (n = 2048, b = 8: 120 steps with a host read each -> 32 without, 41.7 -> 16.5 ms).
+#include <atomic>
+
 #include "tdc_common.cuh"
 
 namespace tdc {
@@ -879,7 +881,7 @@ static cudaError_t bd_sort(const BdLevel& L, int use_z, cudaStream_t s) {
 cudaError_t launch_bd_term(const BdLevel& L, int term, cudaStream_t s) {
   if (L.max_nn > kBdDefMaxN) return cudaErrorInvalidValue;
   const size_t smem = 2 * sizeof(unsigned) * (size_t)((std::max<int64_t>(L.max_nn, 1) + 31) / 32);
-  static bool attr[64] = {false};  // once per device
+  static std::atomic<bool> attr[64];  // once per device
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;

@@ -31,6 +31,8 @@
 // division and leaves z_l = 0 for a tau_l = 0 reflector.  G = V^T V and Y = V^T X are
 // split products cut along k into segments (partial sums added in a fixed order), then
 // X += V Z with Z = -T Y is one more split product.
+#include <atomic>
+
 #include "tdc_common.cuh"
 #include "tdc_trd_rule.cuh"
 
@@ -835,7 +837,7 @@ cudaError_t launch_range_unscale(double* x, int64_t n, const int* escale, cudaSt
 }
 
 int trd_panel_grid() {
-  static int grid[64] = {0};
+  static std::atomic<int> grid[64];  // per device; threads that come at once all store the same
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
   if (!grid[dev]) {
@@ -877,11 +879,10 @@ static size_t trd_resident_smem(int64_t m, int grid) {
 
 // The largest trailing order k_trd_resident takes on this device (0: none).
 int64_t trd_resident_max() {
-  static int64_t best[64] = {0};
-  static bool known[64] = {false};
+  static std::atomic<int64_t> known[64];  // per device: the order + 1; threads that come at once all store the same
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
-  if (!known[dev]) {
+  if (known[dev] == 0) {
     const int grid = trd_panel_grid();
     int optin = 0;
     cudaFuncAttributes fa;
@@ -894,10 +895,9 @@ int64_t trd_resident_max() {
       return 0;
     int64_t m = std::min<int64_t>(kTrdResMax, (int64_t)kResCols * grid);
     while (m > 0 && (int64_t)trd_resident_smem(m, grid) > room) --m;
-    best[dev] = m;
-    known[dev] = true;
+    known[dev] = m + 1;
   }
-  return best[dev];
+  return known[dev] - 1;
 }
 
 cudaError_t launch_trd_resident(const TrdResident& P, int grid, cudaStream_t s) {
@@ -1131,7 +1131,7 @@ cudaError_t launch_orm_step(const OrmStep& O, const double* A, int64_t lda, cuda
   if (e != cudaSuccess) return e;
   e = launch_seg_split(O.list1, 2 * O.ns, O.S, O.status, O.budget, O.img, O.chunk_steps, s);
   if (e != cudaSuccess) return e;
-  static bool attr[64] = {false};
+  static std::atomic<bool> attr[64];
   int dev = 0;
   e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
