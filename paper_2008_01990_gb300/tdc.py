@@ -199,6 +199,27 @@ def _stream(stream=None):
     return ctypes.c_void_p(s.cuda_stream)
 
 
+def _lend(stream, *made):
+    """Handle of the stream a call runs on.  `made` are the buffers that the wrapper itself
+    allocated or wrote on the current stream (outputs, workspaces, copies): before another
+    stream uses them it waits for the work queued so far, copies and earlier users of the same
+    memory among it, and the allocator keeps them until that stream is done with them (the
+    calls only enqueue).  Buffers of the caller's own are the caller's to order."""
+    cur = torch.cuda.current_stream()
+    if stream is None or stream.cuda_stream == cur.cuda_stream:
+        return ctypes.c_void_p(cur.cuda_stream)
+    made = [t for t in made if t is not None]
+    if made:
+        s = stream if isinstance(stream, torch.cuda.Stream) else torch.cuda.ExternalStream(stream.cuda_stream)
+        with torch.cuda.stream(s):
+            capturing = torch.cuda.is_current_stream_capturing()
+        if not capturing:  # a capture takes no wait for work outside it
+            s.wait_stream(cur)
+        for t in made:
+            t.record_stream(s)
+    return ctypes.c_void_p(stream.cuda_stream)
+
+
 def default_opts(**kw) -> Opts:
     o = Opts()
     lib().tdc_default_opts(ctypes.byref(o))
@@ -226,15 +247,19 @@ def eig(d: torch.Tensor, e: torch.Tensor, opts: Opts | None = None, ws: torch.Te
     returned as a column-major n x n matrix (a transposed view of row-major storage)."""
     n = d.numel()
     dev = d.device
+    made = []
     if lam is None:
         lam = torch.empty(n, dtype=torch.float64, device=dev)
+        made.append(lam)
     if Q is None:
         Q = torch.empty(n, n, dtype=torch.float64, device=dev).t()  # column-major storage
+        made.append(Q)
     if ws is None:
         ws = workspace(workspace_size(n, opts), dev)
+        made.append(ws)
     ld = Q.stride(1) if n > 0 else 1
     st = lib().tdc_eig(n, _ptr(d), _ptr(e), _ptr(lam), _ptr(Q), max(ld, 1), _ptr(ws), ws.numel(),
-                       ctypes.byref(opts) if opts else None, _stream(stream))
+                       ctypes.byref(opts) if opts else None, _lend(stream, *made))
     _check("tdc_eig", st)
     if check:
         _check("tdc_eig (device status)", sync_status(stream))
@@ -257,11 +282,12 @@ def eig_batched(sizes, d: torch.Tensor, e: torch.Tensor, off_de, off_q, lam: tor
     nh = np.ascontiguousarray(sizes, dtype=np.int64)
     od = np.ascontiguousarray(off_de, dtype=np.int64)
     oq = np.ascontiguousarray(off_q, dtype=np.int64)
+    made = None
     if ws is None:
-        ws = workspace(batched_workspace_size(nh, opts), d.device)
+        ws = made = workspace(batched_workspace_size(nh, opts), d.device)
     st = lib().tdc_eig_batched(len(nh), nh.ctypes.data_as(ctypes.c_void_p), od.ctypes.data_as(ctypes.c_void_p),
                                oq.ctypes.data_as(ctypes.c_void_p), _ptr(d), _ptr(e), _ptr(lam), _ptr(Q), _ptr(ws),
-                               ws.numel(), ctypes.byref(opts) if opts else None, _stream(stream))
+                               ws.numel(), ctypes.byref(opts) if opts else None, _lend(stream, made))
     _check("tdc_eig_batched", st)
     if check:
         _check("tdc_eig_batched (device status)", sync_status(stream))
@@ -280,7 +306,8 @@ def rank_one(D: torch.Tensor, z: torch.Tensor, rho: float, max_iter: int = 64, s
     _check("tdc_rank_one_workspace_size", lib().tdc_rank_one_workspace_size(K, ctypes.byref(b)))
     ws = workspace(b.value, dev)
     _check("tdc_rank_one", lib().tdc_rank_one(K, _ptr(D), _ptr(z), float(rho), _ptr(org), _ptr(tau), _ptr(zhat),
-                                              _ptr(s), int(max_iter), _ptr(ws), ws.numel(), _stream(stream)))
+                                              _ptr(s), int(max_iter), _ptr(ws), ws.numel(),
+                                              _lend(stream, org, tau, zhat, s, ws)))
     if check:
         _check("tdc_rank_one (device status)", sync_status(stream))
     return org, tau, zhat, s
@@ -301,12 +328,13 @@ def cauchy_gemm(A: torch.Tensor, D: torch.Tensor, org: torch.Tensor, tau: torch.
     m, K = A.shape
     lda = A.stride(1) if K > 0 else max(m, 1)
     C = torch.empty(K, m, dtype=torch.float64, device=A.device).t()
+    made = None
     if ws is None:
-        ws = workspace(cauchy_gemm_workspace_size(m, K, mode, opts), A.device)
+        ws = made = workspace(cauchy_gemm_workspace_size(m, K, mode, opts), A.device)
     _check("tdc_cauchy_gemm", lib().tdc_cauchy_gemm(m, K, _ptr(A), max(lda, 1), _ptr(D), _ptr(org), _ptr(tau),
                                                     _ptr(zhat), _ptr(s), _ptr(C), max(m, 1), mode,
                                                     ctypes.byref(opts) if opts else None, _ptr(ws), ws.numel(),
-                                                    _stream(stream)))
+                                                    _lend(stream, C, made)))
     if check:
         _check("tdc_cauchy_gemm (device status)", sync_status(stream))
     return C
@@ -326,7 +354,7 @@ def cauchy_like_gemm(A: torch.Tensor, d: torch.Tensor, w: torch.Tensor, u: torch
     _check("tdc_cauchy_like_gemm", lib().tdc_cauchy_like_gemm(m, n, _ptr(A), max(lda, 1), _ptr(d), _ptr(w), _ptr(u),
                                                               _ptr(v), _ptr(C), max(m, 1), mode,
                                                               ctypes.byref(opts) if opts else None, _ptr(ws),
-                                                              ws.numel(), _stream(stream)))
+                                                              ws.numel(), _lend(stream, C, ws)))
     if check:
         _check("tdc_cauchy_like_gemm (device status)", sync_status(stream))
     return C
@@ -345,7 +373,8 @@ def cauchy_like_ranks(d: torch.Tensor, w: torch.Tensor, u: torch.Tensor, v: torc
                                                                                               ctypes.byref(b)))
     ws = workspace(b.value, d.device)
     _check("tdc_cauchy_like_ranks", lib().tdc_cauchy_like_ranks(n, _ptr(d), _ptr(w), _ptr(u), _ptr(v), ctypes.byref(o),
-                                                                _ptr(ranks), _ptr(ws), ws.numel(), _stream(stream)))
+                                                                _ptr(ranks), _ptr(ws), ws.numel(),
+                                                                _lend(stream, ranks, ws)))
     _check("tdc_cauchy_like_ranks (device status)", sync_status(stream))
     return ranks
 
@@ -372,7 +401,7 @@ def sytrd(A: torch.Tensor, opts: Opts | None = None, stream=None, check: bool = 
     _check("tdc_sytrd_workspace_size", lib().tdc_sytrd_workspace_size(n, ctypes.byref(b)))
     ws = workspace(b.value, dev)
     _check("tdc_sytrd", lib().tdc_sytrd(n, _ptr(R), max(n, 1), _ptr(d), _ptr(e), _ptr(tau), _ptr(ws), ws.numel(),
-                                        ctypes.byref(opts) if opts else None, _stream(stream)))
+                                        ctypes.byref(opts) if opts else None, _lend(stream, R, d, e, tau, ws)))
     if check:
         _check("tdc_sytrd (device status)", sync_status(stream))
     return d[:n], e[:max(n - 1, 0)], tau[:max(n - 1, 0)], R
@@ -390,7 +419,8 @@ def ormtr(R: torch.Tensor, tau: torch.Tensor, X: torch.Tensor, opts: Opts | None
     ws = workspace(b.value, X.device)
     ldx = X.stride(1) if ncols > 1 else max(n, 1)
     _check("tdc_ormtr", lib().tdc_ormtr(n, ncols, _ptr(R), max(R.stride(1), n, 1), _ptr(tau), _ptr(X), max(ldx, n, 1),
-                                        _ptr(ws), ws.numel(), ctypes.byref(opts) if opts else None, _stream(stream)))
+                                        _ptr(ws), ws.numel(), ctypes.byref(opts) if opts else None,
+                                        _lend(stream, ws)))
     if check:
         _check("tdc_ormtr (device status)", sync_status(stream))
     return X
@@ -413,11 +443,13 @@ def syevd(A: torch.Tensor, opts: Opts | None = None, ws: torch.Tensor | None = N
     R = A if (overwrite and (A.stride(0) == 1 or n <= 1)) else _colmajor_copy(A)
     lam = torch.empty(max(n, 1), dtype=torch.float64, device=A.device)
     Z = torch.empty(n, n, dtype=torch.float64, device=A.device).t()
+    made = [lam, Z] if R is A else [R, lam, Z]
     if ws is None:
         ws = workspace(syevd_workspace_size(n, opts), A.device)
+        made.append(ws)
     _check("tdc_syevd", lib().tdc_syevd(n, _ptr(R), max(R.stride(1) if n > 1 else n, n, 1), _ptr(lam), _ptr(Z),
                                         max(n, 1), _ptr(ws), ws.numel(), ctypes.byref(opts) if opts else None,
-                                        _stream(stream)))
+                                        _lend(stream, *made)))
     if check:
         _check("tdc_syevd (device status)", sync_status(stream))
     return lam[:n], Z
@@ -441,7 +473,7 @@ def structured_gemm(A: torch.Tensor, t: torch.Tensor, kind: int = TOEPLITZ, mode
     ws = workspace(b.value, A.device)
     _check("tdc_structured_gemm", lib().tdc_structured_gemm(m, n, _ptr(A), max(lda, m, 1), kind, _ptr(t), _ptr(C),
                                                             max(m, 1), mode, ctypes.byref(opts) if opts else None,
-                                                            _ptr(ws), ws.numel(), _stream(stream)))
+                                                            _ptr(ws), ws.numel(), _lend(stream, C, ws)))
     if check:
         _check("tdc_structured_gemm (device status)", sync_status(stream))
     return C
@@ -459,7 +491,7 @@ def dft_gemm(A: torch.Tensor, mode: int = MERGE_DENSE, opts: Opts | None = None,
     ws = workspace(b.value, A.device)
     _check("tdc_dft_gemm", lib().tdc_dft_gemm(m, n, _ptr(A), max(lda, m, 1), _ptr(Cr), _ptr(Ci), max(m, 1), mode,
                                               ctypes.byref(opts) if opts else None, _ptr(ws), ws.numel(),
-                                              _stream(stream)))
+                                              _lend(stream, Cr, Ci, ws)))
     if check:
         _check("tdc_dft_gemm (device status)", sync_status(stream))
     return Cr, Ci
@@ -479,10 +511,8 @@ def sbevd(AB: torch.Tensor, opts: Opts | None = None, stream=None, check: bool =
                                                                       ctypes.byref(nb)))
     ws = workspace(nb.value, AB.device)
     _check("tdc_sbevd", lib().tdc_sbevd(n, b, _ptr(ABc), max(b1, 1), _ptr(lam), _ptr(Q), max(n, 1), _ptr(ws),
-                                        ws.numel(), ctypes.byref(opts) if opts else None, _stream(stream)))
-    if stream is not None:  # the call only enqueues: its buffers live until that stream is done with them
-        for t in (ABc, lam, Q, ws):
-            t.record_stream(stream)
+                                        ws.numel(), ctypes.byref(opts) if opts else None,
+                                        _lend(stream, ABc, lam, Q, ws)))
     if check:
         _check("tdc_sbevd (device status)", sync_status(stream))
     return lam[:n], Q
@@ -503,7 +533,7 @@ def bdsdc(d: torch.Tensor, e: torch.Tensor, opts: Opts | None = None, stream=Non
     ws = workspace(b.value, dev)
     _check("tdc_bdsdc", lib().tdc_bdsdc(n, _ptr(d), _ptr(e), _ptr(sigma), _ptr(U), max(n, 1), _ptr(VT), max(n, 1),
                                         _ptr(ws), ws.numel(), ctypes.byref(opts) if opts else None,
-                                        _stream(stream)))
+                                        _lend(stream, sigma, U, VT, ws)))
     if check:
         _check("tdc_bdsdc (device status)", sync_status(stream))
     return sigma[:n], U, VT
@@ -526,7 +556,7 @@ def eig_backward(lam: torch.Tensor, Q: torch.Tensor, lam_bar=None, Q_bar=None, s
     ws = workspace(b.value, dev)
     _check("tdc_eig_backward", lib().tdc_eig_backward(n, _ptr(lam), _ptr(Qc), max(Qc.stride(1), 1), _ptr(lb),
                                                       _ptr(Qb), _ptr(d_bar), _ptr(e_bar), _ptr(ws), ws.numel(),
-                                                      _stream(stream)))
+                                                      _lend(stream, Qc, lb, Qb, d_bar, e_bar, ws)))
     return d_bar, e_bar
 
 
@@ -542,9 +572,10 @@ def eig_backward_batched(lam: torch.Tensor, Qs: torch.Tensor, lam_bar=None, Qs_b
     ws = workspace(b.value, dev)
     lb = None if lam_bar is None else lam_bar.contiguous()
     qb = None if Qs_bar is None else Qs_bar.contiguous()
+    lc, qc = lam.contiguous(), Qs.contiguous()
     _check("tdc_eig_backward_batched",
-           lib().tdc_eig_backward_batched(B, n, _ptr(lam.contiguous()), _ptr(Qs.contiguous()), _ptr(lb), _ptr(qb),
-                                          _ptr(d_bar), _ptr(e_bar), _ptr(ws), ws.numel(), _stream(stream)))
+           lib().tdc_eig_backward_batched(B, n, _ptr(lc), _ptr(qc), _ptr(lb), _ptr(qb), _ptr(d_bar), _ptr(e_bar),
+                                          _ptr(ws), ws.numel(), _lend(stream, lc, qc, lb, qb, d_bar, e_bar, ws)))
     return d_bar, e_bar
 
 
