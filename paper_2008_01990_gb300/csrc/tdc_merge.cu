@@ -2013,6 +2013,18 @@ __device__ __forceinline__ void far_weights(const double* rec, double x, double&
   }
 }
 
+// Where the FP32 side of the iterations below holds its stated accuracy.  1 / rho and the
+// interval's width within FP32's range with room for their products:
+__device__ __forceinline__ bool fp32_range(float irho, float width) {
+  return irho > 1e-18f && irho < 1e18f && width > 1e-30f && width < 1e30f;
+}
+// A slope gp of 2^-20 relative accuracy: the window's terms z^2 / delta^2, delta >= dist, are
+// made of an FP32 z^2, z^2 / delta and their product, each of which may round by half of the
+// smallest subnormal (2^-150), 32 terms: 2^-145 (1 + 1 / dist + 1 / dist^2) in all.
+__device__ __forceinline__ bool fp32_slope(float gp, float dist) {
+  return dist > 1e-36f && dist < 1e30f && gp < 1e37f && gp > 1e-36f && gp * dist > 1e-36f && gp * dist * dist > 1e-36f;
+}
+
 // FP64 Newton iteration for root j from a close starting point (the FP32 estimate), as a
 // rule with a single pass over all poles.  In that pass, at tau1, the far terms (outside the
 // window of the 32 poles nearest the root, one per lane) are summed: t, t r and t r^2 with
@@ -2021,8 +2033,10 @@ __device__ __forceinline__ void far_weights(const double* rec, double x, double&
 //   t_i(tau1 + e) = t_i / (1 - e r_i) = t_i (1 + e r_i + (e r_i)^2) + rest_i,
 //   |sum of rest_i| <= (sum of far |t_i|) q^3 / (1 - q),  q = |e| / (distance from
 //   tau1 to the nearest far pole).
-// What decides the root's accuracy, the sums of t and of t r and the value g, is FP64; the
-// slope, the sums of magnitudes and the tests are FP32.  A root is accepted when |g| plus
+// What decides the root's accuracy, the far sums and the value g, is FP64 (the sum of t r^2
+// too: it is 1 / rho over the square of the poles' distances, and held in FP32 it underflowed
+// for distances from 1e13 on, with 3e-13 of the root); the slope, the sums of magnitudes and
+// the tests are FP32.  A root is accepted when |g| plus
 // the bound is at rounding level of 1/rho + sum |t|, or after a Newton step h below 2^-33 of
 // the distance to the nearest pole: the quadratic error (2^-66) and the FP32 slope's (2^-20
 // of h) are then below the rounding of tau.  A step that leaves the expansion's range
@@ -2035,7 +2049,7 @@ __device__ bool secular_certified(const double* D, const double* zz, int K, int 
                                   double& tau, int max_passes, int& passes, const double* far) {
   const int lane = threadIdx.x & 31;
   const float irf = (float)irho, wf = (float)width;
-  if (!(irf > 1e-18f && irf < 1e18f && wf > 1e-30f)) return false;  // FP32 tests out of range
+  if (!fp32_range(irf, wf)) return false;
   const bool last = j == K - 1;
   const double dorg = D[org];
   const int w0 = max(0, min(j - 15, K - 32));
@@ -2047,26 +2061,25 @@ __device__ bool secular_certified(const double* D, const double* zz, int K, int 
   const bool use_far = n0 > 0 || n1 < K;
   double tau1 = tau;
   for (passes = 1; passes <= max_passes; ++passes) {
-    double F = 0.0, A1 = 0.0;
-    float S = 0.0f, A2 = 0.0f, A1f = 0.0f, rdmin = 0.0f;
+    double F = 0.0, A1 = 0.0, A2 = 0.0;
+    float S = 0.0f, A1f = 0.0f, rdmin = 0.0f;
     if (K > 32) {
       // this lane's far poles are i = lane (mod 32): those below the window lie left of the
       // root, those above it right
-      double a0 = 0.0, b0 = 0.0, a2 = 0.0;
+      double a0 = 0.0, b0 = 0.0;
       for (int i = n0 + ((lane - n0) & 31); i < w0; i += 32) {
         const double r = rcp_nr((D[i] - dorg) - tau1);
         const double t = zz[i] * r, tr = t * r;
-        a0 += t; A1 += tr; a2 = fma(tr, r, a2);
+        a0 += t; A1 += tr; A2 = fma(tr, r, A2);
       }
       for (int i = iw + 32; i < n1; i += 32) {
         const double r = rcp_nr((D[i] - dorg) - tau1);
         const double t = zz[i] * r, tr = t * r;
-        b0 += t; A1 += tr; a2 = fma(tr, r, a2);
+        b0 += t; A1 += tr; A2 = fma(tr, r, A2);
       }
       F = a0 + b0;
       S = warp_sumf((float)(b0 - a0));
-      A2 = warp_sumf((float)a2);
-      warp_sum2(F, A1);
+      warp_sum3(F, A1, A2);
       A1f = (float)A1;
       // 1 / (distance from tau1 to the nearest far pole), below the window (lower half-warp)
       // and above it (poles are sorted)
@@ -2096,7 +2109,7 @@ __device__ bool secular_certified(const double* D, const double* zz, int K, int 
       A1 += (double)slope;
       A1f += slope;
     }
-    const double A2d = (double)A2;
+    const float A2f = (float)A2;
     double tc = tau1, e = 0.0;
     float ef = 0.0f, q = 0.0f;
     for (int it = 0; it < 8; ++it) {
@@ -2111,7 +2124,7 @@ __device__ bool secular_certified(const double* D, const double* zz, int K, int 
       }
       wsf = warp_sumf(wsf);
       wdf = warp_sumf(wdf);
-      const double gv = (irho + F + e * fma(e, A2d, A1)) + warp_sum(wt);
+      const double gv = (irho + F + e * fma(e, A2, A1)) + warp_sum(wt);
       const float gf = (float)gv, sabs = irf + S + Sf + wsf;
       // remainders: third order of the poles summed here, second of the far ones (whose FP32
       // slope is good to 2^-20)
@@ -2119,9 +2132,9 @@ __device__ bool secular_certified(const double* D, const double* zz, int K, int 
       const float rest = it > 0 ? S * q * q * q / (1.0f - q) + Sf * qf * (2.0f * qf + 0x1p-20f) : 0.0f;
       tau = tc;
       if (fabsf(gf) + rest <= 8.0f * (float)kEps * sabs) return true;
-      const float gp = A1f + 2.0f * ef * A2 + wdf;
+      const float gp = A1f + 2.0f * ef * A2f + wdf;
       const float tf = fabsf((float)tc), dist = last ? tf : fminf(tf, wf - tf);
-      if (!(gp > 0.0f && gp < 1e37f && dist > 1e-36f)) return false;
+      if (!fp32_slope(gp, dist)) return false;
       const float h = -gf / gp;
       if (!(fabsf(h) <= 0.015625f * dist)) return false;
       tc += (double)h;
@@ -2435,7 +2448,7 @@ __device__ bool secular_certified_thread(const double* D, const double* zz, int 
                                          double width, double& tau) {
   constexpr int kWin = 6;
   const float irf = (float)irho, wf = (float)width;
-  if (!(irf > 1e-18f && irf < 1e18f && wf > 1e-30f)) return false;  // FP32 tests out of range
+  if (!fp32_range(irf, wf)) return false;
   const bool last = j == K - 1;
   const double dorg = D[org];
   const int w0 = max(0, j - 2), w1 = min(K, j + 4);
@@ -2486,7 +2499,7 @@ __device__ bool secular_certified_thread(const double* D, const double* zz, int 
     if (fabsf(gf) + rest <= 8.0f * (float)kEps * sabs + sum_err) return true;
     const float gp = A1f + 2.0f * ef * A2f + wd;
     const float tf = fabsf((float)tc), dist = last ? tf : fminf(tf, wf - tf);
-    if (!(gp > 0.0f && gp < 1e37f && dist > 1e-36f)) return false;
+    if (!fp32_slope(gp, dist)) return false;
     const float h = -__fdividef(gf, gp);
     if (!(fabsf(h) <= 0.015625f * dist)) return false;
     tc += (double)h;
