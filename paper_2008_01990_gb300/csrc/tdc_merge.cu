@@ -2039,7 +2039,9 @@ __device__ __forceinline__ bool fp32_slope(float gp, float dist) {
 // the tests are FP32.  A root is accepted when |g| plus
 // the bound is at rounding level of 1/rho + sum |t|, or after a Newton step h below 2^-33 of
 // the distance to the nearest pole: the quadratic error (2^-66) and the FP32 slope's (2^-20
-// of h) are then below the rounding of tau.  A step that leaves the expansion's range
+// of h) are then below the rounding of tau.  A root accepted by its |g| still takes that last
+// step: without it the errors spread over all of the test's 8 eps, where g itself is good to
+// about one.  A step that leaves the expansion's range
 // (q >= 4e-6) starts another pass there.  Returns true when accepted (tau updated); else tau
 // is the last iterate inside the bracket and the caller continues with the safeguarded
 // iteration.  Bound by FP64 issue: 16 FP64 instructions a root, 20 an iterate and 10 a pole
@@ -2131,12 +2133,15 @@ __device__ bool secular_certified(const double* D, const double* zz, int K, int 
       const float qf = fabsf(ef) * rd3;
       const float rest = it > 0 ? S * q * q * q / (1.0f - q) + Sf * qf * (2.0f * qf + 0x1p-20f) : 0.0f;
       tau = tc;
-      if (fabsf(gf) + rest <= 8.0f * (float)kEps * sabs) return true;
       const float gp = A1f + 2.0f * ef * A2f + wdf;
       const float tf = fabsf((float)tc), dist = last ? tf : fminf(tf, wf - tf);
-      if (!fp32_slope(gp, dist)) return false;
-      const float h = -gf / gp;
-      if (!(fabsf(h) <= 0.015625f * dist)) return false;
+      const bool slope = fp32_slope(gp, dist);
+      const float h = slope ? -__fdividef(gf, gp) : 0.0f;
+      if (fabsf(gf) + rest <= 8.0f * (float)kEps * sabs) {
+        if (fabsf(h) <= 0x1p-33f * dist) tau = tc + (double)h;
+        return true;
+      }
+      if (!slope || !(fabsf(h) <= 0.015625f * dist)) return false;
       tc += (double)h;
       if (fabsf(h) <= 0x1p-33f * dist && rest <= (float)kEps * sabs) {
         tau = tc;
@@ -2496,12 +2501,15 @@ __device__ bool secular_certified_thread(const double* D, const double* zz, int 
     const float gf = (float)gv, sabs = irf + S + ws;
     const float rest = it > 0 ? S * q * q * q / (1.0f - q) : 0.0f;
     tau = tc;
-    if (fabsf(gf) + rest <= 8.0f * (float)kEps * sabs + sum_err) return true;
     const float gp = A1f + 2.0f * ef * A2f + wd;
     const float tf = fabsf((float)tc), dist = last ? tf : fminf(tf, wf - tf);
-    if (!fp32_slope(gp, dist)) return false;
-    const float h = -__fdividef(gf, gp);
-    if (!(fabsf(h) <= 0.015625f * dist)) return false;
+    const bool slope = fp32_slope(gp, dist);
+    const float h = slope ? -__fdividef(gf, gp) : 0.0f;
+    if (fabsf(gf) + rest <= 8.0f * (float)kEps * sabs + sum_err) {
+      if (fabsf(h) <= 0x1p-33f * dist) tau = tc + (double)h;
+      return true;
+    }
+    if (!slope || !(fabsf(h) <= 0.015625f * dist)) return false;
     tc += (double)h;
     if (fabsf(h) <= 0x1p-33f * dist && rest <= (float)kEps * sabs) {
       tau = tc;

@@ -66,3 +66,22 @@ def test_roots_at_far_scales(tdc, scale, K):
         t, sabs, gp = true_root(D, z, rho, j, int(org[j]), tau[j])
         err = abs(Decimal(float(tau[j])) - t)
         assert err <= Decimal((21 + K / 32) * EPS) * sabs / gp + abs(t) * Decimal(2 * EPS), (j, float(err / abs(t)))
+
+
+@pytest.mark.parametrize("K", [3, 16, 33, 100, 300])
+def test_roots_take_the_last_step(tdc, K):
+    """g at an accepted root is known to its own rounding, not only to the test's 8 eps sum, and the step
+    that this leaves is taken: errors in units of eps sum / slope are those of g's evaluation.  With 6
+    independent roundings of at most one unit a term (0.6 rms each) and up to 5 + K / 32 + 2 in the sums,
+    (0.6 sqrt(13 + K / 32)) <= 2.9 units rms for K <= 300, the stopping test alone leaves 8 / sqrt(3) = 4.6."""
+    x = []
+    for seed in range(12):
+        r = np.random.default_rng(100 * K + seed)
+        D, z = np.sort(r.uniform(0, 1, K)), r.uniform(0.05, 1, K)
+        z /= np.linalg.norm(z)
+        org, tau, _, _ = tdc.rank_one(torch.tensor(D, device=DEV), torch.tensor(z, device=DEV), 0.7, check=True)
+        org, tau = org.cpu().numpy(), tau.cpu().numpy()
+        for j in range(0, K, max(1, K // 10)):
+            t, sabs, gp = true_root(D, z, 0.7, j, int(org[j]), tau[j])
+            x.append(float((Decimal(float(tau[j])) - t) * gp / sabs / Decimal(EPS)))
+    assert np.sqrt(np.mean(np.square(x))) <= 2.9, np.sqrt(np.mean(np.square(x)))
