@@ -169,7 +169,7 @@ int tdc_workspace_size(int64_t n, const tdc_opts* o, size_t* bytes);
  * A non-finite entry of d or e is read as zero (in every problem of a batch alike) and
  * the stream's status records TDC_ENONFINITE: lam and Q are then the finite
  * eigendecomposition of the input with those entries zeroed.  A problem whose largest
- * finite |d|, |e| lies outside [2^-400, 2^400] is solved scaled by the power of two that
+ * finite |d|, |e| lies outside [2^-2, 2^32] is solved scaled by the power of two that
  * puts it in [1, 2) (exact), its eigenvalues scaled back (they overflow only where the
  * exact ones exceed the FP64 range); other problems are solved as given. */
 int tdc_eig(int64_t n, const double* d, const double* e, double* lam, double* Q, int64_t ldq, void* ws,
@@ -374,7 +374,7 @@ int tdc_dft_gemm(int64_t m, int64_t n, const double* A, int64_t lda, double* Cre
  * modifications D + z z^T with z = Q^T (x_k; y_k): sort, deflation (Section 3.2's two
  * tests), the secular equation, the Cauchy-like update of the non-deflated columns (split
  * tensor-core product from K = 128 on).  A band whose largest finite |entry| lies
- * outside [2^-400, 2^400] is solved scaled by the power of two that puts it in [1, 2)
+ * outside [2^-2, 2^32] is solved scaled by the power of two that puts it in [1, 2)
  * (exact; AB itself is not modified) and lam scaled back.  lam[n] ascending, Q n x n
  * (ldq >= n).  The nodes of a tree level take their terms in the same launches, and every
  * count stays on the device: the call only enqueues.  ws of tdc_sbevd_workspace_size(n, b, o) bytes.  Errors: -1 n, -2 b,

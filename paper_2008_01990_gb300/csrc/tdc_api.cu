@@ -1776,10 +1776,10 @@ int sbevd_run(int64_t n, int64_t b, const double* AB, int64_t ldab, double* lam,
   band_levels(nodes, band_leafmax(b), inner, first);
   BdNode* dnodes = (BdNode*)(base + L.nodes);
   if (launch_bd_copy_band(n, (int)b, AB, ldab, ABw, cs) != cudaSuccess) return TDC_ECUDA;
-  // entries outside [2^-400, 2^400]: the band copy scaled by a power of two
+  // entries outside [kScaleLow, kScaleHigh]: the band copy scaled by a power of two
   unsigned long long* rmx = (unsigned long long*)(base + L.cnt + 40);
   int* res = (int*)(base + L.cnt + 48);
-  if (launch_range_scale(ABw, ldw, n, ldw, 0, rmx, res, cs) != cudaSuccess) return TDC_ECUDA;
+  if (launch_range_scale(ABw, ldw, n, ldw, 0, kScaleLow, kScaleHigh, rmx, res, cs) != cudaSuccess) return TDC_ECUDA;
   if (launch_bd_zero(n, n, Q, ldq, cs) != cudaSuccess) return TDC_ECUDA;
   // the inner nodes' table (by kernel parameter, copied at launch) and their tearings
   for (size_t c0 = 0; c0 < inner.size(); c0 += kBdNodeChunk) {
@@ -2037,7 +2037,7 @@ int tdc_syevd(int64_t n, double* A, int64_t lda, double* lam, double* Z, int64_t
   char* rest = base + syevd_vec_bytes(n);
   const size_t rest_bytes = ws_bytes - (size_t)(rest - (char*)ws);
   // entries outside [2^-400, 2^400]: solved scaled by a power of two (A is destroyed anyway)
-  if (launch_range_scale(A, n, n, lda, 1, rmx, res, cs) != cudaSuccess) return TDC_ECUDA;
+  if (launch_range_scale(A, n, n, lda, 1, 0x1p-400, 0x1p400, rmx, res, cs) != cudaSuccess) return TDC_ECUDA;
   int r = sytrd_run(n, A, lda, d, e, tau, rest, op, st, cs);
   if (r != TDC_OK) return r;
   r = tdc_eig(n, d, e, lam, Z, ldz, rest, rest_bytes, &op, stream);

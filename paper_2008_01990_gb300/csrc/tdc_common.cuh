@@ -369,9 +369,14 @@ __device__ __forceinline__ double finite_or_zero(double x) { return isfinite(x) 
 
 // An entry of the caller's d or e as the solver reads it: non-finite as zero, then times
 // 2^-escale (exact).  A problem whose largest finite |d|, |e| lies outside
-// [2^-400, 2^400] is solved scaled by the power of two that brings it into [1, 2), so
-// that no square, product or sum of its entries overflows or underflows; escale is 0
-// otherwise and the values enter unchanged.
+// [kScaleLow, kScaleHigh] is solved scaled by the power of two that brings it into [1, 2);
+// escale is 0 otherwise and the values enter unchanged.  Below, because the deflation's
+// tolerance 8 eps max(|D|, |z|) is relative to the unit vector z once the poles are smaller
+// than it: entries of 2^-20 were solved to 1e-9 of themselves, entries of 2^-53 and less not
+// at all (every pole deflated).  Above, because the roots' FP32 estimates want poles and
+// 1 / rho well inside FP32's range (at 2^64 the solve of n = 3000 took a third longer); and
+// no square, product or sum of entries overflows or underflows.
+constexpr double kScaleLow = 0x1p-2, kScaleHigh = 0x1p32;
 __device__ __forceinline__ double input_entry(double x, int escale) {
   return escale ? scale2(finite_or_zero(x), -escale) : finite_or_zero(x);
 }
@@ -748,13 +753,15 @@ struct BdLeafArgs {
 };
 cudaError_t launch_bd_leaf_trd(const BdLeafArgs& A, const BdLeafTable& T, cudaStream_t s);
 cudaError_t launch_bd_leaf_back(const BdLeafArgs& A, const BdLeafTable& T, cudaStream_t s);
-// Overflow guard of the dense and band solvers: the largest finite |entry| of a column-major
+// Range guard of the dense and band solvers: the largest finite |entry| of a column-major
 // rows x cols block (lower != 0: its lower triangle only) and, when that lies outside
-// [2^-400, 2^400], the block times the power of two 2^-escale that puts it in [1, 2)
-// (exact); *escale = 0 otherwise.  mx and escale: 8 and 4 bytes of device scratch.
+// [low, high], the block times the power of two 2^-escale that puts it in [1, 2)
+// (exact); *escale = 0 otherwise.  The dense reduction only has to keep clear of overflow
+// (its tridiagonal takes input_entry's scale); the band tree deflates in the matrix's own
+// units and takes [kScaleLow, kScaleHigh].  mx and escale: 8 and 4 bytes of device scratch.
 // launch_range_unscale: x[0:n) times 2^escale.
-cudaError_t launch_range_scale(double* A, int64_t rows, int64_t cols, int64_t ld, int lower, unsigned long long* mx,
-                               int* escale, cudaStream_t s);
+cudaError_t launch_range_scale(double* A, int64_t rows, int64_t cols, int64_t ld, int lower, double low, double high,
+                               unsigned long long* mx, int* escale, cudaStream_t s);
 cudaError_t launch_range_unscale(double* x, int64_t n, const int* escale, cudaStream_t s);
 // The band tree's inner nodes on one level: node g holds rows [lo, lo + nn) and splits at row
 // mid; its arrays are entries lo .. lo + nn - 1 of the arrays below (columns of Qw: nn x nn at

@@ -60,7 +60,7 @@ __global__ void k_dmod(Plan P) {
 }
 
 // Each problem's input scale (a block per problem): the largest finite |d|, |e|, and
-// escale = its binary exponent when that lies outside [2^-400, 2^400], else 0.
+// escale = its binary exponent when that lies outside [kScaleLow, kScaleHigh], else 0.
 __global__ void __launch_bounds__(256) k_input_scale(Plan P) {
   __shared__ double red[8];
   for (int pi = blockIdx.x; pi < P.nprob; pi += gridDim.x) {
@@ -77,7 +77,7 @@ __global__ void __launch_bounds__(256) k_input_scale(Plan P) {
     if (threadIdx.x == 0) {
       for (int w = 1; w < (int)(blockDim.x >> 5); ++w) m = fmax(m, red[w]);
       m = fmax(m, red[0]);
-      const bool out = m > 0x1p400 || (m > 0.0 && m < 0x1p-400);
+      const bool out = m > kScaleHigh || (m > 0.0 && m < kScaleLow);
       const_cast<Problem*>(P.prob)[pi].escale = out ? ilogb(m) : 0;
     }
   }

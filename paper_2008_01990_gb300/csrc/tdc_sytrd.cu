@@ -795,14 +795,15 @@ __global__ void __launch_bounds__(256) k_range_max(const double* A, int64_t rows
   if ((threadIdx.x & 31) == 0) atomicMax(mx, (unsigned long long)__double_as_longlong(m));
 }
 
-__device__ __forceinline__ int range_exp(const unsigned long long* mx) {
+__device__ __forceinline__ int range_exp(const unsigned long long* mx, double low, double high) {
   const double m = __longlong_as_double((long long)*mx);
-  return (m > 0x1p400 || (m > 0.0 && m < 0x1p-400)) ? ilogb(m) : 0;
+  return (m > high || (m > 0.0 && m < low)) ? ilogb(m) : 0;
 }
 
 __global__ void __launch_bounds__(256) k_range_apply(double* A, int64_t rows, int64_t cols, int64_t ld, int lower,
-                                                    const unsigned long long* mx, int* escale) {
-  const int es = range_exp(mx);
+                                                    double low, double high, const unsigned long long* mx,
+                                                    int* escale) {
+  const int es = range_exp(mx, low, high);
   if (blockIdx.x == 0 && threadIdx.x == 0) *escale = es;
   if (es == 0) return;
   for (int64_t j = blockIdx.y; j < cols; j += gridDim.y)
@@ -818,15 +819,15 @@ __global__ void __launch_bounds__(256) k_range_unscale(double* x, int64_t n, con
     x[t] = scale2(x[t], es);
 }
 
-cudaError_t launch_range_scale(double* A, int64_t rows, int64_t cols, int64_t ld, int lower, unsigned long long* mx,
-                               int* escale, cudaStream_t s) {
+cudaError_t launch_range_scale(double* A, int64_t rows, int64_t cols, int64_t ld, int lower, double low, double high,
+                               unsigned long long* mx, int* escale, cudaStream_t s) {
   cudaError_t e = cudaMemsetAsync(mx, 0, sizeof(unsigned long long), s);
   if (e != cudaSuccess) return e;
   // columns over grid.y, rows of a column over grid.x (coalesced, no index division)
   const dim3 g((unsigned)std::max<int64_t>(1, std::min<int64_t>((rows + 255) / 256, 8)),
                (unsigned)std::max<int64_t>(1, std::min<int64_t>(cols, 1216)));
   k_range_max<<<g, 256, 0, s>>>(A, rows, cols, ld, lower, mx);
-  k_range_apply<<<g, 256, 0, s>>>(A, rows, cols, ld, lower, mx, escale);
+  k_range_apply<<<g, 256, 0, s>>>(A, rows, cols, ld, lower, low, high, mx, escale);
   return cudaGetLastError();
 }
 
