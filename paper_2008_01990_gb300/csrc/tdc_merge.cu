@@ -27,6 +27,7 @@
 #include <utility>
 
 #include "tdc_common.cuh"
+#include "tdc_far.cuh"
 
 namespace tdc {
 
@@ -1732,11 +1733,6 @@ __device__ __forceinline__ FarIn far_in(const BdLevel& L, int, int64_t g) {
   return f;
 }
 
-__device__ __forceinline__ int* far_range(double* rec) { return reinterpret_cast<int*>(rec + 5 * kFarM); }
-__device__ __forceinline__ const int* far_range(const double* rec) {
-  return reinterpret_cast<const int*>(rec + 5 * kFarM);
-}
-
 // The block's interval, its near poles, points and weights.
 template <typename C>
 __global__ void __launch_bounds__(32) k_far_setup(C ctx, int level) {
@@ -1991,28 +1987,6 @@ __device__ __forceinline__ const double* far_record(const double* tab, int K, in
   return tab && K >= kFarMinK ? tab + (int64_t)(j / far_block(K)) * kFarRec : nullptr;
 }
 
-// Barycentric weights of the block's points for position x (relative to the block's pole
-// ref): bw in lanes below kFarM, and 1 / (x - y); a point that x falls on takes all of it.
-__device__ __forceinline__ void far_weights(const double* rec, double x, double& bw, double& rd) {
-  const int lane = threadIdx.x & 31;
-  bw = 0.0;
-  rd = 0.0;
-  bool hit = false;
-  if (lane < kFarM) {
-    const double d = x - rec[lane];
-    hit = !in_range(fabs(d));
-    if (!hit) {
-      rd = rcp_nr(d);
-      bw = rec[kFarM + lane] * rd;
-    }
-  }
-  const unsigned h = __ballot_sync(0xffffffffu, hit);
-  if (h) {
-    bw = lane == __ffs(h) - 1 ? 1.0 : 0.0;
-    rd = 0.0;
-  }
-}
-
 // Where the FP32 side of the iterations below holds its stated accuracy.  1 / rho and the
 // interval's width within FP32's range with room for their products:
 __device__ __forceinline__ bool fp32_range(float irho, float width) {
@@ -2093,19 +2067,9 @@ __device__ bool secular_certified(const double* D, const double* zz, int K, int 
     // the far poles' sum and slope by interpolation; Sf bounds their sum |t|, rd3 1 / distance
     float Sf = 0.0f, rd3 = 0.0f;
     if (use_far) {
-      double bw, rd, ff = 0.0;
-      far_weights(far, (dorg - D[far_range(far)[4]]) + tau1, bw, rd);
-      if (lane < kFarM) {
-        ff = far[2 * kFarM + lane];
-        Sf = (float)far[3 * kFarM + lane];
-      }
-      double num = bw * ff, den = bw;
-      warp_sum2(num, den);
-      const double rden = rcp_nr(den), p = num * rden;
-      const float slope = warp_sumf((float)(bw * (p - ff)) * (float)rd) * (float)rden;
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) Sf = fmaxf(Sf, __shfl_xor_sync(0xffffffffu, Sf, o));
-      rd3 = (float)far[5 * kFarM + 1];
+      double p;
+      float slope;
+      far_value(far, (dorg - D[far_range(far)[4]]) + tau1, p, slope, Sf, rd3);
       rdmin = fmaxf(rdmin, rd3);
       F += p;
       A1 += (double)slope;
