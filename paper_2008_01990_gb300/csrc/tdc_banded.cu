@@ -433,22 +433,6 @@ __device__ __forceinline__ int block_scan_bd(int f, int* wcnt, int& total) {
   return before + __popc(m & ((1u << lane) - 1u));
 }
 
-// w = hypot(zj, zp), c = zj / w, s = -zp / w from a refined reciprocal square root where the
-// squares stay in range (nine FP64 operations for some fifty).
-__device__ __forceinline__ void bd_rotation(double zj, double zp, double& w, double& c, double& s) {
-  const double t2 = fma(zj, zj, zp * zp);
-  if (in_range(t2)) {
-    const double ri = rsqrt_cubic(t2);
-    w = t2 * ri;
-    c = zj * ri;
-    s = -zp * ri;
-  } else {
-    w = hypot(zj, zp);
-    c = zj / w;
-    s = -zp / w;
-  }
-}
-
 __global__ void __launch_bounds__(kBdDefThreads) k_bd_deflate(BdLevel L) {
   extern __shared__ unsigned rotbit[];  // speculative outcome of survivor pair (q - 1, q), then dbit
   __shared__ double red[32];

@@ -530,6 +530,22 @@ __device__ __forceinline__ void reflector(double alpha, double s, double& tau, d
   }
 }
 
+// w = hypot(zj, zp), c = zj / w, s = -zp / w from a refined reciprocal square root where the
+// squares stay in range (nine FP64 operations for some fifty).
+__device__ __forceinline__ void bd_rotation(double zj, double zp, double& w, double& c, double& s) {
+  const double t2 = fma(zj, zj, zp * zp);
+  if (in_range(t2)) {
+    const double ri = rsqrt_cubic(t2);
+    w = t2 * ri;
+    c = zj * ri;
+    s = -zp * ri;
+  } else {
+    w = hypot(zj, zp);
+    c = zj / w;
+    s = -zp / w;
+  }
+}
+
 // A call's status slot is two words: status[0] the first error (first writer wins),
 // status[1] warning bits (results written, accuracy possibly reduced).
 __device__ __forceinline__ void set_status(int* status, int code) {
