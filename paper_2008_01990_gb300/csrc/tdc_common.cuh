@@ -501,12 +501,6 @@ __device__ __forceinline__ void warp_sum3(double& a, double& b, double& c) {
   c = __shfl_sync(0xffffffffu, v, 16);
 }
 
-__device__ __forceinline__ double warp_prod(double v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v *= __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
-}
-
 __device__ __forceinline__ double warp_max(double v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
