@@ -670,7 +670,7 @@ def config_dense(args, n=4096, steps=3):
             "stage_ms": {"sytrd": ms_trd, "eig": ms_eig, "ormtr": ms_orm},
             "checks": {"residual": res, "orthogonality": orth, "paper_residual": paper_res, "columns": "all",
                        "within_bounds": bool(res <= 50 and orth <= 50)},
-            "roofline": {"bound": "alu", "kernel": "k_trd_panel (FP64 symv of the one-stage reduction)",
+            "roofline": {"bound": "alu", "kernel": "k_trd_panel and k_trd_resident (FP64 symv of the one-stage reduction, its last columns in shared memory)",
                          "achieved": achieved, "peak": fp64_peak, "unit": "TFLOP/s", "frac": achieved / fp64_peak,
                          "note": "symv flops 2 sum m^2 over the whole tdc_sytrd time (trailing updates included); "
                                  "peak derived from unit counts (152 SMs x 2 DFMA/clk x 2.07 GHz)"},

@@ -377,9 +377,11 @@ int tdc_dft_gemm(int64_t m, int64_t n, const double* A, int64_t lda, double* Cre
  * outside [2^-2, 2^32] is solved scaled by the power of two that puts it in [1, 2)
  * (exact; AB itself is not modified) and lam scaled back.  lam[n] ascending, Q n x n
  * (ldq >= n).  The nodes of a tree level take their terms in the same launches, and every
- * count stays on the device: the call only enqueues.  ws of tdc_sbevd_workspace_size(n, b, o) bytes.  Errors: -1 n, -2 b,
- * -3 AB, -4 ldab, -5 lam, -6 Q, -7 ldq, -10 options, TDC_ENOWS, TDC_ECUDA, or those of
- * the steps. */
+ * count stays on the device: like the other solvers the call only enqueues, so lam and Q
+ * are there once the stream has been synchronised, and what goes wrong on the device shows
+ * in the stream's status (tdc_sync_status).  ws of tdc_sbevd_workspace_size(n, b, o) bytes.
+ * Errors: -1 n, -2 b, -3 AB, -4 ldab, -5 lam, -6 Q, -7 ldq, -10 options, TDC_ENOWS,
+ * TDC_ECUDA, or those of the steps. */
 int tdc_sbevd_workspace_size(int64_t n, int64_t b, const tdc_opts* o, size_t* bytes);
 int tdc_sbevd(int64_t n, int64_t b, const double* AB, int64_t ldab, double* lam, double* Q, int64_t ldq, void* ws,
               size_t ws_bytes, const tdc_opts* o, tdc_stream_t stream);

@@ -184,7 +184,15 @@ __device__ __forceinline__ double struct_entry(const GemmSeg& sg, int64_t k, int
 constexpr int kFarM = 20;        // Chebyshev nodes of a block
 constexpr int kFarRec = 5 * kFarM + 4;
 constexpr int kFarMinK = 1024;
-constexpr int kFarMinN = 2048;   // host: levels whose largest merge has at least this order
+// Host: levels whose largest merge has at least this order.  With tables / without (us): one
+// merge of 2048 on top, disordered chain 1617 / 1591 (runs differ by as much), band of b = 8
+// 15,604 / 15,680 (uniform) and 16,672 / 16,622 (coupled chain); n = 2150 1949 / 2142, 2500
+// 2282 / 2483, 4096 4138 / 4665; the levels of 2048 under larger merges gain as well (line at
+// 2049: n = 4096 4167 -> 4333, 16384 31.2 -> 31.8 ms).  Bands: n = 2250 to 2400 lose 0.5 to 5 %
+// with tables, 2500 22.3 / 22.7 ms, 4096 52.8 / 55.7, 8192 (b = 2) 70.1 / 75.8; a line of their own at 2500
+// costs n = 4096 1.4 %.  Matrices that deflate almost all poles (uniform) pay 1 to 3 % for tables
+// without blocks, at every order.
+constexpr int kFarMinN = 2048;
 constexpr int64_t kFarMaxMerges = 64;  // and at most so many merges
 constexpr int kFarSplit = 512;   // far poles a block of threads takes
 __host__ __device__ inline int far_block(int64_t K) { return K < 4096 ? 64 : (K < 12288 ? 128 : 256); }

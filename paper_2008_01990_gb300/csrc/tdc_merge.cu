@@ -284,15 +284,6 @@ __global__ void __launch_bounds__(64) k_leaf(Plan P, int64_t nleaves) {
   }
 }
 
-// Leaves of at most LM = 8, 16 or 32 rows: GL = LM / R lanes per leaf, each holding R rows
-// of the eigenvector block, and all of the leaf's d and e, in registers.  Every lane of a
-// leaf runs the same implicit QL/QR chase (the recurrence of EISPACK's imtql2, run from the
-// top) and applies each rotation to its own rows at once, so a leaf needs no shared memory,
-// no barrier and no hand-over of rotations.  Bound by FP64 issue: an FP64 warp instruction
-// holds its quarter of the SM for 64 clocks (measured, whatever the number of active lanes),
-// and a rotation takes 19 of them for the chase and 4 R for the rows.  With few leaves R = 1
-// is shortest (the leaves spread over the SMs), with many a larger R shares a chase among
-// more leaves of the warp.  64 leaves of 16 rows: 1393 -> 415 us.
 // f(0), ..., f(N-1) with the index a compile-time constant in each call, so that register
 // arrays indexed by it are scalars from the start (an unrolled loop with tests on a runtime
 // k was turned back into indexed accesses of local memory)
@@ -314,6 +305,15 @@ __device__ __forceinline__ double twice(double x) {
   return __hiloint2double(h + 0x100000, __double2loint(x));
 }
 
+// Leaves of at most LM = 8, 16 or 32 rows: GL = LM / R lanes per leaf, each holding R rows
+// of the eigenvector block, and all of the leaf's d and e, in registers.  Every lane of a
+// leaf runs the same implicit QL/QR chase (the recurrence of EISPACK's imtql2, run from the
+// top) and applies each rotation to its own rows at once, so a leaf needs no shared memory,
+// no barrier and no hand-over of rotations.  Bound by FP64 issue: an FP64 warp instruction
+// holds its quarter of the SM for 64 clocks (measured, whatever the number of active lanes),
+// and a rotation takes 19 of them for the chase and 4 R for the rows.  With few leaves R = 1
+// is shortest (the leaves spread over the SMs), with many a larger R shares a chase among
+// more leaves of the warp.  64 leaves of 16 rows: 1393 -> 415 us.
 template <int LM, int R, int NL>
 __global__ void __launch_bounds__(32) k_leaf_rows(Plan P, int64_t nleaves, const int* only) {
   constexpr int GL = LM / R;  // lanes per leaf; NL leaves per warp
@@ -671,8 +671,13 @@ __global__ void __launch_bounds__(1024) k_leaf_multi(Plan P, int64_t nleaves, in
 // tangent of the 2 x 2 problem's rotation, for which I + E is that rotation up to a scale.
 // The error is squared each time: two iterations as a rule.  s_ij at rounding level of
 // |lam_i| + |lam_j| counts as zero (the QR iteration's own criterion).  A leaf whose E does
-// not fall below 2^-30 in six iterations (clusters closer than FP32 resolves in groups of
-// three or more, entries below its range) is flagged and left to k_leaf_rows.
+// not fall below 2^-30 in six iterations is flagged and left to k_leaf_rows: clusters closer
+// than FP32 resolves in groups of three or more, entries below its range, and close pairs of
+// eigenvalues small against ||T||, whose s_ij rounds by eps ||T|| and so keeps above the test
+// (relative to ||T|| it would give up the graded accuracy below).  Counted over 15 families of
+// orders 1024 to 16384: two iterations for 97 to 100 % of the leaves of 13 of them, three to
+// five where all diagonal entries are equal and e about 1e-3, none left over in either; glued
+// Wilkinson matrices leave 4 to 5 %.
 // Per leaf of 16 rows 0.8 M FP64 clocks of one quarter SM become 35 k clocks of FP32 chase
 // and 10 k FP64 clocks an iteration over four quarters: 64 leaves 417 -> 54 us, 12,000
 // leaves 2.11 -> 1.38 ms.  Residual and orthogonality of 16-row leaves (eps): 5.3 and 10 -> 0.8 and
@@ -1687,9 +1692,8 @@ __device__ __forceinline__ void dnorm(double& x, int& ex) {
 // near range grows to what the 4 h ask for; past 3/4 of the poles the block stays direct.
 // FP64 instructions a root at K = 16384 (direct sums in brackets): secular 580 (5180),
 // Loewner 480 (2560), norms with rows 620 (4600).  disordered chain n = 16384 57.3 -> 42.3 ms
-// (the sums over K >= 4096 had been 18 ms of it), Hermite matrix n = 4999 6.74 -> 6.29 ms;
-// band n = 2048 (one such level) 16.2 -> 16.4 ms: there the tables cost what they save, hence
-// kFarMinN.
+// (the sums over K >= 4096 had been 18 ms of it), Hermite matrix n = 4999 6.74 -> 6.29 ms.
+// Where the line lies: at kFarMinN.
 // ---------------------------------------------------------------------------
 // record: points y[M] (relative to pole ref), barycentric weights w[M], f0, f1, f2[M]; then
 // {n0, n1} (the near poles), 1 / (3 h), {ref, -}, -.
@@ -2018,7 +2022,7 @@ __device__ __forceinline__ bool fp32_slope(float gp, float dist) {
 // about one.  A step that leaves the expansion's range
 // (q >= 4e-6) starts another pass there.  Returns true when accepted (tau updated); else tau
 // is the last iterate inside the bracket and the caller continues with the safeguarded
-// iteration.  Bound by FP64 issue: 16 FP64 instructions a root, 20 an iterate and 10 a pole
+// iteration.  Bound by FP64 issue: 17 FP64 instructions a root, 20 an iterate and 10 a pole
 // and pass of 32; the earlier form (four FP64 sums, divisions and a square root an iterate)
 // took 24,000 clocks a root of a small merge, this one 5,000.
 __device__ bool secular_certified(const double* D, const double* zz, int K, int j, double irho, int org, double width,
@@ -2656,9 +2660,12 @@ __device__ __forceinline__ void for_warp_roots(const Plan& P, int64_t M, int sma
   }
 }
 
-// Block sizes of the root-side kernels are chosen so that a block fits on an SM
-// beside a resident split-GEMM CTA (about 17.9K registers and 59 KB of shared
-// memory left): the roots of the next level run while this level's products do.
+// Block sizes of the root-side kernels are chosen so that a block fits on an SM beside a
+// resident CTA of a tree's split product (k_gemm_split_shared, 18 warps of 80 registers): 3,584
+// registers of two of the SM's quarters, 6,144 of the other two and 59 KB of shared memory are
+// left, which takes 128 threads (a warp a quarter) of up to 112 registers.  So the roots of the
+// next level run while this level's products do; the blocks of k_prepare and k_finalize are
+// larger and take the kSpareSms SMs that the products leave free.
 constexpr int kSecThreads = 128;
 
 static dim3 warp_root_grid(const LevelLaunch& L, bool listed) {
@@ -2742,8 +2749,8 @@ __global__ void __launch_bounds__(kSecThreads) k_secular_fixup(Plan P, int level
 }
 
 // Warp per root over the merges with K > small_k (for_warp_roots).  At most 80 registers a
-// thread: four warps then fit on an SM beside a resident CTA of the split product (96 x 576
-// of the 65,536 registers), whose stream runs during the next level's roots.
+// thread: six blocks on an SM of its own, one beside a resident CTA of the previous level's
+// split product (kSecThreads).
 __global__ void __launch_bounds__(kSecThreads, 6) k_secular(Plan P, int level, int64_t M, int small_k, bool listed) {
   for_warp_roots(P, M, small_k, listed, [&](int64_t g, int K, int jw) {
     const Node nd = make_node(P, level, g);
