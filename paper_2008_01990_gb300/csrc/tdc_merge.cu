@@ -2022,7 +2022,7 @@ __device__ __forceinline__ bool fp32_slope(float gp, float dist) {
 // about one.  A step that leaves the expansion's range
 // (q >= 4e-6) starts another pass there.  Returns true when accepted (tau updated); else tau
 // is the last iterate inside the bracket and the caller continues with the safeguarded
-// iteration.  Bound by FP64 issue: 17 FP64 instructions a root, 20 an iterate and 10 a pole
+// iteration.  Bound by FP64 issue: 19 FP64 instructions a root, 17 an iterate and 10 a pole
 // and pass of 32; the earlier form (four FP64 sums, divisions and a square root an iterate)
 // took 24,000 clocks a root of a small merge, this one 5,000.
 __device__ bool secular_certified(const double* D, const double* zz, int K, int j, double irho, int org, double width,
@@ -2079,7 +2079,7 @@ __device__ bool secular_certified(const double* D, const double* zz, int K, int 
       A1 += (double)slope;
       A1f += slope;
     }
-    const float A2f = (float)A2;
+    const float A2f = (float)A2, t1f = (float)tau1;
     double tc = tau1, e = 0.0;
     float ef = 0.0f, q = 0.0f;
     for (int it = 0; it < 8; ++it) {
@@ -2102,7 +2102,7 @@ __device__ bool secular_certified(const double* D, const double* zz, int K, int 
       const float rest = it > 0 ? S * q * q * q / (1.0f - q) + Sf * qf * (2.0f * qf + 0x1p-20f) : 0.0f;
       tau = tc;
       const float gp = A1f + 2.0f * ef * A2f + wdf;
-      const float tf = fabsf((float)tc), dist = last ? tf : fminf(tf, wf - tf);
+      const float tf = fabsf(t1f + ef), dist = last ? tf : fminf(tf, wf - tf);
       const bool slope = fp32_slope(gp, dist);
       const float h = slope ? -__fdividef(gf, gp) : 0.0f;
       if (fabsf(gf) + rest <= 8.0f * (float)kEps * sabs) {
@@ -2110,13 +2110,14 @@ __device__ bool secular_certified(const double* D, const double* zz, int K, int 
         return true;
       }
       if (!slope || !(fabsf(h) <= 0.015625f * dist)) return false;
-      tc += (double)h;
       if (fabsf(h) <= 0x1p-33f * dist && rest <= (float)kEps * sabs) {
-        tau = tc;
+        tau = tc + (double)h;
         return true;
       }
-      e = tc - tau1;
-      ef = (float)e;
+      // any point near the step's end will do for the next iterate: an FP32 offset
+      ef += h;
+      e = (double)ef;
+      tc = tau1 + e;
       q = fabsf(ef) * rdmin;
       if (!(q < 4e-6f)) break;
     }
@@ -2450,6 +2451,7 @@ __device__ bool secular_certified_thread(const double* D, const double* zz, int 
   const float fa = (float)fabs(a0), fb = (float)b0, S = fa + fb, A1f = (float)A1, A2f = (float)a2;
   const float sum_err = (float)kEps * ((float)w0 * fa + (float)(K - w1) * fb);
   const double F = a0 + b0, tau1 = tc;
+  const float t1f = (float)tau1;
   double e = 0.0;
   float ef = 0.0f, q = 0.0f;
   for (int it = 0; it < 8; ++it) {
@@ -2470,7 +2472,7 @@ __device__ bool secular_certified_thread(const double* D, const double* zz, int 
     const float rest = it > 0 ? S * q * q * q / (1.0f - q) : 0.0f;
     tau = tc;
     const float gp = A1f + 2.0f * ef * A2f + wd;
-    const float tf = fabsf((float)tc), dist = last ? tf : fminf(tf, wf - tf);
+    const float tf = fabsf(t1f + ef), dist = last ? tf : fminf(tf, wf - tf);
     const bool slope = fp32_slope(gp, dist);
     const float h = slope ? -__fdividef(gf, gp) : 0.0f;
     if (fabsf(gf) + rest <= 8.0f * (float)kEps * sabs + sum_err) {
@@ -2478,13 +2480,13 @@ __device__ bool secular_certified_thread(const double* D, const double* zz, int 
       return true;
     }
     if (!slope || !(fabsf(h) <= 0.015625f * dist)) return false;
-    tc += (double)h;
     if (fabsf(h) <= 0x1p-33f * dist && rest <= (float)kEps * sabs) {
-      tau = tc;
+      tau = tc + (double)h;
       return true;
     }
-    e = tc - tau1;
-    ef = (float)e;
+    ef += h;
+    e = (double)ef;
+    tc = tau1 + e;
     q = fabsf(ef) * rdmin;
     if (!(q < 4e-6f)) return false;
   }
