@@ -128,19 +128,21 @@ __global__ void __launch_bounds__(64) k_leaf(Plan P, int64_t nleaves) {
   double* dd = Qs + L * L;         // L
   double* ee = dd + L;             // L
   double* cs = ee + L;             // 2 buffers x 2L (c, s of each rotation)
-  int* ctrl = (int*)(cs + 4 * L);  // [b][0..1] = pp, q of the sweep in buffer b; [4] = done
+  int* ctrl = (int*)(cs + 4 * L);  // [b][0..1] = pp, q of the sweep in buffer b
   int* perm = ctrl + 6;            // L
   for (int k = tid; k < L * L; k += blockDim.x) Qs[k] = ((k % L) == (k / L)) ? 1.0 : 0.0;
   for (int k = tid; k < L; k += blockDim.x) {
     dd[k] = P.v.dmod[p.voff + lo + k];
     ee[k] = (k < L - 1) ? input_entry(P.e[p.off_de + lo + k], p.escale) : 0.0;
   }
-  if (tid == 0) ctrl[4] = (L <= 1) ? 1 : 0;
   __syncthreads();
   const int max_sweeps = 40 * (L > 0 ? L : 1);
   int sweep = 0;
-  while (!ctrl[4]) {
+  // the end of the iteration travels with the loop's barrier: a flag in shared memory that the
+  // next round may set could be seen by one warp and not by the other
+  for (bool last = L <= 1; !last;) {
     const int b = sweep & 1;
+    bool end = false;
     if (warp == 0) {
       // negligible off-diagonals (all lanes), then the trailing unreduced block
       unsigned long long nz = 0ull;
@@ -157,11 +159,11 @@ __global__ void __launch_bounds__(64) k_leaf(Plan P, int64_t nleaves) {
       __syncwarp();
       if (lane == 0) {
         if (nz == 0ull) {
-          ctrl[4] = 1;
+          end = true;
           ctrl[2 * b] = 0;
           ctrl[2 * b + 1] = 0;
         } else if (sweep >= max_sweeps) {
-          ctrl[4] = 1;
+          end = true;
           ctrl[2 * b] = 0;
           ctrl[2 * b + 1] = 0;
           set_status(P.status, TDC_ENOCONV);
@@ -236,7 +238,7 @@ __global__ void __launch_bounds__(64) k_leaf(Plan P, int64_t nleaves) {
         if (two) Qs[r1 + q * L] = v1;
       }
     }
-    __syncthreads();
+    last = __syncthreads_or(end ? 1 : 0) != 0;
     ++sweep;
   }
   // the sweep in the last buffer (if any) is still to be applied

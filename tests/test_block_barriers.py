@@ -1,0 +1,45 @@
+"""Barriers that a block's warps depend on, walked through in the kernels' sources (a missing one
+cannot be shown safely by running it)."""
+import os
+import re
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2008_01990_gb300", "csrc")
+
+
+def body_after(text, start):
+    """The braced body that follows `start`, without comments."""
+    text = re.sub(r"//[^\n]*", "", text)
+    at = text.index("{", text.index(start))
+    depth, i = 0, at
+    while True:
+        depth += {"{": 1, "}": -1}.get(text[i], 0)
+        if depth == 0:
+            return text[at + 1:i]
+        i += 1
+
+
+def source(name):
+    return open(os.path.join(CSRC, name)).read()
+
+
+def shared_exit_flags(body):
+    """Loop conditions that read shared memory which the loop itself writes: one warp may already
+    have set it in the next round when another evaluates the condition."""
+    found = []
+    for m in re.finditer(r"\bwhile \(!?(\w+)\[(\w+)\]\)\s*\{", body):
+        inner = body_after(body[m.start():], "while")
+        if re.search(r"\b%s\[%s\]\s*=(?!=)" % (m.group(1), m.group(2)), inner):
+            found.append(m.group(0))
+    return found
+
+
+def test_leaf_iteration_ends_at_a_barrier():
+    """The two warps of a leaf leave the QR iteration together: its end comes out of the barrier."""
+    body = body_after(source("tdc_merge.cu"), "k_leaf(Plan P, int64_t nleaves)")
+    assert shared_exit_flags(body) == []
+    assert re.search(r"last = __syncthreads_or\(end \? 1 : 0\) != 0;\s*\+\+sweep;\s*\}", body)
+
+
+def test_a_shared_exit_flag_is_found():
+    body = "ctrl[4] = 0; __syncthreads(); while (!ctrl[4]) { if (warp == 0) ctrl[4] = 1; __syncthreads(); }"
+    assert len(shared_exit_flags(body)) == 1
