@@ -163,6 +163,8 @@ __device__ __forceinline__ void dense_tile(const Plan& P, const Node& nd, int64_
       }
     }
   }
+  // a half that no kept pole has support in runs no k-step, and so none of the loop's barriers
+  if (qlo >= qhi) __syncthreads();
   // epilogue: write to the node's output columns
 #pragma unroll
   for (int c = 0; c < TN; ++c) {

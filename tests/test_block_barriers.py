@@ -43,3 +43,14 @@ def test_leaf_iteration_ends_at_a_barrier():
 def test_a_shared_exit_flag_is_found():
     body = "ctrl[4] = 0; __syncthreads(); while (!ctrl[4]) { if (warp == 0) ctrl[4] = 1; __syncthreads(); }"
     assert len(shared_exit_flags(body)) == 1
+
+
+def test_fp64_tiles_meet_before_their_columns_are_stored():
+    """A tile's column places and scales, written by its first threads, are read by all in the epilogue:
+    the pole loop's barriers lie in between, and where the half has no pole a barrier of its own."""
+    body = body_after(source("tdc_gemm_dense.cu"), "void dense_tile(")
+    write, read = body.index("sc.Pos[tid] ="), body.index("const int pos = sc.Pos[")
+    between = body[write:read]
+    assert "for (int k0 = qlo; k0 < qhi; k0 += BK) {" in between
+    after_loop = between[between.index("for (int k0 = qlo"):]
+    assert re.search(r"if \(qlo >= qhi\) __syncthreads\(\);", after_loop)
