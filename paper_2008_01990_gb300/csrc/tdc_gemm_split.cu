@@ -144,7 +144,8 @@ int64_t split_img_elems(int64_t rows_top, int64_t rows_bot, int64_t kk_bound, in
 // ---------------------------------------------------------------------------
 // One block: each thread counts the digit tiles, output tiles and image elements
 // of a contiguous range of merges, a block scan gives every range its offsets,
-// then the threads write their segments.
+// then the threads write their segments.  A half that no kept pole supports (kk = 0) has
+// no images but keeps its segment: its output tiles store the zeros of its rows.
 // When every non-deflated pole has support in both halves (cross rotations pair
 // each pole of one child with one of the other, as for equal spectra), the two
 // pole lists are the same and the bottom part reuses the top part's Qhat image.
@@ -190,7 +191,7 @@ __global__ void __launch_bounds__(1024) k_split_segs(Plan P, int level, int64_t 
     int64_t ta, tb, tt, el;
     split_seg_counts(P, level, g0 + w / 2, S, (int)(w & 1), ta, tb, tt, el);
     cta += ta; ctb += tb; ctt += tt; cel += el;
-    cns += el > 0 ? 1 : 0;
+    cns += tt > 0 ? 1 : 0;
   }
   int64_t v[4] = {cta, ctb, ctt, cel};
   block_excl_scan4(v, sc);
@@ -203,7 +204,7 @@ __global__ void __launch_bounds__(1024) k_split_segs(Plan P, int level, int64_t 
     const int p = (int)(w & 1);
     int64_t ta, tb, tt, el;
     split_seg_counts(P, level, g, S, p, ta, tb, tt, el);
-    if (el == 0) continue;
+    if (tt == 0) continue;
     const Node nd = make_node(P, level, g);
     const int n = (int)(nd.hi - nd.lo), n1 = (int)(nd.mid - nd.lo);
     const int K = P.m.K[g];
@@ -236,7 +237,7 @@ __global__ void __launch_bounds__(1024) k_split_segs(Plan P, int level, int64_t 
       split_seg_counts(P, level, g, S, 0, ta0, tb0, tt0, el0);
       sg.b_img = e - el0 + ta0 * S * kATileElems;
     }
-    if (el > 0 && P.stats) {
+    if (P.stats) {
       const unsigned long long r = (unsigned long long)sg.rows, kq = (unsigned long long)sg.kk,
                                kc = (unsigned long long)K;
       atomicAdd(&P.stats->split_flops, 2ull * r * kq * kc);

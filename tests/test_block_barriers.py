@@ -54,3 +54,12 @@ def test_fp64_tiles_meet_before_their_columns_are_stored():
     assert "for (int k0 = qlo; k0 < qhi; k0 += BK) {" in between
     after_loop = between[between.index("for (int k0 = qlo"):]
     assert re.search(r"if \(qlo >= qhi\) __syncthreads\(\);", after_loop)
+
+
+def test_split_segments_are_kept_and_counted_alike():
+    """The split path's list holds exactly the merge parts whose output tiles its offsets count: a part
+    without a pole (no digit images) has output tiles too, and skipping it would leave its rows unwritten
+    and tiles that belong to no segment."""
+    body = body_after(source("tdc_gemm_split.cu"), "k_split_segs(Plan P, int level")
+    assert re.search(r"cns \+= tt > 0 \? 1 : 0;", body) and re.search(r"if \(tt == 0\) continue;", body)
+    assert not re.search(r"if \(el == 0\) continue", body)

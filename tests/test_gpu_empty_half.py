@@ -21,10 +21,10 @@ def tdc():
 def half_empty(n, side):
     """Diagonal on one half of the top split (eigenvectors are unit vectors, the one at the split has
     weight 1 / sqrt 2 in z), a Toeplitz matrix on the other (weights at most sqrt(1 / n2)), coupled by
-    b: rho / sqrt 2 > tol >= rho sqrt(1 / n2) for rho = 2 |b| = 3 tol, tol = 8 2^-53 max |D|, n2 >= 16."""
+    b: rho / sqrt 2 > tol >= rho sqrt(1 / n2) for rho = 2 |b| = 1.5 tol, tol = 8 2^-52 max |D|, n2 >= 16."""
     n1 = n // 2
     d, e = np.full(n, 2.0), np.ones(n - 1)
-    e[n1 - 1] = 1.5 * 8 * 2.0 ** -53 * 4.0
+    e[n1 - 1] = 0.75 * 8 * 2.0 ** -52 * 4.0
     lo, hi = (0, n1) if side == "bottom" else (n1, n)
     d[lo:hi] = np.linspace(-3.5, 3.5, hi - lo)
     e[lo:hi - 1] = 0.0
@@ -70,3 +70,30 @@ def test_many_problems(tdc):
     for k, (a, b) in enumerate(parts):
         n = int(sizes[k])
         check(a, b, lam[off[k]:off[k + 1]], Q[offq[k]:offq[k + 1]].view(n, n).t())
+
+
+@pytest.mark.parametrize("side", ["top", "bottom"])
+@pytest.mark.parametrize("n", [2000, 4000, 5001])
+def test_empty_half_on_the_split_path(tdc, n, side):
+    """The same with more kept poles than the split path's threshold: the full half's eigenvectors at the
+    split spread over 200 rows (weights up to sqrt(1 / 201)), the empty half's over all of its n / 2 rows
+    (up to sqrt(2 / n)), rho at 0.95 of what would keep the largest of those."""
+    n1 = n // 2
+    d, e = np.full(n, 2.0), np.ones(n - 1)
+    lo, hi, cut = (0, n1, n1 - 200) if side == "bottom" else (n1, n, n1 + 200)
+    if side == "bottom":
+        d[lo:cut] = np.linspace(-3.5, -0.5, cut - lo)
+        e[lo:cut] = 0.0
+    else:
+        d[cut:hi] = np.linspace(-3.5, -0.5, hi - cut)
+        e[cut - 1:hi - 1] = 0.0
+    tol = 8 * 2.0 ** -52 * 4.0
+    n2 = n - n1 if side == "bottom" else n1
+    e[n1 - 1] = 0.5 * 0.95 * tol / np.sqrt(1.0 / (n2 + 1))
+    o = tdc.default_opts(collect_stats=1)
+    ws = torch.full(((tdc.workspace_size(n, o) + 7) // 8,), float("nan"), dtype=torch.float64, device=DEV)
+    lam = torch.full((n,), float("nan"), dtype=torch.float64, device=DEV)
+    Q = torch.full((n, n), float("nan"), dtype=torch.float64, device=DEV).t()
+    tdc.eig(torch.tensor(d, device=DEV), torch.tensor(e, device=DEV), o, ws=ws.view(torch.uint8), lam=lam, Q=Q, check=True)
+    assert 128 <= tdc.get_stats()["sum_K"][0] <= 200
+    check(d, e, lam, Q)
