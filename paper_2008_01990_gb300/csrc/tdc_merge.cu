@@ -2024,7 +2024,7 @@ __device__ __forceinline__ bool fp32_slope(float gp, float dist) {
 // about one.  A step that leaves the expansion's range
 // (q >= 4e-6) starts another pass there.  Returns true when accepted (tau updated); else tau
 // is the last iterate inside the bracket and the caller continues with the safeguarded
-// iteration.  Bound by FP64 issue: 19 FP64 instructions a root, 17 an iterate and 10 a pole
+// iteration.  Bound by FP64 issue: 19 FP64 instructions a root, 19 an iterate and 10 a pole
 // and pass of 32; the earlier form (four FP64 sums, divisions and a square root an iterate)
 // took 24,000 clocks a root of a small merge, this one 5,000.
 __device__ bool secular_certified(const double* D, const double* zz, int K, int j, double irho, int org, double width,
@@ -2116,10 +2116,9 @@ __device__ bool secular_certified(const double* D, const double* zz, int K, int 
         tau = tc + (double)h;
         return true;
       }
-      // any point near the step's end will do for the next iterate: an FP32 offset
-      ef += h;
-      e = (double)ef;
-      tc = tau1 + e;
+      tc += (double)h;
+      e = tc - tau1;
+      ef = (float)e;
       q = fabsf(ef) * rdmin;
       if (!(q < 4e-6f)) break;
     }
@@ -2486,9 +2485,9 @@ __device__ bool secular_certified_thread(const double* D, const double* zz, int 
       tau = tc + (double)h;
       return true;
     }
-    ef += h;
-    e = (double)ef;
-    tc = tau1 + e;
+    tc += (double)h;
+    e = tc - tau1;
+    ef = (float)e;
     q = fabsf(ef) * rdmin;
     if (!(q < 4e-6f)) return false;
   }
